@@ -11,12 +11,14 @@ _SUBMODULES = ("binding", "synth", "build", "dp")
 
 
 def __getattr__(name):
+    # (found names stay in the module: looking one up through here again costs more than a microsecond
+    # of every call of a serving loop)
     if name in _SUBMODULES:
-        return importlib.import_module("." + name, __name__)
+        return globals().setdefault(name, importlib.import_module("." + name, __name__))
     if name.startswith("__"):
         raise AttributeError(name)
     binding = importlib.import_module(".binding", __name__)
     try:
-        return getattr(binding, name)
+        return globals().setdefault(name, getattr(binding, name))
     except AttributeError:
         raise AttributeError(f"module {__name__!r} has no attribute {name!r}") from None

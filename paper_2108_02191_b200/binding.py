@@ -1,9 +1,14 @@
-"""Thin ctypes binding of librobe.so: argument marshalling only.
+"""Thin binding of librobe.so: argument marshalling only.
 
 Every function has the name of the C entry point it calls (see include/robe.h) and does
 no arithmetic of the method itself.  torch is used for device memory and streams.  There
-is no fallback: if the shared library is missing or does not load, importing this module
+is no fallback: if a shared library is missing or does not load, importing this module
 raises.
+
+The calls of a training or serving loop go through `_robe_py` (csrc/robe_py.cpp), which reads the
+tensors in native code: through ctypes alone a call costs about 8 us of Python, more than the
+smallest lookups take on the GPU.  It declines, without calling anything, what is not plainly the
+right kind of argument; the ctypes path below then makes the call or says what is wrong.
 """
 from __future__ import annotations
 
@@ -64,6 +69,7 @@ if not os.path.exists(LIB_PATH):
         "(there is no CPU or PyTorch fallback)")
 
 _lib = C.CDLL(LIB_PATH)
+from . import _robe_py as _native  # noqa: E402  (built beside the library; missing: ImportError)
 
 _vp, _i64, _u64, _u32 = C.c_void_p, C.c_int64, C.c_uint64, C.c_uint32
 _lib.robe_create.argtypes = [C.POINTER(_vp), _u64, _u32, _u32, _u32, _u64]
@@ -92,6 +98,11 @@ _lib.robe_status_string.restype = C.c_char_p
 for _name in EXPORTS:
     if _name not in ("robe_backward_workspace_bytes", "robe_status_string"):
         getattr(_lib, _name).restype = C.c_int
+
+_native.set_calls(*(C.cast(getattr(_lib, _name), _vp).value for _name in (
+    "robe_set_option", "robe_forward", "robe_forward_keep", "robe_backward", "robe_backward_kept",
+    "robe_backward_adam", "robe_backward_adagrad", "robe_apply_sgd")))
+_NOT_TAKEN = 1  # from _native: nothing was called
 
 
 class RobeError(RuntimeError):
@@ -175,6 +186,9 @@ def robe_get_hash_constants(h):
 
 
 def robe_forward(h, indices, offsets, batch: int, out, stream=None) -> None:
+    rc = _native.forward(h, indices, offsets, batch, out, stream)
+    if rc != _NOT_TAKEN:
+        return _check(rc, "robe_forward")
     _state_index_type(h, indices)
     _check(_lib.robe_forward(h, _ids_ptr(indices), _dev_ptr(offsets, torch.int64),
                              batch, indices.numel(), _dev_ptr(out, torch.float32),
@@ -183,6 +197,9 @@ def robe_forward(h, indices, offsets, batch: int, out, stream=None) -> None:
 
 def robe_forward_keep(h, indices, offsets, batch: int, out, workspace, stream=None) -> None:
     """robe_forward that also leaves the block starts in `workspace` for robe_backward_kept."""
+    rc = _native.forward_keep(h, indices, offsets, batch, out, workspace, stream)
+    if rc != _NOT_TAKEN:
+        return _check(rc, "robe_forward_keep")
     _state_index_type(h, indices)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check(_lib.robe_forward_keep(h, _ids_ptr(indices), _dev_ptr(offsets, torch.int64),
@@ -196,6 +213,9 @@ def robe_backward_workspace_bytes(h, batch: int, nnz: int) -> int:
 
 def robe_backward(h, grad_out, indices, offsets, batch: int, grad_array=None, lr: float = 0.0,
                   workspace=None, stream=None) -> None:
+    rc = _native.backward(h, grad_out, indices, offsets, batch, grad_array, lr, workspace, stream)
+    if rc != _NOT_TAKEN:
+        return _check(rc, "robe_backward")
     _state_index_type(h, indices)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check(_lib.robe_backward(h, _dev_ptr(grad_out, torch.float32), _ids_ptr(indices),
@@ -207,6 +227,9 @@ def robe_backward(h, grad_out, indices, offsets, batch: int, grad_array=None, lr
 def robe_backward_kept(h, grad_out, indices, offsets, batch: int, grad_array=None, lr: float = 0.0,
                        workspace=None, stream=None) -> None:
     """robe_backward on the block starts that robe_forward_keep left in `workspace`."""
+    rc = _native.backward_kept(h, grad_out, indices, offsets, batch, grad_array, lr, workspace, stream)
+    if rc != _NOT_TAKEN:
+        return _check(rc, "robe_backward_kept")
     _state_index_type(h, indices)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check(_lib.robe_backward_kept(h, _dev_ptr(grad_out, torch.float32), _ids_ptr(indices),
@@ -229,6 +252,10 @@ def robe_backward_deterministic_static(h, grad_out, indices, offsets, batch: int
 
 def robe_backward_adam(h, grad_out, indices, offsets, batch: int, m1, m2, lr: float, beta1: float,
                        beta2: float, eps: float, step: int, workspace, stream=None) -> None:
+    rc = _native.backward_adam(h, grad_out, indices, offsets, batch, m1, m2, lr, beta1, beta2, eps, step,
+                               workspace, stream)
+    if rc != _NOT_TAKEN:
+        return _check(rc, "robe_backward_adam")
     _state_index_type(h, indices)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check(_lib.robe_backward_adam(
@@ -239,6 +266,9 @@ def robe_backward_adam(h, grad_out, indices, offsets, batch: int, m1, m2, lr: fl
 
 def robe_backward_adagrad(h, grad_out, indices, offsets, batch: int, sum_sq, lr: float, eps: float,
                           workspace, stream=None) -> None:
+    rc = _native.backward_adagrad(h, grad_out, indices, offsets, batch, sum_sq, lr, eps, workspace, stream)
+    if rc != _NOT_TAKEN:
+        return _check(rc, "robe_backward_adagrad")
     _state_index_type(h, indices)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     _check(_lib.robe_backward_adagrad(
@@ -249,6 +279,9 @@ def robe_backward_adagrad(h, grad_out, indices, offsets, batch: int, sum_sq, lr:
 
 def robe_apply_sgd(h, grad_array, lr: float, zero_grad: bool = True, stream=None) -> None:
     """Dense SGD apply of the data-parallel step: array <- fma(-lr, grad_array, array)."""
+    rc = _native.apply_sgd(h, grad_array, lr, zero_grad, stream)
+    if rc != _NOT_TAKEN:
+        return _check(rc, "robe_apply_sgd")
     _check(_lib.robe_apply_sgd(h, _dev_ptr(grad_array, torch.float32), lr, 1 if zero_grad else 0,
                                _stream_ptr(stream)), "robe_apply_sgd")
 

@@ -1,10 +1,12 @@
-"""Builds librobe.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds librobe.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _robe_py.so (the
+binding's native marshalling) with g++ against the installed torch."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
@@ -34,7 +36,27 @@ def build(force: bool = False, verbose: bool = False) -> str:
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB] + sources()
         subprocess.run(cmd, check=True)
+    build_native(force)
     return LIB
+
+
+NATIVE = os.path.join(_HERE, "_robe_py.so")
+
+
+def build_native(force: bool = False) -> str:
+    src = os.path.join(CSRC, "robe_py.cpp")
+    header = os.path.join(_HERE, "..", "include", "robe.h")
+    if force or not os.path.exists(NATIVE) or os.path.getmtime(NATIVE) < max(map(os.path.getmtime, (src, header))):
+        import torch
+        root = os.path.dirname(torch.__file__)
+        cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+        inc = [os.path.join(root, "include"), sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+        subprocess.run(
+            ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *("-isystem" + i for i in inc),
+             "-o", NATIVE, src, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"],
+            check=True)
+    return NATIVE
 
 
 DEBUG_LIB = os.path.join(_HERE, "librobe_debug.so")
