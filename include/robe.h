@@ -64,9 +64,11 @@ typedef enum {
                                returns ROBE_OK.  Read it with robe_last_device_status
                                and zero it yourself before going on.                      */
 #define ROBE_OPT_FWD_KERNEL 4 /* forward kernel; every variant gives the same bits.
-                                 0 automatic (default): the lane-hashed kernel for Z <= 2 on arrays of
-                                   up to 192 MB, the staged kernel for rows of up to 128 elements, else
-                                   the direct kernel
+                                 0 automatic (default).  One-hot: the rows kernel (repeats of an id
+                                   gathered once) for large batches with more than 16 chunks per row,
+                                   else the flat kernel (rows of any length as one run of elements);
+                                   pooled: the lane-hashed kernel for Z <= 2 on arrays of up to 192 MB,
+                                   the staged kernel for rows of up to 128 elements, else the direct one
                                  1 direct: any (Z, d); every lane hashes its element's chunk per id
                                  2 staged: d <= 128; block starts of a batch of ids through shared
                                    memory, 4-byte loads, lanes on consecutive slots of a block
@@ -78,7 +80,9 @@ typedef enum {
                                  A variant asked for a call it cannot take returns
                                  ROBE_ERR_UNSUPPORTED and launches nothing.                          */
 #define ROBE_OPT_BWD_KERNEL 5 /* kernel of the ATOMIC backward (all within the atomic bound):
-                                 0 automatic (default): staged for d <= 128, else direct
+                                 0 automatic (default).  One-hot: the rows kernel (repeats of an id
+                                   summed first) for large batches, else the flat kernel; pooled:
+                                   staged for d <= 128, else direct
                                  1 direct   2 staged (scalar red.global.add.f32, lanes on consecutive slots)
                                  3 vector: red.global.add.v4.f32 on the aligned middle of a block,
                                    scalar head and tail; d, Z, M multiples of 4, d <= 128, sign off

@@ -2,7 +2,7 @@
 // ceil(d/Z) blocks M[h(e,x,c) : h(e,x,c)+Z] read circularly; Section 3.1 for the optional
 // element-wise sign).  Sum pooling over a bag is sequential in fp32 in bag order.
 //
-// Two kernels:
+// Kernels (one-hot rows mostly go to those of robe_flat.cu and robe_rows.cu, see launch_forward):
 //   fwd_direct_kernel  any Z, any d: every lane hashes the chunk of its own element.
 //   fwd_staged_kernel  d <= 128: a warp first evaluates the block starts of a whole batch of
 //                      ids (one (id, chunk) pair per lane) into a warp-private staging area in
@@ -379,10 +379,14 @@ static void launch_vec(const FwdArgs& a, bool bags, cudaStream_t st) {
 // for (MINB, see kStagedCtas*).  Measured on B200: the time of the HBM-resident gather does not move
 // between 4 and 16 ids in flight - the random 64-byte requests themselves are the limit.
 
+// One-hot rows of 128 from a bf16 array are the exception (131072 x 26 rows on 50 MB, us): 6 CTAs and 2 ids
+// 498, 5 and 4 484, 4 and 8 477, 3 and 8 505, 8 and 2 566.
+
 template <int EPL, int DT, bool SIGN, bool FULLD, int MINB>
 static void launch_staged_minb(const FwdArgs& a, bool bags, cudaStream_t st) {
     constexpr int UB = (EPL == 4) ? 2 : 4;
-    constexpr int UO = (EPL == 4) ? 2 : 4;
+    constexpr int UO = (EPL == 4) ? (DT == 1 && !SIGN ? 8 : 2) : 4;
+    constexpr int MINO = (EPL == 4 && DT == 1 && !SIGN) ? 4 : MINB;
     const uint32_t ipb = staged_ids_per_batch(a.mp, bags, SIGN);
     const uint32_t cmagic = chunk_magic(a.mp);
     const int64_t warps = bags ? a.nbags : (a.nbags + ipb - 1) / ipb;
@@ -390,7 +394,7 @@ static void launch_staged_minb(const FwdArgs& a, bool bags, cudaStream_t st) {
     if (bags)
         fwd_staged_kernel<EPL, DT, SIGN, true, FULLD, MINB, UB><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
     else
-        fwd_staged_kernel<EPL, DT, SIGN, false, FULLD, MINB, UO><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
+        fwd_staged_kernel<EPL, DT, SIGN, false, FULLD, MINO, UO><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
 }
 
 template <int EPL, int DT, bool SIGN, bool FULLD>
@@ -559,17 +563,32 @@ cudaError_t launch_forward(const Problem& pb, float* out, int variant, cudaStrea
         launch_vec(a, bags, st);
         return cudaGetLastError();
     }
-    // Short blocks: every lane hashes its own chunks (keeps nothing for a sort-based backward).
-    // Automatic for arrays of L2 size, where the staged kernel is bound by its instruction count
-    // (measured on B200, Z = 1 / 2: 1 MB array 2.27 -> 1.72 ms / 1.72 -> 1.00 ms, 100 MB 3.59 -> 3.40 /
-    // 2.14 -> 2.09); on a 10 GB array the staged kernel's higher occupancy keeps more DRAM requests
-    // in flight and stays ahead (9.5 vs 10.2 ms), so it keeps those.
+    // Pooled short blocks: every lane hashes its own chunks (keeps nothing for a sort-based backward).
+    // Automatic for arrays of L2 size, where the staged kernel is bound by its instruction count; on a
+    // 10 GB array the staged kernel's higher occupancy keeps more DRAM requests in flight.
     const bool l2_sized = (uint64_t)pb.mp.m * (pb.dtype == 0 ? 4u : 2u) <= kL2SizedBytes;
-    if (variant == 4 || (variant == 0 && pb.mp.Z <= 2 && l2_sized && lanehash_ok(pb) && keep_keys == nullptr)) {
+    if (variant == 4 ||
+        (variant == 0 && bags && pb.mp.Z <= 2 && l2_sized && lanehash_ok(pb) && keep_keys == nullptr)) {
         if (!lanehash_ok(pb)) return cudaErrorInvalidValue;
         if (pb.dtype == 0) launch_lanehash<0>(a, bags, st);
         else launch_lanehash<1>(a, bags, st);
         return cudaGetLastError();
+    }
+    if (variant == 0 && keep_keys == nullptr && !bags) {  // (the kernels of these two keep no block starts)
+        // Many short blocks per row: gathering a repeated id once saves more than finding the repeats
+        // costs (B200, 26 x 32768 rows of 128 on 100 MB, Zipf ids, us: Z = 1 / 2 / 4 507 -> 370,
+        // 302 -> 240, 253 -> 185; ids that never repeat 880 -> 900, 525 -> 505 .. 550).  From Z = 8 on
+        // the flat kernel is ahead (150 against 156, but 266 against 240 where nothing repeats), and a
+        // few thousand rows hold too few repeats.
+        if (pb.mp.C > 16 && pb.nbags >= 32768 && rows_ok(pb)) return launch_forward_rows(pb, out, st);
+        // Otherwise the flat kernel, except where the staged one measured ahead of it: bf16 arrays with
+        // rows of 64 or 128 (477 against 505 us, 131072 x 26 rows, Z = 32) and rows that fill three
+        // quarters of the staged kernel's lanes with a short last block (d = 100, Z = 32: 74 against 78).
+        const uint32_t lanes = pb.mp.d <= 32 ? 32u : (pb.mp.d <= 64 ? 64u : 128u);
+        const bool ragged = pb.mp.d % pb.mp.Z != 0;
+        const bool staged = warp_ok && pb.nbags >= 32768 &&
+                            ((pb.dtype != 0 && pb.mp.d % 64 == 0) || (ragged && 4 * pb.mp.d >= 3 * lanes));
+        if (!staged && flat_ok(pb)) return launch_forward_flat(pb, out, st);
     }
     const bool use_warp = variant == 2 || (variant == 0 && warp_ok);
     if (use_warp) {

@@ -33,6 +33,18 @@ cudaError_t launch_forward(const Problem& pb, float* out, int variant, cudaStrea
                            uint32_t* keep_keys = nullptr, uint32_t* keep_vals = nullptr,
                            bool* kept = nullptr);
 
+// one-hot rows of any length as one run of elements (robe_flat.cu)
+bool flat_ok(const Problem& pb);
+cudaError_t launch_forward_flat(const Problem& pb, float* out, cudaStream_t st);
+cudaError_t launch_backward_flat(const Problem& pb, const float* grad_out, float* target, float scale,
+                                 cudaStream_t st);
+
+// one-hot rows with the repeats of an id served together (robe_rows.cu)
+bool rows_ok(const Problem& pb);
+cudaError_t launch_forward_rows(const Problem& pb, float* out, cudaStream_t st);
+cudaError_t launch_backward_rows(const Problem& pb, const float* grad_out, float* target, float scale,
+                                 cudaStream_t st);
+
 // atomic backward: adds scale * g * grad_out into target (fp32 [M])
 cudaError_t launch_backward_atomic(const Problem& pb, const float* grad_out, float* target,
                                    float scale, int variant, cudaStream_t st);

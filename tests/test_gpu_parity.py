@@ -332,6 +332,27 @@ def test_backward_merged_rows_kernel(d, Z, M, table_major):
             c.backward(g_d, "atomic", kernel=5)
 
 
+# Batches large enough for the kernels that serve the repeats of an id together (131072 rows and more):
+# block starts listed per row or hashed per lane, one / two / four elements per lane, short last blocks,
+# arrays that wrap all the time, tables of few ids beside tables whose ids hardly repeat, a last CTA and a
+# last warp that are not full; and rows beyond 128 elements in one run.
+@pytest.mark.parametrize("table_major", [False, True])
+@pytest.mark.parametrize("d,Z,M", [(16, 16, 5003), (16, 1, 5003), (33, 1, 64), (64, 4, 100_003), (128, 8, 4099),
+                                   (128, 128, 129), (100, 5, 262_144), (128, 1, 100_003), (256, 64, 70_001),
+                                   (130, 48, 5003), (300, 2, 5003)])
+def test_large_one_hot_batches(d, Z, M, table_major):
+    batch = 131072 // 3 + 5 if d <= 128 else 1001
+    w = small(d=d, Z=Z, M=M, batch=batch, vocab_arg=(3, 1000, 40_000_000), id_dist="uniform")
+    with Case(w, table_major=table_major) as c:
+        assert_bits_equal(c.forward().cpu().numpy().reshape(-1), c.oracle_forward().reshape(-1), "forward")
+        shape = (c.T, c.B, d) if table_major else (c.B, c.T, d)
+        g_h = np.random.default_rng(3).integers(-2, 3, size=shape).astype(np.float32)
+        delta64, _ = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+        # small integers: exact in any order and grouping (sums stay below 2^24)
+        assert_bits_equal(c.backward(torch.from_numpy(g_h).to(c.dev), "atomic").cpu().numpy(),
+                          delta64.astype(np.float32), "backward, integer gradient")
+
+
 @pytest.mark.parametrize("mode", ["atomic", "det"])
 def test_cfg1_backward_dense_and_sgd(mode):
     for sign in (False, True):
