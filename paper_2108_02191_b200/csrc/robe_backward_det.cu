@@ -23,12 +23,14 @@ namespace robe {
 
 namespace {
 
-constexpr int kSortThreads = 256;
+constexpr int kSortThreads = 512;                       // of the count and scatter kernels
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 16;                          // keys per thread per tile
+constexpr int kSortItems = 8;                           // keys per thread per tile
 constexpr int kSortTile = kSortThreads * kSortItems;    // 4096
 constexpr int kRadix = 256;
-constexpr int kSortMaxGrid = 148 * 4;
+constexpr int kSortCtas = 2;                            // per SM (3, with 40 registers: spills, 6 % slower)
+constexpr int kSortMaxGrid = 148 * kSortCtas;
+constexpr int kScanThreads = 256;
 
 inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -125,7 +127,7 @@ __global__ void __launch_bounds__(kSortThreads)
 sort_count_kernel(const uint32_t* keys, uint32_t* counts, uint64_t nb, uint64_t tiles,
                   uint32_t shift, uint32_t mask) {
     __shared__ uint32_t hist[kSortWarps][kRadix];
-    for (int k = 0; k < kSortWarps; ++k) hist[k][threadIdx.x] = 0;
+    for (int k = threadIdx.x; k < kSortWarps * kRadix; k += kSortThreads) (&hist[0][0])[k] = 0;
     __syncthreads();
     uint64_t first, count;
     cta_tiles(tiles, gridDim.x, blockIdx.x, first, count);
@@ -136,14 +138,16 @@ sort_count_kernel(const uint32_t* keys, uint32_t* counts, uint64_t nb, uint64_t 
     for (uint64_t i = begin + threadIdx.x; i < end; i += kSortThreads)
         atomicAdd(&mine[(keys[i] >> shift) & mask], 1u);
     __syncthreads();
+    if (threadIdx.x >= kRadix) return;
     uint32_t total = 0;
     for (int k = 0; k < kSortWarps; ++k) total += hist[k][threadIdx.x];
     counts[(uint64_t)threadIdx.x * gridDim.x + blockIdx.x] = total;
 }
 
-// Exclusive scan of the 256 values held one per thread (value v of thread t): returns the sum
-// of the values of threads below t.  All 256 threads of the CTA call it; contains __syncthreads.
-__device__ __forceinline__ uint32_t cta_exclusive_scan_256(uint32_t v, uint32_t* warp_sums) {
+// Exclusive scan of the values held one per thread (value v of thread t): returns the sum of the values
+// of threads below t.  All threads of the CTA call it; warp_sums holds a word per warp; contains
+// __syncthreads.
+__device__ __forceinline__ uint32_t cta_exclusive_scan(uint32_t v, uint32_t* warp_sums) {
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t inc = v;
 #pragma unroll
@@ -161,19 +165,19 @@ __device__ __forceinline__ uint32_t cta_exclusive_scan_256(uint32_t v, uint32_t*
 
 // ---- kernel 2: one CTA per digit: exclusive scan of that digit's per-CTA counts, in place, and
 // the digit's total into totals[digit]
-__global__ void __launch_bounds__(kSortThreads)
+__global__ void __launch_bounds__(kScanThreads)
 sort_scan_kernel(uint32_t* counts, uint32_t* totals, uint32_t grid) {
-    __shared__ uint32_t warp_sums[kSortWarps];
+    __shared__ uint32_t warp_sums[kScanThreads / 32];
     uint32_t* row = counts + (uint64_t)blockIdx.x * grid;
     uint32_t carry = 0;
-    for (uint32_t b0 = 0; b0 < grid; b0 += kSortThreads) {
+    for (uint32_t b0 = 0; b0 < grid; b0 += kScanThreads) {
         const uint32_t b = b0 + threadIdx.x;
         const uint32_t v = b < grid ? row[b] : 0u;
-        const uint32_t ex = cta_exclusive_scan_256(v, warp_sums);
+        const uint32_t ex = cta_exclusive_scan(v, warp_sums);
         if (b < grid) row[b] = carry + ex;
         // total of this chunk = exclusive prefix of the last thread + its value
         __shared__ uint32_t chunk_total;
-        if (threadIdx.x == kSortThreads - 1) chunk_total = ex + v;
+        if (threadIdx.x == kScanThreads - 1) chunk_total = ex + v;
         __syncthreads();
         carry += chunk_total;
         __syncthreads();
@@ -182,110 +186,190 @@ sort_scan_kernel(uint32_t* counts, uint32_t* totals, uint32_t grid) {
 }
 
 // ---- kernel 3: ranked scatter (STABLE: keeps the input order inside a digit - the LSD sort needs
-// that; the binned backward does not and takes ranks from shared-memory counters).  Per tile of 4096 pairs: every warp ranks its 512 pairs
-// by digit (16 rounds of ballots, earlier rounds and lower lanes first), the ranks are
-// extended over the warps, the pairs are laid out in shared memory in (digit, original order),
-// and then written out so that each digit's pairs go to consecutive addresses.
-template <bool STABLE>
-__global__ void __launch_bounds__(kSortThreads, 4)
-sort_scatter_kernel(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                    uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
-                    const uint32_t* __restrict__ cta_offsets, const uint32_t* __restrict__ totals,
-                    uint64_t nb, uint64_t tiles, uint32_t shift, uint32_t mask) {
-    __shared__ uint32_t skey[kSortTile];
-    __shared__ uint32_t sval[kSortTile];
-    __shared__ uint32_t wcnt[kSortWarps][kRadix];
-    __shared__ uint32_t base[kRadix];    // where the next pair of this digit goes, minus dstart
-    __shared__ uint32_t dstart[kRadix];  // start of the digit's run inside the tile
-    __shared__ uint32_t warp_sums[kSortWarps];
-    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
-    {
-        // start of this digit in the output = pairs of lower digits + this digit's pairs in
-        // lower CTAs
-        const uint32_t below = cta_exclusive_scan_256(totals[threadIdx.x], warp_sums);
-        base[threadIdx.x] = below + cta_offsets[(uint64_t)threadIdx.x * gridDim.x + blockIdx.x];
-    }
-    uint64_t first, count;
-    cta_tiles(tiles, gridDim.x, blockIdx.x, first, count);
-    for (uint64_t t = first; t < first + count; ++t) {
-        for (int k = 0; k < kSortWarps; ++k) wcnt[k][threadIdx.x] = 0;
-        __syncthreads();
-        const uint64_t tbegin = t * kSortTile;
-        const uint64_t wbegin = tbegin + (uint64_t)w * (32 * kSortItems);
-        uint32_t key[kSortItems], rank[kSortItems];
+// that; the binned backward does not and takes ranks from shared-memory counters).  Per tile of 4096
+// pairs: every warp ranks its 256 pairs by digit (8 rounds of ballots, earlier rounds and lower lanes
+// first), the ranks are extended over the warps, the pairs are laid out in shared memory in (digit,
+// original order), and then written out so that each digit's pairs go to consecutive addresses.
+//
+// Bound by the latency of a tile's phases, ranking most of all (34 M pairs, 7-bit digits: a plain copy
+// through the same phases takes 94 us, ranking without the final stores 158, all of it 192).  So: one
+// ballot per digit bit that the pass has (BITS), no bounds checks in full tiles, 32-bit positions, and the
+// next tile's pairs asked for before this one is written out.  Measured (B200, same pairs, us per pass,
+// before -> here): 247 -> 192; unstable with 6-bit digits 142 -> 130.  Finding the lanes of a digit by an
+// atomicOr into a shared word instead of ballots takes as long.
+template <bool STABLE, int BITS>
+struct ScatterSmem {
+    uint2 pair[kSortTile];
+    // STABLE: per warp, pairs of each digit, then where they start in the tile
+    uint16_t warp_digit[STABLE ? kSortWarps : 1][1 << BITS];
+    uint32_t counter[1 << BITS];  // not STABLE: the same for the whole tile
+    uint32_t base[1 << BITS];     // where the next pair of this digit goes, minus its place in the tile
+    uint32_t warp_sums[kSortWarps];
+};
+
+// The pairs of the tile that starts at tbegin, warp-striped.  (nb may be close to 2^32: positions are
+// compared relative to the tile, so that nothing overflows.)
+__device__ __forceinline__ void scatter_load(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+                                             uint32_t tbegin, uint32_t nb, uint32_t (&key)[kSortItems],
+                                             uint32_t (&val)[kSortItems]) {
+    const uint32_t left = nb - tbegin, local = (threadIdx.x >> 5) * (32 * kSortItems) + (threadIdx.x & 31);
+    kin += tbegin;
+    vin += tbegin;
+    if (left >= (uint32_t)kSortTile) {
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) key[r] = __ldcs(kin + (local + r * 32));
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) val[r] = __ldcs(vin + (local + r * 32));
+    } else {
 #pragma unroll
         for (int r = 0; r < kSortItems; ++r) {
-            const uint64_t idx = wbegin + r * 32 + lane;
-            key[r] = idx < nb ? kin[idx] : 0u;
+            key[r] = local + r * 32 < left ? __ldcs(kin + (local + r * 32)) : 0u;
+            val[r] = local + r * 32 < left ? __ldcs(vin + (local + r * 32)) : 0u;
         }
-        if (!STABLE) {
-            // any order inside a digit will do: the rank is what a shared-memory counter hands out
+    }
+}
+
+template <bool STABLE, int BITS, bool FULL>
+__device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, const uint32_t* __restrict__ kin,
+                                             const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
+                                             uint32_t* __restrict__ vout, uint32_t nb, uint32_t tbegin,
+                                             uint32_t shift, uint32_t (&key)[kSortItems],
+                                             uint32_t (&val)[kSortItems], bool more) {
+    constexpr uint32_t R = 1u << BITS, mask = R - 1u;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t left = nb - tbegin, local = w * (32 * kSortItems) + lane;  // (see scatter_load)
+    if (STABLE) {
+        for (uint32_t k = tid; k < kSortWarps * R / 2; k += kSortThreads)
+            reinterpret_cast<uint32_t*>(&sm.warp_digit[0][0])[k] = 0;
+    } else if (tid < R) {
+        sm.counter[tid] = 0;
+    }
+    __syncthreads();
+    uint32_t rank[kSortItems];
 #pragma unroll
-            for (int r = 0; r < kSortItems; ++r) {
-                rank[r] = 0;
-                if (wbegin + r * 32 + lane < nb) rank[r] = atomicAdd(&wcnt[w][(key[r] >> shift) & mask], 1u);
-            }
-        }
-#pragma unroll
-        for (int r = 0; STABLE && r < kSortItems; ++r) {
-            const bool valid = wbegin + r * 32 + lane < nb;
-            const uint32_t dg = valid ? ((key[r] >> shift) & mask) : 0u;
+    for (int r = 0; r < kSortItems; ++r) {
+        const bool valid = FULL || local + r * 32 < left;
+        const uint32_t dg = (key[r] >> shift) & mask;
+        rank[r] = 0;
+        if (!STABLE) {  // any order inside a digit will do: the rank is what a shared-memory counter hands out
+            if (valid) rank[r] = atomicAdd(&sm.counter[dg], 1u);
+        } else {
             // lanes holding the same digit: one ballot per digit bit (a fixed cost, where
             // __match_any_sync takes time in proportion to the number of distinct digits)
-            uint32_t peers = __ballot_sync(0xFFFFFFFFu, valid);
+            uint32_t peers = FULL ? 0xFFFFFFFFu : __ballot_sync(0xFFFFFFFFu, valid);
 #pragma unroll
-            for (int b = 0; b < 8; ++b) {
+            for (int b = 0; b < BITS; ++b) {
                 const bool bit = (dg >> b) & 1u;
                 const uint32_t bal = __ballot_sync(0xFFFFFFFFu, bit);
                 peers &= bit ? bal : ~bal;
             }
-            uint32_t before = 0;
-            if (valid) before = wcnt[w][dg];
+            const uint32_t before = sm.warp_digit[w][dg];
             __syncwarp();
-            if (valid && (peers & lt) == 0) wcnt[w][dg] = before + __popc(peers);
+            if (valid && (peers & lt) == 0) sm.warp_digit[w][dg] = (uint16_t)(before + __popc(peers));
             __syncwarp();
             rank[r] = before + __popc(peers & lt);
         }
-        __syncthreads();
-        // per digit: exclusive prefix over the warps of this tile, and the tile's total
-        uint32_t tile_total = 0;
-        for (int k = 0; k < kSortWarps; ++k) {
-            const uint32_t c = wcnt[k][threadIdx.x];
-            wcnt[k][threadIdx.x] = tile_total;
-            tile_total += c;
-        }
-        const uint32_t ds = cta_exclusive_scan_256(tile_total, warp_sums);  // syncs inside
-        dstart[threadIdx.x] = ds;
-        // from here base[] holds (output position of the digit's next pair) - (its position in
-        // the tile), so that a pair at tile position lp goes to base[digit] + lp
-        base[threadIdx.x] -= ds;
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
-            const uint64_t idx = wbegin + r * 32 + lane;
-            if (idx < nb) {
-                const uint32_t dg = (key[r] >> shift) & mask;
-                const uint32_t lp = dstart[dg] + wcnt[w][dg] + rank[r];
-                if (!ROBE_CHK(lp < (uint32_t)kSortTile, ROBE_DBG_SHARED)) continue;
-                skey[lp] = key[r];
-                sval[lp] = vin[idx];  // payloads are only passed through: read them this late
-            }
-        }
-        __syncthreads();
-        const uint32_t in_tile = (uint32_t)(nb - tbegin < (uint64_t)kSortTile ? nb - tbegin
-                                                                               : (uint64_t)kSortTile);
-        for (uint32_t lp = threadIdx.x; lp < in_tile; lp += kSortThreads) {
-            const uint32_t k = skey[lp];
-            const uint32_t dst = base[(k >> shift) & mask] + lp;
-            if (!ROBE_CHK((uint64_t)dst < nb, ROBE_DBG_SORT_POS)) continue;
-            kout[dst] = k;
-            vout[dst] = sval[lp];
-        }
-        __syncthreads();
-        base[threadIdx.x] += ds + tile_total;  // undo the shift, advance past this tile's pairs
-        // (the next tile's first barrier orders this update before its readers)
     }
+    __syncthreads();
+    // per digit: start of each warp's pairs inside the tile, and the tile's total
+    uint32_t tile_total = 0;
+    if (tid < R) {
+        if (STABLE) {
+#pragma unroll
+            for (int k = 0; k < kSortWarps; ++k) tile_total += sm.warp_digit[k][tid];
+        } else {
+            tile_total = sm.counter[tid];
+        }
+    }
+    const uint32_t ds = cta_exclusive_scan(tile_total, sm.warp_sums);  // syncs inside
+    if (tid < R) {
+        if (STABLE) {
+            uint32_t from = ds;
+#pragma unroll
+            for (int k = 0; k < kSortWarps; ++k) {
+                const uint32_t n = sm.warp_digit[k][tid];
+                sm.warp_digit[k][tid] = (uint16_t)from;
+                from += n;
+            }
+        } else {
+            sm.counter[tid] = ds;
+        }
+        sm.base[tid] -= ds;  // a pair at tile position lp goes to base[digit] + lp
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        if (FULL || local + r * 32 < left) {
+            const uint32_t dg = (key[r] >> shift) & mask;
+            const uint32_t lp = (STABLE ? sm.warp_digit[w][dg] : sm.counter[dg]) + rank[r];
+            if (!ROBE_CHK(lp < (uint32_t)kSortTile, ROBE_DBG_SHARED)) continue;
+            sm.pair[lp] = make_uint2(key[r], val[r]);
+        }
+    }
+    __syncthreads();
+    if (more) scatter_load(kin, vin, tbegin + kSortTile, nb, key, val);
+    const uint32_t in_tile = FULL ? kSortTile : left;
+#pragma unroll 4
+    for (uint32_t lp = tid; lp < in_tile; lp += kSortThreads) {
+        const uint2 p = sm.pair[lp];
+        const uint32_t dst = sm.base[(p.x >> shift) & mask] + lp;
+        if (!ROBE_CHK(dst < nb, ROBE_DBG_SORT_POS)) continue;
+        kout[dst] = p.x;
+        vout[dst] = p.y;
+    }
+    __syncthreads();
+    if (tid < R) sm.base[tid] += ds + tile_total;  // undo the shift, advance past this tile's pairs
+    // (the next tile's first barrier orders this update before its readers)
+}
+
+template <bool STABLE, int BITS>
+__global__ void __launch_bounds__(kSortThreads, kSortCtas)
+sort_scatter_kernel(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+                    uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
+                    const uint32_t* __restrict__ cta_offsets, const uint32_t* __restrict__ totals,
+                    uint32_t nb, uint32_t tiles, uint32_t shift) {
+    __shared__ ScatterSmem<STABLE, BITS> sm;
+    const uint32_t tid = threadIdx.x;
+    {
+        // start of this digit in the output = pairs of lower digits + this digit's pairs in
+        // lower CTAs
+        const bool on = tid < (1u << BITS);
+        const uint32_t below = cta_exclusive_scan(on ? totals[tid] : 0u, sm.warp_sums);
+        if (on) sm.base[tid] = below + cta_offsets[(uint64_t)tid * gridDim.x + blockIdx.x];
+    }
+    uint64_t first, count;
+    cta_tiles(tiles, gridDim.x, blockIdx.x, first, count);
+    if (count == 0) return;
+    uint32_t key[kSortItems], val[kSortItems];
+    scatter_load(kin, vin, (uint32_t)first * kSortTile, nb, key, val);
+    for (uint32_t t = (uint32_t)first; t < (uint32_t)(first + count); ++t) {
+        const uint32_t tbegin = t * kSortTile;
+        const bool more = t + 1 < (uint32_t)(first + count);
+        if (nb - tbegin >= (uint32_t)kSortTile)
+            scatter_tile<STABLE, BITS, true>(sm, kin, vin, kout, vout, nb, tbegin, shift, key, val, more);
+        else
+            scatter_tile<STABLE, BITS, false>(sm, kin, vin, kout, vout, nb, tbegin, shift, key, val, more);
+    }
+}
+
+// One pass: count, scan, scatter by `width` bits at `shift`.  A pass may sort by a few bits more than asked
+// (those of the next pass, which sorts by them again): three builds serve all widths.
+template <bool STABLE, int BITS>
+void launch_sort_pass_bits(const SortPlan& sp, const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
+                           uint32_t* counts, uint32_t* totals, uint32_t shift, cudaStream_t st) {
+    sort_count_kernel<<<sp.grid, kSortThreads, 0, st>>>(kin, counts, sp.nb, sp.tiles, shift, (1u << BITS) - 1u);
+    sort_scan_kernel<<<1 << BITS, kScanThreads, 0, st>>>(counts, totals, sp.grid);
+    sort_scatter_kernel<STABLE, BITS><<<sp.grid, kSortThreads, 0, st>>>(kin, vin, kout, vout, counts, totals,
+                                                                       (uint32_t)sp.nb, (uint32_t)sp.tiles, shift);
+}
+
+template <bool STABLE>
+void launch_sort_pass(const SortPlan& sp, const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
+                      uint32_t* counts, uint32_t* totals, uint32_t shift, uint32_t width, cudaStream_t st) {
+    if (width <= 6) launch_sort_pass_bits<STABLE, 6>(sp, kin, vin, kout, vout, counts, totals, shift, st);
+    else if (width == 7) launch_sort_pass_bits<STABLE, 7>(sp, kin, vin, kout, vout, counts, totals, shift, st);
+    else launch_sort_pass_bits<STABLE, 8>(sp, kin, vin, kout, vout, counts, totals, shift, st);
 }
 
 // A round of the apply kernel whose walks got long, handed over to the long-walk kernel: where
@@ -1274,11 +1358,7 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
         // be updated in L2, large enough that the scatter writes long runs) unless that would
         // need more than 256 bins or the array is smaller than one such span.
         const uint32_t shift = bits > 30 ? bits - 8 : (bits > 22 ? 22 : (bits > 8 ? bits - 8 : 0));
-        const uint32_t mask = (1u << (bits - shift)) - 1u;
-        sort_count_kernel<<<sp.grid, kSortThreads, 0, st>>>(kA, counts, nb, sp.tiles, shift, mask);
-        sort_scan_kernel<<<kRadix, kSortThreads, 0, st>>>(counts, totals, sp.grid);
-        sort_scatter_kernel<false><<<sp.grid, kSortThreads, 0, st>>>(kA, vA, kB, vB, counts, totals, nb,
-                                                                    sp.tiles, shift, mask);
+        launch_sort_pass<false>(sp, kA, vA, kB, vB, counts, totals, shift, bits - shift, st);
         ApplyArgs ab{mp, grad_out, pb.indices, target, lr, nb, pb.status, AdamState{}, nullptr, nullptr, 0,
                      nullptr, nullptr, 0, (uint64_t)pb.nbags * mp.d, pb.l2_keep};
         uint32_t log2Zp = 0;
@@ -1300,11 +1380,7 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
     for (uint32_t pass = 0; pass < npass; ++pass) {
         const uint32_t shift = pass * bpp;
         const uint32_t width = bits - shift < bpp ? bits - shift : bpp;
-        const uint32_t mask = (1u << width) - 1u;
-        sort_count_kernel<<<sp.grid, kSortThreads, 0, st>>>(kA, counts, nb, sp.tiles, shift, mask);
-        sort_scan_kernel<<<kRadix, kSortThreads, 0, st>>>(counts, totals, sp.grid);
-        sort_scatter_kernel<true><<<sp.grid, kSortThreads, 0, st>>>(kA, vA, kB, vB, counts, totals, nb,
-                                                                   sp.tiles, shift, mask);
+        launch_sort_pass<true>(sp, kA, vA, kB, vB, counts, totals, shift, width, st);
         uint32_t* t = kA; kA = kB; kB = t;
         t = vA; vA = vB; vB = t;
     }
