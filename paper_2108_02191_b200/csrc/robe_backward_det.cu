@@ -16,8 +16,11 @@
 //                      by a small second kernel (those terms come last: their keys are the largest).
 //                      Walks over hundreds of blocks (an id repeated many times in the batch)
 //                      are finished by a third kernel that keeps a whole step of terms in flight.
+//                      Arrays that the call touches densely are served slot by slot instead
+//                      (robe_strips.cu), in the same order.
 // No atomics on floating-point data and no waits between CTAs: the result is bit-reproducible.
 #include "robe_internal.h"
+#include "robe_update.cuh"
 
 namespace robe {
 
@@ -396,11 +399,6 @@ struct ApplyArgs {
     uint32_t* long_count;    // number of handed-over rounds (may run past long_cap)
     LongWalk* long_walks;
     uint32_t long_cap;
-    // window apply (densely touched arrays): per array window of 2^win_log2 slots, did the window kernel
-    // leave it to the position-tile kernel?  nullptr = there is no window kernel in this call
-    const uint8_t* win_left;
-    const uint32_t* any_left;  // number of windows left over (0: the tile kernel has nothing to do)
-    uint32_t win_log2;         // log2 of the window length
     uint64_t grad_elems;       // elements of grad_out (read by the debug build's index checks only)
     int l2_keep;               // binned adds: the reductions carry the L2 "keep" policy
 };
@@ -433,36 +431,6 @@ __device__ __forceinline__ bool block_term(const ApplyArgs& a, const uint32_t* b
     return true;
 }
 
-// What a served slot does with its sum delta (MODE): 0 - add it to a dense gradient; 1 - the
-// SGD step M[j] = fma(-lr, delta, M[j]); 3 - the Adagrad step; 2 - the Adam step (Kingma & Ba, Algorithm 1; the paper
-// trains five of its six models with Adam, Section 5) on the slot and its two moment slots, every
-// operation a separate correctly rounded fp32 one.  `old` is target[j].
-template <int MODE>
-__device__ __forceinline__ void commit_slot(const ApplyArgs& a, uint32_t j, float delta, float old) {
-    if (!ROBE_CHK(j < a.mp.m, ROBE_DBG_ARRAY_SLOT)) return;
-    if (MODE == 0) {
-        a.target[j] = __fadd_rn(old, delta);
-    } else if (MODE == 1) {
-        a.target[j] = __fmaf_rn(-a.lr, delta, old);
-    } else if (MODE == 3) {
-        // Adagrad (Duchi, Hazan, Singer): one accumulator of squared gradients per slot
-        const AdamState& ad = a.adam;  // m2 = the accumulators, eps
-        const float s = __fadd_rn(ad.m2[j], __fmul_rn(delta, delta));
-        ad.m2[j] = s;
-        const float den = __fadd_rn(__fsqrt_rn(s), ad.eps);
-        a.target[j] = __fsub_rn(old, __fmul_rn(a.lr, __fdiv_rn(delta, den)));
-    } else {
-        const AdamState& ad = a.adam;
-        const float m = __fadd_rn(__fmul_rn(ad.beta1, ad.m1[j]), __fmul_rn(__fsub_rn(1.0f, ad.beta1), delta));
-        const float v = __fadd_rn(__fmul_rn(ad.beta2, ad.m2[j]),
-                                  __fmul_rn(__fsub_rn(1.0f, ad.beta2), __fmul_rn(delta, delta)));
-        ad.m1[j] = m;
-        ad.m2[j] = v;
-        const float den = __fadd_rn(__fsqrt_rn(__fdiv_rn(v, ad.bias2)), ad.eps);
-        a.target[j] = __fsub_rn(old, __fmul_rn(a.lr, __fdiv_rn(__fdiv_rn(m, ad.bias1), den)));
-    }
-}
-
 // Slots j in [Z-1, m).  The sorted blocks that reach slot j are those with key in [j-Z+1, j];
 // the slot is served from the FIRST of them: position i serves slot K[i]+u iff i starts a run of
 // equal keys and the previous key is below K[i]+u-Z+1, i.e. u >= Z - min(Z, K[i]-K[i-1]).  The
@@ -480,12 +448,6 @@ __device__ __forceinline__ void commit_slot(const ApplyArgs& a, uint32_t j, floa
 // rounds is full does it go on here, 16 positions per step, with the gradient rows of the
 // positions after those asked into L2 ahead of time.
 constexpr uint32_t kRing = 128;
-// window apply: the array is cut into windows of 2^8 .. 2^11 slots, one CTA each
-constexpr uint32_t kWinLog2Min = 9, kWinLog2Max = 11;
-constexpr uint32_t kWinThreads = 512;     // threads of the window kernel (<= the shortest window)
-constexpr uint32_t kWinMaxZ = 128;        // longest block the window kernel takes
-constexpr uint32_t kWinEnt = 512;         // sorted blocks per chunk, at most
-constexpr uint32_t kWinStage = 6144;      // gradient elements per chunk, at most (>= kWinMaxZ)
 constexpr uint32_t kNoKey = 0xFFFFFFFFu;  // above every slot number (m + d <= 2^32)
 
 struct ApplyTile {
@@ -631,7 +593,6 @@ det_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __
                                               // measured slower on Zipf ids, 32 no faster)
     __shared__ uint2 ring_s[8][kRing];
     if (a.status != nullptr && *a.status != 0) return;
-    if (a.any_left != nullptr && *a.any_left == 0) return;  // the window kernel served every slot
     const MapParams& mp = a.mp;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     ApplyTile tl;
@@ -688,7 +649,6 @@ det_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __
         const uint64_t j64 = (uint64_t)s + u;
         // j64 >= m: wrapped part, j64 < Z-1: low slots - both belong to the other kernel
         bool active = idx < total && u >= lo_e && u < mp.Z && j64 < mp.m && j64 + 1 >= mp.Z;
-        if (active && a.win_left != nullptr) active = a.win_left[j64 >> a.win_log2] != 0;
         if (__ballot_sync(0xFFFFFFFFu, active) == 0) continue;
         const uint32_t j = (uint32_t)j64;
         float old = 0.0f;
@@ -740,172 +700,6 @@ det_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __
         }
         if (wk.touched) commit_slot<MODE>(a, j, wk.acc, old);
     }
-}
-
-// ---- window apply: the slot-major way, for arrays that a call touches densely (plain blocks
-// of full length).  The array is cut into windows of W = 2^win_log2 slots.
-//
-// lo_of[b] = first sorted position whose block reaches slot b*W or a later one (key + Z-1 >= b*W),
-// hi_of[b] = first sorted position whose key is >= b*W; both for b = 0 .. number of windows.
-constexpr int kBoundsPer = 8;  // sorted positions per thread
-
-__global__ void __launch_bounds__(256)
-det_bounds_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* lo_of, uint32_t* hi_of,
-                  uint32_t nwin, uint32_t win_log2, uint32_t Z, const int32_t* status) {
-    // after a failed input check K was not written: the loops below rely on sorted keys
-    if (status != nullptr && *status != 0) return;
-    const uint64_t i0 = ((uint64_t)blockIdx.x * 256 + threadIdx.x) * kBoundsPer;
-    if (i0 > nb) return;
-    uint64_t k[kBoundsPer + 1];  // k[t] = key before position i0 + t
-    k[0] = i0 > 0 ? (uint64_t)__ldg(K + i0 - 1) : 0;
-#pragma unroll
-    for (int t = 0; t < kBoundsPer; ++t) k[t + 1] = i0 + t < nb ? (uint64_t)__ldg(K + i0 + t) : ~0ull;
-#pragma unroll
-    for (int t = 0; t < kBoundsPer; ++t) {
-        const uint64_t i = i0 + t;
-        if (i > nb) break;
-        // windows b with b*W in (k[t], k[t+1]] get hi_of[b] = i (and b = 0 at i = 0)
-        uint64_t from = i > 0 ? (k[t] >> win_log2) + 1 : 0;
-        uint64_t to = i < nb ? (k[t + 1] >> win_log2) : nwin;
-        for (uint64_t b = from; b <= to && b <= nwin; ++b)
-            if (ROBE_CHK(b <= (uint64_t)nwin, ROBE_DBG_WINDOW)) hi_of[b] = (uint32_t)i;
-        from = i > 0 ? ((k[t] + (Z - 1)) >> win_log2) + 1 : 0;
-        to = i < nb ? ((k[t + 1] + (Z - 1)) >> win_log2) : nwin;
-        for (uint64_t b = from; b <= to && b <= nwin; ++b) lo_of[b] = (uint32_t)i;
-    }
-}
-
-// win_left[b] = 1 for a window reached by more than n_max sorted blocks (an id that occurs very
-// often in the batch falls there): the position-tile kernel and the long-walk kernel serve the
-// slots of such windows, the window kernel all others.  *any_left counts them.
-__global__ void __launch_bounds__(256)
-det_window_classify_kernel(const uint32_t* __restrict__ lo_of, const uint32_t* __restrict__ hi_of,
-                           uint32_t nwin, uint32_t n_max, uint8_t* win_left, uint32_t* any_left,
-                           const int32_t* status) {
-    if (status != nullptr && *status != 0) return;
-    const uint32_t b = blockIdx.x * 256 + threadIdx.x;
-    const bool left = b < nwin && hi_of[b + 1] - lo_of[b] > n_max;
-    if (b < nwin) win_left[b] = left ? 1 : 0;
-    const uint32_t votes = __ballot_sync(0xFFFFFFFFu, left);
-    if ((threadIdx.x & 31) == 0 && votes != 0) atomicAdd(any_left, (uint32_t)__popc(votes));
-}
-
-// One CTA per window of W = 2^LOG2W slots.  The sorted blocks that reach the window are positions
-// [lo_of[b], hi_of[b+1]); with their keys taken relative to w0 - (Z-1) ("offsets", 0 .. W+Z-2)
-// pre[t] = number of those blocks with offset < t, so that slot w0 + s is reached by the blocks
-// lo + [pre[s], pre[s+Z]) - those with key in [j-Z+1, j] - already in sorted order.  pre[] is
-// written straight from the sorted keys: the block at relative position e stores e into
-// pre[offset of block e-1 + 1 .. its own offset].  The blocks then stream through shared memory in
-// chunks, each chunk with its gradient elements (fetched by coalesced loads); every thread owns
-// the slots tid, tid+T, ... (T threads) of the window and adds, per chunk, the terms of its slots' ranges
-// from first to last, keeping the running sums in registers.  All slots are committed at the end.
-template <int MODE, int LOG2W>
-__global__ void __launch_bounds__(kWinThreads, 4)
-det_apply_window_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V,
-                        const uint32_t* __restrict__ lo_of, const uint32_t* __restrict__ hi_of,
-                        uint32_t chunk, int vec4) {
-    constexpr uint32_t W = 1u << LOG2W;
-    constexpr int kSlots = W / kWinThreads;
-    __shared__ uint2 ent[kWinEnt];  // .x = (row of the block in stage[]) - key, .y = payload
-    __shared__ __align__(16) float stage[kWinStage];
-    __shared__ uint32_t pre[W + kWinMaxZ + 8];
-    if (a.status != nullptr && *a.status != 0) return;
-    const MapParams& mp = a.mp;
-    const uint32_t tid = threadIdx.x;
-    const uint32_t b = blockIdx.x;
-    const uint32_t lo = lo_of[b], hi = hi_of[b + 1];
-    if (a.win_left[b] != 0) return;
-    const uint32_t Z = mp.Z;
-    const uint64_t w0 = (uint64_t)b << LOG2W;
-    const uint32_t n = hi - lo;
-    if (n == 0) return;
-    if (tid < W / 32) {  // ask the window's target lines into L2 for the commit at the end
-        const uint64_t j = w0 + ((uint64_t)tid << 5);
-        if (j < mp.m) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.target + j));
-    }
-    const bool one_chunk = n <= chunk;
-    const uint32_t span = W + Z - 1;           // offsets 0 .. span-1; pre[0 .. span]
-    const uint32_t bias = (uint32_t)w0 - (Z - 1);  // offset = key - bias (mod 2^32; keys reach >= bias)
-    for (uint32_t e = tid; e <= n; e += kWinThreads) {
-        const uint32_t from = e > 0 ? __ldg(K + lo + e - 1) - bias + 1 : 0;
-        uint32_t to = span;
-        if (e < n) {
-            const uint32_t k = __ldg(K + lo + e);
-            to = k - bias;
-            if (one_chunk && ROBE_CHK(e < kWinEnt, ROBE_DBG_SHARED)) ent[e] = make_uint2(e * Z - k, __ldg(V + lo + e));
-        }
-        for (uint32_t t = from; t <= to; ++t)
-            if (ROBE_CHK(t < W + kWinMaxZ + 8, ROBE_DBG_SHARED)) pre[t] = e;
-    }
-    __syncthreads();
-    // a window in the middle of the array: every slot exists and none is a low slot
-    const bool inner = b != 0 && w0 + W <= (uint64_t)mp.m;
-    const uint32_t j0 = (uint32_t)w0 + tid;  // the thread's first slot
-    float acc[kSlots];
-#pragma unroll
-    for (int q = 0; q < kSlots; ++q) acc[q] = 0.0f;
-    for (uint32_t c0 = 0; c0 < n; c0 += chunk) {
-        const uint32_t c1 = c0 + chunk < n ? c0 + chunk : n;
-        const uint32_t ne = c1 - c0;
-        if (!one_chunk) {
-            if (c0 != 0) __syncthreads();  // the chunk before has been used
-            for (uint32_t e = tid; e < ne; e += kWinThreads)
-                if (ROBE_CHK(e < kWinEnt && (uint64_t)lo + c0 + e < a.nb, ROBE_DBG_SHARED))
-                    ent[e] = make_uint2(e * Z - __ldg(K + lo + c0 + e), __ldg(V + lo + c0 + e));
-            __syncthreads();
-        }
-        if (vec4) {
-            const uint32_t zq = Z >> 2, tot = ne * zq;
-            const bool pow2 = mp.log2Z != 0xFFFFFFFFu;
-            for (uint32_t t = tid; t < tot; t += kWinThreads) {
-                const uint32_t e = pow2 ? t >> (mp.log2Z - 2) : t / zq, o = t - e * zq;
-                if (ROBE_CHK(4u * t + 3u < kWinStage && (uint64_t)ent[e].y + 4u * o + 3u < a.grad_elems,
-                             ROBE_DBG_GRAD_POS))
-                    reinterpret_cast<float4*>(stage)[t] =
-                        __ldg(reinterpret_cast<const float4*>(a.grad_out + ent[e].y) + o);
-            }
-        } else {
-            const uint32_t tot = ne * Z;
-            for (uint32_t t = tid; t < tot; t += kWinThreads) {
-                const uint32_t e = t / Z, o = t - e * Z;
-                if (ROBE_CHK(t < kWinStage && (uint64_t)ent[e].y + o < a.grad_elems, ROBE_DBG_GRAD_POS))
-                    stage[t] = __ldg(a.grad_out + ((uint64_t)ent[e].y + o));
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < kSlots; ++q) {
-            const uint32_t sl = tid + q * kWinThreads;
-            const uint32_t first = pre[sl], last = pre[sl + Z];
-            const uint32_t f = (first > c0 ? first : c0) - c0;
-            const uint32_t l = (last < c1 ? last : c1) - c0;  // (wraps when last < c0: then f >= l)
-            if (first < c1 && last > c0) {
-                const uint32_t j = j0 + q * kWinThreads;  // (a slot past the array is dropped at the commit)
-                float s = acc[q];
-                for (uint32_t e = f; e < l; ++e)
-                    if (ROBE_CHK(e < kWinEnt && ent[e].x + j < kWinStage, ROBE_DBG_SHARED))
-                        s = __fadd_rn(s, stage[ent[e].x + j]);
-                acc[q] = s;
-            }
-        }
-    }
-    // commit: the old values of all the thread's slots are asked for together
-    float old[kSlots];
-    bool has[kSlots];
-#pragma unroll
-    for (int q = 0; q < kSlots; ++q) {
-        const uint32_t sl = tid + q * kWinThreads;
-        has[q] = pre[sl + Z] != pre[sl];
-        if (!inner) {
-            // low slots belong to the low-slot kernel; past the array lie the wrapped tails (the same)
-            const uint64_t j64 = w0 + sl;
-            has[q] = has[q] && j64 < mp.m && j64 + 1 >= Z;
-        }
-        old[q] = has[q] ? a.target[j0 + q * kWinThreads] : 0.0f;
-    }
-#pragma unroll
-    for (int q = 0; q < kSlots; ++q)
-        if (has[q]) commit_slot<MODE>(a, j0 + q * kWinThreads, acc[q], old[q]);
 }
 
 // Long walks (plain blocks only).  One CTA of eight warps per handed-over round, in steps of
@@ -1156,20 +950,11 @@ uint32_t bits_for(uint32_t m) {  // bits needed for keys in [0, m)
 }
 
 struct Layout {
-    size_t keysA, keysB, valsA, valsB, bag_of, counts, totals, long_count, long_walks, bounds, win_left,
-        total;
-    uint32_t long_cap, nwin, win_log2;
+    size_t keysA, keysB, valsA, valsB, bag_of, counts, totals, long_count, long_walks, strips, total;
+    uint32_t long_cap;
 };
 
-// Window length of the window apply: 2048 slots, fewer for a small array so that there are
-// still several CTAs per SM.
-uint32_t window_log2(uint32_t m) {
-    uint32_t l = kWinLog2Max;
-    while (l > kWinLog2Min && (m >> l) < 1024u) --l;
-    return l;
-}
-
-Layout make_layout(uint64_t nb, int64_t nnz, bool bags, uint32_t m) {
+Layout make_layout(uint64_t nb, int64_t nnz, bool bags, const MapParams& mp) {
     Layout L;
     size_t off = 0;
     const size_t kb = align256((nb ? nb : 1) * sizeof(uint32_t));
@@ -1186,91 +971,63 @@ Layout make_layout(uint64_t nb, int64_t nnz, bool bags, uint32_t m) {
     L.long_cap = (uint32_t)cap;
     L.long_count = off; off += 256;
     L.long_walks = off; off += align256((size_t)cap * sizeof(LongWalk));
-    // window apply: first sorted position of every array window, a left-over flag per window and,
-    // in the flag array's first aligned word past the flags, the count of left-over windows
-    L.win_log2 = window_log2(m);
-    L.nwin = (uint32_t)((((uint64_t)m - 1) >> L.win_log2) + 1);
-    L.bounds = off; off += 2 * align256(((size_t)L.nwin + 1) * sizeof(uint32_t));
-    L.win_left = off; off += align256((size_t)L.nwin + 256);
+    // (the sign option may be switched after the workspace was sized: room for the strips either way)
+    L.strips = off; off += strips_ok(mp, nb, false) ? strips_workspace_bytes(mp, nb) : 0;
     L.total = off;
     return L;
 }
 
-// The window kernel pays when most slots are reached, so that walking every slot is no waste.
-bool use_window_apply(const MapParams& mp, uint64_t nb, bool sign) {
-    if (sign || mp.d % mp.Z != 0 || mp.Z > kWinMaxZ || nb == 0) return false;
-    return nb * mp.Z * 2 >= mp.m;
-}
-
-struct WindowBuffers {
-    uint32_t* lo_of;
-    uint32_t* hi_of;
-    uint8_t* left;
-    uint32_t nwin, win_log2;
-    // second stream for the kernels that serve the left-over windows, or nullptr
-    cudaStream_t side;
+// Second stream for what need not hold up the caller's, or nullptr.
+struct SideStream {
+    cudaStream_t st;
     cudaEvent_t fork_event, join_event;
 };
 
-template <bool SIGN, int MODE>
-void launch_apply(ApplyArgs aa, const uint32_t* K, const uint32_t* V, const uint32_t* bag_of,
-                  const WindowBuffers& wb, cudaStream_t st) {
+// Strips where they pay, and the low slots beside them: the hot strips (a few long-running CTAs) and the
+// low slots in the second stream (of higher priority), all other strips in the caller's.
+template <int MODE>
+void launch_apply_strips(const ApplyArgs& aa, const uint32_t* K, const uint32_t* V, int mode, void* workspace,
+                         const SideStream& side, cudaStream_t st) {
     const MapParams& mp = aa.mp;
-    const bool windows = !SIGN && use_window_apply(mp, aa.nb, SIGN);
-    uint32_t chunk = kWinStage / mp.Z;
-    if (chunk > kWinEnt) chunk = kWinEnt;
-    if (windows) {
-        const size_t flags = ((size_t)wb.nwin + 255) & ~(size_t)255;
-        uint32_t* any_left = (uint32_t*)(wb.left + flags);
-        cudaMemsetAsync(any_left, 0, sizeof(uint32_t), st);
-        const uint64_t per_cta = 256ull * kBoundsPer;
-        det_bounds_kernel<<<(unsigned)(aa.nb / per_cta + 1), 256, 0, st>>>(K, aa.nb, wb.lo_of, wb.hi_of,
-                                                                          wb.nwin, wb.win_log2, mp.Z, aa.status);
-        // a window reached by many times the average number of blocks holds an often repeated id
-        const uint64_t mean = (((uint64_t)1 << wb.win_log2) + mp.Z) * aa.nb / mp.m + 1;
-        const uint64_t n_max = mean * 4 > 512 ? mean * 4 : 512;
-        det_window_classify_kernel<<<(wb.nwin + 255) / 256, 256, 0, st>>>(
-            wb.lo_of, wb.hi_of, wb.nwin, (uint32_t)(n_max < 0xFFFFFFFFull ? n_max : 0xFFFFFFFFull), wb.left,
-            any_left, aa.status);
-        aa.win_left = wb.left;
-        aa.any_left = any_left;
-        aa.win_log2 = wb.win_log2;
-    }
-    // With windows, the kernels below serve the left-over windows only: a few long-running CTAs.
-    // They go to the second stream (of higher priority) and the window kernel runs beside them.
-    const bool forked = windows && wb.side != nullptr;
-    cudaStream_t ts = st;
+    const StripProblem sp{mp, aa.grad_out, aa.grad_elems, aa.target, aa.lr, aa.adam, K, V, aa.nb, aa.status, workspace};
+    launch_strips_prepare(sp, st);
+    const bool forked = side.st != nullptr;
     if (forked) {
-        cudaEventRecord(wb.fork_event, st);
-        cudaStreamWaitEvent(wb.side, wb.fork_event, 0);
-        ts = wb.side;
+        cudaEventRecord(side.fork_event, st);
+        cudaStreamWaitEvent(side.st, side.fork_event, 0);
     }
+    const cudaStream_t ts = forked ? side.st : st;
+    launch_strips(sp, mode, st, ts);
+    if (mp.Z > 1) {
+        const unsigned low_blocks = (mp.Z - 1 + kLowWarps - 1) / kLowWarps;
+        if (mp.d % mp.Z != 0) det_apply_low_kernel<false, MODE, true><<<low_blocks, 32 * kLowWarps, 0, ts>>>(aa, K, V, nullptr);
+        else det_apply_low_kernel<false, MODE, false><<<low_blocks, 32 * kLowWarps, 0, ts>>>(aa, K, V, nullptr);
+    }
+    if (forked) {
+        cudaEventRecord(side.join_event, side.st);
+        cudaStreamWaitEvent(st, side.join_event, 0);
+    }
+}
+
+template <bool SIGN, int MODE>
+void launch_apply(const ApplyArgs& aa, const uint32_t* K, const uint32_t* V, const uint32_t* bag_of, cudaStream_t st) {
+    const MapParams& mp = aa.mp;
     const unsigned blocks = (unsigned)((aa.nb + 255) / 256);  // one warp per 32 sorted positions
     const unsigned low_blocks = (mp.Z - 1 + kLowWarps - 1) / kLowWarps;  // one warp per low slot
     if (mp.d % mp.Z != 0) {
-        det_apply_kernel<SIGN, MODE, true><<<blocks, 256, 0, ts>>>(aa, K, V, bag_of);
+        det_apply_kernel<SIGN, MODE, true><<<blocks, 256, 0, st>>>(aa, K, V, bag_of);
         if (mp.Z > 1)
-            det_apply_low_kernel<SIGN, MODE, true><<<low_blocks, 32 * kLowWarps, 0, ts>>>(aa, K, V, bag_of);
+            det_apply_low_kernel<SIGN, MODE, true><<<low_blocks, 32 * kLowWarps, 0, st>>>(aa, K, V, bag_of);
     } else {
-        det_apply_kernel<SIGN, MODE, false><<<blocks, 256, 0, ts>>>(aa, K, V, bag_of);
+        det_apply_kernel<SIGN, MODE, false><<<blocks, 256, 0, st>>>(aa, K, V, bag_of);
         if (!SIGN) {
             // the rounds the apply kernel handed over; a grid-stride loop over the list
             const unsigned lblocks = aa.long_cap < 148u * 8u ? aa.long_cap : 148u * 8u;
-            det_apply_long_kernel<MODE><<<lblocks, 32 * kLongWarps, 0, ts>>>(aa, K, V);
+            det_apply_long_kernel<MODE><<<lblocks, 32 * kLongWarps, 0, st>>>(aa, K, V);
         }
         if (mp.Z > 1)
-            det_apply_low_kernel<SIGN, MODE, false><<<low_blocks, 32 * kLowWarps, 0, ts>>>(aa, K, V, bag_of);
+            det_apply_low_kernel<SIGN, MODE, false><<<low_blocks, 32 * kLowWarps, 0, st>>>(aa, K, V, bag_of);
     }
-    if (forked) cudaEventRecord(wb.join_event, wb.side);
-    if (windows) {
-        const int vec4 = mp.Z % 4 == 0 && mp.d % 4 == 0 && ((uintptr_t)aa.grad_out & 15) == 0;
-        switch (wb.win_log2) {
-            case 9: det_apply_window_kernel<MODE, 9><<<wb.nwin, kWinThreads, 0, st>>>(aa, K, V, wb.lo_of, wb.hi_of, chunk, vec4); break;
-            case 10: det_apply_window_kernel<MODE, 10><<<wb.nwin, kWinThreads, 0, st>>>(aa, K, V, wb.lo_of, wb.hi_of, chunk, vec4); break;
-            default: det_apply_window_kernel<MODE, 11><<<wb.nwin, kWinThreads, 0, st>>>(aa, K, V, wb.lo_of, wb.hi_of, chunk, vec4); break;
-        }
-    }
-    if (forked) cudaStreamWaitEvent(st, wb.join_event, 0);
 }
 
 }  // namespace
@@ -1278,12 +1035,12 @@ void launch_apply(ApplyArgs aa, const uint32_t* K, const uint32_t* V, const uint
 size_t det_workspace_bytes(const MapParams& mp, int64_t nbags, int64_t nnz, bool bags) {
     (void)nbags;
     const uint64_t nb = (uint64_t)nnz * mp.C;
-    return make_layout(nb, nnz, bags, mp.m).total;
+    return make_layout(nb, nnz, bags, mp).total;
 }
 
 void block_key_buffers(const Problem& pb, void* workspace, uint32_t** keys, uint32_t** vals) {
     const uint64_t nb = (uint64_t)pb.nnz * pb.mp.C;
-    const Layout L = make_layout(nb, pb.nnz, pb.offsets != nullptr, pb.mp.m);
+    const Layout L = make_layout(nb, pb.nnz, pb.offsets != nullptr, pb.mp);
     *keys = (uint32_t*)((char*)workspace + L.keysA);
     *vals = (uint32_t*)((char*)workspace + L.valsA);
 }
@@ -1303,7 +1060,7 @@ cudaError_t launch_block_keys(const Problem& pb, void* workspace, size_t workspa
     const MapParams& mp = pb.mp;
     const bool bags = pb.offsets != nullptr;
     const uint64_t nb = (uint64_t)pb.nnz * mp.C;
-    const Layout L = make_layout(nb, pb.nnz, bags, mp.m);
+    const Layout L = make_layout(nb, pb.nnz, bags, mp);
     if (workspace == nullptr || workspace_bytes < L.total) return cudaErrorInvalidValue;
     char* ws = (char*)workspace;
     uint32_t* kA = (uint32_t*)(ws + L.keysA);
@@ -1330,7 +1087,7 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
     const MapParams& mp = pb.mp;
     const bool bags = pb.offsets != nullptr;
     const uint64_t nb = (uint64_t)pb.nnz * mp.C;
-    const Layout L = make_layout(nb, pb.nnz, bags, mp.m);
+    const Layout L = make_layout(nb, pb.nnz, bags, mp);
     if (workspace == nullptr || workspace_bytes < L.total) return cudaErrorInvalidValue;
     // the payload of a block is a 32-bit position in grad_out
     if ((uint64_t)pb.nbags * mp.d > (1ull << 32)) return cudaErrorInvalidValue;
@@ -1360,7 +1117,7 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
         const uint32_t shift = bits > 30 ? bits - 8 : (bits > 22 ? 22 : (bits > 8 ? bits - 8 : 0));
         launch_sort_pass<false>(sp, kA, vA, kB, vB, counts, totals, shift, bits - shift, st);
         ApplyArgs ab{mp, grad_out, pb.indices, target, lr, nb, pb.status, AdamState{}, nullptr, nullptr, 0,
-                     nullptr, nullptr, 0, (uint64_t)pb.nbags * mp.d, pb.l2_keep};
+                     (uint64_t)pb.nbags * mp.d, pb.l2_keep};
         uint32_t log2Zp = 0;
         while ((1u << log2Zp) < mp.Z) ++log2Zp;
         const uint64_t groups = (nb + kBinnedPer - 1) / kBinnedPer;
@@ -1386,24 +1143,27 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
     }
 
     uint32_t* long_count = (uint32_t*)(ws + L.long_count);
+    const ApplyArgs aa{mp, grad_out, pb.indices, target, lr, nb, pb.status, adam ? *adam : AdamState{},
+                       long_count, (LongWalk*)(ws + L.long_walks), L.long_cap, (uint64_t)pb.nbags * mp.d, 0};
+    if (strips_ok(mp, nb, pb.sign != 0)) {
+        const SideStream side{pb.side, pb.fork_event, pb.join_event};
+        if (mode == 4) launch_apply_strips<3>(aa, kA, vA, mode, ws + L.strips, side, st);
+        else if (mode == 2) launch_apply_strips<2>(aa, kA, vA, mode, ws + L.strips, side, st);
+        else if (mode == 1) launch_apply_strips<1>(aa, kA, vA, mode, ws + L.strips, side, st);
+        else launch_apply_strips<0>(aa, kA, vA, mode, ws + L.strips, side, st);
+        return cudaGetLastError();
+    }
     cudaMemsetAsync(long_count, 0, 2 * sizeof(uint32_t), st);  // [0] rounds handed over, [1] rounds taken
-    ApplyArgs aa{mp, grad_out, pb.indices, target, lr, nb, pb.status, adam ? *adam : AdamState{},
-                 long_count, (LongWalk*)(ws + L.long_walks), L.long_cap, nullptr, nullptr, 0,
-                 (uint64_t)pb.nbags * mp.d, 0};
-    const WindowBuffers wb{(uint32_t*)(ws + L.bounds),
-                           (uint32_t*)(ws + L.bounds + align256(((size_t)L.nwin + 1) * sizeof(uint32_t))),
-                           (uint8_t*)(ws + L.win_left), L.nwin, L.win_log2,
-                           pb.side, pb.fork_event, pb.join_event};
     if (pb.sign) {
-        if (mode == 4) launch_apply<true, 3>(aa, kA, vA, bag_of, wb, st);
-        else if (mode == 2) launch_apply<true, 2>(aa, kA, vA, bag_of, wb, st);
-        else if (mode == 1) launch_apply<true, 1>(aa, kA, vA, bag_of, wb, st);
-        else launch_apply<true, 0>(aa, kA, vA, bag_of, wb, st);
+        if (mode == 4) launch_apply<true, 3>(aa, kA, vA, bag_of, st);
+        else if (mode == 2) launch_apply<true, 2>(aa, kA, vA, bag_of, st);
+        else if (mode == 1) launch_apply<true, 1>(aa, kA, vA, bag_of, st);
+        else launch_apply<true, 0>(aa, kA, vA, bag_of, st);
     } else {
-        if (mode == 4) launch_apply<false, 3>(aa, kA, vA, bag_of, wb, st);
-        else if (mode == 2) launch_apply<false, 2>(aa, kA, vA, bag_of, wb, st);
-        else if (mode == 1) launch_apply<false, 1>(aa, kA, vA, bag_of, wb, st);
-        else launch_apply<false, 0>(aa, kA, vA, bag_of, wb, st);
+        if (mode == 4) launch_apply<false, 3>(aa, kA, vA, bag_of, st);
+        else if (mode == 2) launch_apply<false, 2>(aa, kA, vA, bag_of, st);
+        else if (mode == 1) launch_apply<false, 1>(aa, kA, vA, bag_of, st);
+        else launch_apply<false, 0>(aa, kA, vA, bag_of, st);
     }
     return cudaGetLastError();
 }

@@ -60,6 +60,28 @@ struct AdamState {
     float bias2;   // 1 - beta2^t
 };
 
+// What the strip apply (robe_strips.cu) takes: the sorted blocks and what their sums are for.
+struct StripProblem {
+    MapParams mp;
+    const float* grad_out;
+    uint64_t grad_elems;
+    float* target;
+    float lr;
+    AdamState adam;
+    const uint32_t* K;
+    const uint32_t* V;
+    uint64_t nb;
+    const int32_t* status;
+    void* workspace;  // strips_workspace_bytes, 256-byte aligned
+};
+bool strips_ok(const MapParams& mp, uint64_t nb, bool sign);
+size_t strips_workspace_bytes(const MapParams& mp, uint64_t nb);
+// first sorted position of every strip; in st
+void launch_strips_prepare(const StripProblem& sp, cudaStream_t st);
+// all slots but [0, Z-1), mode as launch_backward_det's 0, 1, 2, 4.  Strips of often repeated ids are served
+// in hot_st (st itself, or a stream that has been made to wait for launch_strips_prepare).
+void launch_strips(const StripProblem& sp, int mode, cudaStream_t st, cudaStream_t hot_st);
+
 // mode 0: target[j] += delta; 1: target = attached array, target[j] = fma(-lr, delta, target[j]);
 // 2: Adam step on the attached array with the moments in *adam; 4: Adagrad step on the attached
 // array with the accumulators in adam->m2 and adam->eps; 3: binned atomic adds of

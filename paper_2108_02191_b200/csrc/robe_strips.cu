@@ -1,0 +1,541 @@
+// Strip apply: the slot-major last step of the deterministic backward, for arrays that a call touches
+// densely (sign off, blocks of up to 128 elements, short last blocks included).
+//
+// The array is cut into strips of 64 .. 256 slots.  With the blocks sorted by start, those that reach a
+// strip are one stretch of the sorted list.  A group of LP lanes (LP = 8, 16, 32 by the block length)
+// serves a strip, several groups to a warp: it keeps the strip's sums in shared memory and takes the
+// stretch block after block - lane o of the group fetches gradient element o and adds it to slot
+// start + o.  Blocks come one after the other, so every slot adds its terms in the canonical order, and
+// there is nothing to search and nothing to stage: the keys say where to add.
+//   * The gradient loads of eight blocks are in flight together, the next keys are asked for ahead.
+//   * The sums start from -0 and a -0 element is made +0 first: x + -0 is x for every x, and -0 remains
+//     exactly where nothing was added (the canonical sum starts from +0, adds the same terms, and is never
+//     -0).  So an untouched slot is known by its sum.
+// No barriers between warps, nothing waits but a warp for its own loads.  Bound by instruction issue
+// (12 per block and lane group) and the random gradient reads.
+// Measured (B200, us, a CTA per 2048 slots with position-tile and long-walk kernels for often repeated ids
+// -> here): 34 M blocks of 16 on 250 M slots 1690 -> 895; Adam on 852 K blocks of 8 from Zipf ids, 540 K slots
+// 137 -> 50 (the longest id's chain: 9100 terms); the whole Adam step 257 -> 157.
+// Rejected: a lane per four slots with the blocks' rows staged in shared memory and the blocks of each lane
+// found by bisection or a scan - 385 .. 518 instructions per strip of 128 against about 200.
+//
+// A strip reached by very many blocks (an id that the batch repeats hundreds of times) would keep one group
+// busy for long; such strips go to strip_hot_kernel, one CTA each: eight warps copy gradient elements
+// ahead (cp.async), a warp per 32 slots adds.
+// Slots [0, Z-1) also receive the wrapped tails of the array's last blocks: another kernel's.
+#include "robe_internal.h"
+#include "robe_update.cuh"
+
+namespace robe {
+
+namespace {
+
+constexpr uint32_t kStripMinLog2 = 6, kStripMaxLog2 = 8;
+constexpr int kStripWarps = 8;
+constexpr uint32_t kStripMaxZ = 128;
+constexpr int kHotCopiers = 8;            // warps of the hot kernel that copy
+constexpr int kHotAdders = 8;             // and that add: 32 slots each
+constexpr uint32_t kHotBufs = 3;          // steps staged: one being added, two on their way
+constexpr uint32_t kHotMin = 256;         // a strip is hot from this many blocks on, at least
+
+struct StripArgs {
+    MapParams mp;
+    const float* grad_out;
+    float* target;
+    float lr;
+    AdamState adam;
+    const uint32_t* K;         // sorted block starts
+    const uint32_t* V;         // bag*d + c*Z of each: its first gradient element
+    const int32_t* status;
+    const uint32_t* lo_of;     // [strips + 1]: first sorted position whose block reaches the strip or one beyond
+    const uint32_t* hi_of;     // [strips + 1]: first sorted position whose key is in the strip or beyond
+    uint32_t strips, log2w;    // strips of 2^log2w slots
+    uint32_t n_hot;
+    uint32_t* hot_count;       // [0] strips at the front of the list, [1] at its back, [2] taken
+    uint32_t* hot_list;
+    uint32_t hot_cap;
+    uint32_t hot_entries;      // blocks copied at a time by a warp: 32, 16 or 8
+    uint32_t hot_magic;        // ceil(2^32 / Z); 0: Z is 1
+    int vec_commit;            // target and moments are 16-byte aligned
+    uint64_t grad_elems;       // of grad_out (read by the debug build's index checks only)
+};
+
+constexpr uint32_t kBoundsGap = 256;  // longer gaps are filled by the whole warp
+
+// lo_of and hi_of for b = 0 .. strips.  A thread takes eight sorted positions; position i begins the strips
+// whose first slot lies past the key before it and not past its own (lo_of: the same of the blocks' last slots).
+__global__ void __launch_bounds__(256)
+strip_bounds_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* __restrict__ lo_of,
+                    uint32_t* __restrict__ hi_of, uint32_t strips, uint32_t log2w, uint32_t reach, const int32_t* status) {
+    if (status != nullptr && *status != 0) return;  // after a failed input check K was not written
+    const uint64_t i0 = ((uint64_t)blockIdx.x * 256 + threadIdx.x) * 8;
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t k[9];  // k[0]: the key before
+    if (i0 + 8 <= nb) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(K + i0)), y = __ldg(reinterpret_cast<const uint4*>(K + i0) + 1);
+        k[1] = x.x; k[2] = x.y; k[3] = x.z; k[4] = x.w;
+        k[5] = y.x; k[6] = y.y; k[7] = y.z; k[8] = y.w;
+    } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) k[t + 1] = i0 + t < nb ? __ldg(K + i0 + t) : 0u;
+    }
+    k[0] = __shfl_up_sync(0xFFFFFFFFu, k[8], 1);
+    if (lane == 0 && i0 > 0 && i0 <= nb) k[0] = __ldg(K + i0 - 1);
+    if (__all_sync(0xFFFFFFFFu, i0 > 0 && i0 + 8 <= nb && ((k[8] + reach) >> log2w) - (k[0] >> log2w) <= kBoundsGap)) {
+        // in the middle of the list (most threads): a position begins a strip, or a few, or none
+        uint32_t h = k[0] >> log2w, l = (k[0] + reach) >> log2w;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const uint32_t hi = k[t + 1] >> log2w, to = (k[t + 1] + reach) >> log2w;
+            while (h != hi) {
+                ++h;
+                if (ROBE_CHK(h <= strips, ROBE_DBG_WINDOW)) hi_of[h] = (uint32_t)(i0 + t);
+            }
+            while (l != to) {
+                ++l;
+                if (l <= strips) lo_of[l] = (uint32_t)(i0 + t);  // (a block may reach past the array's end)
+            }
+        }
+        return;
+    }
+    bool gap = false;
+    // strips from .. to begin at position i0 + t  (reach = Z - 1; key + reach < 2^32)
+    auto span = [&](int t, uint32_t past, uint32_t& from, uint32_t& n) {
+        const uint64_t i = i0 + t;
+        from = i > 0 ? ((k[t] + past) >> log2w) + 1 : 0u;
+        uint32_t to = i < nb ? (k[t + 1] + past) >> log2w : strips;
+        if (to > strips) to = strips;
+        n = i <= nb && to >= from ? to - from + 1 : 0u;
+    };
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        uint32_t from, n;
+        span(t, 0, from, n);
+        if (n > kBoundsGap) gap = true;
+        else
+            for (uint32_t b = 0; b < n; ++b)
+                if (ROBE_CHK(from + b <= strips, ROBE_DBG_WINDOW)) hi_of[from + b] = (uint32_t)(i0 + t);
+        span(t, reach, from, n);
+        if (n > kBoundsGap) gap = true;
+        else
+            for (uint32_t b = 0; b < n; ++b)
+                if (ROBE_CHK(from + b <= strips, ROBE_DBG_WINDOW)) lo_of[from + b] = (uint32_t)(i0 + t);
+    }
+    if (!__any_sync(0xFFFFFFFFu, gap)) return;
+    for (int t = 0; t < 16; ++t) {
+        uint32_t* const of = t < 8 ? hi_of : lo_of;
+        uint32_t from = 0, n = 0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c == (t & 7)) span(c, t < 8 ? 0u : reach, from, n);
+        for (uint32_t wide = __ballot_sync(0xFFFFFFFFu, n > kBoundsGap); wide != 0; wide &= wide - 1) {
+            const int src = __ffs((int)wide) - 1;
+            const uint32_t f = __shfl_sync(0xFFFFFFFFu, from, src), c = __shfl_sync(0xFFFFFFFFu, n, src);
+            const uint32_t p = __shfl_sync(0xFFFFFFFFu, (uint32_t)(i0 + (t & 7)), src);
+            for (uint32_t b = lane; b < c; b += 32)
+                if (ROBE_CHK(f + b <= strips, ROBE_DBG_WINDOW)) of[f + b] = p;
+        }
+    }
+}
+
+// The list of hot strips: the hottest at its front, so that they are begun first.
+__global__ void __launch_bounds__(256) strip_hot_list_kernel(StripArgs a) {
+    if (a.status != nullptr && *a.status != 0) return;
+    const uint32_t b = blockIdx.x * 256 + threadIdx.x;
+    if (b >= a.strips) return;
+    const uint32_t n = a.hi_of[b + 1] - a.lo_of[b];
+    if (n <= a.n_hot) return;
+    const bool front = n > 4 * a.n_hot;
+    const uint32_t at = atomicAdd(a.hot_count + (front ? 0 : 1), 1u);
+    if (ROBE_CHK(at < a.hot_cap, ROBE_DBG_LONG_WALK)) a.hot_list[front ? at : a.hot_cap - 1 - at] = b;
+}
+
+// elements of the block with payload v
+template <bool SHORT>
+__device__ __forceinline__ uint32_t strip_len(const MapParams& mp, uint32_t v) {
+    if (!SHORT) return mp.Z;
+    const uint32_t left = mp.d - v % mp.d;
+    return left < mp.Z ? left : mp.Z;
+}
+
+__device__ __forceinline__ bool strip_touched(float sum) { return __float_as_uint(sum) != 0x80000000u; }
+
+template <int MODE, int LP, int EPL, bool SHORT>
+__global__ void __launch_bounds__(32 * kStripWarps, 5)
+strip_apply_kernel(StripArgs a) {
+    extern __shared__ float4 strip_smem[];
+    if (a.status != nullptr && *a.status != 0) return;
+    constexpr uint32_t G = 32 / LP;               // groups per warp
+    constexpr int U = EPL == 4 ? 4 : 8;           // blocks whose loads are in flight together
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t g = lane / LP, ol = lane % LP;
+    const uint32_t b = (blockIdx.x * kStripWarps + w) * G + g;
+    const uint32_t Z = a.mp.Z, W = 1u << a.log2w;
+    volatile float* const sum = reinterpret_cast<float*>(strip_smem) + (w * G + g) * W;
+    uint32_t lo = 0, n = 0;
+    if (b < a.strips) {
+        lo = __ldg(a.lo_of + b);
+        n = __ldg(a.hi_of + b + 1) - lo;
+        if (n > a.n_hot) n = 0;  // the hot kernel's
+    }
+    const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n);
+    if (most == 0) return;
+    const uint32_t w0 = b << a.log2w;
+    if (n != 0 && ol < W / 32 && (uint64_t)w0 + 32 * ol < a.mp.m)  // wanted at the end: the lines of the target
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.target + w0 + 32 * ol));
+    for (uint32_t i = ol; i < W / 4; i += LP)
+        reinterpret_cast<float4*>(strip_smem)[((w * G + g) * W >> 2) + i] = make_float4(-0.0f, -0.0f, -0.0f, -0.0f);
+    // lane ol holds block ol of the present LP: start relative to the strip, payload
+    uint32_t nk = 0, nv = 0;
+    if (ol < n) {
+        nk = __ldg(a.K + lo + ol);
+        nv = __ldg(a.V + lo + ol);
+    }
+    __syncwarp();
+    for (uint32_t c0 = 0; c0 < most; c0 += LP) {
+        // a block past the stretch starts beyond every strip
+        const uint32_t rel = c0 + ol < n ? nk - w0 : 0x40000000u, v = nv;
+        const uint32_t len = SHORT ? strip_len<SHORT>(a.mp, v) : 0u;
+        if (c0 + LP + ol < n) {
+            nk = __ldg(a.K + lo + c0 + LP + ol);
+            nv = __ldg(a.V + lo + c0 + LP + ol);
+        }
+#pragma unroll 1
+        for (uint32_t u0 = 0; u0 < LP && c0 + u0 < most; u0 += U) {
+            float x[U][EPL];
+            uint32_t slot[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int src = (int)(g * LP + u0 + u);
+                const uint32_t r = __shfl_sync(0xFFFFFFFFu, rel, src), p = __shfl_sync(0xFFFFFFFFu, v, src) + ol;
+                const uint32_t l = SHORT ? __shfl_sync(0xFFFFFFFFu, len, src) : Z;
+                slot[u] = r + ol;  // (below the strip: wraps to a large number)
+#pragma unroll
+                for (int q = 0; q < EPL; ++q) {
+                    x[u][q] = -0.0f;
+                    if (slot[u] + 32 * q < W && ol + 32 * q < l &&
+                        ROBE_CHK((uint64_t)p + 32 * q < a.grad_elems, ROBE_DBG_GRAD_POS))
+                        x[u][q] = __ldg(a.grad_out + (p + 32 * q)) + 0.0f;  // -0 -> +0
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+#pragma unroll
+                for (int q = 0; q < EPL; ++q) {
+                    // (a lane past the block's end adds -0 to a slot that is no other lane's in this step)
+                    const uint32_t s = slot[u] + 32 * q;
+                    if (s < W) sum[s] = __fadd_rn(sum[s], x[u][q]);
+                }
+                __syncwarp();
+            }
+        }
+    }
+    if (n == 0) return;
+    const bool inner = a.vec_commit && w0 + 1 >= Z && (uint64_t)w0 + W <= a.mp.m;
+    const float4* const sum4 = strip_smem + ((w * G + g) * W >> 2);
+    for (uint32_t i = ol; i < W / 4; i += LP) {
+        const float4 s = sum4[i];
+        const bool t0 = strip_touched(s.x), t1 = strip_touched(s.y), t2 = strip_touched(s.z), t3 = strip_touched(s.w);
+        const uint32_t j = w0 + 4 * i;
+        if (!(t0 || t1 || t2 || t3)) continue;
+        if (inner) {  // all of the strip inside the array and above the low slots, vectors aligned
+            if (!ROBE_CHK((uint64_t)j + 3 < a.mp.m, ROBE_DBG_ARRAY_SLOT)) continue;
+            float4 old = *reinterpret_cast<const float4*>(a.target + j), m1 = make_float4(0, 0, 0, 0), m2 = m1;
+            if (MODE == 2) m1 = *reinterpret_cast<const float4*>(a.adam.m1 + j);
+            if (MODE >= 2) m2 = *reinterpret_cast<const float4*>(a.adam.m2 + j);
+            if (t0) old.x = slot_step<MODE>(a.adam, a.lr, s.x, old.x, m1.x, m2.x);
+            if (t1) old.y = slot_step<MODE>(a.adam, a.lr, s.y, old.y, m1.y, m2.y);
+            if (t2) old.z = slot_step<MODE>(a.adam, a.lr, s.z, old.z, m1.z, m2.z);
+            if (t3) old.w = slot_step<MODE>(a.adam, a.lr, s.w, old.w, m1.w, m2.w);
+            *reinterpret_cast<float4*>(a.target + j) = old;
+            if (MODE == 2) *reinterpret_cast<float4*>(a.adam.m1 + j) = m1;
+            if (MODE >= 2) *reinterpret_cast<float4*>(a.adam.m2 + j) = m2;
+            continue;
+        }
+        const float one[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+        for (uint32_t q = 0; q < 4; ++q)
+            if (strip_touched(one[q]) && (uint64_t)j + q < a.mp.m && j + q + 1 >= Z)
+                commit_slot<MODE>(a, j + q, one[q], a.target[j + q]);
+    }
+}
+
+__device__ __forceinline__ float lds1(uint32_t at) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(at));
+    return v;
+}
+__device__ __forceinline__ float4 lds4(uint32_t at) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at));
+    return v;
+}
+__device__ __forceinline__ float add4(float acc, const float4 x) {
+    return __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(acc, x.x), x.y), x.z), x.w);
+}
+
+// acc + one slot's terms of `units` times eight blocks, in order: units of 32 bytes at `at`, `per_chunk` (a power
+// of two) of them side by side and `skip` bytes on to the next chunk.  The reads run a unit ahead of the adds.
+__device__ __forceinline__ float hot_add_units(float acc, uint32_t at, uint32_t units, uint32_t per_chunk, uint32_t skip) {
+    float4 x = lds4(at), y = lds4(at + 16);
+#pragma unroll 4
+    for (uint32_t u = 1; u < units; ++u) {
+        at += 32;
+        if ((u & (per_chunk - 1)) == 0) at += skip;
+        const float4 x1 = lds4(at), y1 = lds4(at + 16);
+        acc = add4(add4(acc, x), y);
+        x = x1;
+        y = y1;
+    }
+    return add4(add4(acc, x), y);
+}
+
+// Hot strips.  The chain of dependent adds of a slot is the definition's, and one warp's issue is what it
+// costs beyond that: the copies are laid out slot by slot, so that a lane reads four blocks' terms at once,
+// and a whole step of repeats of one start is one loop.  One barrier per step of eight copiers' blocks,
+// whose copies were issued two steps ahead.
+// Measured (B200, ns per repeat of one start): 9.3 with a row per block, 4 here; the chain itself: 2.1.
+template <int MODE, bool SHORT>
+__global__ void __launch_bounds__(32 * (kHotCopiers + kHotAdders))
+strip_hot_kernel(StripArgs a) {
+    extern __shared__ float4 strip_smem[];
+    __shared__ int2 ent_s[kHotBufs][kHotCopiers][32];  // (start relative to the strip, length) of each block
+    __shared__ int4 all_s[kHotBufs][kHotCopiers];      // of the blocks of one copier: their number; all alike? start, length
+    __shared__ uint32_t item_s;
+    if (a.status != nullptr && *a.status != 0) return;
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool copier = w >= (uint32_t)kHotAdders;
+    const uint32_t cw = w - kHotAdders;
+    const uint32_t Z = a.mp.Z, W = 1u << a.log2w, E = a.hot_entries, per_step = E * kHotCopiers;
+    const uint32_t n_front = a.hot_count[0], n_items = n_front + a.hot_count[1];
+    float* const stage = reinterpret_cast<float*>(strip_smem);
+    const uint32_t pitch = E + 4, chunk = pitch * Z;  // element o of block e at o * pitch + e
+    for (;;) {
+        __syncthreads();  // item_s and the buffers are free
+        if (threadIdx.x == 0) item_s = atomicAdd(a.hot_count + 2, 1u);
+        __syncthreads();
+        const uint32_t item = item_s;
+        if (item >= n_items) break;
+        const uint32_t b = a.hot_list[item < n_front ? item : a.hot_cap - 1 - (item - n_front)];
+        const uint32_t w0 = b << a.log2w;
+        const uint32_t lo = a.lo_of[b], n = a.hi_of[b + 1] - lo;
+        const uint32_t steps = (n + per_step - 1) / per_step;
+        uint32_t k = 0, v = 0;  // copiers: the block of this lane in the step to be copied next
+        // blocks of this copier in step s: positions from lo + s*per_step + cw*E, this many
+        auto count = [&](uint32_t s) -> uint32_t {
+            const uint64_t at = (uint64_t)s * per_step + cw * E;
+            return at >= n ? 0u : (n - at < E ? (uint32_t)(n - at) : E);
+        };
+        auto fetch = [&](uint32_t s) {
+            if (lane < count(s)) {
+                const uint32_t at = lo + s * per_step + cw * E + lane;
+                k = __ldg(a.K + at);
+                v = __ldg(a.V + at);
+            }
+        };
+        auto copy = [&](uint32_t s) {  // one commit group per call
+            const uint32_t ne = count(s);
+            float* const rows = stage + ((s % kHotBufs) * kHotCopiers + cw) * chunk;
+            const int rel = (int)(k - w0);
+            const int len = (int)(lane < ne ? strip_len<SHORT>(a.mp, v) : 0u);
+            ent_s[s % kHotBufs][cw][lane] = make_int2(rel, len);
+            const int rel0 = __shfl_sync(0xFFFFFFFFu, rel, 0), len0 = __shfl_sync(0xFFFFFFFFu, len, 0);
+            const bool alike = __all_sync(0xFFFFFFFFu, lane >= ne || (rel == rel0 && len == len0));
+            if (lane == 0) all_s[s % kHotBufs][cw] = make_int4((int)ne, alike ? 1 : 0, rel0, len0);
+            const uint32_t total = ne * Z;
+            for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+                const uint32_t t = t0 + lane, e = a.hot_magic != 0 ? __umulhi(t, a.hot_magic) : t, o = t - e * Z;
+                const int r = __shfl_sync(0xFFFFFFFFu, rel, e);
+                const uint32_t p = __shfl_sync(0xFFFFFFFFu, v, e) + o;
+                const uint32_t l = SHORT ? (uint32_t)__shfl_sync(0xFFFFFFFFu, len, e) : Z;
+                const int first = r + (int)o;
+                if (t < total && first >= 0 && first < (int)W && o < l && ROBE_CHK(p < a.grad_elems, ROBE_DBG_GRAD_POS)) {
+                    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(rows + o * pitch + e);
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(a.grad_out + p) : "memory");
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        if (copier) {
+            fetch(0);
+            copy(0);
+            fetch(1);
+            if (steps > 1) copy(1);
+            fetch(2);
+        }
+        const int slot = (int)(32 * w + lane);  // adders: within the strip
+        float acc = -0.0f;
+        for (uint32_t s = 0; s < steps; ++s) {
+            if (copier) {
+                if (s + 1 < steps) asm volatile("cp.async.wait_group 1;" ::: "memory");
+                else asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();  // step s is in; step s - 1 has been added
+            if (copier) {
+                if (s + 2 < steps) {
+                    copy(s + 2);
+                    fetch(s + 3);
+                }
+                continue;
+            }
+            if (32 * w >= W) continue;
+            const uint32_t stage_at = (uint32_t)__cvta_generic_to_shared(stage + (s % kHotBufs) * kHotCopiers * chunk);
+            const int4 lead = all_s[s % kHotBufs][0], its = all_s[s % kHotBufs][lane % kHotCopiers];
+            if (__all_sync(0xFFFFFFFFu, its.x == (int)E && its.y != 0 && its.z == lead.z && its.w == lead.w)) {
+                // a whole step of repeats (-0 turns +0 at the first term: see strip_apply_kernel)
+                const uint32_t d = (uint32_t)(slot - lead.z);
+                if (d < (uint32_t)lead.w)
+                    acc = hot_add_units(acc + 0.0f, stage_at + 4 * pitch * d, kHotCopiers * (E / 8), E / 8, 4 * (chunk - E));
+                continue;
+            }
+            for (uint32_t c = 0; c < (uint32_t)kHotCopiers; ++c) {
+                const int4 all = all_s[s % kHotBufs][c];
+                const uint32_t ne = (uint32_t)all.x;
+                if (ne == 0) break;
+                const uint32_t rows_at = stage_at + 4 * chunk * c;
+                if (all.y) {  // every block covers the same slots
+                    const uint32_t d = (uint32_t)(slot - all.z);
+                    if (d < (uint32_t)all.w) {
+                        acc += 0.0f;
+                        const uint32_t at = rows_at + 4 * pitch * d;
+                        if (ne >= 8) acc = hot_add_units(acc, at, ne / 8, 32, 0);
+                        for (uint32_t e = ne & ~7u; e < ne; ++e) acc = __fadd_rn(acc, lds1(at + 4 * e));
+                    }
+                    __syncwarp();
+                    continue;
+                }
+                // (-0 for a block that does not reach the slot, +0 for a term -0)
+                const int2 mine = ent_s[s % kHotBufs][c][lane];
+                for (uint32_t e0 = 0; e0 < ne; e0 += 8) {
+                    float x[8];
+#pragma unroll
+                    for (uint32_t u = 0; u < 8; ++u) {
+                        const uint32_t d = (uint32_t)(slot - __shfl_sync(0xFFFFFFFFu, mine.x, e0 + u));
+                        const uint32_t l = (uint32_t)__shfl_sync(0xFFFFFFFFu, mine.y, e0 + u);  // (0 past the last block)
+                        x[u] = -0.0f;
+                        if (d < l) x[u] = lds1(rows_at + 4 * (d * pitch + e0 + u)) + 0.0f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc = __fadd_rn(acc, x[u]);
+                }
+            }
+        }
+        if (!copier && strip_touched(acc)) {
+            const uint64_t j = (uint64_t)w0 + (uint32_t)slot;
+            if (j < a.mp.m && j + 1 >= Z) commit_slot<MODE>(a, (uint32_t)j, acc, a.target[j]);
+        }
+    }
+}
+
+inline size_t align_256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+struct StripLayout {
+    size_t lo_of, hi_of, list, total;
+    uint32_t strips, hot_cap, log2w;
+};
+
+StripLayout strip_layout(uint64_t nb, uint32_t m) {
+    StripLayout L;
+    // Long strips (fewer blocks that reach two of them), unless that leaves warps without work
+    L.log2w = kStripMaxLog2;
+    while (L.log2w > kStripMinLog2 && (m >> L.log2w) < 148u * 64u) --L.log2w;
+    L.strips = ((m - 1) >> L.log2w) + 1;
+    const uint64_t cap = 3 * nb / kHotMin + 1;  // (a block of up to 128 elements reaches at most three strips)
+    L.hot_cap = (uint32_t)(cap < L.strips ? cap : L.strips);
+    L.lo_of = 256;  // the counters come first
+    L.hi_of = L.lo_of + align_256(((size_t)L.strips + 1) * sizeof(uint32_t));
+    L.list = L.hi_of + align_256(((size_t)L.strips + 1) * sizeof(uint32_t));
+    L.total = L.list + align_256((size_t)L.hot_cap * sizeof(uint32_t));
+    return L;
+}
+
+template <int MODE, int LP, int EPL, bool SHORT>
+void launch_strip_kernels(const StripArgs& a, cudaStream_t st, cudaStream_t hot_st) {
+    const size_t hot_smem = (size_t)kHotBufs * kHotCopiers * (a.hot_entries + 4) * a.mp.Z * sizeof(float);
+    if (hot_smem > 36 * 1024)  // (with the static part above the default limit)
+        cudaFuncSetAttribute(strip_hot_kernel<MODE, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hot_smem);
+    uint32_t hot_grid = 148 * 3;
+    if (hot_grid > a.hot_cap) hot_grid = a.hot_cap;
+    strip_hot_kernel<MODE, SHORT><<<hot_grid, 32 * (kHotCopiers + kHotAdders), hot_smem, hot_st>>>(a);
+    const uint32_t per_cta = kStripWarps * (32 / LP);
+    const size_t smem = ((size_t)per_cta << a.log2w) * sizeof(float);
+    strip_apply_kernel<MODE, LP, EPL, SHORT><<<(a.strips + per_cta - 1) / per_cta, 32 * kStripWarps, smem, st>>>(a);
+}
+
+template <int MODE, bool SHORT>
+void launch_strip_lanes(const StripArgs& a, cudaStream_t st, cudaStream_t hot_st) {
+    if (a.mp.Z <= 8) launch_strip_kernels<MODE, 8, 1, SHORT>(a, st, hot_st);
+    else if (a.mp.Z <= 16) launch_strip_kernels<MODE, 16, 1, SHORT>(a, st, hot_st);
+    else if (a.mp.Z <= 32) launch_strip_kernels<MODE, 32, 1, SHORT>(a, st, hot_st);
+    else if (a.mp.Z <= 64) launch_strip_kernels<MODE, 32, 2, SHORT>(a, st, hot_st);
+    else launch_strip_kernels<MODE, 32, 4, SHORT>(a, st, hot_st);
+}
+
+template <int MODE>
+void launch_strip_mode(const StripArgs& a, cudaStream_t st, cudaStream_t hot_st) {
+    if (a.mp.d % a.mp.Z != 0) launch_strip_lanes<MODE, true>(a, st, hot_st);
+    else launch_strip_lanes<MODE, false>(a, st, hot_st);
+}
+
+StripArgs strip_args(const StripProblem& sp) {
+    const MapParams& mp = sp.mp;
+    const StripLayout L = strip_layout(sp.nb, mp.m);
+    char* ws = (char*)sp.workspace;
+    auto aligned = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
+    StripArgs a{};
+    a.mp = mp;
+    a.grad_out = sp.grad_out;
+    a.target = sp.target;
+    a.lr = sp.lr;
+    a.adam = sp.adam;
+    a.K = sp.K;
+    a.V = sp.V;
+    a.status = sp.status;
+    a.lo_of = (const uint32_t*)(ws + L.lo_of);
+    a.hi_of = (const uint32_t*)(ws + L.hi_of);
+    a.strips = L.strips;
+    a.log2w = L.log2w;
+    a.hot_count = (uint32_t*)ws;
+    a.hot_list = (uint32_t*)(ws + L.list);
+    a.hot_cap = L.hot_cap;
+    a.hot_entries = mp.Z <= 32 ? 32 : (mp.Z <= 64 ? 16 : 8);
+    a.hot_magic = mp.Z == 1 ? 0u : (uint32_t)((0x100000000ull + mp.Z - 1) / mp.Z);
+    a.vec_commit = aligned(sp.target) && aligned(sp.adam.m1) && aligned(sp.adam.m2);
+    a.grad_elems = sp.grad_elems;
+    // hot: twice the average number of blocks, and enough of them to be worth a CTA (26 x 16384 Zipf rows on
+    // 540 K slots, twice / four times: 34 / 53 us beside the hot kernel's 50; a floor of 128 blocks instead
+    // of 256 made a 250 M-slot array 3 % slower, 512 none faster)
+    const uint64_t mean = (uint64_t)((double)((1u << L.log2w) + mp.Z) * (double)sp.nb / mp.m) + 1;
+    const uint64_t hot = mean * 2 > kHotMin ? mean * 2 : kHotMin;
+    a.n_hot = (uint32_t)(hot < 0x20000000ull ? hot : 0x20000000ull);
+    return a;
+}
+
+}  // namespace
+
+// Strips pay when most slots are reached, so that walking every strip is no waste.  (Positions advance by up
+// to a few hundred in 32 bits: nb stays a little below 2^32.)
+bool strips_ok(const MapParams& mp, uint64_t nb, bool sign) {
+    return !sign && mp.Z <= kStripMaxZ && nb != 0 && nb < 0xFFFFF000ull && nb * mp.Z * 2 >= mp.m;
+}
+
+size_t strips_workspace_bytes(const MapParams& mp, uint64_t nb) { return strip_layout(nb, mp.m).total; }
+
+void launch_strips_prepare(const StripProblem& sp, cudaStream_t st) {
+    const StripLayout L = strip_layout(sp.nb, sp.mp.m);
+    char* ws = (char*)sp.workspace;
+    cudaMemsetAsync(ws, 0, 3 * sizeof(uint32_t), st);
+    strip_bounds_kernel<<<(unsigned)(sp.nb / 2048 + 1), 256, 0, st>>>(
+        sp.K, sp.nb, (uint32_t*)(ws + L.lo_of), (uint32_t*)(ws + L.hi_of), L.strips, L.log2w, sp.mp.Z - 1, sp.status);
+}
+
+void launch_strips(const StripProblem& sp, int mode, cudaStream_t st, cudaStream_t hot_st) {
+    const StripArgs a = strip_args(sp);
+    strip_hot_list_kernel<<<(a.strips + 255) / 256, 256, 0, hot_st>>>(a);
+    if (mode == 4) launch_strip_mode<3>(a, st, hot_st);
+    else if (mode == 2) launch_strip_mode<2>(a, st, hot_st);
+    else if (mode == 1) launch_strip_mode<1>(a, st, hot_st);
+    else launch_strip_mode<0>(a, st, hot_st);
+}
+
+}  // namespace robe

@@ -500,6 +500,28 @@ def test_deterministic_window_apply(case):
         assert_bits_equal(c.array.cpu().numpy(), want, "window apply, SGD")
 
 
+# The strips that arrays of this kind are cut into, at the sizes where they can go wrong: every lane group
+# (blocks of up to 8, 16, 32, 64, 128 elements), short last blocks, blocks longer than a strip, arrays of a
+# few slots, ids repeated so often that whole steps, parts of steps or only mixed lots of a strip's blocks
+# are repeats.
+STRIP_CASES = [
+    dict(d=16, Z=8, M=40_003, batch=5000, vocab_arg=(3, 40, 10**6), id_dist="zipf1.05"),
+    dict(d=20, Z=8, M=40_003, batch=5000, vocab_arg=(3, 40, 10**6), id_dist="zipf1.05"),
+    dict(d=53, Z=32, M=30_011, batch=3000, vocab_arg=(3, 700, 10**6), id_dist="zipf1.05"),
+    dict(d=64, Z=64, M=50_007, batch=3000, vocab_arg=(5, 10**5, 10**6)),
+    dict(d=100, Z=48, M=50_007, batch=2000, vocab_arg=(2, 10**5, 10**6), id_dist="zipf1.05"),
+    dict(d=128, Z=100, M=50_008, batch=2500, vocab_arg=(2, 30, 10**6)),
+    dict(d=128, Z=128, M=129, batch=300, vocab_arg=(2, 30, 10**6)),
+    dict(d=6, Z=3, M=7, batch=700, vocab_arg=(2, 30, 10**6)),
+    dict(d=33, Z=1, M=65, batch=90, vocab_arg=(4, 30, 10**6)),
+]
+
+
+@pytest.mark.parametrize("case", STRIP_CASES, ids=lambda k: f"d{k['d']}_Z{k['Z']}_M{k['M']}")
+def test_deterministic_strips(case):
+    test_deterministic_window_apply(case)
+
+
 # robe_forward_keep + robe_backward_kept: one hash of every id per training step.  The pair must
 # give what robe_forward and robe_backward give: the forward bit for bit, the deterministic
 # backward bit for bit, the binned and atomic ones within the atomic bound.  Shapes: rows of every
