@@ -581,13 +581,23 @@ cudaError_t launch_forward(const Problem& pb, float* out, int variant, cudaStrea
         // the flat kernel is ahead (150 against 156, but 266 against 240 where nothing repeats), and a
         // few thousand rows hold too few repeats.
         if (pb.mp.C > 16 && pb.nbags >= 32768 && rows_ok(pb)) return launch_forward_rows(pb, out, st);
-        // Otherwise the flat kernel, except where the staged one measured ahead of it: bf16 arrays with
-        // rows of 64 or 128 (477 against 505 us, 131072 x 26 rows, Z = 32) and rows that fill three
-        // quarters of the staged kernel's lanes with a short last block (d = 100, Z = 32: 74 against 78).
+        // Otherwise the flat kernel, except where the staged one measured ahead of it in large calls
+        // (B200, us, flat / staged):
+        //   rows of 64 or 128, several blocks each: 26 x 4096 rows, d = 128, Z = 32, 100 MB 22.9 / 20.8;
+        //     7 x 38574, d = 64, Z = 32, 29.1 / 26.4; 26 x 131072, Z = 32, 10 GB 753 / 742; bf16 arrays
+        //     505 / 477 - but not blocks of 8 on a small fp32 array (26 x 32768, d = 128, 2 MB 118 / 126)
+        //   rows of 32 on an array beyond the L2: 7 x 38574, Z = 8, 1 GB 38.6 / 34.1 (100 MB 23.2 / 24.8)
+        //   a short last block, where rows fill three quarters of the staged kernel's lanes (d = 100,
+        //     Z = 32 78 / 74), or half of them on a small array (7 x 38574, d = 73, Z = 32, 2 MB 31 / 26;
+        //     100 MB, 26 x 32768 103 / 107)
         const uint32_t lanes = pb.mp.d <= 32 ? 32u : (pb.mp.d <= 64 ? 64u : 128u);
         const bool ragged = pb.mp.d % pb.mp.Z != 0;
-        const bool staged = warp_ok && pb.nbags >= 32768 &&
-                            ((pb.dtype != 0 && pb.mp.d % 64 == 0) || (ragged && 4 * pb.mp.d >= 3 * lanes));
+        const bool few = (uint64_t)pb.mp.m * (pb.dtype == 0 ? 4u : 2u) <= (16ull << 20);
+        bool staged = false;
+        if (ragged) staged = 4 * pb.mp.d >= 3 * lanes || (few && 2 * pb.mp.d >= lanes);
+        else if (pb.mp.d == 64 || pb.mp.d == 128) staged = pb.dtype != 0 || (pb.mp.C > 1 && pb.mp.Z >= (few ? 16u : 8u));
+        else if (pb.mp.d == 32) staged = !l2_sized && pb.mp.C > 1 && pb.mp.Z >= 8;
+        staged = staged && warp_ok && pb.nbags >= (ragged || pb.dtype != 0 ? 32768 : 65536);
         if (!staged && flat_ok(pb)) return launch_forward_flat(pb, out, st);
     }
     const bool use_warp = variant == 2 || (variant == 0 && warp_ok);
