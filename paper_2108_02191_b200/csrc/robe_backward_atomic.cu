@@ -548,6 +548,7 @@ cudaError_t launch_backward_atomic(const Problem& pb, const float* grad_out, flo
             return launch_backward_rows(pb, grad_out, target, scale, st);
         if (flat_ok(pb)) return launch_backward_flat(pb, grad_out, target, scale, st);
     }
+    if (variant == 0 && bags && pool_ok(pb, true)) return launch_backward_pool(pb, grad_out, target, scale, st);
     const bool use_warp = variant == 2 || (variant == 0 && warp_ok);
     if (use_warp) {
         launch_bwd_staged_epl(a, bags, pb.sign != 0, st);

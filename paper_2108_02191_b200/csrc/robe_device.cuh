@@ -167,6 +167,14 @@ __device__ __forceinline__ float sign_of(const MapParams& mp, uint64_t gbase, ui
     return (t & 1ull) ? 1.0f : -1.0f;
 }
 
+// g(e,x,i) * v, given the sign-hash base of (e,x) and gterm = (C_g i) mod P: the sum of the two reduced
+// mod P loses the odd number P where it reaches it, i.e. flips its parity; an even one negates v.
+__device__ __forceinline__ float with_sign(uint64_t gbase, uint64_t gterm, float v) {
+    const uint64_t t = gbase + gterm;
+    const uint32_t odd = ((uint32_t)t ^ (t >= kP61 ? 1u : 0u)) & 1u;
+    return __uint_as_float(__float_as_uint(v) ^ ((odd ^ 1u) << 31));
+}
+
 // chunk id and in-chunk offset of element i
 __device__ __forceinline__ void chunk_of(const MapParams& mp, uint32_t i, uint32_t& c, uint32_t& o) {
     if (mp.log2Z != 0xFFFFFFFFu) {

@@ -600,6 +600,11 @@ cudaError_t launch_forward(const Problem& pb, float* out, int variant, cudaStrea
         staged = staged && warp_ok && pb.nbags >= (ragged || pb.dtype != 0 ? 32768 : 65536);
         if (!staged && flat_ok(pb)) return launch_forward_flat(pb, out, st);
     }
+    if (variant == 0 && bags && pool_ok(pb, false)) {
+        if (kept != nullptr) *kept = keep_keys != nullptr;
+        if (keep_keys != nullptr) keep_gaps_kernel<<<8, 256, 0, st>>>(a);
+        return launch_forward_pool(pb, out, keep_keys, keep_vals, st);
+    }
     const bool use_warp = variant == 2 || (variant == 0 && warp_ok);
     if (use_warp) {
         if (kept != nullptr) *kept = keep_keys != nullptr;  // (the direct kernel keeps nothing)

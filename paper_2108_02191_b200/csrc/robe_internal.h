@@ -45,6 +45,11 @@ cudaError_t launch_forward_rows(const Problem& pb, float* out, cudaStream_t st);
 cudaError_t launch_backward_rows(const Problem& pb, const float* grad_out, float* target, float scale,
                                  cudaStream_t st);
 
+// pooled rows of short bags, a run of bags per warp (robe_pool.cu); the forward keeps block starts when asked
+bool pool_ok(const Problem& pb, bool backward);
+cudaError_t launch_forward_pool(const Problem& pb, float* out, uint32_t* keep_keys, uint32_t* keep_vals, cudaStream_t st);
+cudaError_t launch_backward_pool(const Problem& pb, const float* grad_out, float* target, float scale, cudaStream_t st);
+
 // atomic backward: adds scale * g * grad_out into target (fp32 [M])
 cudaError_t launch_backward_atomic(const Problem& pb, const float* grad_out, float* target,
                                    float scale, int variant, cudaStream_t st);

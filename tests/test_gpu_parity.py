@@ -353,6 +353,34 @@ def test_large_one_hot_batches(d, Z, M, table_major):
                           delta64.astype(np.float32), "backward, integer gradient")
 
 
+# A run of short bags per warp: runs that end inside the last warp, empty bags at either end of a run and in
+# rows, bags that go on over several batches of staged ids, one element and 128 per row, arrays that wrap,
+# rows clubbed into one block, and offsets that are no stretch (a warp then takes its bags one by one).
+@pytest.mark.parametrize("d,Z,M", [(16, 8, 4099), (1, 1, 5), (33, 4, 70), (64, 16, 100_003), (100, 32, 1013), (128, 128, 128),
+                                   (128, 1, 4099), (16, 64, 1000)])
+@pytest.mark.parametrize("batch,bags", [(8191, (2, 0, 9)), (4001, (1, 0, 300)), (70_000, (1, 0, 4))])
+def test_short_bags(d, Z, M, batch, bags):
+    w = small(d=d, Z=Z, M=M, bag_rule=bags, batch=batch)
+    for sign in (False, True):
+        with Case(w, sign=sign) as c:
+            want = c.oracle_forward()
+            assert_bits_equal(c.forward().cpu().numpy(), want, "forward")
+            g_h, g_d = _grad(c, 21)
+            delta64, l1 = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+            assert_within_l1(c.backward(g_d, "atomic").cpu().numpy(), delta64, l1, what="backward")
+            if batch == 8191:
+                can, _ = c.oracle.backward_canonical(g_h, c.indices_h, c.offsets_h, c.B)
+                out, det = c.step_sharing_keys(g_d, "det")
+                assert_bits_equal(out.cpu().numpy(), want, "forward that keeps its block starts")
+                assert_bits_equal(det.cpu().numpy(), can, "deterministic on the kept starts")
+                # offsets out of order: bag k holds [off[k], max(off[k], off[k + 1])), as for a warp per bag
+                bad = c.offsets.clone()
+                bad[5:c.nbags - 3:7] = 3
+                c.offsets = bad
+                one = c.forward(2).cpu().numpy()
+                assert_bits_equal(c.forward().cpu().numpy(), one, "offsets out of order")
+
+
 @pytest.mark.parametrize("mode", ["atomic", "det"])
 def test_cfg1_backward_dense_and_sgd(mode):
     for sign in (False, True):
