@@ -167,12 +167,15 @@ __device__ __forceinline__ float sign_of(const MapParams& mp, uint64_t gbase, ui
     return (t & 1ull) ? 1.0f : -1.0f;
 }
 
-// g(e,x,i) * v, given the sign-hash base of (e,x) and gterm = (C_g i) mod P: the sum of the two reduced
-// mod P loses the odd number P where it reaches it, i.e. flips its parity; an even one negates v.
-__device__ __forceinline__ float with_sign(uint64_t gbase, uint64_t gterm, float v) {
-    const uint64_t t = gbase + gterm;
-    const uint32_t odd = ((uint32_t)t ^ (t >= kP61 ? 1u : 0u)) & 1u;
-    return __uint_as_float(__float_as_uint(v) ^ ((odd ^ 1u) << 31));
+// The sign of an element without its product: with gbase the sign-hash base of (e,x) and gterm = (C_g i) mod
+// P, the sum of the two reduced mod P loses the odd number P where it reaches it, i.e. flips its parity; an
+// even one negates.  Kept per id: P - gbase (whose parity is the other one) ..
+__device__ __forceinline__ uint64_t sign_limit(uint64_t gbase) { return kP61 - gbase; }
+// .. and per element gterm and its parity as a sign bit; +- v from the three.
+__device__ __forceinline__ float with_sign(uint64_t limit, uint64_t gterm, uint32_t gparity, float v) {
+    // negated where parity(gbase) ^ parity(gterm) ^ [gterm >= limit] is even; parity(gbase) = !parity(limit)
+    const uint32_t bits = __float_as_uint(v) ^ gparity ^ ((uint32_t)limit << 31);
+    return __uint_as_float(gterm >= limit ? bits ^ 0x80000000u : bits);
 }
 
 // chunk id and in-chunk offset of element i

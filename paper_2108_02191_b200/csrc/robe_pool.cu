@@ -14,6 +14,7 @@ namespace robe {
 namespace {
 
 constexpr uint32_t kPoolBags = 16;  // bags per warp, at most
+constexpr int kPoolCtas = 5, kPoolCtasSign = 4;  // per SM
 
 struct PoolArgs {
     MapParams mp;
@@ -69,7 +70,7 @@ __device__ __forceinline__ bool pool_stage(PoolSmem& sm, const PoolArgs& a, int6
                 sm.stage.piece[w][t] = (uint32_t)(x - xh * mp.R) * mp.d;
             }
             base_s[t] = addmod_p61(table_term(mp.h, e), mulmod_p61_any(mp.h.B, xh));
-            if (SIGN) gbase_s[t] = addmod_p61(table_term(mp.g, e), mulmod_p61_any(mp.g.B, x));
+            if (SIGN) gbase_s[t] = sign_limit(addmod_p61(table_term(mp.g, e), mulmod_p61_any(mp.g.B, x)));
         }
     }
     __syncwarp();
@@ -151,7 +152,7 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
                 uint32_t j = l.col[u][g0 + g] + l.off[u];
                 if (wraps && j >= mp.m) j -= mp.m;
                 if ((FULL || (uint32_t)g < n) && l.live[u] && ROBE_CHK(j < mp.m, ROBE_DBG_ARRAY_SLOT))
-                    red_add(a.io + j, SIGN ? with_sign(gbase_s[g0 + g], l.gelem[u], l.acc[u]) : l.acc[u], pol);
+                    red_add(a.io + j, SIGN ? with_sign(gbase_s[g0 + g], l.gelem[u], (uint32_t)l.gelem[u] << 31, l.acc[u]) : l.acc[u], pol);
             }
         }
     } else {
@@ -171,7 +172,7 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
             if (!FULL && (uint32_t)g >= n) break;
 #pragma unroll
             for (int u = 0; u < EPL; ++u)
-                l.acc[u] = l.acc[u] + (SIGN ? with_sign(gbase_s[g0 + g], l.gelem[u], v[g][u]) : v[g][u]);
+                l.acc[u] = l.acc[u] + (SIGN ? with_sign(gbase_s[g0 + g], l.gelem[u], (uint32_t)l.gelem[u] << 31, v[g][u]) : v[g][u]);
             if ((bag[g] & kPoolLast) != 0) {
                 float* orow = a.io + (k0 + (bag[g] & ~kPoolLast)) * (int64_t)mp.d + lane;
 #pragma unroll
@@ -186,7 +187,7 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
 
 // MODE 0: forward, fp32 array; 1: forward, bf16 array; 2: backward
 template <int MODE, int EPL, bool SIGN>
-__global__ void __launch_bounds__(256, SIGN ? 4 : 5)
+__global__ void __launch_bounds__(256, SIGN ? kPoolCtasSign : kPoolCtas)
 pool_kernel(PoolArgs a) {
     __shared__ PoolSmem sm;
     const MapParams& mp = a.mp;
@@ -279,6 +280,12 @@ uint32_t pool_bags(const Problem& pb, bool backward) {
     int64_t bags = ids / mean;
     const int64_t spread = pb.nbags / (148 * 40) + 1;
     if (bags > spread) bags = spread;
+    // a last wave that is nearly empty costs a whole one: rather a bag more per warp
+    const int64_t wave = 148 * 8 * (pb.sign != 0 ? kPoolCtasSign : kPoolCtas);
+    if (bags > 1) {
+        const int64_t waves = ((pb.nbags + bags - 1) / bags + wave / 2) / wave;
+        if (waves >= 1 && waves <= 3) bags = (pb.nbags + waves * wave - 1) / (waves * wave);
+    }
     if (bags > (int64_t)kPoolBags) bags = kPoolBags;
     return bags < 1 ? 1u : (uint32_t)bags;
 }

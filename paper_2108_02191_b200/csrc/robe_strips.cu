@@ -35,7 +35,8 @@ constexpr int kStripWarps = 8;
 constexpr uint32_t kStripMaxZ = 128;
 constexpr int kHotCopiers = 8;            // warps of the hot kernel that copy
 constexpr int kHotAdders = 8;             // and that add: 32 slots each
-constexpr uint32_t kHotBufs = 3;          // steps staged: one being added, two on their way
+constexpr uint32_t kHotAhead = 3;         // steps that the copies, and again as many that the keys, are asked for ahead
+constexpr uint32_t kHotBufs = kHotAhead + 1;
 constexpr uint32_t kHotMin = 256;         // a strip is hot from this many blocks on, at least
 
 struct StripArgs {
@@ -54,15 +55,44 @@ struct StripArgs {
     uint32_t* hot_count;       // [0] strips at the front of the list, [1] at its back, [2] taken
     uint32_t* hot_list;
     uint32_t hot_cap;
-    uint32_t hot_entries;      // blocks copied at a time by a warp: 32, 16 or 8
-    uint32_t hot_magic;        // ceil(2^32 / Z); 0: Z is 1
     int vec_commit;            // target and moments are 16-byte aligned
     uint64_t grad_elems;       // of grad_out (read by the debug build's index checks only)
 };
 
 constexpr uint32_t kBoundsGap = 256;  // longer gaps are filled by the whole warp
 
-// lo_of and hi_of for b = 0 .. strips.  A thread takes eight sorted positions; position i begins the strips
+// lo_of and hi_of for b = 0 .. strips, for many strips: a thread per strip, by a bisection that shares all but its
+// last steps with its neighbours', and a gallop back from there for lo_of.  34 M keys, 977 K strips: 58 us
+// against 90 of the scan below; 852 K keys, 8437 strips: 12 (a warp per strip, 32 probes at a time: 7)
+// against 5.
+__global__ void __launch_bounds__(256)
+strip_bounds_search_kernel(const uint32_t* __restrict__ K, uint32_t nb, uint32_t* __restrict__ lo_of,
+                           uint32_t* __restrict__ hi_of, uint32_t strips, uint32_t log2w, uint32_t reach,
+                           const int32_t* status) {
+    if (status != nullptr && *status != 0) return;  // after a failed input check K was not written
+    const uint32_t b = blockIdx.x * 256 + threadIdx.x;
+    if (b > strips) return;
+    // first position in [from, to] whose key is at least `least`: the keys before `from` are below it, that of
+    // `to` (or what lies past the list) is not
+    auto search = [&](uint32_t from, uint32_t to, uint64_t least) {
+        while (from < to) {
+            const uint32_t mid = from + ((to - from) >> 1);
+            if ((uint64_t)__ldg(K + mid) >= least) to = mid; else from = mid + 1;
+        }
+        return from;
+    };
+    const uint64_t first_slot = (uint64_t)b << log2w, least = first_slot > reach ? first_slot - reach : 0;
+    const uint32_t hi = search(0, nb, first_slot);
+    uint32_t to = hi, step = 1;
+    while (to >= step && (uint64_t)__ldg(K + (to - step)) >= least) {
+        to -= step;
+        step <<= 1;  // (the steps add up to less than nb)
+    }
+    hi_of[b] = hi;
+    lo_of[b] = search(to >= step ? to - step + 1 : 0, to, least);
+}
+
+// The same for few strips, by reading the list.  A thread takes eight sorted positions; position i begins the strips
 // whose first slot lies past the key before it and not past its own (lo_of: the same of the blocks' last slots).
 __global__ void __launch_bounds__(256)
 strip_bounds_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* __restrict__ lo_of,
@@ -159,6 +189,9 @@ __device__ __forceinline__ uint32_t strip_len(const MapParams& mp, uint32_t v) {
 }
 
 __device__ __forceinline__ bool strip_touched(float sum) { return __float_as_uint(sum) != 0x80000000u; }
+
+// blocks that a copying warp of the hot kernel takes at a time, by the elements per lane of a block
+__host__ __device__ constexpr uint32_t hot_blocks(int epl) { return epl == 1 ? 32u : (epl == 2 ? 16u : 8u); }
 
 template <int MODE, int LP, int EPL, bool SHORT>
 __global__ void __launch_bounds__(32 * kStripWarps, 5)
@@ -274,14 +307,13 @@ __device__ __forceinline__ float add4(float acc, const float4 x) {
     return __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(acc, x.x), x.y), x.z), x.w);
 }
 
-// acc + one slot's terms of `units` times eight blocks, in order: units of 32 bytes at `at`, `per_chunk` (a power
-// of two) of them side by side and `skip` bytes on to the next chunk.  The reads run a unit ahead of the adds.
-__device__ __forceinline__ float hot_add_units(float acc, uint32_t at, uint32_t units, uint32_t per_chunk, uint32_t skip) {
+// acc + one slot's terms of n blocks side by side at `at`, n a multiple of eight; the reads of eight run ahead
+// of the adds of the eight before
+__device__ __forceinline__ float hot_add_chunk(float acc, uint32_t at, uint32_t n) {
     float4 x = lds4(at), y = lds4(at + 16);
 #pragma unroll 4
-    for (uint32_t u = 1; u < units; ++u) {
+    for (uint32_t e = 8; e < n; e += 8) {
         at += 32;
-        if ((u & (per_chunk - 1)) == 0) at += skip;
         const float4 x1 = lds4(at), y1 = lds4(at + 16);
         acc = add4(add4(acc, x), y);
         x = x1;
@@ -290,26 +322,51 @@ __device__ __forceinline__ float hot_add_units(float acc, uint32_t at, uint32_t 
     return add4(add4(acc, x), y);
 }
 
+// The same for `pairs` times two lots of 16 blocks, the second `odd` bytes after the first, the next pair `step`
+// bytes on: 16 reads ahead and nothing else inside (the chain of adds is what this loop should wait for).
+__device__ __forceinline__ float hot_add_step(float acc, uint32_t at, uint32_t pairs, uint32_t odd, uint32_t step) {
+    float4 x[4], y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = lds4(at + 16 * u);
+#pragma unroll 2
+    for (uint32_t c = 0; c < pairs; ++c) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) y[u] = lds4(at + odd + 16 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = add4(acc, x[u]);
+        if (c + 1 < pairs) at += step;  // (else the last lot again, not used)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = lds4(at + 16 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = add4(acc, y[u]);
+    }
+    return acc;
+}
+
 // Hot strips.  The chain of dependent adds of a slot is the definition's, and one warp's issue is what it
 // costs beyond that: the copies are laid out slot by slot, so that a lane reads four blocks' terms at once,
 // and a whole step of repeats of one start is one loop.  One barrier per step of eight copiers' blocks,
-// whose copies were issued two steps ahead.
-// Measured (B200, ns per repeat of one start): 9.3 with a row per block, 4 here; the chain itself: 2.1.
-template <int MODE, bool SHORT>
-__global__ void __launch_bounds__(32 * (kHotCopiers + kHotAdders))
+// whose copies were issued three steps ahead.
+// Measured (B200, ns per repeat of one start): 9.3 with a row per block, 4.1 with divisions and a pass over all
+// blocks in the copiers, 3.7 here (of a step, 1308 clocks are adds, 330 what stands before them); the chain itself: 2.1.
+template <int MODE, int LP, int EPL, bool SHORT>
+__global__ void __launch_bounds__(32 * (kHotCopiers + kHotAdders), 2)
 strip_hot_kernel(StripArgs a) {
     extern __shared__ float4 strip_smem[];
     __shared__ int2 ent_s[kHotBufs][kHotCopiers][32];  // (start relative to the strip, length) of each block
     __shared__ int4 all_s[kHotBufs][kHotCopiers];      // of the blocks of one copier: their number; all alike? start, length
+    __shared__ uint2 keys_s[2 * kHotBufs][kHotCopiers][32];  // (start, payload) of steps yet to be copied
     __shared__ uint32_t item_s;
     if (a.status != nullptr && *a.status != 0) return;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const bool copier = w >= (uint32_t)kHotAdders;
     const uint32_t cw = w - kHotAdders;
-    const uint32_t Z = a.mp.Z, W = 1u << a.log2w, E = a.hot_entries, per_step = E * kHotCopiers;
+    const uint32_t Z = a.mp.Z, W = 1u << a.log2w;
+    constexpr uint32_t E = hot_blocks(EPL), per_step = E * kHotCopiers;
     const uint32_t n_front = a.hot_count[0], n_items = n_front + a.hot_count[1];
     float* const stage = reinterpret_cast<float*>(strip_smem);
-    const uint32_t pitch = E + 4, chunk = pitch * Z;  // element o of block e at o * pitch + e
+    constexpr uint32_t pitch = E + 4;  // element o of block e at o * pitch + e
+    const uint32_t chunk = pitch * Z;
     for (;;) {
         __syncthreads();  // item_s and the buffers are free
         if (threadIdx.x == 0) item_s = atomicAdd(a.hot_count + 2, 1u);
@@ -320,20 +377,25 @@ strip_hot_kernel(StripArgs a) {
         const uint32_t w0 = b << a.log2w;
         const uint32_t lo = a.lo_of[b], n = a.hi_of[b + 1] - lo;
         const uint32_t steps = (n + per_step - 1) / per_step;
-        uint32_t k = 0, v = 0;  // copiers: the block of this lane in the step to be copied next
         // blocks of this copier in step s: positions from lo + s*per_step + cw*E, this many
+        const uint32_t share = n > cw * E ? n - cw * E : 0u;
         auto count = [&](uint32_t s) -> uint32_t {
-            const uint64_t at = (uint64_t)s * per_step + cw * E;
-            return at >= n ? 0u : (n - at < E ? (uint32_t)(n - at) : E);
+            const uint32_t before = s * per_step;  // (the steps asked about end at most six past the last)
+            return before >= share ? 0u : (share - before < E ? share - before : E);
         };
+        // The keys of this lane's block of step s, and the elements of the blocks of step s: one group of copies
+        // per step has the elements kHotAhead steps ahead of what is added and the keys as much again ahead.
         auto fetch = [&](uint32_t s) {
             if (lane < count(s)) {
                 const uint32_t at = lo + s * per_step + cw * E + lane;
-                k = __ldg(a.K + at);
-                v = __ldg(a.V + at);
+                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&keys_s[s % (2 * kHotBufs)][cw][lane]);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(a.K + at) : "memory");
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4), "l"(a.V + at) : "memory");
             }
         };
-        auto copy = [&](uint32_t s) {  // one commit group per call
+        auto copy = [&](uint32_t s) {
+            const uint2 kv = keys_s[s % (2 * kHotBufs)][cw][lane];
+            const uint32_t k = kv.x, v = kv.y;
             const uint32_t ne = count(s);
             float* const rows = stage + ((s % kHotBufs) * kHotCopiers + cw) * chunk;
             const int rel = (int)(k - w0);
@@ -342,40 +404,63 @@ strip_hot_kernel(StripArgs a) {
             const int rel0 = __shfl_sync(0xFFFFFFFFu, rel, 0), len0 = __shfl_sync(0xFFFFFFFFu, len, 0);
             const bool alike = __all_sync(0xFFFFFFFFu, lane >= ne || (rel == rel0 && len == len0));
             if (lane == 0) all_s[s % kHotBufs][cw] = make_int4((int)ne, alike ? 1 : 0, rel0, len0);
-            const uint32_t total = ne * Z;
-            for (uint32_t t0 = 0; t0 < total; t0 += 32) {
-                const uint32_t t = t0 + lane, e = a.hot_magic != 0 ? __umulhi(t, a.hot_magic) : t, o = t - e * Z;
-                const int r = __shfl_sync(0xFFFFFFFFu, rel, e);
-                const uint32_t p = __shfl_sync(0xFFFFFFFFu, v, e) + o;
-                const uint32_t l = SHORT ? (uint32_t)__shfl_sync(0xFFFFFFFFu, len, e) : Z;
-                const int first = r + (int)o;
-                if (t < total && first >= 0 && first < (int)W && o < l && ROBE_CHK(p < a.grad_elems, ROBE_DBG_GRAD_POS)) {
-                    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(rows + o * pitch + e);
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(a.grad_out + p) : "memory");
+            // lane: element lane % LP (+ 32, ..) of every (32 / LP)-th block
+            constexpr uint32_t G = 32 / LP;
+            const uint32_t o0 = lane % LP, e0 = lane / LP;
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(rows + o0 * pitch + e0);
+            if (alike && ne == E) {  // the same elements of every block are wanted
+                bool on[EPL];
+#pragma unroll
+                for (int i = 0; i < EPL; ++i)
+                    on[i] = o0 + 32 * i < (uint32_t)len0 && (uint32_t)rel0 + o0 + 32 * i < W;
+#pragma unroll
+                for (uint32_t q = 0; q < E / G; ++q) {
+                    const uint32_t p = __shfl_sync(0xFFFFFFFFu, v, e0 + q * G) + o0;
+#pragma unroll
+                    for (int i = 0; i < EPL; ++i)
+                        if (on[i] && ROBE_CHK((uint64_t)p + 32 * i < a.grad_elems, ROBE_DBG_GRAD_POS))
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * (q * G + 32 * i * pitch)),
+                                         "l"(a.grad_out + (p + 32 * i))
+                                         : "memory");
+                }
+            } else {
+#pragma unroll 4
+                for (uint32_t q = 0; q < E / G; ++q) {
+                    if (q * G >= ne) break;  // (warp-uniform)
+                    const uint32_t e = e0 + q * G;
+                    const uint32_t r = __shfl_sync(0xFFFFFFFFu, (uint32_t)rel, e), p = __shfl_sync(0xFFFFFFFFu, v, e) + o0;
+                    const uint32_t l = (uint32_t)__shfl_sync(0xFFFFFFFFu, len, e);  // (0 past the last block)
+#pragma unroll
+                    for (int i = 0; i < EPL; ++i)
+                        if (o0 + 32 * i < l && r + o0 + 32 * i < W &&
+                            ROBE_CHK((uint64_t)p + 32 * i < a.grad_elems, ROBE_DBG_GRAD_POS))
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * (q * G + 32 * i * pitch)),
+                                         "l"(a.grad_out + (p + 32 * i))
+                                         : "memory");
                 }
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
         };
+        auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
         if (copier) {
-            fetch(0);
-            copy(0);
-            fetch(1);
-            if (steps > 1) copy(1);
-            fetch(2);
+            for (uint32_t s = 0; s < kHotAhead; ++s) fetch(s);
+            commit();
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            for (uint32_t s = 0; s < kHotAhead; ++s) {
+                if (s < steps) copy(s);
+                fetch(s + kHotAhead);
+                commit();
+            }
         }
         const int slot = (int)(32 * w + lane);  // adders: within the strip
         float acc = -0.0f;
         for (uint32_t s = 0; s < steps; ++s) {
-            if (copier) {
-                if (s + 1 < steps) asm volatile("cp.async.wait_group 1;" ::: "memory");
-                else asm volatile("cp.async.wait_group 0;" ::: "memory");
-            }
+            // (the group of step s has the elements of step s and the keys of step s + kHotAhead)
+            if (copier) asm volatile("cp.async.wait_group %0;" ::"n"(kHotAhead - 1) : "memory");
             __syncthreads();  // step s is in; step s - 1 has been added
             if (copier) {
-                if (s + 2 < steps) {
-                    copy(s + 2);
-                    fetch(s + 3);
-                }
+                if (s + kHotAhead < steps) copy(s + kHotAhead);
+                fetch(s + 2 * kHotAhead);
+                commit();
                 continue;
             }
             if (32 * w >= W) continue;
@@ -384,8 +469,14 @@ strip_hot_kernel(StripArgs a) {
             if (__all_sync(0xFFFFFFFFu, its.x == (int)E && its.y != 0 && its.z == lead.z && its.w == lead.w)) {
                 // a whole step of repeats (-0 turns +0 at the first term: see strip_apply_kernel)
                 const uint32_t d = (uint32_t)(slot - lead.z);
-                if (d < (uint32_t)lead.w)
-                    acc = hot_add_units(acc + 0.0f, stage_at + 4 * pitch * d, kHotCopiers * (E / 8), E / 8, 4 * (chunk - E));
+                if (d < (uint32_t)lead.w) {
+                    const uint32_t at = stage_at + 4 * pitch * d;
+                    acc += 0.0f;
+                    if (E == 32) acc = hot_add_step(acc, at, kHotCopiers, 64, 4 * chunk);
+                    else if (E == 16) acc = hot_add_step(acc, at, kHotCopiers / 2, 4 * chunk, 8 * chunk);
+                    else
+                        for (uint32_t c = 0; c < (uint32_t)kHotCopiers; ++c) acc = hot_add_chunk(acc, at + 4 * chunk * c, E);
+                }
                 continue;
             }
             for (uint32_t c = 0; c < (uint32_t)kHotCopiers; ++c) {
@@ -398,7 +489,7 @@ strip_hot_kernel(StripArgs a) {
                     if (d < (uint32_t)all.w) {
                         acc += 0.0f;
                         const uint32_t at = rows_at + 4 * pitch * d;
-                        if (ne >= 8) acc = hot_add_units(acc, at, ne / 8, 32, 0);
+                        if (ne >= 8) acc = hot_add_chunk(acc, at, ne & ~7u);
                         for (uint32_t e = ne & ~7u; e < ne; ++e) acc = __fadd_rn(acc, lds1(at + 4 * e));
                     }
                     __syncwarp();
@@ -420,6 +511,7 @@ strip_hot_kernel(StripArgs a) {
                 }
             }
         }
+        if (copier) asm volatile("cp.async.wait_group 0;" ::: "memory");
         if (!copier && strip_touched(acc)) {
             const uint64_t j = (uint64_t)w0 + (uint32_t)slot;
             if (j < a.mp.m && j + 1 >= Z) commit_slot<MODE>(a, (uint32_t)j, acc, a.target[j]);
@@ -451,12 +543,13 @@ StripLayout strip_layout(uint64_t nb, uint32_t m) {
 
 template <int MODE, int LP, int EPL, bool SHORT>
 void launch_strip_kernels(const StripArgs& a, cudaStream_t st, cudaStream_t hot_st) {
-    const size_t hot_smem = (size_t)kHotBufs * kHotCopiers * (a.hot_entries + 4) * a.mp.Z * sizeof(float);
-    if (hot_smem > 36 * 1024)  // (with the static part above the default limit)
-        cudaFuncSetAttribute(strip_hot_kernel<MODE, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hot_smem);
-    uint32_t hot_grid = 148 * 3;
+    const size_t hot_smem = (size_t)kHotBufs * kHotCopiers * (hot_blocks(EPL) + 4) * a.mp.Z * sizeof(float);
+    if (hot_smem > 23 * 1024)  // (with the static part above the default limit)
+        cudaFuncSetAttribute(strip_hot_kernel<MODE, LP, EPL, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hot_smem);
+    const uint32_t per_sm = (uint32_t)(220 * 1024 / (hot_smem + 26 * 1024));  // (26 KB: the static part and a margin)
+    uint32_t hot_grid = 148 * (per_sm > 2 ? 2 : (per_sm < 1 ? 1 : per_sm));
     if (hot_grid > a.hot_cap) hot_grid = a.hot_cap;
-    strip_hot_kernel<MODE, SHORT><<<hot_grid, 32 * (kHotCopiers + kHotAdders), hot_smem, hot_st>>>(a);
+    strip_hot_kernel<MODE, LP, EPL, SHORT><<<hot_grid, 32 * (kHotCopiers + kHotAdders), hot_smem, hot_st>>>(a);
     const uint32_t per_cta = kStripWarps * (32 / LP);
     const size_t smem = ((size_t)per_cta << a.log2w) * sizeof(float);
     strip_apply_kernel<MODE, LP, EPL, SHORT><<<(a.strips + per_cta - 1) / per_cta, 32 * kStripWarps, smem, st>>>(a);
@@ -498,8 +591,6 @@ StripArgs strip_args(const StripProblem& sp) {
     a.hot_count = (uint32_t*)ws;
     a.hot_list = (uint32_t*)(ws + L.list);
     a.hot_cap = L.hot_cap;
-    a.hot_entries = mp.Z <= 32 ? 32 : (mp.Z <= 64 ? 16 : 8);
-    a.hot_magic = mp.Z == 1 ? 0u : (uint32_t)((0x100000000ull + mp.Z - 1) / mp.Z);
     a.vec_commit = aligned(sp.target) && aligned(sp.adam.m1) && aligned(sp.adam.m2);
     a.grad_elems = sp.grad_elems;
     // hot: twice the average number of blocks, and enough of them to be worth a CTA (26 x 16384 Zipf rows on
@@ -525,8 +616,13 @@ void launch_strips_prepare(const StripProblem& sp, cudaStream_t st) {
     const StripLayout L = strip_layout(sp.nb, sp.mp.m);
     char* ws = (char*)sp.workspace;
     cudaMemsetAsync(ws, 0, 3 * sizeof(uint32_t), st);
-    strip_bounds_kernel<<<(unsigned)(sp.nb / 2048 + 1), 256, 0, st>>>(
-        sp.K, sp.nb, (uint32_t*)(ws + L.lo_of), (uint32_t*)(ws + L.hi_of), L.strips, L.log2w, sp.mp.Z - 1, sp.status);
+    uint32_t *lo_of = (uint32_t*)(ws + L.lo_of), *hi_of = (uint32_t*)(ws + L.hi_of);
+    if (L.strips > 148u * 256u)
+        strip_bounds_search_kernel<<<L.strips / 256 + 1, 256, 0, st>>>(sp.K, (uint32_t)sp.nb, lo_of, hi_of, L.strips,
+                                                                      L.log2w, sp.mp.Z - 1, sp.status);
+    else
+        strip_bounds_kernel<<<(unsigned)(sp.nb / 2048 + 1), 256, 0, st>>>(sp.K, sp.nb, lo_of, hi_of, L.strips, L.log2w,
+                                                                         sp.mp.Z - 1, sp.status);
 }
 
 void launch_strips(const StripProblem& sp, int mode, cudaStream_t st, cudaStream_t hot_st) {
