@@ -16,6 +16,7 @@ constexpr int kApplyVecPerThread = 4;  // float4 pairs in flight per thread
 template <bool ZERO>
 __global__ void __launch_bounds__(kApplyThreads)
 dense_sgd_apply_kernel(float* __restrict__ array, float* __restrict__ grad, uint64_t m, float lr) {
+    follow();
     const uint64_t nvec = m >> 2;
     float4* a4 = reinterpret_cast<float4*>(array);
     float4* g4 = reinterpret_cast<float4*>(grad);
@@ -76,9 +77,9 @@ cudaError_t launch_dense_sgd_apply(float* array, float* grad, uint64_t m, float 
     if (want > cap) want = cap;
     if (want < 1) want = 1;
     if (zero_grad)
-        dense_sgd_apply_kernel<true><<<(unsigned)want, kApplyThreads, 0, st>>>(array, grad, m, lr);
+        launch_next(dense_sgd_apply_kernel<true>, (unsigned)want, kApplyThreads, 0, st, array, grad, m, lr);
     else
-        dense_sgd_apply_kernel<false><<<(unsigned)want, kApplyThreads, 0, st>>>(array, grad, m, lr);
+        launch_next(dense_sgd_apply_kernel<false>, (unsigned)want, kApplyThreads, 0, st, array, grad, m, lr);
     return cudaGetLastError();
 }
 

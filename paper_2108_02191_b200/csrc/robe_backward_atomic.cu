@@ -74,6 +74,7 @@ bwd_atomic_staged_kernel(BwdArgs a, uint32_t ids_per_batch, uint32_t cmagic) {
     const int64_t warp = (int64_t)blockIdx.x * 8 + w;
 
     stage_init(sm, mp);
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
 
     int64_t lo, hi;
@@ -467,9 +468,9 @@ static void launch_bwd_staged_minb(const BwdArgs& a, bool bags, cudaStream_t st)
     const int64_t warps = bags ? a.nbags : (a.nbags + ipb - 1) / ipb;
     const unsigned blocks = (unsigned)((warps + 7) / 8);
     if (bags)
-        bwd_atomic_staged_kernel<EPL, SIGN, true, FULLD, MINB><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
+        launch_next(bwd_atomic_staged_kernel<EPL, SIGN, true, FULLD, MINB>, blocks, 256, 0, st, a, ipb, cmagic);
     else
-        bwd_atomic_staged_kernel<EPL, SIGN, false, FULLD, MINB><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
+        launch_next(bwd_atomic_staged_kernel<EPL, SIGN, false, FULLD, MINB>, blocks, 256, 0, st, a, ipb, cmagic);
 }
 
 template <int EPL, bool SIGN, bool FULLD>
@@ -521,9 +522,9 @@ cudaError_t launch_backward_atomic(const Problem& pb, const float* grad_out, flo
         const int64_t warps = ((batch + ipb - 1) / ipb) * pb.mp.T;
         const unsigned blocks = (unsigned)((warps + 7) / 8);
         const uint32_t cmagic = chunk_magic(a.mp);
-        if (a.mp.d <= 32) bwd_atomic_staged_kernel<1, false, false, false, 6, true><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
-        else if (a.mp.d <= 64) bwd_atomic_staged_kernel<2, false, false, false, 6, true><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
-        else bwd_atomic_staged_kernel<4, false, false, false, 5, true><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
+        if (a.mp.d <= 32) launch_next(bwd_atomic_staged_kernel<1, false, false, false, 6, true>, blocks, 256, 0, st, a, ipb, cmagic);
+        else if (a.mp.d <= 64) launch_next(bwd_atomic_staged_kernel<2, false, false, false, 6, true>, blocks, 256, 0, st, a, ipb, cmagic);
+        else launch_next(bwd_atomic_staged_kernel<4, false, false, false, 5, true>, blocks, 256, 0, st, a, ipb, cmagic);
         return cudaGetLastError();
     }
     if (variant == 3 || variant == 4) {  // 16-byte reductions; 4: duplicates of an id merged first

@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(256) det_bag_of_kernel(KeyArgs a, uint32_t* ba
 template <bool SIGN>
 __global__ void __launch_bounds__(256)
 det_keys_kernel(KeyArgs a, const uint32_t* bag_of, uint32_t* keys, uint32_t* vals) {
+    follow<true>();
     const uint64_t p = (uint64_t)blockIdx.x * 256 + threadIdx.x;
     if (p >= (uint64_t)a.nnz) return;
     const MapParams& mp = a.mp;
@@ -112,6 +113,7 @@ template <bool SIGN>
 __global__ void __launch_bounds__(256)
 det_keys_by_block_kernel(KeyArgs a, const uint32_t* bag_of, uint32_t* keys, uint32_t* vals,
                          uint64_t nb) {
+    follow<true>();
     const uint64_t q = (uint64_t)blockIdx.x * 256 + threadIdx.x;
     if (q >= nb) return;
     const MapParams& mp = a.mp;
@@ -130,6 +132,7 @@ __global__ void __launch_bounds__(kSortThreads)
 sort_count_kernel(const uint32_t* keys, uint32_t* counts, uint64_t nb, uint64_t tiles,
                   uint32_t shift, uint32_t mask) {
     __shared__ uint32_t hist[kSortWarps][kRadix];
+    follow<true>();
     for (int k = threadIdx.x; k < kSortWarps * kRadix; k += kSortThreads) (&hist[0][0])[k] = 0;
     __syncthreads();
     uint64_t first, count;
@@ -171,6 +174,7 @@ __device__ __forceinline__ uint32_t cta_exclusive_scan(uint32_t v, uint32_t* war
 __global__ void __launch_bounds__(kScanThreads)
 sort_scan_kernel(uint32_t* counts, uint32_t* totals, uint32_t grid) {
     __shared__ uint32_t warp_sums[kScanThreads / 32];
+    follow<true>();
     uint32_t* row = counts + (uint64_t)blockIdx.x * grid;
     uint32_t carry = 0;
     for (uint32_t b0 = 0; b0 < grid; b0 += kScanThreads) {
@@ -334,6 +338,7 @@ sort_scatter_kernel(const uint32_t* __restrict__ kin, const uint32_t* __restrict
                     uint32_t nb, uint32_t tiles, uint32_t shift) {
     __shared__ ScatterSmem<STABLE, BITS> sm;
     const uint32_t tid = threadIdx.x;
+    follow<true>();
     {
         // start of this digit in the output = pairs of lower digits + this digit's pairs in
         // lower CTAs
@@ -361,9 +366,9 @@ sort_scatter_kernel(const uint32_t* __restrict__ kin, const uint32_t* __restrict
 template <bool STABLE, int BITS>
 void launch_sort_pass_bits(const SortPlan& sp, const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
                            uint32_t* counts, uint32_t* totals, uint32_t shift, cudaStream_t st) {
-    sort_count_kernel<<<sp.grid, kSortThreads, 0, st>>>(kin, counts, sp.nb, sp.tiles, shift, (1u << BITS) - 1u);
-    sort_scan_kernel<<<1 << BITS, kScanThreads, 0, st>>>(counts, totals, sp.grid);
-    sort_scatter_kernel<STABLE, BITS><<<sp.grid, kSortThreads, 0, st>>>(kin, vin, kout, vout, counts, totals,
+    launch_next(sort_count_kernel, sp.grid, kSortThreads, 0, st, kin, counts, sp.nb, sp.tiles, shift, (1u << BITS) - 1u);
+    launch_next(sort_scan_kernel, 1 << BITS, kScanThreads, 0, st, counts, totals, sp.grid);
+    launch_next(sort_scatter_kernel<STABLE, BITS>, sp.grid, kSortThreads, 0, st, kin, vin, kout, vout, counts, totals,
                                                                        (uint32_t)sp.nb, (uint32_t)sp.tiles, shift);
 }
 
@@ -914,6 +919,7 @@ template <bool SIGN, bool SHORT>
 __global__ void __launch_bounds__(256)
 binned_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V,
                     const uint32_t* __restrict__ bag_of, uint32_t log2Zp) {
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
     const MapParams& mp = a.mp;
     const uint64_t tid = (uint64_t)blockIdx.x * 256 + threadIdx.x;
@@ -1070,12 +1076,12 @@ cudaError_t launch_block_keys(const Problem& pb, void* workspace, size_t workspa
     if (bags) launch_bag_of(pb, L, ws, st);
     if (mp.C <= 8) {
         const unsigned kb = (unsigned)((pb.nnz + 255) / 256);
-        if (pb.sign) det_keys_kernel<true><<<kb, 256, 0, st>>>(ka, bag_of, kA, vA);
-        else det_keys_kernel<false><<<kb, 256, 0, st>>>(ka, bag_of, kA, vA);
+        if (pb.sign) launch_next(det_keys_kernel<true>, kb, 256, 0, st, ka, bag_of, kA, vA);
+        else launch_next(det_keys_kernel<false>, kb, 256, 0, st, ka, bag_of, kA, vA);
     } else {
         const unsigned kb = (unsigned)((nb + 255) / 256);
-        if (pb.sign) det_keys_by_block_kernel<true><<<kb, 256, 0, st>>>(ka, bag_of, kA, vA, nb);
-        else det_keys_by_block_kernel<false><<<kb, 256, 0, st>>>(ka, bag_of, kA, vA, nb);
+        if (pb.sign) launch_next(det_keys_by_block_kernel<true>, kb, 256, 0, st, ka, bag_of, kA, vA, nb);
+        else launch_next(det_keys_by_block_kernel<false>, kb, 256, 0, st, ka, bag_of, kA, vA, nb);
     }
     return cudaGetLastError();
 }
@@ -1127,11 +1133,11 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
         const unsigned blocks = (unsigned)(((groups << log2Zp) + 255) / 256);
         const bool shortb = mp.d % mp.Z != 0;
         if (pb.sign) {
-            if (shortb) binned_apply_kernel<true, true><<<blocks, 256, 0, st>>>(ab, kB, vB, bag_of, log2Zp);
-            else binned_apply_kernel<true, false><<<blocks, 256, 0, st>>>(ab, kB, vB, bag_of, log2Zp);
+            if (shortb) launch_next(binned_apply_kernel<true, true>, blocks, 256, 0, st, ab, kB, vB, bag_of, log2Zp);
+            else launch_next(binned_apply_kernel<true, false>, blocks, 256, 0, st, ab, kB, vB, bag_of, log2Zp);
         } else {
-            if (shortb) binned_apply_kernel<false, true><<<blocks, 256, 0, st>>>(ab, kB, vB, bag_of, log2Zp);
-            else binned_apply_kernel<false, false><<<blocks, 256, 0, st>>>(ab, kB, vB, bag_of, log2Zp);
+            if (shortb) launch_next(binned_apply_kernel<false, true>, blocks, 256, 0, st, ab, kB, vB, bag_of, log2Zp);
+            else launch_next(binned_apply_kernel<false, false>, blocks, 256, 0, st, ab, kB, vB, bag_of, log2Zp);
         }
         return cudaGetLastError();
     }

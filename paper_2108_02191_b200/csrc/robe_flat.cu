@@ -162,11 +162,12 @@ flat_kernel(FlatArgs a) {
     __shared__ FlatSmem sm;
     const MapParams& mp = a.mp;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (uint32_t c = threadIdx.x; c < mp.C; c += 32 * kFlatWarps) {
+    for (uint32_t c = threadIdx.x; c < mp.C; c += 32 * kFlatWarps) {  // (needs nothing of the kernel before)
         sm.cterm[c] = mulmod_p61_u32(mp.h.C, c);
         sm.ct[c] = mod_m(sm.cterm[c], mp.m, mp.mu);
     }
     __syncthreads();
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
     const int64_t row0 = ((int64_t)blockIdx.x * kFlatWarps + w) * a.rows;
     if (row0 >= a.nbags) return;
@@ -210,9 +211,9 @@ static cudaError_t launch_flat(const Problem& pb, const float* grad_out, float* 
     const unsigned blocks = (unsigned)((warps + kFlatWarps - 1) / kFlatWarps);
     const bool ragged = mp.d % mp.Z != 0, pow2 = mp.log2Z != 0xFFFFFFFFu;
     auto pick = [&](auto plain, auto any, auto rag) {
-        if (ragged) rag<<<blocks, 32 * kFlatWarps, 0, st>>>(a);
-        else if (pow2) plain<<<blocks, 32 * kFlatWarps, 0, st>>>(a);
-        else any<<<blocks, 32 * kFlatWarps, 0, st>>>(a);
+        if (ragged) launch_next(rag, blocks, 32 * kFlatWarps, 0, st, a);
+        else if (pow2) launch_next(plain, blocks, 32 * kFlatWarps, 0, st, a);
+        else launch_next(any, blocks, 32 * kFlatWarps, 0, st, a);
     };
     if (mode == 0) pick(flat_kernel<0, true, false>, flat_kernel<0, false, false>, flat_kernel<0, false, true>);
     else if (mode == 1) pick(flat_kernel<1, true, false>, flat_kernel<1, false, false>, flat_kernel<1, false, true>);

@@ -165,6 +165,7 @@ fwd_staged_kernel(FwdArgs a, uint32_t ids_per_batch, uint32_t cmagic) {
     const int64_t warp = (int64_t)blockIdx.x * 8 + w;
 
     stage_init(sm, mp);
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
 
     int64_t lo, hi;
@@ -392,9 +393,9 @@ static void launch_staged_minb(const FwdArgs& a, bool bags, cudaStream_t st) {
     const int64_t warps = bags ? a.nbags : (a.nbags + ipb - 1) / ipb;
     const unsigned blocks = (unsigned)((warps + 7) / 8);
     if (bags)
-        fwd_staged_kernel<EPL, DT, SIGN, true, FULLD, MINB, UB><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
+        launch_next(fwd_staged_kernel<EPL, DT, SIGN, true, FULLD, MINB, UB>, blocks, 256, 0, st, a, ipb, cmagic);
     else
-        fwd_staged_kernel<EPL, DT, SIGN, false, FULLD, MINO, UO><<<blocks, 256, 0, st>>>(a, ipb, cmagic);
+        launch_next(fwd_staged_kernel<EPL, DT, SIGN, false, FULLD, MINO, UO>, blocks, 256, 0, st, a, ipb, cmagic);
 }
 
 template <int EPL, int DT, bool SIGN, bool FULLD>

@@ -193,6 +193,7 @@ pool_kernel(PoolArgs a) {
     const MapParams& mp = a.mp;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     stage_init(sm.stage, mp);
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
     const PoolRun run = pool_run(a, w, lane);
     if (run.bags == 0) return;
@@ -249,9 +250,9 @@ pool_kernel(PoolArgs a) {
 
 template <int MODE, bool SIGN>
 void launch_pool_epl(const PoolArgs& a, unsigned blocks, cudaStream_t st) {
-    if (a.mp.d <= 32) pool_kernel<MODE, 1, SIGN><<<blocks, 256, 0, st>>>(a);
-    else if (a.mp.d <= 64) pool_kernel<MODE, 2, SIGN><<<blocks, 256, 0, st>>>(a);
-    else pool_kernel<MODE, 4, SIGN><<<blocks, 256, 0, st>>>(a);
+    if (a.mp.d <= 32) launch_next(pool_kernel<MODE, 1, SIGN>, blocks, 256, 0, st, a);
+    else if (a.mp.d <= 64) launch_next(pool_kernel<MODE, 2, SIGN>, blocks, 256, 0, st, a);
+    else launch_next(pool_kernel<MODE, 4, SIGN>, blocks, 256, 0, st, a);
 }
 
 uint32_t pool_ids(const Problem& pb) { return staged_ids_per_batch(pb.mp, true, pb.sign != 0); }

@@ -205,6 +205,7 @@ fwd_rows_kernel(RowsArgs a) {
     __shared__ uint32_t lists[LISTED ? kRowsWarps : 1][LISTED ? kRowsMaxC * 33 : 1];
     const MapParams& mp = a.mp;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
     const uint32_t first = blockIdx.x * a.rows_per_cta;
     if (first >= a.nbags) return;
@@ -260,6 +261,7 @@ bwd_rows_kernel(RowsArgs a) {
     __shared__ uint32_t lists[LISTED ? kRowsWarps : 1][LISTED ? kRowsMaxC * 33 : 1];
     const MapParams& mp = a.mp;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
     const uint32_t first = blockIdx.x * a.rows_per_cta;
     if (first >= a.nbags) return;
@@ -367,8 +369,8 @@ static RowsArgs rows_args(const Problem& pb, bool whole_waves, unsigned& grid) {
 
 template <int EPL, bool LISTED, bool M30>
 static void launch_fwd_rows(const RowsArgs& a, int dtype, unsigned grid, cudaStream_t st) {
-    if (dtype == 0) fwd_rows_kernel<EPL, 0, LISTED, M30, 4><<<grid, kRowsThreads, 0, st>>>(a);
-    else fwd_rows_kernel<EPL, 1, LISTED, M30, 4><<<grid, kRowsThreads, 0, st>>>(a);
+    if (dtype == 0) launch_next(fwd_rows_kernel<EPL, 0, LISTED, M30, 4>, grid, kRowsThreads, 0, st, a);
+    else launch_next(fwd_rows_kernel<EPL, 1, LISTED, M30, 4>, grid, kRowsThreads, 0, st, a);
 }
 
 template <int EPL>
@@ -391,9 +393,9 @@ cudaError_t launch_forward_rows(const Problem& pb, float* out, cudaStream_t st) 
 template <int EPL>
 static void launch_bwd_rows(const RowsArgs& a, unsigned grid, cudaStream_t st) {
     constexpr int U = EPL == 4 ? 2 : 4;
-    if (a.mp.C <= kRowsMaxC) bwd_rows_kernel<EPL, true, false, U><<<grid, kRowsThreads, 0, st>>>(a);
-    else if (a.mp.m < (1u << 30)) bwd_rows_kernel<EPL, false, true, U><<<grid, kRowsThreads, 0, st>>>(a);
-    else bwd_rows_kernel<EPL, false, false, U><<<grid, kRowsThreads, 0, st>>>(a);
+    if (a.mp.C <= kRowsMaxC) launch_next(bwd_rows_kernel<EPL, true, false, U>, grid, kRowsThreads, 0, st, a);
+    else if (a.mp.m < (1u << 30)) launch_next(bwd_rows_kernel<EPL, false, true, U>, grid, kRowsThreads, 0, st, a);
+    else launch_next(bwd_rows_kernel<EPL, false, false, U>, grid, kRowsThreads, 0, st, a);
 }
 
 cudaError_t launch_backward_rows(const Problem& pb, const float* grad_out, float* target, float scale,

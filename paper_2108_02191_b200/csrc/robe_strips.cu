@@ -68,7 +68,9 @@ constexpr uint32_t kBoundsGap = 256;  // longer gaps are filled by the whole war
 __global__ void __launch_bounds__(256)
 strip_bounds_search_kernel(const uint32_t* __restrict__ K, uint32_t nb, uint32_t* __restrict__ lo_of,
                            uint32_t* __restrict__ hi_of, uint32_t strips, uint32_t log2w, uint32_t reach,
-                           const int32_t* status) {
+                           const int32_t* status, uint32_t* hot_count) {
+    follow<true>();
+    if (blockIdx.x == 0 && threadIdx.x < 3) hot_count[threadIdx.x] = 0;  // (for the kernels after this one)
     if (status != nullptr && *status != 0) return;  // after a failed input check K was not written
     const uint32_t b = blockIdx.x * 256 + threadIdx.x;
     if (b > strips) return;
@@ -96,7 +98,10 @@ strip_bounds_search_kernel(const uint32_t* __restrict__ K, uint32_t nb, uint32_t
 // whose first slot lies past the key before it and not past its own (lo_of: the same of the blocks' last slots).
 __global__ void __launch_bounds__(256)
 strip_bounds_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* __restrict__ lo_of,
-                    uint32_t* __restrict__ hi_of, uint32_t strips, uint32_t log2w, uint32_t reach, const int32_t* status) {
+                    uint32_t* __restrict__ hi_of, uint32_t strips, uint32_t log2w, uint32_t reach, const int32_t* status,
+                    uint32_t* hot_count) {
+    follow<true>();
+    if (blockIdx.x == 0 && threadIdx.x < 3) hot_count[threadIdx.x] = 0;  // (for the kernels after this one)
     if (status != nullptr && *status != 0) return;  // after a failed input check K was not written
     const uint64_t i0 = ((uint64_t)blockIdx.x * 256 + threadIdx.x) * 8;
     const uint32_t lane = threadIdx.x & 31;
@@ -170,6 +175,7 @@ strip_bounds_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* __res
 
 // The list of hot strips: the hottest at its front, so that they are begun first.
 __global__ void __launch_bounds__(256) strip_hot_list_kernel(StripArgs a) {
+    follow<true>();
     if (a.status != nullptr && *a.status != 0) return;
     const uint32_t b = blockIdx.x * 256 + threadIdx.x;
     if (b >= a.strips) return;
@@ -197,6 +203,7 @@ template <int MODE, int LP, int EPL, bool SHORT>
 __global__ void __launch_bounds__(32 * kStripWarps, 5)
 strip_apply_kernel(StripArgs a) {
     extern __shared__ float4 strip_smem[];
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
     constexpr uint32_t G = 32 / LP;               // groups per warp
     constexpr int U = EPL == 4 ? 4 : 8;           // blocks whose loads are in flight together
@@ -357,6 +364,7 @@ strip_hot_kernel(StripArgs a) {
     __shared__ int4 all_s[kHotBufs][kHotCopiers];      // of the blocks of one copier: their number; all alike? start, length
     __shared__ uint2 keys_s[2 * kHotBufs][kHotCopiers][32];  // (start, payload) of steps yet to be copied
     __shared__ uint32_t item_s;
+    follow();
     if (a.status != nullptr && *a.status != 0) return;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const bool copier = w >= (uint32_t)kHotAdders;
@@ -549,10 +557,10 @@ void launch_strip_kernels(const StripArgs& a, cudaStream_t st, cudaStream_t hot_
     const uint32_t per_sm = (uint32_t)(220 * 1024 / (hot_smem + 26 * 1024));  // (26 KB: the static part and a margin)
     uint32_t hot_grid = 148 * (per_sm > 2 ? 2 : (per_sm < 1 ? 1 : per_sm));
     if (hot_grid > a.hot_cap) hot_grid = a.hot_cap;
-    strip_hot_kernel<MODE, LP, EPL, SHORT><<<hot_grid, 32 * (kHotCopiers + kHotAdders), hot_smem, hot_st>>>(a);
+    launch_next(strip_hot_kernel<MODE, LP, EPL, SHORT>, hot_grid, 32 * (kHotCopiers + kHotAdders), hot_smem, hot_st, a);
     const uint32_t per_cta = kStripWarps * (32 / LP);
     const size_t smem = ((size_t)per_cta << a.log2w) * sizeof(float);
-    strip_apply_kernel<MODE, LP, EPL, SHORT><<<(a.strips + per_cta - 1) / per_cta, 32 * kStripWarps, smem, st>>>(a);
+    launch_next(strip_apply_kernel<MODE, LP, EPL, SHORT>, (a.strips + per_cta - 1) / per_cta, 32 * kStripWarps, smem, st, a);
 }
 
 template <int MODE, bool SHORT>
@@ -615,19 +623,18 @@ size_t strips_workspace_bytes(const MapParams& mp, uint64_t nb) { return strip_l
 void launch_strips_prepare(const StripProblem& sp, cudaStream_t st) {
     const StripLayout L = strip_layout(sp.nb, sp.mp.m);
     char* ws = (char*)sp.workspace;
-    cudaMemsetAsync(ws, 0, 3 * sizeof(uint32_t), st);
     uint32_t *lo_of = (uint32_t*)(ws + L.lo_of), *hi_of = (uint32_t*)(ws + L.hi_of);
     if (L.strips > 148u * 256u)
-        strip_bounds_search_kernel<<<L.strips / 256 + 1, 256, 0, st>>>(sp.K, (uint32_t)sp.nb, lo_of, hi_of, L.strips,
-                                                                      L.log2w, sp.mp.Z - 1, sp.status);
+        launch_next(strip_bounds_search_kernel, L.strips / 256 + 1, 256, 0, st, sp.K, (uint32_t)sp.nb, lo_of, hi_of, L.strips,
+                    L.log2w, sp.mp.Z - 1, sp.status, (uint32_t*)ws);
     else
-        strip_bounds_kernel<<<(unsigned)(sp.nb / 2048 + 1), 256, 0, st>>>(sp.K, sp.nb, lo_of, hi_of, L.strips, L.log2w,
-                                                                         sp.mp.Z - 1, sp.status);
+        launch_next(strip_bounds_kernel, (unsigned)(sp.nb / 2048 + 1), 256, 0, st, sp.K, sp.nb, lo_of, hi_of, L.strips,
+                    L.log2w, sp.mp.Z - 1, sp.status, (uint32_t*)ws);
 }
 
 void launch_strips(const StripProblem& sp, int mode, cudaStream_t st, cudaStream_t hot_st) {
     const StripArgs a = strip_args(sp);
-    strip_hot_list_kernel<<<(a.strips + 255) / 256, 256, 0, hot_st>>>(a);
+    launch_next(strip_hot_list_kernel, (a.strips + 255) / 256, 256, 0, hot_st, a);
     if (mode == 4) launch_strip_mode<3>(a, st, hot_st);
     else if (mode == 2) launch_strip_mode<2>(a, st, hot_st);
     else if (mode == 1) launch_strip_mode<1>(a, st, hot_st);

@@ -447,6 +447,31 @@ def test_backward_adam_matches_oracle_over_steps(bags):
                 robe.robe_backward_adam(c.h, g_d, c.indices, c.offsets, c.B, m1_d, m2_d, lr, b1, b2, eps, 0, ws)
 
 
+# Kernels are set up while the one before still runs: a training loop that never waits must leave the bits of
+# one that waits for the GPU after every call (lookups read what the step before wrote, on the same SMs).
+@pytest.mark.parametrize("bags", [None, (3, 0, 9), (20, 1, 80)])
+@pytest.mark.parametrize("d,Z,M,batch", [(16, 8, 4099, 300), (64, 16, 30_011, 2000), (100, 32, 1013, 500), (128, 1, 8209, 300)])
+def test_back_to_back_steps_see_each_other(d, Z, M, batch, bags):
+    w = small(d=d, Z=Z, M=M, bag_rule=bags, batch=batch)
+    arrays, rows = [], []
+    for wait in (False, True):
+        with Case(w) as c:
+            robe.robe_set_option(c.h, robe.ROBE_OPT_BWD_MODE, robe.ROBE_BWD_DETERMINISTIC)
+            ws = torch.empty(robe.robe_backward_workspace_bytes(c.h, c.B, c.indices.numel()), dtype=torch.uint8, device=c.dev)
+            out = torch.empty(c.nbags, d, device=c.dev)
+            for step in range(20):
+                robe.robe_forward(c.h, c.indices, c.offsets, c.B, out)
+                if wait:
+                    torch.cuda.synchronize()
+                robe.robe_backward(c.h, out, c.indices, c.offsets, c.B, None, 1e-3, ws)
+                if wait:
+                    torch.cuda.synchronize()
+            arrays.append(c.array.cpu().numpy())
+            rows.append(out.cpu().numpy())
+    assert_bits_equal(rows[0], rows[1], "rows")
+    assert_bits_equal(arrays[0], arrays[1], "array")
+
+
 @pytest.mark.parametrize("bags", [None, (3, 0, 9)])
 def test_backward_adagrad_matches_oracle_over_steps(bags):
     # three Adagrad steps in a row (array and accumulators carried over), bit for bit; the dense
