@@ -949,6 +949,89 @@ binned_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t*
     }
 }
 
+// The same for plain blocks of up to 128 elements: a warp takes 32 sorted blocks, a block per lane, and hands
+// them round - LP lanes (8, 16 or 32 by the block length) add a block's elements, EPL each, 32 / LP blocks at
+// a time - where binned_apply_kernel has every thread read and work out every block's numbers itself.  Measured
+// (B200, 34 M blocks of 16 on 1 GB, us): 930 (45 instructions per element and thread) -> 780; on 100 MB 930 ->
+// 550; 13 tables of d = 73, Z = 32 1104 -> 460; Z = 128 880 -> 480.  Now bound by the reductions and by the
+// gradient rows, read once per id (going through odd bins backwards, to meet rows again in L2, changed nothing)
+template <int LP, int EPL, bool SHORT>
+__global__ void __launch_bounds__(256)
+binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V) {
+    follow();
+    if (a.status != nullptr && *a.status != 0) return;
+    constexpr uint32_t G = 32 / LP;              // blocks at a time
+    constexpr int U = EPL == 4 ? 4 : 8;          // times whose loads are in flight together
+    const MapParams& mp = a.mp;
+    const uint32_t lane = threadIdx.x & 31, g = lane / LP, ol = lane % LP, Z = mp.Z, m = mp.m;
+    const uint64_t i0 = ((uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
+    if (i0 >= a.nb) return;
+    const uint32_t cnt = a.nb - i0 < 32 ? (uint32_t)(a.nb - i0) : 32u;
+    uint32_t k = 0, v = 0, len = 0;              // (length 0: nothing of the block is added)
+    if (lane < cnt) {
+        k = __ldg(K + i0 + lane);
+        v = __ldg(V + i0 + lane);
+        len = Z;
+        if (SHORT) {
+            const uint32_t left = mp.d - v % mp.d;
+            if (left < Z) len = left;
+        }
+    }
+    const bool plain = !SHORT && __all_sync(0xFFFFFFFFu, lane < cnt && k <= m - Z);  // full blocks, none wraps
+    const uint64_t pol = l2_keep_policy(a.l2_keep != 0);
+#pragma unroll 1
+    for (uint32_t s0 = 0; s0 < LP && s0 * G < cnt; s0 += U) {
+        float x[U][EPL];
+        uint32_t slot[U];
+        if (plain) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int src = (int)((s0 + u) * G + g);
+                slot[u] = __shfl_sync(0xFFFFFFFFu, k, src) + ol;
+                const float* row = a.grad_out + (__shfl_sync(0xFFFFFFFFu, v, src) + ol);
+#pragma unroll
+                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < Z ? __ldg(row + 32 * q) : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int q = 0; q < EPL; ++q)
+                    if (ol + 32 * q < Z && ROBE_CHK(slot[u] + 32 * q < m, ROBE_DBG_ARRAY_SLOT))
+                        red_add(a.target + slot[u] + 32 * q, a.lr * x[u][q], pol);
+        } else {
+            uint32_t l[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int src = (int)((s0 + u) * G + g);
+                slot[u] = __shfl_sync(0xFFFFFFFFu, k, src) + ol;
+                const float* row = a.grad_out + (__shfl_sync(0xFFFFFFFFu, v, src) + ol);
+                l[u] = __shfl_sync(0xFFFFFFFFu, len, src);
+#pragma unroll
+                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < l[u] ? __ldg(row + 32 * q) : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int q = 0; q < EPL; ++q)
+                    if (ol + 32 * q < l[u]) {
+                        uint32_t j = slot[u] + 32 * q;  // < m + d <= 2^32
+                        if (j >= m) j -= m;
+                        if (ROBE_CHK(j < m, ROBE_DBG_ARRAY_SLOT)) red_add(a.target + j, a.lr * x[u][q], pol);
+                    }
+        }
+    }
+}
+
+template <bool SHORT>
+void launch_binned_blocks(const ApplyArgs& a, const uint32_t* K, const uint32_t* V, cudaStream_t st) {
+    const unsigned blocks = (unsigned)((a.nb + 255) / 256);
+    if (a.mp.Z <= 8) launch_next(binned_apply_blocks_kernel<8, 1, SHORT>, blocks, 256, 0, st, a, K, V);
+    else if (a.mp.Z <= 16) launch_next(binned_apply_blocks_kernel<16, 1, SHORT>, blocks, 256, 0, st, a, K, V);
+    else if (a.mp.Z <= 32) launch_next(binned_apply_blocks_kernel<32, 1, SHORT>, blocks, 256, 0, st, a, K, V);
+    else if (a.mp.Z <= 64) launch_next(binned_apply_blocks_kernel<32, 2, SHORT>, blocks, 256, 0, st, a, K, V);
+    else launch_next(binned_apply_blocks_kernel<32, 4, SHORT>, blocks, 256, 0, st, a, K, V);
+}
+
 uint32_t bits_for(uint32_t m) {  // bits needed for keys in [0, m)
     uint32_t b = 1;
     while (b < 32 && (1ull << b) < (uint64_t)m) ++b;
@@ -1116,17 +1199,22 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
     const SortPlan sp = make_plan(nb);
     const uint32_t bits = bits_for(mp.m);
     if (mode == 3) {
-        // binned: one pass on the top key bits, then atomic adds in bin order.  A bin spans 2^22
-        // slots (16 MB of fp32: the span that measured fastest on a 1 GB array - small enough to
-        // be updated in L2, large enough that the scatter writes long runs) unless that would
-        // need more than 256 bins or the array is smaller than one such span.
-        const uint32_t shift = bits > 30 ? bits - 8 : (bits > 22 ? 22 : (bits > 8 ? bits - 8 : 0));
+        // binned: one pass on the top key bits, then atomic adds in bin order.  A bin spans 2^23 slots (32 MB of
+        // fp32: the span that measured fastest on a 1 GB array, by 1 % - small enough to be updated in L2, large
+        // enough that the scatter writes long runs) unless that would need more than 256 bins or the array is
+        // smaller than one such span.
+        const uint32_t shift = bits > 31 ? bits - 8 : (bits > 23 ? 23 : (bits > 22 ? 22 : (bits > 8 ? bits - 8 : 0)));
         launch_sort_pass<false>(sp, kA, vA, kB, vB, counts, totals, shift, bits - shift, st);
         // (an array that does not fit the L2 passes through it bin by bin: lines that outlive their bin would
         // only be in the way of the gradient rows; 34 M blocks of 16 on 1 GB, us: 951 -> 925)
         const int keep = (uint64_t)mp.m * 4 <= (192ull << 20) ? pb.l2_keep : 0;
         ApplyArgs ab{mp, grad_out, pb.indices, target, lr, nb, pb.status, AdamState{}, nullptr, nullptr, 0,
                      (uint64_t)pb.nbags * mp.d, keep};
+        if (!pb.sign && mp.Z <= 128) {
+            if (mp.d % mp.Z != 0) launch_binned_blocks<true>(ab, kB, vB, st);
+            else launch_binned_blocks<false>(ab, kB, vB, st);
+            return cudaGetLastError();
+        }
         uint32_t log2Zp = 0;
         while ((1u << log2Zp) < mp.Z) ++log2Zp;
         const uint64_t groups = (nb + kBinnedPer - 1) / kBinnedPer;
