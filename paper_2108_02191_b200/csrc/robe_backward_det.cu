@@ -1199,11 +1199,11 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
     const SortPlan sp = make_plan(nb);
     const uint32_t bits = bits_for(mp.m);
     if (mode == 3) {
-        // binned: one pass on the top key bits, then atomic adds in bin order.  A bin spans 2^23 slots (32 MB of
-        // fp32: the span that measured fastest on a 1 GB array, by 1 % - small enough to be updated in L2, large
-        // enough that the scatter writes long runs) unless that would need more than 256 bins or the array is
-        // smaller than one such span.
-        const uint32_t shift = bits > 31 ? bits - 8 : (bits > 23 ? 23 : (bits > 22 ? 22 : (bits > 8 ? bits - 8 : 0)));
+        // binned: one pass on the top key bits, then atomic adds in bin order.  A bin spans 2^22
+        // slots (16 MB of fp32: the span that measured fastest on a 1 GB array - small enough to
+        // be updated in L2, large enough that the scatter writes long runs; 32 MB: adds 850 us against
+        // 805) unless that would need more than 256 bins or the array is smaller than one such span.
+        const uint32_t shift = bits > 30 ? bits - 8 : (bits > 22 ? 22 : (bits > 8 ? bits - 8 : 0));
         launch_sort_pass<false>(sp, kA, vA, kB, vB, counts, totals, shift, bits - shift, st);
         // (an array that does not fit the L2 passes through it bin by bin: lines that outlive their bin would
         // only be in the way of the gradient rows; 34 M blocks of 16 on 1 GB, us: 951 -> 925)
