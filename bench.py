@@ -44,18 +44,18 @@ UNIT = "ids/s"
 NCU_TRAFFIC_RECORDS = {
     # (workload, backward variant, block starts shared, id type, bag layout)
     ("cfg4_multihot", "binned", True, "int64", "sample-major"): {
-        "forward": 4_412_000_000, "backward": 4_838_700_000,
+        "forward": 4_411_400_000, "backward": 4_822_100_000,
         "source": "profiles/launches_cfg4_multihot.md: full-size one-pass ncu capture of `python bench.py --steps 3 "
                   "--warmup 3 --no-cpu-baseline`; forward = fwd_staged_kernel, backward = sort_count + sort_scan + "
-                  "sort_scatter + binned_apply"},
+                  "sort_scatter + binned_apply_blocks"},
     ("cfg4_multihot", "atomic", False, "int64", "sample-major"): {
         "forward": 4_130_800_000, "backward": 7_378_600_000,
         "source": "profiles/launches_cfg4_multihot.md: full-size one-pass ncu capture of `python bench.py --steps 3 "
                   "--warmup 3 --no-cpu-baseline --backward atomic`"},
     ("cfg4_multihot", "det", True, "int64", "sample-major"): {
-        "forward": 4_411_800_000, "backward": 7_246_000_000,
+        "forward": 4_411_900_000, "backward": 7_445_500_000,
         "source": "profiles/launches_cfg4_multihot.md: full-size one-pass ncu capture of `python bench.py --steps 3 "
-                  "--warmup 3 --no-cpu-baseline --backward det`; backward = 4 sort passes, window bounds and classes, "
+                  "--warmup 3 --no-cpu-baseline --backward det`; backward = 4 sort passes, strip bounds, "
                   "apply kernels"},
 }
 
@@ -417,10 +417,11 @@ def run_ours(args, w):
         zb = min(w.Z, w.d)
         bwd_launches = ((1 if bags else 0) + 1 + 3 * npass + 1 + (1 if w.d % zb == 0 else 0)
                         + (1 if zb > 1 else 0))
-        # a densely touched array: window bounds, window classes and the window kernel as well
-        terms = float(np.mean([len(b[0]) for b in batches])) * w.d
-        if w.d % zb == 0 and zb <= 128 and 2 * terms >= w.M:
-            bwd_launches += 3
+        # a densely touched array is served by strips: their bounds, the list of hot ones, the two apply
+        # kernels (and the low slots) instead
+        nblocks = float(np.mean([len(b[0]) for b in batches])) * -(-w.d // zb)
+        if zb <= 128 and 2 * nblocks * zb >= w.M:
+            bwd_launches = (1 if bags else 0) + 1 + 3 * npass + 4 + (1 if zb > 1 else 0)
     # One training step hashes every id once: the forward leaves the block starts in the workspace
     # and the sort-based backward takes them from there (rows of up to 128 elements; longer rows
     # use a forward kernel that keeps nothing, and the key kernels then run inside the forward call).
@@ -565,10 +566,10 @@ def run_ours(args, w):
 
     peak, peak_kind = measured_peaks()
     fwd_bytes, bwd_bytes = algorithmic_bytes(w, nbags, nnz_per_step, bags, id_bytes)
-    fwd_kernel = "fwd_staged_kernel" if d <= 128 else "fwd_direct_kernel"
-    bwd_label = {"atomic": "bwd_atomic_staged_kernel" if d <= 128 else "bwd_atomic_direct_kernel",
-                 "binned": "composite: keys, sort_count, sort_scan, sort_scatter, binned_apply kernels",
-                 "det": "composite: keys, sort passes, window bounds/classes, apply kernels"}[args.backward]
+    fwd_kernel = "fwd_staged_kernel" if bags and d <= 128 else "forward kernel (automatic choice)"
+    bwd_label = {"atomic": "bwd_atomic_staged_kernel" if bags and d <= 128 else "atomic backward kernel (automatic choice)",
+                 "binned": "composite: keys, sort_count, sort_scan, sort_scatter, binned_apply_blocks kernels",
+                 "det": "composite: keys, sort passes, strip bounds, apply kernels"}[args.backward]
     if share_keys:
         bwd_label = bwd_label.replace("keys, ", "")
     # a traffic record applies to the configuration it was captured on, and to no other
