@@ -949,6 +949,105 @@ binned_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t*
     }
 }
 
+// answer = do starts repeat among 32 neighbours of the sorted list?  128 places looked at, a quarter of them with a
+// repeat is a yes.
+__global__ void __launch_bounds__(1024) binned_sample_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* answer) {
+    follow();
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t found = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < 4; ++q) {
+        const uint64_t at = (nb - 32) / 128 * (w * 4 + q) + lane;  // (nb is large)
+        const uint32_t k = __ldg(K + at);
+        found += __any_sync(0xFFFFFFFFu, __popc(__match_any_sync(0xFFFFFFFFu, k)) > 1) ? 1u : 0u;
+    }
+    __shared__ uint32_t total_s;
+    if (threadIdx.x == 0) total_s = 0;
+    __syncthreads();
+    if (lane == 0) atomicAdd(&total_s, found);
+    __syncthreads();
+    if (threadIdx.x == 0) *answer = total_s >= 32u ? 1u : 0u;
+}
+
+// Repeats of one start (an id that the batch draws often) would be reductions on the same slots, one after the
+// other in L2.  The CTA's 256 blocks are brought together by a counting sort on a hash of their starts, and
+// the gradient rows of equal starts among 32 neighbours are summed before one reduction.
+// Measured (B200, 34 M blocks of 16 from Zipf ids on 1 GB, us): 5380 -> 2360; 13 tables of d = 73, Z = 32
+// 2580 -> 1170.  Spread ids gain nothing from it (805 -> 905), nor do small calls (1.1 M blocks 46 -> 71): the
+// launcher asks for it from 8 M blocks on, and a sample of the sorted list says whether starts repeat.
+template <int LP, int EPL, bool SHORT>
+__device__ __forceinline__ void binned_add_merged(const ApplyArgs& a, uint32_t k, uint32_t v, uint2* sorted, uint32_t* count,
+                                                  uint32_t* warp_sums) {
+    constexpr uint32_t G = 32 / LP;
+    const MapParams& mp = a.mp;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, g = lane / LP, ol = lane % LP, Z = mp.Z, m = mp.m;
+    const uint32_t bin = (k * 0x9E3779B1u) >> 24;
+    count[tid] = 0;
+    __syncthreads();
+    const uint32_t rank = atomicAdd(&count[bin], 1u);
+    __syncthreads();
+    const uint32_t start = cta_exclusive_scan(count[tid], warp_sums);  // syncs inside
+    count[tid] = start;
+    __syncthreads();
+    if (ROBE_CHK(count[bin] + rank < 256u, ROBE_DBG_SHARED)) sorted[count[bin] + rank] = make_uint2(k, v);
+    __syncthreads();
+    const uint2 kv = sorted[tid];
+    k = kv.x;
+    v = kv.y;
+    uint32_t len = k == kNoKey ? 0u : Z;
+    if (SHORT && len != 0) {
+        const uint32_t left = mp.d - v % mp.d;
+        if (left < Z) len = left;
+    }
+    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, k);
+    const uint64_t pol = l2_keep_policy(a.l2_keep != 0);
+    uint32_t rest = __ballot_sync(0xFFFFFFFFu, len != 0 && (peers & ((1u << lane) - 1u)) == 0);  // first of each start
+    while (rest != 0) {
+        uint32_t left = rest;  // group g takes the g-th start that is left
+#pragma unroll
+        for (uint32_t i = 0; i + 1 < G; ++i)
+            if (i < g) left &= left - 1;
+#pragma unroll
+        for (uint32_t i = 0; i < G; ++i) rest &= rest - 1;
+        const int src = left != 0 ? __ffs((int)left) - 1 : 0;
+        uint32_t from = __shfl_sync(0xFFFFFFFFu, peers, src);
+        const uint32_t first = __shfl_sync(0xFFFFFFFFu, k, src);
+        if (left == 0) from = 0;
+        float sum[EPL];
+        uint32_t reach = 0;  // longest of the blocks
+#pragma unroll
+        for (int q = 0; q < EPL; ++q) sum[q] = 0.0f;
+        while (__any_sync(0xFFFFFFFFu, from != 0)) {
+            float x[4][EPL];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = from != 0 ? __ffs((int)from) - 1 : 0;
+                const uint32_t row = __shfl_sync(0xFFFFFFFFu, v, p) + ol;
+                uint32_t l = __shfl_sync(0xFFFFFFFFu, len, p);
+                if (from == 0) l = 0;
+                if (l > reach) reach = l;
+                from &= from - 1;
+#pragma unroll
+                for (int q = 0; q < EPL; ++q)
+                    x[u][q] = ol + 32 * q < l && ROBE_CHK((uint64_t)row + 32 * q < a.grad_elems, ROBE_DBG_GRAD_POS)
+                                  ? __ldg(a.grad_out + (row + 32 * q))
+                                  : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int q = 0; q < EPL; ++q) sum[q] += x[u][q];
+        }
+#pragma unroll
+        for (int q = 0; q < EPL; ++q)
+            if (ol + 32 * q < reach) {
+                uint32_t j = first + ol + 32 * q;  // < m + d <= 2^32
+                if (j >= m) j -= m;
+                if (ROBE_CHK(j < m, ROBE_DBG_ARRAY_SLOT)) red_add(a.target + j, a.lr * sum[q], pol);
+            }
+    }
+}
+
 // The same for plain blocks of up to 128 elements: a warp takes 32 sorted blocks, a block per lane, and hands
 // them round - LP lanes (8, 16 or 32 by the block length) add a block's elements, EPL each, 32 / LP blocks at
 // a time - where binned_apply_kernel has every thread read and work out every block's numbers itself.  Measured
@@ -964,10 +1063,12 @@ binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const ui
     constexpr int U = EPL == 4 ? 4 : 8;          // times whose loads are in flight together
     const MapParams& mp = a.mp;
     const uint32_t lane = threadIdx.x & 31, g = lane / LP, ol = lane % LP, Z = mp.Z, m = mp.m;
+    __shared__ uint2 sorted_s[256];
+    __shared__ uint32_t count_s[256];
+    __shared__ uint32_t warp_sums[8];
     const uint64_t i0 = ((uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;
-    if (i0 >= a.nb) return;
-    const uint32_t cnt = a.nb - i0 < 32 ? (uint32_t)(a.nb - i0) : 32u;
-    uint32_t k = 0, v = 0, len = 0;              // (length 0: nothing of the block is added)
+    const uint32_t cnt = i0 >= a.nb ? 0u : (a.nb - i0 < 32 ? (uint32_t)(a.nb - i0) : 32u);
+    uint32_t k = kNoKey, v = 0, len = 0;         // (length 0: nothing of the block is added)
     if (lane < cnt) {
         k = __ldg(K + i0 + lane);
         v = __ldg(V + i0 + lane);
@@ -976,6 +1077,10 @@ binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const ui
             const uint32_t left = mp.d - v % mp.d;
             if (left < Z) len = left;
         }
+    }
+    if (a.long_count != nullptr && *a.long_count != 0) {  // (binned_sample_kernel's answer)
+        binned_add_merged<LP, EPL, SHORT>(a, k, v, sorted_s, count_s, warp_sums);
+        return;
     }
     const bool plain = !SHORT && __all_sync(0xFFFFFFFFu, lane < cnt && k <= m - Z);  // full blocks, none wraps
     const uint64_t pol = l2_keep_policy(a.l2_keep != 0);
@@ -1211,6 +1316,10 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
         ApplyArgs ab{mp, grad_out, pb.indices, target, lr, nb, pb.status, AdamState{}, nullptr, nullptr, 0,
                      (uint64_t)pb.nbags * mp.d, keep};
         if (!pb.sign && mp.Z <= 128) {
+            if (nb >= (8u << 20)) {
+                ab.long_count = (uint32_t*)(ws + L.long_count);
+                launch_next(binned_sample_kernel, 1, 1024, 0, st, kB, nb, ab.long_count);
+            }
             if (mp.d % mp.Z != 0) launch_binned_blocks<true>(ab, kB, vB, st);
             else launch_binned_blocks<false>(ab, kB, vB, st);
             return cudaGetLastError();
