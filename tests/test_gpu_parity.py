@@ -381,6 +381,19 @@ def test_short_bags(d, Z, M, batch, bags):
                 assert_bits_equal(c.forward().cpu().numpy(), one, "offsets out of order")
 
 
+# Binned adds of a call large enough to look for repeats of a start (8 M blocks): hot ids, whose blocks are added
+# together, in full and in short last blocks, and ids that hardly repeat.
+@pytest.mark.parametrize("d,Z,batch,vocab", [(64, 1, 46_000, (5, 50, 3000)), (64, 3, 130_000, (5, 50, 10**6)),
+                                             (64, 1, 46_000, (10**6, 10**6, 10**6))])
+def test_binned_adds_of_repeated_blocks(d, Z, batch, vocab):
+    w = small(d=d, Z=Z, M=4_000_037, batch=batch, vocab_arg=vocab)
+    with Case(w) as c:
+        assert c.indices.numel() * -(-d // Z) >= 8 << 20
+        g_h, g_d = _grad(c, 31)
+        delta64, l1 = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+        assert_within_l1(c.backward(g_d, "binned").cpu().numpy(), delta64, l1, what="binned")
+
+
 @pytest.mark.parametrize("mode", ["atomic", "det"])
 def test_cfg1_backward_dense_and_sgd(mode):
     for sign in (False, True):
