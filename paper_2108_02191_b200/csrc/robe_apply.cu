@@ -15,7 +15,7 @@ constexpr int kApplyVecPerThread = 4;  // float4 pairs in flight per thread
 
 template <bool ZERO>
 __global__ void __launch_bounds__(kApplyThreads)
-dense_sgd_apply_kernel(float* __restrict__ array, float* __restrict__ grad, uint64_t m, float lr) {
+dense_sgd_apply_kernel(float* array, float* grad, uint64_t m, float lr) {
     follow();
     const uint64_t nvec = m >> 2;
     float4* a4 = reinterpret_cast<float4*>(array);

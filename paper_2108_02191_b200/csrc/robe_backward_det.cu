@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(256) det_bag_of_kernel(KeyArgs a, uint32_t* ba
     const int64_t k = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
     const uint32_t lane = threadIdx.x & 31;
     if (k >= a.nbags) return;
-    int64_t lo = __ldg(a.offsets + k), hi = __ldg(a.offsets + k + 1);
+    int64_t lo = __ldca(a.offsets + k), hi = __ldca(a.offsets + k + 1);
     lo = lo < 0 ? 0 : (lo > a.nnz ? a.nnz : lo);
     hi = hi < lo ? lo : (hi > a.nnz ? a.nnz : hi);
     for (int64_t p = lo + lane; p < hi; p += 32) bag_of[p] = (uint32_t)k;
@@ -216,7 +216,7 @@ struct ScatterSmem {
 
 // The pairs of the tile that starts at tbegin, warp-striped.  (nb may be close to 2^32: positions are
 // compared relative to the tile, so that nothing overflows.)
-__device__ __forceinline__ void scatter_load(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+__device__ __forceinline__ void scatter_load(const uint32_t* kin, const uint32_t* vin,
                                              uint32_t tbegin, uint32_t nb, uint32_t (&key)[kSortItems],
                                              uint32_t (&val)[kSortItems]) {
     const uint32_t left = nb - tbegin, local = (threadIdx.x >> 5) * (32 * kSortItems) + (threadIdx.x & 31);
@@ -237,9 +237,9 @@ __device__ __forceinline__ void scatter_load(const uint32_t* __restrict__ kin, c
 }
 
 template <bool STABLE, int BITS, bool FULL>
-__device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, const uint32_t* __restrict__ kin,
-                                             const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-                                             uint32_t* __restrict__ vout, uint32_t nb, uint32_t tbegin,
+__device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, const uint32_t* kin,
+                                             const uint32_t* vin, uint32_t* kout,
+                                             uint32_t* vout, uint32_t nb, uint32_t tbegin,
                                              uint32_t shift, uint32_t (&key)[kSortItems],
                                              uint32_t (&val)[kSortItems], bool more) {
     constexpr uint32_t R = 1u << BITS, mask = R - 1u;
@@ -332,9 +332,9 @@ __device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, cons
 
 template <bool STABLE, int BITS>
 __global__ void __launch_bounds__(kSortThreads, kSortCtas)
-sort_scatter_kernel(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-                    uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
-                    const uint32_t* __restrict__ cta_offsets, const uint32_t* __restrict__ totals,
+sort_scatter_kernel(const uint32_t* kin, const uint32_t* vin,
+                    uint32_t* kout, uint32_t* vout,
+                    const uint32_t* cta_offsets, const uint32_t* totals,
                     uint32_t nb, uint32_t tiles, uint32_t shift) {
     __shared__ ScatterSmem<STABLE, BITS> sm;
     const uint32_t tid = threadIdx.x;
@@ -421,18 +421,18 @@ __device__ __forceinline__ bool block_term(const ApplyArgs& a, const uint32_t* b
             if (cz + o >= mp.d) return false;
         }
         if (!ROBE_CHK((uint64_t)v + o < a.grad_elems, ROBE_DBG_GRAD_POS)) return false;
-        term = __ldg(a.grad_out + (uint64_t)v + o);
+        term = __ldca(a.grad_out + (uint64_t)v + o);
         return true;
     }
     const uint32_t p = v / mp.C;  // v = q
     const uint32_t c = v - p * mp.C;
     const uint32_t i = c * mp.Z + o;
     if (i >= mp.d) return false;
-    const uint64_t bag = bag_of ? (uint64_t)__ldg(bag_of + p) : (uint64_t)p;
+    const uint64_t bag = bag_of ? (uint64_t)__ldca(bag_of + p) : (uint64_t)p;
     if (!ROBE_CHK(bag * mp.d + i < a.grad_elems, ROBE_DBG_GRAD_POS)) return false;
     const uint32_t e = table_of_bag(bag, mp);
     const uint64_t x = (uint64_t)a.indices.load(p);
-    term = sign_of(mp, hash_base(mp.g, e, x), i) * __ldg(a.grad_out + bag * mp.d + i);
+    term = sign_of(mp, hash_base(mp.g, e, x), i) * __ldca(a.grad_out + bag * mp.d + i);
     return true;
 }
 
@@ -466,7 +466,7 @@ struct ApplyTile {
     __device__ __forceinline__ uint2 fetch(uint32_t r) const {
         const uint64_t idx = i0 + r;
         if (idx >= nb) return make_uint2(kNoKey, 0u);
-        return make_uint2(__ldg(K + idx), __ldg(V + idx));
+        return make_uint2(__ldca(K + idx), __ldca(V + idx));
     }
 };
 
@@ -570,7 +570,7 @@ __device__ __forceinline__ bool walk_deep(const ApplyArgs& a, ApplyTile& tl, App
             term[t] = 0.0f;
             if ((uint32_t)t < n_max) {
                 if ((uint32_t)t < n_in && ROBE_CHK((uint64_t)at[t] < a.grad_elems, ROBE_DBG_GRAD_POS))
-                    term[t] = __ldg(a.grad_out + at[t]);
+                    term[t] = __ldca(a.grad_out + at[t]);
             }
         }
 #pragma unroll
@@ -590,8 +590,8 @@ __device__ __forceinline__ bool walk_deep(const ApplyArgs& a, ApplyTile& tl, App
 
 template <bool SIGN, int MODE, bool SHORT>
 __global__ void __launch_bounds__(256)
-det_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V,
-                 const uint32_t* __restrict__ bag_of) {
+det_apply_kernel(ApplyArgs a, const uint32_t* K, const uint32_t* V,
+                 const uint32_t* bag_of) {
     constexpr int UN = 8;
     constexpr uint32_t kDeepAfter = 64;       // positions after which a walk takes 16 per step, if it stays here
     constexpr uint32_t kHandOverAfter = 64;   // positions after which it goes to the long-walk kernel (128 and 256
@@ -614,7 +614,7 @@ det_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __
 
     // first offset served from this lane's position (Z = none)
     uint32_t kprev = __shfl_up_sync(0xFFFFFFFFu, mine.x, 1);
-    if (lane == 0 && tl.i0 > 0) kprev = __ldg(K + tl.i0 - 1);
+    if (lane == 0 && tl.i0 > 0) kprev = __ldca(K + tl.i0 - 1);
     uint32_t own_lo = mp.Z;
     if (tl.i0 + lane < a.nb) {
         if (tl.i0 + lane == 0) own_lo = 0;
@@ -730,7 +730,7 @@ static_assert(kLongStep == 64, "the scout warp brings in two keys per lane and s
 
 template <int MODE>
 __global__ void __launch_bounds__(32 * kLongWarps)
-det_apply_long_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V) {
+det_apply_long_kernel(ApplyArgs a, const uint32_t* K, const uint32_t* V) {
     __shared__ float terms_s[kLongBufs][kLongStep][32];
     __shared__ uint2 ring[kLongRing];
     __shared__ uint32_t reach_s[2][32];  // by step parity: positions of the step that reach each slot
@@ -762,7 +762,7 @@ det_apply_long_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_
         auto fetch = [&](uint32_t r) -> uint2 {
             const uint64_t idx = i0 + r;
             if (idx >= a.nb) return make_uint2(kNoKey, 0u);
-            return make_uint2(__ldg(K + idx), __ldg(V + idx));
+            return make_uint2(__ldca(K + idx), __ldca(V + idx));
         };
         // This copier warp's share of the copies of the step that starts at tile-relative position `base`.
         auto issue = [&](uint32_t base, uint32_t buf) {
@@ -861,8 +861,8 @@ det_apply_long_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_
 constexpr unsigned kLowWarps = 4;
 
 template <bool SIGN, bool SHORT>
-__device__ __forceinline__ void low_walk(const ApplyArgs& a, const uint32_t* __restrict__ K,
-                                         const uint32_t* __restrict__ V, const uint32_t* bag_of,
+__device__ __forceinline__ void low_walk(const ApplyArgs& a, const uint32_t* K,
+                                         const uint32_t* V, const uint32_t* bag_of,
                                          uint64_t from, uint64_t to, uint64_t j_plus, float& acc,
                                          bool& touched) {
     const uint32_t lane = threadIdx.x & 31;
@@ -870,7 +870,7 @@ __device__ __forceinline__ void low_walk(const ApplyArgs& a, const uint32_t* __r
         const uint64_t i = i0 + lane;
         float term = 0.0f;
         bool ok = false;
-        if (i < to) ok = block_term<SIGN, SHORT>(a, bag_of, __ldg(V + i), (uint32_t)(j_plus - __ldg(K + i)), term);
+        if (i < to) ok = block_term<SIGN, SHORT>(a, bag_of, __ldca(V + i), (uint32_t)(j_plus - __ldca(K + i)), term);
         const uint32_t oks = __ballot_sync(0xFFFFFFFFu, ok);
         if (oks != 0) touched = true;
         for (uint32_t rest = oks; rest != 0; rest &= rest - 1) {
@@ -881,19 +881,19 @@ __device__ __forceinline__ void low_walk(const ApplyArgs& a, const uint32_t* __r
 }
 
 // first sorted position with key >= bound (warp-uniform)
-__device__ __forceinline__ uint64_t first_at_least(const uint32_t* __restrict__ K, uint64_t nb, uint64_t bound) {
+__device__ __forceinline__ uint64_t first_at_least(const uint32_t* K, uint64_t nb, uint64_t bound) {
     uint64_t lo = 0, hi = nb;
     while (lo < hi) {
         const uint64_t mid = lo + ((hi - lo) >> 1);
-        if ((uint64_t)__ldg(K + mid) >= bound) hi = mid; else lo = mid + 1;
+        if ((uint64_t)__ldca(K + mid) >= bound) hi = mid; else lo = mid + 1;
     }
     return lo;
 }
 
 template <bool SIGN, int MODE, bool SHORT>
 __global__ void __launch_bounds__(32 * kLowWarps)
-det_apply_low_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V,
-                     const uint32_t* __restrict__ bag_of) {
+det_apply_low_kernel(ApplyArgs a, const uint32_t* K, const uint32_t* V,
+                     const uint32_t* bag_of) {
     if (a.status != nullptr && *a.status != 0) return;
     const MapParams& mp = a.mp;
     const uint32_t j = blockIdx.x * kLowWarps + (threadIdx.x >> 5);
@@ -917,8 +917,8 @@ constexpr int kBinnedPer = 8;  // sorted blocks per thread group, all their load
 
 template <bool SIGN, bool SHORT>
 __global__ void __launch_bounds__(256)
-binned_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V,
-                    const uint32_t* __restrict__ bag_of, uint32_t log2Zp) {
+binned_apply_kernel(ApplyArgs a, const uint32_t* K, const uint32_t* V,
+                    const uint32_t* bag_of, uint32_t log2Zp) {
     follow();
     if (a.status != nullptr && *a.status != 0) return;
     const MapParams& mp = a.mp;
@@ -930,8 +930,8 @@ binned_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t*
 #pragma unroll
     for (int t = 0; t < kBinnedPer; ++t) {
         const uint64_t i = i0 + t < a.nb ? i0 + t : a.nb - 1;
-        k[t] = __ldg(K + i);
-        v[t] = __ldg(V + i);
+        k[t] = __ldca(K + i);
+        v[t] = __ldca(V + i);
     }
     const uint64_t pol = l2_keep_policy(a.l2_keep != 0);
     float term[kBinnedPer];
@@ -951,14 +951,14 @@ binned_apply_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t*
 
 // answer = do starts repeat among 32 neighbours of the sorted list?  128 places looked at, a quarter of them with a
 // repeat is a yes.
-__global__ void __launch_bounds__(1024) binned_sample_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* answer) {
+__global__ void __launch_bounds__(1024) binned_sample_kernel(const uint32_t* K, uint64_t nb, uint32_t* answer) {
     follow();
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t found = 0;
 #pragma unroll
     for (uint32_t q = 0; q < 4; ++q) {
         const uint64_t at = (nb - 32) / 128 * (w * 4 + q) + lane;  // (nb is large)
-        const uint32_t k = __ldg(K + at);
+        const uint32_t k = __ldca(K + at);
         found += __any_sync(0xFFFFFFFFu, __popc(__match_any_sync(0xFFFFFFFFu, k)) > 1) ? 1u : 0u;
     }
     __shared__ uint32_t total_s;
@@ -1030,7 +1030,7 @@ __device__ __forceinline__ void binned_add_merged(const ApplyArgs& a, uint32_t k
 #pragma unroll
                 for (int q = 0; q < EPL; ++q)
                     x[u][q] = ol + 32 * q < l && ROBE_CHK((uint64_t)row + 32 * q < a.grad_elems, ROBE_DBG_GRAD_POS)
-                                  ? __ldg(a.grad_out + (row + 32 * q))
+                                  ? __ldca(a.grad_out + (row + 32 * q))
                                   : 0.0f;
             }
 #pragma unroll
@@ -1056,7 +1056,7 @@ __device__ __forceinline__ void binned_add_merged(const ApplyArgs& a, uint32_t k
 // gradient rows, read once per id (going through odd bins backwards, to meet rows again in L2, changed nothing)
 template <int LP, int EPL, bool SHORT>
 __global__ void __launch_bounds__(256)
-binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const uint32_t* __restrict__ V) {
+binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* K, const uint32_t* V) {
     follow();
     if (a.status != nullptr && *a.status != 0) return;
     constexpr uint32_t G = 32 / LP;              // blocks at a time
@@ -1070,8 +1070,8 @@ binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const ui
     const uint32_t cnt = i0 >= a.nb ? 0u : (a.nb - i0 < 32 ? (uint32_t)(a.nb - i0) : 32u);
     uint32_t k = kNoKey, v = 0, len = 0;         // (length 0: nothing of the block is added)
     if (lane < cnt) {
-        k = __ldg(K + i0 + lane);
-        v = __ldg(V + i0 + lane);
+        k = __ldca(K + i0 + lane);
+        v = __ldca(V + i0 + lane);
         len = Z;
         if (SHORT) {
             const uint32_t left = mp.d - v % mp.d;
@@ -1095,7 +1095,7 @@ binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const ui
                 slot[u] = __shfl_sync(0xFFFFFFFFu, k, src) + ol;
                 const float* row = a.grad_out + (__shfl_sync(0xFFFFFFFFu, v, src) + ol);
 #pragma unroll
-                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < Z ? __ldg(row + 32 * q) : 0.0f;
+                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < Z ? __ldca(row + 32 * q) : 0.0f;
             }
 #pragma unroll
             for (int u = 0; u < U; ++u)
@@ -1112,7 +1112,7 @@ binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* __restrict__ K, const ui
                 const float* row = a.grad_out + (__shfl_sync(0xFFFFFFFFu, v, src) + ol);
                 l[u] = __shfl_sync(0xFFFFFFFFu, len, src);
 #pragma unroll
-                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < l[u] ? __ldg(row + 32 * q) : 0.0f;
+                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < l[u] ? __ldca(row + 32 * q) : 0.0f;
             }
 #pragma unroll
             for (int u = 0; u < U; ++u)

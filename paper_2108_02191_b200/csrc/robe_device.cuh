@@ -51,17 +51,33 @@ __device__ __forceinline__ void follow() {
     if (EARLY) asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// The same; the kernel after this one may take its place once all of this one's CTAs have begun AND all kernels
+// before it have finished: what those wrote is read-only for the next kernel from its first instruction on.
+__device__ __forceinline__ void follow_settled() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+
+// Loads.  A kernel launched by launch_next is resident while the kernel before it still writes, so what that one
+// may write - ids, offsets, gradients, the array, sorted blocks - is not read-only for its lifetime, which is
+// what ld.global.nc (__ldg, const __restrict__ parameters) asks for; and nothing keeps an invariant load, or an
+// asm that is not volatile, behind the wait of follow().  So the kernels load with __ldca, __ldcs (volatile,
+// ld.global) or plainly.  Only a kernel whose predecessor is a follow_settled() one may read with this what
+// still earlier kernels wrote.  It pays in a loop of loads and warp barriers (strip apply on 34 M blocks of 16:
+// 917 us, 1035 with coherent loads).
+template <class T>
+__device__ __forceinline__ T load_settled(const T* p) { return __ldg(p); }
 
 struct HashConsts {  // all < P
     uint64_t A, B, C, D;
 };
 
-// The ids of a call: int64 (default) or int32 elements, read through the read-only path.
+// The ids of a call: int64 (default) or int32 elements.
 struct IdList {
     const void* p;
     int i32;  // 0: int64_t elements, 1: int32_t elements
     __device__ __forceinline__ int64_t load(int64_t pos) const {
-        return i32 ? (int64_t)__ldg((const int32_t*)p + pos) : __ldg((const int64_t*)p + pos);
+        return i32 ? (int64_t)((const int32_t*)p)[pos] : ((const int64_t*)p)[pos];
     }
 };
 
@@ -206,13 +222,10 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
 
 template <int DT>
 __device__ __forceinline__ float load_elem(const void* array, uint32_t j) {
-    if (DT == 0) return __ldg((const float*)array + j);
-    return bf16_bits_to_float(__ldg((const unsigned short*)array + j));
+    if (DT == 0) return __ldca((const float*)array + j);
+    return bf16_bits_to_float(__ldca((const unsigned short*)array + j));
 }
 
-// Array read of the gather kernels: read-only path, with the 64-byte L2 fetch hint.  Random
-// Z-blocks gain nothing from the wider default fetch; measured on B200 this hint shortens a
-// random 64-byte-block gather from a 1 GB array by about 13 %.
 // L2 cache policy "keep": lines fetched under it are the last to be evicted.  For an array about
 // the size of the L2 that shares it with gigabytes of streamed ids, output rows and gradients.
 // 0 stands for "no policy" (createpolicy never returns 0 for evict_last).
@@ -230,31 +243,18 @@ __device__ __forceinline__ void red_add(float* p, float v, uint64_t pol) {
         atomicAdd(p, v);
 }
 
+// Array read of the gather kernels, with the 64-byte L2 fetch hint.  Random Z-blocks gain nothing from the
+// wider default fetch; measured on B200 this hint shortens a random 64-byte-block gather from a 1 GB array by
+// about 13 %.
 template <int DT>
-__device__ __forceinline__ float gather_elem(const void* array, uint32_t j, uint64_t pol = 0) {
-    if (pol != 0) {  // (warp-uniform)
-        if (DT == 0) {
-            float v;
-            asm("ld.global.nc.L2::cache_hint.L2::64B.f32 %0, [%1], %2;"
-                : "=f"(v)
-                : "l"((const float*)array + j), "l"(pol));
-            return v;
-        }
-        unsigned short b;
-        asm("ld.global.nc.L2::cache_hint.L2::64B.u16 %0, [%1], %2;"
-            : "=h"(b)
-            : "l"((const unsigned short*)array + j), "l"(pol));
-        return bf16_bits_to_float(b);
-    }
+__device__ __forceinline__ float gather_elem(const void* array, uint32_t j) {
     if (DT == 0) {
         float v;
-        asm("ld.global.nc.L2::64B.f32 %0, [%1];" : "=f"(v) : "l"((const float*)array + j));
+        asm volatile("ld.global.L2::64B.f32 %0, [%1];" : "=f"(v) : "l"((const float*)array + j));
         return v;
     }
     unsigned short b;
-    asm("ld.global.nc.L2::64B.u16 %0, [%1];"
-                 : "=h"(b)
-                 : "l"((const unsigned short*)array + j));
+    asm volatile("ld.global.L2::64B.u16 %0, [%1];" : "=h"(b) : "l"((const unsigned short*)array + j));
     return bf16_bits_to_float(b);
 }
 

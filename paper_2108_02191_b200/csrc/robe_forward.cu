@@ -236,7 +236,7 @@ fwd_staged_kernel(FwdArgs a, uint32_t ids_per_batch, uint32_t cmagic) {
 // the lanes of the first id hold the sum and fetch the other ids' vectors by shuffle, in order.
 __device__ __forceinline__ float4 ldg_f4_64B(const float* p) {
     float4 v;
-    asm("ld.global.nc.L2::64B.v4.f32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L2::64B.v4.f32 {%0, %1, %2, %3}, [%4];"
         : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
         : "l"(p));
     return v;

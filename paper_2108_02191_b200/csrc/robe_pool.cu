@@ -110,7 +110,7 @@ __device__ __forceinline__ PoolRun pool_run(const PoolArgs& a, uint32_t w, uint3
     const int64_t left = a.nbags - r.k0;
     r.bags = left <= 0 ? 0u : (left < (int64_t)a.bags ? (uint32_t)left : a.bags);
     r.off = 0;
-    if (r.bags != 0) r.off = clamp64(__ldg(a.offsets + r.k0 + (lane < r.bags ? lane : r.bags)), 0, a.nnz);
+    if (r.bags != 0) r.off = clamp64(__ldca(a.offsets + r.k0 + (lane < r.bags ? lane : r.bags)), 0, a.nnz);
     const int64_t next = __shfl_down_sync(0xFFFFFFFFu, r.off, 1);
     r.stretch = __all_sync(0xFFFFFFFFu, lane >= r.bags || next >= r.off);
     return r;

@@ -16,8 +16,8 @@ __device__ __forceinline__ void bag_range(const int64_t* offsets, int64_t nnz, i
         lo = k;
         hi = k + 1;
     } else {
-        lo = clamp64(__ldg(offsets + k), 0, nnz);
-        hi = clamp64(__ldg(offsets + k + 1), lo, nnz);
+        lo = clamp64(__ldca(offsets + k), 0, nnz);
+        hi = clamp64(__ldca(offsets + k + 1), lo, nnz);
     }
 }
 

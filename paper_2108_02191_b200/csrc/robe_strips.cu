@@ -66,10 +66,10 @@ constexpr uint32_t kBoundsGap = 256;  // longer gaps are filled by the whole war
 // against 90 of the scan below; 852 K keys, 8437 strips: 12 (a warp per strip, 32 probes at a time: 7)
 // against 5.
 __global__ void __launch_bounds__(256)
-strip_bounds_search_kernel(const uint32_t* __restrict__ K, uint32_t nb, uint32_t* __restrict__ lo_of,
-                           uint32_t* __restrict__ hi_of, uint32_t strips, uint32_t log2w, uint32_t reach,
+strip_bounds_search_kernel(const uint32_t* K, uint32_t nb, uint32_t* lo_of,
+                           uint32_t* hi_of, uint32_t strips, uint32_t log2w, uint32_t reach,
                            const int32_t* status, uint32_t* hot_count) {
-    follow<true>();
+    follow_settled();
     if (blockIdx.x == 0 && threadIdx.x < 3) hot_count[threadIdx.x] = 0;  // (for the kernels after this one)
     if (status != nullptr && *status != 0) return;  // after a failed input check K was not written
     const uint32_t b = blockIdx.x * 256 + threadIdx.x;
@@ -79,14 +79,14 @@ strip_bounds_search_kernel(const uint32_t* __restrict__ K, uint32_t nb, uint32_t
     auto search = [&](uint32_t from, uint32_t to, uint64_t least) {
         while (from < to) {
             const uint32_t mid = from + ((to - from) >> 1);
-            if ((uint64_t)__ldg(K + mid) >= least) to = mid; else from = mid + 1;
+            if ((uint64_t)K[mid] >= least) to = mid; else from = mid + 1;
         }
         return from;
     };
     const uint64_t first_slot = (uint64_t)b << log2w, least = first_slot > reach ? first_slot - reach : 0;
     const uint32_t hi = search(0, nb, first_slot);
     uint32_t to = hi, step = 1;
-    while (to >= step && (uint64_t)__ldg(K + (to - step)) >= least) {
+    while (to >= step && (uint64_t)K[to - step] >= least) {
         to -= step;
         step <<= 1;  // (the steps add up to less than nb)
     }
@@ -97,25 +97,25 @@ strip_bounds_search_kernel(const uint32_t* __restrict__ K, uint32_t nb, uint32_t
 // The same for few strips, by reading the list.  A thread takes eight sorted positions; position i begins the strips
 // whose first slot lies past the key before it and not past its own (lo_of: the same of the blocks' last slots).
 __global__ void __launch_bounds__(256)
-strip_bounds_kernel(const uint32_t* __restrict__ K, uint64_t nb, uint32_t* __restrict__ lo_of,
-                    uint32_t* __restrict__ hi_of, uint32_t strips, uint32_t log2w, uint32_t reach, const int32_t* status,
+strip_bounds_kernel(const uint32_t* K, uint64_t nb, uint32_t* lo_of,
+                    uint32_t* hi_of, uint32_t strips, uint32_t log2w, uint32_t reach, const int32_t* status,
                     uint32_t* hot_count) {
-    follow<true>();
+    follow_settled();
     if (blockIdx.x == 0 && threadIdx.x < 3) hot_count[threadIdx.x] = 0;  // (for the kernels after this one)
     if (status != nullptr && *status != 0) return;  // after a failed input check K was not written
     const uint64_t i0 = ((uint64_t)blockIdx.x * 256 + threadIdx.x) * 8;
     const uint32_t lane = threadIdx.x & 31;
     uint32_t k[9];  // k[0]: the key before
     if (i0 + 8 <= nb) {
-        const uint4 x = __ldg(reinterpret_cast<const uint4*>(K + i0)), y = __ldg(reinterpret_cast<const uint4*>(K + i0) + 1);
+        const uint4 x = reinterpret_cast<const uint4*>(K + i0)[0], y = reinterpret_cast<const uint4*>(K + i0)[1];
         k[1] = x.x; k[2] = x.y; k[3] = x.z; k[4] = x.w;
         k[5] = y.x; k[6] = y.y; k[7] = y.z; k[8] = y.w;
     } else {
 #pragma unroll
-        for (int t = 0; t < 8; ++t) k[t + 1] = i0 + t < nb ? __ldg(K + i0 + t) : 0u;
+        for (int t = 0; t < 8; ++t) k[t + 1] = i0 + t < nb ? K[i0 + t] : 0u;
     }
     k[0] = __shfl_up_sync(0xFFFFFFFFu, k[8], 1);
-    if (lane == 0 && i0 > 0 && i0 <= nb) k[0] = __ldg(K + i0 - 1);
+    if (lane == 0 && i0 > 0 && i0 <= nb) k[0] = K[i0 - 1];
     if (__all_sync(0xFFFFFFFFu, i0 > 0 && i0 + 8 <= nb && ((k[8] + reach) >> log2w) - (k[0] >> log2w) <= kBoundsGap)) {
         // in the middle of the list (most threads): a position begins a strip, or a few, or none
         uint32_t h = k[0] >> log2w, l = (k[0] + reach) >> log2w;
@@ -203,7 +203,7 @@ template <int MODE, int LP, int EPL, bool SHORT>
 __global__ void __launch_bounds__(32 * kStripWarps, 5)
 strip_apply_kernel(StripArgs a) {
     extern __shared__ float4 strip_smem[];
-    follow();
+    follow();  // (after strip_bounds_*, which are settled: sorted blocks and gradients are read-only here)
     if (a.status != nullptr && *a.status != 0) return;
     constexpr uint32_t G = 32 / LP;               // groups per warp
     constexpr int U = EPL == 4 ? 4 : 8;           // blocks whose loads are in flight together
@@ -214,8 +214,8 @@ strip_apply_kernel(StripArgs a) {
     volatile float* const sum = reinterpret_cast<float*>(strip_smem) + (w * G + g) * W;
     uint32_t lo = 0, n = 0;
     if (b < a.strips) {
-        lo = __ldg(a.lo_of + b);
-        n = __ldg(a.hi_of + b + 1) - lo;
+        lo = a.lo_of[b];
+        n = a.hi_of[b + 1] - lo;
         if (n > a.n_hot) n = 0;  // the hot kernel's
     }
     const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n);
@@ -228,8 +228,8 @@ strip_apply_kernel(StripArgs a) {
     // lane ol holds block ol of the present LP: start relative to the strip, payload
     uint32_t nk = 0, nv = 0;
     if (ol < n) {
-        nk = __ldg(a.K + lo + ol);
-        nv = __ldg(a.V + lo + ol);
+        nk = load_settled(a.K + lo + ol);
+        nv = load_settled(a.V + lo + ol);
     }
     __syncwarp();
     for (uint32_t c0 = 0; c0 < most; c0 += LP) {
@@ -237,8 +237,8 @@ strip_apply_kernel(StripArgs a) {
         const uint32_t rel = c0 + ol < n ? nk - w0 : 0x40000000u, v = nv;
         const uint32_t len = SHORT ? strip_len<SHORT>(a.mp, v) : 0u;
         if (c0 + LP + ol < n) {
-            nk = __ldg(a.K + lo + c0 + LP + ol);
-            nv = __ldg(a.V + lo + c0 + LP + ol);
+            nk = load_settled(a.K + lo + c0 + LP + ol);
+            nv = load_settled(a.V + lo + c0 + LP + ol);
         }
 #pragma unroll 1
         for (uint32_t u0 = 0; u0 < LP && c0 + u0 < most; u0 += U) {
@@ -255,7 +255,7 @@ strip_apply_kernel(StripArgs a) {
                     x[u][q] = -0.0f;
                     if (slot[u] + 32 * q < W && ol + 32 * q < l &&
                         ROBE_CHK((uint64_t)p + 32 * q < a.grad_elems, ROBE_DBG_GRAD_POS))
-                        x[u][q] = __ldg(a.grad_out + (p + 32 * q)) + 0.0f;  // -0 -> +0
+                        x[u][q] = load_settled(a.grad_out + (p + 32 * q)) + 0.0f;  // -0 -> +0
                 }
             }
 #pragma unroll

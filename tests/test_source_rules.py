@@ -1,0 +1,54 @@
+"""Rules that every kernel source keeps and that no run can show to be broken: what would hold only by luck, on
+the code as compiled today."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2108_02191_b200", "csrc")
+SOURCES = sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")))
+
+
+def code(path):
+    """The file without comments."""
+    text = open(path).read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+def body(text, name):
+    """The body of the kernel `name`."""
+    at = text.index("{", re.search(r"\b%s\s*\([^;]*?\)\s*(?=\{)" % name, text).start())
+    depth = 0
+    for k in range(at, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[k], 0)
+        if depth == 0:
+            return text[at:k + 1]
+    raise AssertionError(name)
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_no_read_only_loads(path):
+    # kernels are set up while the one before them still writes (launch_next): nothing of a call's data is
+    # read-only for their lifetime, and an invariant load may be moved to before the wait
+    text = code(path)
+    text = re.sub(r"T load_settled\(const T\* p\) \{[^}]*\}", "", text)
+    assert not re.search(r"\b__ldg\s*\(|\.nc\b|__restrict__", text)
+    # loads in assembly stay behind the wait only as volatile ones
+    assert not re.search(r'asm\s*\(\s*"ld\.global', text)
+
+
+def test_settled_loads_follow_a_settled_kernel():
+    # the one kernel with read-only loads: what it reads with them was written before its predecessors, which
+    # let it take its place only after their own wait
+    text = {os.path.basename(p): code(p) for p in SOURCES}
+    used = {n: len(re.findall(r"\bload_settled\(", t)) for n, t in text.items()}
+    apply = body(text["robe_strips.cu"], "strip_apply_kernel")
+    assert {n for n, k in used.items() if k} == {"robe_device.cuh", "robe_strips.cu"} and used["robe_device.cuh"] == 1
+    assert used["robe_strips.cu"] == len(re.findall(r"\bload_settled\(", apply))
+    assert set(re.findall(r"\bload_settled\(\(?(\w+(?:\.\w+)?)", apply)) <= {"a.K", "a.V", "a.grad_out"}
+    prepare = text["robe_strips.cu"][text["robe_strips.cu"].index("void launch_strips_prepare"):]
+    launched = re.findall(r"launch_next\((\w+)", prepare[:prepare.index("void launch_strips(")])
+    assert launched
+    for name in launched:
+        assert re.match(r"\{\s*follow_settled\(\);", body(text["robe_strips.cu"], name)), name
