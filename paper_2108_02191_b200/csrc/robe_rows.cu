@@ -77,14 +77,21 @@ __device__ __forceinline__ bool rows_sort(const RowsArgs& a, RowsSmem& sm, uint3
     }
     __syncthreads();
     bool repeats = false;
-    for (uint32_t r = tid; r < rows; r += kRowsThreads) {
-        uint32_t e;
-        const uint32_t p = rows_position(a, row0 + r, e);
-        const uint64_t base = addmod_p61(table_term(mp.h, e), mulmod_p61_any(mp.h.B, (uint64_t)a.indices.load(p)));
-        sm.base[r] = base;
-        const uint32_t bin = mod_m(base, mp.m, mp.mu) >> a.shift;
-        if (ROBE_CHK(bin < kRowsBins, ROBE_DBG_SHARED)) atomicAdd(&sm.cursor[bin], 1u);
-        if (r < kRowsThreads) repeats = __popc(__match_any_sync(__activemask(), base)) > 1;
+    for (uint32_t r0 = 0; r0 < rows; r0 += kRowsThreads) {  // (whole warps: the match below takes all lanes)
+        const uint32_t r = r0 + tid;
+        uint64_t base = ~0ull;  // (above every base: rows past the end match one another only)
+        if (r < rows) {
+            uint32_t e;
+            const uint32_t p = rows_position(a, row0 + r, e);
+            base = addmod_p61(table_term(mp.h, e), mulmod_p61_any(mp.h.B, (uint64_t)a.indices.load(p)));
+            sm.base[r] = base;
+            const uint32_t bin = mod_m(base, mp.m, mp.mu) >> a.shift;
+            if (ROBE_CHK(bin < kRowsBins, ROBE_DBG_SHARED)) atomicAdd(&sm.cursor[bin], 1u);
+        }
+        if (r0 == 0) {
+            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, base);
+            repeats = r < rows && __popc(peers) > 1;
+        }
     }
     // No id repeats inside a warp's first 32 rows: the ids are spread so thinly that sorting would bring
     // next to nothing together.

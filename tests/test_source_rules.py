@@ -52,3 +52,9 @@ def test_settled_loads_follow_a_settled_kernel():
     assert launched
     for name in launched:
         assert re.match(r"\{\s*follow_settled\(\);", body(text["robe_strips.cu"], name)), name
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_warp_calls_name_lanes_that_are_sure_to_arrive(path):
+    # the lanes active at one call need not be those at the next: a mask read from the hardware is no promise
+    assert "__activemask" not in code(path)
