@@ -42,7 +42,7 @@ struct Reader {
             return nullptr;
         }
         const at::Tensor& t = THPVariable_Unpack(args[k]);
-        if (!t.is_cuda() || !t.is_contiguous()) {
+        if (!t.is_cuda() || !t.has_storage() || !t.is_contiguous()) {
             ok = false;
             return nullptr;
         }
@@ -129,6 +129,20 @@ struct Reader {
         return p;
     }
 };
+
+// What the interpreter calls.  Torch reports a tensor whose memory cannot be had (sparse, fake, transformed
+// ones) or a device it cannot reach by a C++ exception, which must not pass into the interpreter: such a call
+// is not taken, and the ctypes path raises what there is to raise.  (Arguments are read before the library is
+// called, and the library throws nothing.)
+template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* args, Py_ssize_t n) {
+    try {
+        return F(self, args, n);
+    } catch (const std::exception&) {
+        PyErr_Clear();
+        return PyLong_FromLong(kNotTaken);
+    }
+}
 
 // The call itself, without the interpreter lock: a full launch queue makes a launch wait.
 template <class F>
@@ -287,7 +301,7 @@ PyObject* set_calls(PyObject*, PyObject* const* args, Py_ssize_t n) {
     Py_RETURN_NONE;
 }
 
-#define FAST(f) ((PyCFunction)(void (*)(void))(f))
+#define FAST(...) ((PyCFunction)(void (*)(void))(&guarded<__VA_ARGS__>))
 PyMethodDef methods[] = {
     {"set_calls", FAST(set_calls), METH_FASTCALL, "addresses of the C-ABI functions"},
     {"forward", FAST(forward), METH_FASTCALL, "robe_forward"},

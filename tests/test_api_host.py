@@ -174,3 +174,29 @@ def test_c_program_links_and_calls_the_library(tmp_path):
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, (r.returncode, r.stderr)
     assert int(r.stdout.strip()) == int(orc.hash_constants(7)[1])  # A_h as the oracle draws it
+
+
+FAKE_TENSORS = r"""
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+import paper_2108_02191_b200 as robe
+h = robe.robe_create(4096, 4, 16, 4, 7)
+with FakeTensorMode():  # CUDA tensors without memory, as tracing and shape propagation hand them over
+    ids = torch.empty(8, dtype=torch.int64, device="cuda")
+    out = torch.empty(2, 4, 16, device="cuda")
+for call in (lambda: robe.robe_forward(h, ids, None, 2, out),
+             lambda: robe.robe_backward(h, out, ids, None, 2, out),
+             lambda: robe.robe_apply_sgd(h, out, 0.1)):
+    try:
+        call()
+    except Exception as e:
+        print("raised", type(e).__name__)
+"""
+
+
+def test_tensors_without_memory_raise_and_do_not_end_the_process():
+    import subprocess
+    import sys
+    r = subprocess.run([sys.executable, "-c", FAKE_TENSORS], cwd=ROOT, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
+    assert r.stdout.count("raised") == 3, r.stdout + r.stderr[-2000:]
