@@ -99,7 +99,7 @@ for _name in EXPORTS:
     if _name not in ("robe_backward_workspace_bytes", "robe_status_string"):
         getattr(_lib, _name).restype = C.c_int
 
-_native.set_calls(*(C.cast(getattr(_lib, _name), _vp).value for _name in (
+_native.set_calls(_vp, *(C.cast(getattr(_lib, _name), _vp).value for _name in (
     "robe_set_option", "robe_forward", "robe_forward_keep", "robe_backward", "robe_backward_kept",
     "robe_backward_adam", "robe_backward_adagrad", "robe_apply_sgd")))
 _NOT_TAKEN = 1  # from _native: nothing was called

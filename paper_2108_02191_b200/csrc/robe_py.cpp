@@ -31,6 +31,8 @@ struct Calls {
     decltype(&robe_apply_sgd) apply_sgd;
 } calls;
 
+PyObject* handle_type;  // ctypes.c_void_p
+
 // Reads the arguments of one call; ok turns false at the first one that is not plainly usable.
 struct Reader {
     PyObject* const* args;
@@ -97,11 +99,11 @@ struct Reader {
         }
         return (float)v;
     }
-    // a ctypes.c_void_p: its buffer is the pointer
+    // a ctypes.c_void_p and nothing else that has a buffer: its buffer is the pointer
     robe_handle_t handle(int k) {
         Py_buffer b;
         robe_handle_t h = nullptr;
-        if (!PyObject_CheckBuffer(args[k]) || PyObject_GetBuffer(args[k], &b, PyBUF_SIMPLE) != 0) {
+        if ((PyObject*)Py_TYPE(args[k]) != handle_type || PyObject_GetBuffer(args[k], &b, PyBUF_SIMPLE) != 0) {
             PyErr_Clear();
             ok = false;
             return nullptr;
@@ -283,17 +285,19 @@ PyObject* apply_sgd(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return made([&] { return calls.apply_sgd(h, grad_array, lr, zero, st); });
 }
 
-// (addresses of the C-ABI functions, in the order of Calls)
+// (the type of a handle, addresses of the C-ABI functions in the order of Calls)
 PyObject* set_calls(PyObject*, PyObject* const* args, Py_ssize_t n) {
     void* p[8];
-    if (n != 8) {
-        PyErr_SetString(PyExc_TypeError, "set_calls takes eight addresses");
+    if (n != 9) {
+        PyErr_SetString(PyExc_TypeError, "set_calls takes a type and eight addresses");
         return nullptr;
     }
     for (int k = 0; k < 8; ++k) {
-        p[k] = PyLong_AsVoidPtr(args[k]);
+        p[k] = PyLong_AsVoidPtr(args[k + 1]);
         if (PyErr_Occurred()) return nullptr;
     }
+    Py_INCREF(args[0]);
+    Py_XSETREF(handle_type, args[0]);
     calls = Calls{(decltype(calls.set_option))p[0],       (decltype(calls.forward))p[1],
                   (decltype(calls.forward_keep))p[2],     (decltype(calls.backward))p[3],
                   (decltype(calls.backward_kept))p[4],    (decltype(calls.backward_adam))p[5],
@@ -303,7 +307,7 @@ PyObject* set_calls(PyObject*, PyObject* const* args, Py_ssize_t n) {
 
 #define FAST(...) ((PyCFunction)(void (*)(void))(&guarded<__VA_ARGS__>))
 PyMethodDef methods[] = {
-    {"set_calls", FAST(set_calls), METH_FASTCALL, "addresses of the C-ABI functions"},
+    {"set_calls", FAST(set_calls), METH_FASTCALL, "type of a handle, addresses of the C-ABI functions"},
     {"forward", FAST(forward), METH_FASTCALL, "robe_forward"},
     {"forward_keep", FAST(forward_keep), METH_FASTCALL, "robe_forward_keep"},
     {"backward", FAST(backward<&Calls::backward>), METH_FASTCALL, "robe_backward"},

@@ -200,3 +200,17 @@ def test_tensors_without_memory_raise_and_do_not_end_the_process():
     r = subprocess.run([sys.executable, "-c", FAKE_TENSORS], cwd=ROOT, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
     assert r.stdout.count("raised") == 3, r.stdout + r.stderr[-2000:]
+
+
+def test_only_a_handle_is_taken_for_one():
+    # eight bytes of anything else (an array that holds the address, a plain integer of that size) are refused
+    from types import SimpleNamespace
+    h = robe.robe_create(4096, 4, 16, 4, 7)
+    stream = SimpleNamespace(cuda_stream=0)
+    with pytest.raises(robe.RobeError) as ei:  # the handle itself: the library says what is missing
+        robe.robe_apply_sgd(h, None, 0.1, True, stream)
+    assert ei.value.status == robe.ROBE_ERR_INVALID_ARG
+    for other in (np.array([h.value], dtype=np.uint64), C.c_uint64(h.value), bytearray(C.string_at(C.addressof(h), 8))):
+        with pytest.raises(C.ArgumentError):
+            robe.robe_apply_sgd(other, None, 0.1, True, stream)
+    robe.robe_destroy(h)
