@@ -342,9 +342,8 @@ int robe_apply_sgd(robe_handle_t h, float* grad_array, float lr, int zero_grad, 
  *
  * Limit: the call must fit the fixed array, i.e. the value robe_backward_workspace_bytes
  * reports for it in deterministic mode (about 19 bytes per block, nnz * ceil(d/Z) blocks,
- * plus 4 bytes per id, 0.4 MB of counters and lists, and, where the call touches the array
- * densely, the bounds of its strips: M/8 bytes for small arrays, M/32 from 2.4 M slots on)
- * must not exceed
+ * plus 4 bytes per id, 0.3 MB of counters and lists, and up to 0.25 MB more where a call
+ * touches an array of up to 5.5 M slots densely) must not exceed
  * ROBE_STATIC_SCRATCH_BYTES; a larger call returns ROBE_ERR_WORKSPACE and launches nothing.
  *
  * First call on a device: the function looks up the device address of the array once per

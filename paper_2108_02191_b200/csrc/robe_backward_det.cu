@@ -1144,17 +1144,22 @@ uint32_t bits_for(uint32_t m) {  // bits needed for keys in [0, m)
 }
 
 struct Layout {
-    size_t keysA, keysB, valsA, valsB, bag_of, counts, totals, long_count, long_walks, strips, total;
+    size_t keysA, valsA, keysB, valsB, bag_of, counts, totals, long_count, long_walks, strips, total;
     uint32_t long_cap;
+    bool strips_own, strips_spare;  // the strips' bounds and lists have room of their own / fit the free pair of buffers
 };
+
+// Arrays whose strips can never ask for more than this (up to 5.5 M slots) have room for them in the workspace.
+constexpr size_t kStripRoom = 256 << 10;
 
 Layout make_layout(uint64_t nb, int64_t nnz, bool bags, const MapParams& mp) {
     Layout L;
     size_t off = 0;
     const size_t kb = align256((nb ? nb : 1) * sizeof(uint32_t));
+    // starts and payloads side by side: the pair that the last sort pass read from is free for the strips
     L.keysA = off; off += kb;
-    L.keysB = off; off += kb;
     L.valsA = off; off += kb;
+    L.keysB = off; off += kb;
     L.valsB = off; off += kb;
     L.bag_of = off; off += bags ? align256((size_t)(nnz ? nnz : 1) * sizeof(uint32_t)) : 0;
     L.counts = off; off += align256((size_t)kRadix * kSortMaxGrid * sizeof(uint32_t));
@@ -1165,8 +1170,13 @@ Layout make_layout(uint64_t nb, int64_t nnz, bool bags, const MapParams& mp) {
     L.long_cap = (uint32_t)cap;
     L.long_count = off; off += 256;
     L.long_walks = off; off += align256((size_t)cap * sizeof(LongWalk));
-    // (the sign option may be switched after the workspace was sized: room for the strips either way)
-    L.strips = off; off += strips_ok(mp, nb, false) ? strips_workspace_bytes(mp, nb) : 0;
+    // (The sign option may be switched after the workspace was sized: room for the strips either way.)  The total
+    // must not fall as nb grows: a caller sizes for its largest call.  On a longer array the strips go to the
+    // free pair; where they do not fit that, there is less than a block per strip, and the call goes without.
+    const size_t strips = strips_ok(mp, nb, false) ? strips_workspace_bytes(mp, nb) : 0;
+    L.strips_own = strips != 0 && strips_workspace_bytes(mp, 1ull << 40) <= kStripRoom;
+    L.strips_spare = strips != 0 && !L.strips_own && strips <= 2 * kb;
+    L.strips = off; off += L.strips_own ? strips : 0;
     L.total = off;
     return L;
 }
@@ -1351,12 +1361,13 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
     uint32_t* long_count = (uint32_t*)(ws + L.long_count);
     const ApplyArgs aa{mp, grad_out, pb.indices, target, lr, nb, pb.status, adam ? *adam : AdamState{},
                        long_count, (LongWalk*)(ws + L.long_walks), L.long_cap, (uint64_t)pb.nbags * mp.d, 0};
-    if (strips_ok(mp, nb, pb.sign != 0)) {
+    if ((L.strips_own || L.strips_spare) && strips_ok(mp, nb, pb.sign != 0)) {
         const SideStream side{pb.side, pb.fork_event, pb.join_event};
-        if (mode == 4) launch_apply_strips<3>(aa, kA, vA, mode, ws + L.strips, side, st);
-        else if (mode == 2) launch_apply_strips<2>(aa, kA, vA, mode, ws + L.strips, side, st);
-        else if (mode == 1) launch_apply_strips<1>(aa, kA, vA, mode, ws + L.strips, side, st);
-        else launch_apply_strips<0>(aa, kA, vA, mode, ws + L.strips, side, st);
+        void* const room = L.strips_own ? (void*)(ws + L.strips) : (void*)kB;
+        if (mode == 4) launch_apply_strips<3>(aa, kA, vA, mode, room, side, st);
+        else if (mode == 2) launch_apply_strips<2>(aa, kA, vA, mode, room, side, st);
+        else if (mode == 1) launch_apply_strips<1>(aa, kA, vA, mode, room, side, st);
+        else launch_apply_strips<0>(aa, kA, vA, mode, room, side, st);
         return cudaGetLastError();
     }
     cudaMemsetAsync(long_count, 0, 2 * sizeof(uint32_t), st);  // [0] rounds handed over, [1] rounds taken

@@ -106,6 +106,30 @@ def test_workspace_grows_with_blocks():
     robe.robe_destroy(h)
 
 
+def test_workspace_asks_for_no_more_than_it_used_to():
+    # callers hold workspaces of a size, and the static call has a limit: blocks (four words each), ids (one
+    # word), hand-over records and the counters; bounds of strips may not come on top of that
+    up = lambda v: -(-v // 256) * 256
+    asked = {}
+    for M, d, Z in [(300_000_000, 128, 128), (250_000_000, 64, 16), (2_400_000, 32, 32), (2_600_000, 128, 127),
+                    (540_000, 16, 8), (1_200_000, 128, 128), (4096, 16, 4), (129, 128, 128), (25_000_000, 100, 100),
+                    (5_400_000, 128, 128), (5_800_000, 128, 128)]:
+        h = robe.robe_create(M, Z, d, 1, 1)
+        robe.robe_set_option(h, robe.ROBE_OPT_BWD_MODE, robe.ROBE_BWD_DETERMINISTIC)
+        for nnz in [1, 100, 9375, M // (2 * d) + 1, M // (2 * d) + 500, M // d, 1_300_000]:
+            nb = nnz * -(-d // Z)
+            was = (4 * up(4 * nb) + up(4 * nnz) + 4 * 256 * 592 + 4 * 256 + 256
+                   + up(400 * min(max(nb // 128, 64), 1 << 20)))
+            asked[M, nnz] = robe.robe_backward_workspace_bytes(h, nnz, nnz)
+            assert asked[M, nnz] <= was, (M, d, Z, nnz)
+        # and a workspace sized for the largest call is enough for every smaller one
+        sizes = [robe.robe_backward_workspace_bytes(h, n, n) for n in range(1, 60_000, 7)]
+        assert all(a <= b for a, b in zip(sizes, sizes[1:])), (M, d, Z)
+        robe.robe_destroy(h)
+    # 1.3 M rows of one block that touch 300 M slots densely: within the static call's limit
+    assert asked[300_000_000, 1_300_000] <= robe.ROBE_STATIC_SCRATCH_BYTES
+
+
 def test_sort_based_variants_refuse_sizes_beyond_their_32_bit_numbering():
     # block numbers, bag numbers and gradient positions are 32-bit in the binned / deterministic /
     # Adam paths: larger calls are refused before anything is launched (dummy pointers are never read)

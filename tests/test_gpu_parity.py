@@ -588,6 +588,21 @@ def test_deterministic_strips(case):
     test_deterministic_window_apply(case)
 
 
+# Where the strips' bounds and lists go: room of their own on a short array; on a longer one where the last sort
+# pass read from, or, at just under a block per strip, nowhere (the position-tile kernel then serves a densely
+# touched array).
+ROOM_CASES = [
+    dict(d=128, Z=128, M=5_400_007, batch=7300, vocab_arg=(10**6, 10**6, 30)),
+    dict(d=128, Z=128, M=25_000_000, batch=33_000, vocab_arg=(10**6, 10**6, 30)),
+    dict(d=128, Z=128, M=25_000_000, batch=32_567, vocab_arg=(10**6, 10**6, 30)),
+]
+
+
+@pytest.mark.parametrize("case", ROOM_CASES, ids=lambda k: f"M{k['M']}_batch{k['batch']}")
+def test_deterministic_strip_rooms(case):
+    test_deterministic_window_apply(case)
+
+
 # robe_forward_keep + robe_backward_kept: one hash of every id per training step.  The pair must
 # give what robe_forward and robe_backward give: the forward bit for bit, the deterministic
 # backward bit for bit, the binned and atomic ones within the atomic bound.  Shapes: rows of every

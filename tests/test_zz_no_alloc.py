@@ -131,3 +131,21 @@ def test_largest_and_too_large_calls():
     with Case(w, batch=fits) as c:  # close to the limit: the whole array is in use
         g = _grad(c, 4)
         assert_bits_equal(_static_dense(c, g), _reference_dense(c, g), "static scratch at its limit")
+
+
+def test_large_densely_touched_array_fits():
+    # 1.3 M blocks that touch most of 300 M slots: the strips' bounds take no room of their own
+    w = _workload(d=128, Z=128, M=300_000_000, bag_rule=None, num_tables=4, vocab_arg=(10**6, 10**6, 10**6, 77),
+                  batch=325_000)
+    free, _ = torch.cuda.mem_get_info()
+    if free < 8 * 2**30:
+        pytest.skip("not enough free device memory")
+    with Case(w, host_array=False) as c:
+        g = _grad(c, 6)
+        ga = torch.zeros(w.M, dtype=torch.float32, device=c.dev)
+        robe.robe_backward_deterministic_static(c.h, g, c.indices, c.offsets, c.B, ga, 0.0)
+        torch.cuda.synchronize()
+        for j0, jn in ((0, 100_000), (123_456_789, 100_000), (w.M - 100_000, 100_000)):
+            can, _ = c.oracle.backward_canonical(g.cpu().numpy(), c.indices_h, c.offsets_h, c.B, j0=j0, jn=jn)
+            assert np.any(can)
+            assert_bits_equal(ga[j0:j0 + jn].cpu().numpy(), can, f"static scratch, slots from {j0}")
