@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(256) bwd_atomic_direct_kernel(BwdArgs a) {
     for (uint32_t i = lane; i < mp.d; i += 32) {
         uint32_t c, o;
         chunk_of(mp, i, c, o);
-        const float gv = __ldcs(a.grad_out + k * mp.d + i) * a.scale;
+        const float* const ge = a.grad_out + k * mp.d + i;
+        const float gv = ROBE_CHK_GRAD(ge, a) ? __ldcs(ge) * a.scale : 0.0f;
         for (int64_t p = lo; p < hi; ++p) {
             const uint64_t x = (uint64_t)a.indices.load(p);
             uint32_t j = id_block_start(mp, e, x, c) + o;
@@ -119,7 +120,8 @@ bwd_atomic_staged_kernel(BwdArgs a, uint32_t ids_per_batch, uint32_t cmagic) {
         if (!live[u]) i = mp.d - 1;
         chunk_of(mp, i, chk[u], off[u]);
         gv[u] = 0.0f;
-        if (BAGS && live[u]) gv[u] = __ldcs(a.grad_out + warp * (int64_t)mp.d + i) * a.scale;
+        const float* const ge = a.grad_out + warp * (int64_t)mp.d + i;
+        if (BAGS && live[u] && ROBE_CHK_GRAD(ge, a)) gv[u] = __ldcs(ge) * a.scale;
     }
     const uint32_t* start_s = sm.start[w];
     const uint64_t* gbase_s = sm.base[w] + kStageIds / 2;
@@ -152,14 +154,15 @@ bwd_atomic_staged_kernel(BwdArgs a, uint32_t ids_per_batch, uint32_t cmagic) {
                     const int64_t row = p0 + (int64_t)((g & ~31u) + (uint32_t)(__ffs((int)rest) - 1)) * pstride;
 #pragma unroll
                     for (int u = 0; u < EPL; ++u)
-                        if (live[u]) gv[u] += __ldcs(a.grad_out + row * (int64_t)mp.d + lane + 32u * u);
+                        if (live[u] && ROBE_CHK_GRAD(a.grad_out + row * (int64_t)mp.d + lane + 32u * u, a))
+                            gv[u] += __ldcs(a.grad_out + row * (int64_t)mp.d + lane + 32u * u);
                 }
 #pragma unroll
                 for (int u = 0; u < EPL; ++u) gv[u] *= a.scale;
             } else if (!BAGS) {
 #pragma unroll
                 for (int u = 0; u < EPL; ++u)
-                    if (live[u])
+                    if (live[u] && ROBE_CHK_GRAD(a.grad_out + (p0 + g) * (int64_t)mp.d + lane + 32u * u, a))
                         gv[u] = __ldcs(a.grad_out + (p0 + g) * (int64_t)mp.d + lane + 32u * u) * a.scale;
             }
 #pragma unroll
@@ -273,6 +276,7 @@ __device__ __forceinline__ void vec_scatter_batch(const BwdArgs& a, const uint32
                 gn = gk;
                 for (uint32_t rest = mk; rest != 0; rest &= rest - 1) {
                     const int64_t row = p0 + (t & ~31u) + (uint32_t)(__ffs((int)rest) - 1);
+                    if (!ROBE_CHK_GRAD((const float*)(rows + row * vpr + k) + (last_in_block ? 3 : 7), a)) continue;
                     const float4 x = __ldcs(rows + row * vpr + k);
                     gk.x += x.x; gk.y += x.y; gk.z += x.z; gk.w += x.w;
                     if (!last_in_block) {
@@ -282,6 +286,7 @@ __device__ __forceinline__ void vec_scatter_batch(const BwdArgs& a, const uint32
                 }
             } else {
                 const int64_t row = p0 + t;
+                if (!ROBE_CHK_GRAD((const float*)(rows + row * vpr + k) + (last_in_block ? 3 : 7), a)) continue;
                 gk = __ldcs(rows + row * vpr + k);
                 gn = last_in_block ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : __ldcs(rows + row * vpr + k + 1);
             }
@@ -327,8 +332,8 @@ bwd_atomic_vec_kernel(BwdArgs a, uint32_t ids_per_batch, uint32_t cmagic) {
     float4 gk = make_float4(0.0f, 0.0f, 0.0f, 0.0f), gn = gk;
     if (BAGS && lane_on) {  // the bag's gradient row: once for all its ids
         const float4* row = reinterpret_cast<const float4*>(a.grad_out + warp * (int64_t)mp.d);
-        gk = scaled(__ldcs(row + k), a.scale);
-        if (!last_in_block) gn = scaled(__ldcs(row + k + 1), a.scale);
+        if (ROBE_CHK_GRAD((const float*)(row + k) + 3, a)) gk = scaled(__ldcs(row + k), a.scale);
+        if (!last_in_block && ROBE_CHK_GRAD((const float*)(row + k) + 7, a)) gn = scaled(__ldcs(row + k + 1), a.scale);
     }
 
     for (int64_t p0 = lo; p0 < hi; p0 += ids_per_batch) {
@@ -404,7 +409,8 @@ bwd_atomic_lanehash_kernel(BwdArgs a, uint32_t padj) {
 #pragma unroll
                     for (int u = 0; u < EPL; ++u) {
                         gv[gg][u] = 0.0f;
-                        if (g + gg < n && lc.live[u])
+                        if (g + gg < n && lc.live[u] &&
+                            ROBE_CHK_GRAD(a.grad_out + (r0 + g + gg) * (int64_t)mp.d + lane + 32u * u, a))
                             gv[gg][u] = __ldcs(a.grad_out + (r0 + g + gg) * (int64_t)mp.d + lane + 32u * u) * a.scale;
                     }
                 scatter_id(bm, thr, (int)g, gv[0]);
@@ -421,7 +427,8 @@ bwd_atomic_lanehash_kernel(BwdArgs a, uint32_t padj) {
 #pragma unroll
             for (int u = 0; u < EPL; ++u) {
                 gv[u] = 0.0f;
-                if (lc.live[u]) gv[u] = __ldcs(a.grad_out + bag * (int64_t)mp.d + lane + 32u * u) * a.scale;
+                if (lc.live[u] && ROBE_CHK_GRAD(a.grad_out + bag * (int64_t)mp.d + lane + 32u * u, a))
+                    gv[u] = __ldcs(a.grad_out + bag * (int64_t)mp.d + lane + 32u * u) * a.scale;
             }
             for (int64_t p0 = lo; p0 < hi; p0 += 32) {
                 uint32_t bm = 0;

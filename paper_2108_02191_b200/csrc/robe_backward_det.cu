@@ -1095,7 +1095,10 @@ binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* K, const uint32_t* V) {
                 slot[u] = __shfl_sync(0xFFFFFFFFu, k, src) + ol;
                 const float* row = a.grad_out + (__shfl_sync(0xFFFFFFFFu, v, src) + ol);
 #pragma unroll
-                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < Z ? __ldca(row + 32 * q) : 0.0f;
+                for (int q = 0; q < EPL; ++q)
+                    x[u][q] = ol + 32 * q < Z && ROBE_CHK((uint64_t)(row + 32 * q - a.grad_out) < a.grad_elems, ROBE_DBG_GRAD_POS)
+                                  ? __ldca(row + 32 * q)
+                                  : 0.0f;
             }
 #pragma unroll
             for (int u = 0; u < U; ++u)
@@ -1112,7 +1115,10 @@ binned_apply_blocks_kernel(ApplyArgs a, const uint32_t* K, const uint32_t* V) {
                 const float* row = a.grad_out + (__shfl_sync(0xFFFFFFFFu, v, src) + ol);
                 l[u] = __shfl_sync(0xFFFFFFFFu, len, src);
 #pragma unroll
-                for (int q = 0; q < EPL; ++q) x[u][q] = ol + 32 * q < l[u] ? __ldca(row + 32 * q) : 0.0f;
+                for (int q = 0; q < EPL; ++q)
+                    x[u][q] = ol + 32 * q < l[u] && ROBE_CHK((uint64_t)(row + 32 * q - a.grad_out) < a.grad_elems, ROBE_DBG_GRAD_POS)
+                                  ? __ldca(row + 32 * q)
+                                  : 0.0f;
             }
 #pragma unroll
             for (int u = 0; u < U; ++u)

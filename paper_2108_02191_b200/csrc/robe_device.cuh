@@ -40,6 +40,8 @@ __device__ __forceinline__ bool robe_dbg_ok(bool cond, int32_t code) {
 #else
 #define ROBE_CHK(cond, code) true
 #endif
+// .. of a gradient element (or of the last one of a vector) at address p of the call with arguments a
+#define ROBE_CHK_GRAD(p, a) ROBE_CHK((uint64_t)((p) - (a).grad_out) < (uint64_t)(a).nbags * (a).mp.d, ROBE_DBG_GRAD_POS)
 
 // First statement of a kernel launched by launch_next, in every thread: waits until the kernel before it in the
 // stream has finished and its writes are seen.  EARLY: the kernel after this one may take its place on the SMs

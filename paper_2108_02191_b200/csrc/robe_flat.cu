@@ -53,6 +53,7 @@ __device__ __forceinline__ bool flat_hash(const FlatArgs& a, FlatSmem& sm, int64
                                           uint32_t lane) {
     const MapParams& mp = a.mp;
     for (uint32_t t = lane; t < cnt; t += 32) {
+        if (!ROBE_CHK(t < kFlatRows, ROBE_DBG_SHARED)) break;
         const uint32_t e = table_of_bag((uint64_t)(row0 + t), mp);
         const uint64_t x = (uint64_t)a.indices.load(row0 + t);
         if (mp.R > 1) {  // rows clubbed into one block: its start is all there is
@@ -100,7 +101,7 @@ __device__ __forceinline__ uint32_t flat_slot(const FlatArgs& a, const uint32_t*
         q = flat_div(f, a.zmagic);
         off = f - q * mp.Z;
     }
-    uint32_t j = start[q] + off;  // < m + d <= 2^32
+    uint32_t j = (ROBE_CHK(q < kFlatEntries, ROBE_DBG_SHARED) ? start[q] : 0u) + off;  // < m + d <= 2^32
     if (WRAP && j >= mp.m) j -= mp.m;
     return j;
 }
@@ -145,7 +146,8 @@ __device__ __forceinline__ void flat_scatter(const FlatArgs& a, const uint32_t* 
     for (uint32_t f = lane; f - lane < n; f += 32 * U) {
         float v[U];
 #pragma unroll
-        for (uint32_t u = 0; u < U; ++u) v[u] = f + 32 * u < n ? __ldcs(grad + f + 32 * u) : 0.0f;
+        for (uint32_t u = 0; u < U; ++u)
+            v[u] = f + 32 * u < n && ROBE_CHK_GRAD(grad + f + 32 * u, a) ? __ldcs(grad + f + 32 * u) : 0.0f;
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u)
             if (f + 32 * u < n) {

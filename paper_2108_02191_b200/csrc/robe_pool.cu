@@ -141,7 +141,8 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
             const float* row = a.grad_out + (k0 + (bag[g] & ~kPoolLast)) * (int64_t)mp.d + lane;
             const bool fresh = g == 0 ? begins : (bag[g - 1] & kPoolLast) != 0;  // (warp-uniform)
 #pragma unroll
-            for (int u = 0; u < EPL; ++u) v[g][u] = fresh && l.live[u] && (FULL || (uint32_t)g < n) ? __ldcs(row + 32 * u) : 0.0f;
+            for (int u = 0; u < EPL; ++u)
+                v[g][u] = fresh && l.live[u] && (FULL || (uint32_t)g < n) && ROBE_CHK_GRAD(row + 32 * u, a) ? __ldcs(row + 32 * u) : 0.0f;
         }
 #pragma unroll
         for (int g = 0; g < U; ++g) {

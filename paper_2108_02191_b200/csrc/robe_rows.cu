@@ -80,7 +80,7 @@ __device__ __forceinline__ bool rows_sort(const RowsArgs& a, RowsSmem& sm, uint3
     for (uint32_t r0 = 0; r0 < rows; r0 += kRowsThreads) {  // (whole warps: the match below takes all lanes)
         const uint32_t r = r0 + tid;
         uint64_t base = ~0ull;  // (above every base: rows past the end match one another only)
-        if (r < rows) {
+        if (r < rows && ROBE_CHK(r < kRowsCap, ROBE_DBG_SHARED)) {
             uint32_t e;
             const uint32_t p = rows_position(a, row0 + r, e);
             base = addmod_p61(table_term(mp.h, e), mulmod_p61_any(mp.h.B, (uint64_t)a.indices.load(p)));
@@ -175,7 +175,7 @@ struct RowSlots<EPL, true, M30> {
             uint64_t s = (uint64_t)l.bm + t.ct[c] + (t.cterm[c] >= l.thr ? a.padj : 0u);
             if (s >= m) s -= m;
             if (s >= m) s -= m;
-            list[c * 33u + lane] = (uint32_t)s;
+            if (ROBE_CHK(c < kRowsMaxC, ROBE_DBG_SHARED)) list[c * 33u + lane] = (uint32_t)s;
         }
         __syncwarp();
     }
@@ -295,7 +295,7 @@ bwd_rows_kernel(RowsArgs a) {
         const uint32_t group_end = __shfl_sync(0xFFFFFFFFu, incl, lane < cnt ? __ffs((int)l.peers) - 1 : 31);
         const uint32_t k = group_end - __popc(l.peers >> lane);
         __syncwarp();
-        if (lane < cnt) turn[k] = make_uint2(l.pos, lane);
+        if (lane < cnt && ROBE_CHK(k < 32u, ROBE_DBG_SHARED)) turn[k] = make_uint2(l.pos, lane);
         else turn[lane] = make_uint2(0u, lane);  // (read, not used)
         const uint32_t ends = __reduce_or_sync(0xFFFFFFFFu, lead ? 1u << (incl - 1) : 0u);
         __syncwarp();
@@ -305,7 +305,8 @@ bwd_rows_kernel(RowsArgs a) {
             for (int q = 0; q < U; ++q) {
                 const float* row = grad + (size_t)turn[k0 + q].x * mp.d;
 #pragma unroll
-                for (int u = 0; u < EPL; ++u) nxt[q][u] = k0 + q < cnt && rs.live(u) ? __ldcs(row + 32 * u) : 0.0f;
+                for (int u = 0; u < EPL; ++u)
+                    nxt[q][u] = k0 + q < cnt && rs.live(u) && ROBE_CHK_GRAD(row + 32 * u, a) ? __ldcs(row + 32 * u) : 0.0f;
             }
         };
         load(0);

@@ -56,7 +56,7 @@ struct StripArgs {
     uint32_t* hot_list;
     uint32_t hot_cap;
     int vec_commit;            // target and moments are 16-byte aligned
-    uint64_t grad_elems;       // of grad_out (read by the debug build's index checks only)
+    uint64_t grad_elems, nb;   // of grad_out; sorted blocks (read by the debug build's index checks only)
 };
 
 constexpr uint32_t kBoundsGap = 256;  // longer gaps are filled by the whole warp
@@ -227,7 +227,7 @@ strip_apply_kernel(StripArgs a) {
         reinterpret_cast<float4*>(strip_smem)[((w * G + g) * W >> 2) + i] = make_float4(-0.0f, -0.0f, -0.0f, -0.0f);
     // lane ol holds block ol of the present LP: start relative to the strip, payload
     uint32_t nk = 0, nv = 0;
-    if (ol < n) {
+    if (ol < n && ROBE_CHK((uint64_t)lo + ol < a.nb, ROBE_DBG_SORT_POS)) {
         nk = load_settled(a.K + lo + ol);
         nv = load_settled(a.V + lo + ol);
     }
@@ -236,7 +236,7 @@ strip_apply_kernel(StripArgs a) {
         // a block past the stretch starts beyond every strip
         const uint32_t rel = c0 + ol < n ? nk - w0 : 0x40000000u, v = nv;
         const uint32_t len = SHORT ? strip_len<SHORT>(a.mp, v) : 0u;
-        if (c0 + LP + ol < n) {
+        if (c0 + LP + ol < n && ROBE_CHK((uint64_t)lo + c0 + LP + ol < a.nb, ROBE_DBG_SORT_POS)) {
             nk = load_settled(a.K + lo + c0 + LP + ol);
             nv = load_settled(a.V + lo + c0 + LP + ol);
         }
@@ -396,6 +396,7 @@ strip_hot_kernel(StripArgs a) {
         auto fetch = [&](uint32_t s) {
             if (lane < count(s)) {
                 const uint32_t at = lo + s * per_step + cw * E + lane;
+                if (!ROBE_CHK((uint64_t)at < a.nb, ROBE_DBG_SORT_POS)) return;
                 const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&keys_s[s % (2 * kHotBufs)][cw][lane]);
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(a.K + at) : "memory");
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4), "l"(a.V + at) : "memory");
@@ -601,6 +602,7 @@ StripArgs strip_args(const StripProblem& sp) {
     a.hot_cap = L.hot_cap;
     a.vec_commit = aligned(sp.target) && aligned(sp.adam.m1) && aligned(sp.adam.m2);
     a.grad_elems = sp.grad_elems;
+    a.nb = sp.nb;
     // hot: twice the average number of blocks, and enough of them to be worth a CTA (26 x 16384 Zipf rows on
     // 540 K slots, twice / four times: 34 / 53 us beside the hot kernel's 50; a floor of 128 blocks instead
     // of 256 made a 250 M-slot array 3 % slower, 512 none faster)

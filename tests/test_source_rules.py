@@ -58,3 +58,12 @@ def test_settled_loads_follow_a_settled_kernel():
 def test_warp_calls_name_lanes_that_are_sure_to_arrive(path):
     # the lanes active at one call need not be those at the next: a mask read from the hardware is no promise
     assert "__activemask" not in code(path)
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_every_gradient_read_is_checked_in_the_index_check_build(path):
+    # a read of grad_out stands behind a check that names it, at most four lines further up
+    lines = code(path).splitlines()
+    for n, line in enumerate(lines):
+        if re.search(r"(__ldcs|__ldca|load_settled)\((rows? \+|grad \+|ge\)|a\.grad_out)", line):
+            assert re.search("ROBE_CHK_GRAD|ROBE_DBG_GRAD_POS", " ".join(lines[max(0, n - 4):n + 1])), (n + 1, line)
