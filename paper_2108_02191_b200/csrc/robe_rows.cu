@@ -26,7 +26,7 @@ constexpr int kRowsWarps = kRowsThreads / 32;
 constexpr uint32_t kRowsCap = 512;      // rows per CTA, at most
 constexpr uint32_t kRowsMin = 64;       // and at least
 constexpr uint32_t kRowsBins = 512;     // of the counting sort: two per thread
-constexpr uint32_t kRowsMaxC = 16;      // chunks per row whose starts are listed (see RowSlots)
+constexpr uint32_t kRowsMaxC = 16;      // backward: chunks per row whose starts are listed (see RowSlots)
 
 struct RowsArgs {
     MapParams mp;
@@ -143,8 +143,8 @@ __device__ __forceinline__ RowsLane rows_fetch(const RowsArgs& a, const RowsSmem
     return l;
 }
 
-// Where the rows' slots come from while a warp serves 32 rows.  Few chunks per row (C <= kRowsMaxC):
-// every lane evaluates the block starts of its row into a list that the warp shares, and a lane that
+// Where the rows' slots come from while a warp serves 32 rows.  Few chunks per row (C <= kRowsMaxC; the
+// backward only, launch_forward sends such rows elsewhere): every lane evaluates the block starts of its row into a list that the warp shares, and a lane that
 // owns element i reads the start of chunk i / Z.  Many chunks: each lane hashes the chunks of its own
 // elements (LaneChunks) from what the row's lane hands round.
 template <int EPL, bool LISTED, bool M30>
@@ -205,11 +205,10 @@ struct RowSlots<EPL, false, M30> {
 
 // Forward: the first row of a group is gathered, every row of it written; the gathers of U groups in
 // flight.
-template <int EPL, int DT, bool LISTED, bool M30, int U>
+template <int EPL, int DT, bool M30, int U>
 __global__ void __launch_bounds__(kRowsThreads, kRowsCtas)
 fwd_rows_kernel(RowsArgs a) {
     __shared__ RowsSmem sm;
-    __shared__ uint32_t lists[LISTED ? kRowsWarps : 1][LISTED ? kRowsMaxC * 33 : 1];
     const MapParams& mp = a.mp;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     follow();
@@ -217,14 +216,12 @@ fwd_rows_kernel(RowsArgs a) {
     const uint32_t first = blockIdx.x * a.rows_per_cta;
     if (first >= a.nbags) return;
     const uint32_t rows = a.nbags - first < a.rows_per_cta ? a.nbags - first : a.rows_per_cta;
-    uint32_t* list = lists[LISTED ? w : 0];
-    const bool sorted = rows_sort<LISTED>(a, sm, first, rows);
-    RowSlots<EPL, LISTED, M30> rs(mp, lane, a.padj, list);
+    const bool sorted = rows_sort<false>(a, sm, first, rows);
+    RowSlots<EPL, false, M30> rs(mp, lane, a.padj, nullptr);
     float* const out = a.io + lane;
     for (uint32_t i0 = w * 32; i0 < rows; i0 += kRowsThreads) {
         uint32_t leaders;
         const RowsLane l = rows_fetch(a, sm, first, i0, rows - i0 < 32 ? rows - i0 : 32, lane, sorted, leaders);
-        rs.put(a, sm.terms, list, l, lane);
         while (leaders != 0) {
             float v[U][EPL];
             int src[U];
@@ -375,17 +372,16 @@ static RowsArgs rows_args(const Problem& pb, bool whole_waves, unsigned& grid) {
     return a;
 }
 
-template <int EPL, bool LISTED, bool M30>
+template <int EPL, bool M30>
 static void launch_fwd_rows(const RowsArgs& a, int dtype, unsigned grid, cudaStream_t st) {
-    if (dtype == 0) launch_next(fwd_rows_kernel<EPL, 0, LISTED, M30, 4>, grid, kRowsThreads, 0, st, a);
-    else launch_next(fwd_rows_kernel<EPL, 1, LISTED, M30, 4>, grid, kRowsThreads, 0, st, a);
+    if (dtype == 0) launch_next(fwd_rows_kernel<EPL, 0, M30, 4>, grid, kRowsThreads, 0, st, a);
+    else launch_next(fwd_rows_kernel<EPL, 1, M30, 4>, grid, kRowsThreads, 0, st, a);
 }
 
 template <int EPL>
 static void launch_fwd_rows(const RowsArgs& a, int dtype, unsigned grid, cudaStream_t st) {
-    if (a.mp.C <= kRowsMaxC) launch_fwd_rows<EPL, true, false>(a, dtype, grid, st);
-    else if (a.mp.m < (1u << 30)) launch_fwd_rows<EPL, false, true>(a, dtype, grid, st);
-    else launch_fwd_rows<EPL, false, false>(a, dtype, grid, st);
+    if (a.mp.m < (1u << 30)) launch_fwd_rows<EPL, true>(a, dtype, grid, st);
+    else launch_fwd_rows<EPL, false>(a, dtype, grid, st);
 }
 
 cudaError_t launch_forward_rows(const Problem& pb, float* out, cudaStream_t st) {
