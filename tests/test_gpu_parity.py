@@ -381,6 +381,32 @@ def test_short_bags(d, Z, M, batch, bags):
                 assert_bits_equal(c.forward().cpu().numpy(), one, "offsets out of order")
 
 
+# The same in calls of so many bags that a warp takes up to 16 (mean 2) or 10 (mean 3) of them, unsigned rows of
+# every length in the backward too; full batches of staged ids inside a run, long bags among the short ones
+# that go on over several batches, and in the middle of a run.
+@pytest.mark.parametrize("d,Z,M", [(16, 8, 4099), (64, 16, 100_003), (100, 32, 1013), (128, 128, 1283), (128, 8, 100_003)])
+@pytest.mark.parametrize("bags", [(2, 0, 6), (3, 1, 9)])
+def test_long_runs_of_short_bags(d, Z, M, bags):
+    w = small(d=d, Z=Z, M=M, bag_rule=bags, batch=70_000)
+    rng = np.random.default_rng(41)
+    lengths = np.diff(synth.make_ids(w)[1])
+    lengths[::1009] = rng.integers(65, 300, size=len(lengths[::1009]))
+    offsets = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    vocab = np.array(w.vocab_arg)[np.repeat(np.arange(len(lengths)) % w.num_tables, lengths)]
+    ids = rng.integers(0, vocab).astype(np.int64)
+    # what a run of bags per warp asks for, forward and backward (pool_bags in robe_pool.cu)
+    nbags, nnz = len(lengths), int(offsets[-1])
+    assert nbags >= 200_000 and nnz >= nbags and (nnz + nbags // 2) // nbags <= 4 and M * 4 <= 192 << 20
+    for sign in (False, True):
+        with Case(w, sign=sign, ids=(ids, offsets)) as c:
+            want = c.oracle_forward()
+            assert_bits_equal(c.forward().cpu().numpy(), want, "forward")
+            g_h, g_d = _grad(c, 22, integer=True)
+            delta64, _ = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+            assert np.abs(delta64).max() < 2**24  # small integers: exact in any order
+            assert_bits_equal(c.backward(g_d, "atomic").cpu().numpy(), delta64.astype(np.float32), "backward")
+
+
 # Binned adds of a call large enough to look for repeats of a start (8 M blocks): hot ids, whose blocks are added
 # together, in full and in short last blocks, and ids that hardly repeat.
 @pytest.mark.parametrize("d,Z,batch,vocab", [(64, 1, 46_000, (5, 50, 3000)), (64, 3, 130_000, (5, 50, 10**6)),
@@ -524,11 +550,46 @@ def test_deterministic_is_bit_reproducible_and_order_sensitive_case():
             assert_bits_equal(r, can, "hot id deterministic")
 
 
-# Densely touched arrays take the slot-major kernel (one CTA per window of 256..2048 slots); the
-# cases span its branches: windows of every length, a ragged last window, blocks that wrap, ids
-# repeated so often that their windows go back to the position-tile and long-walk kernels while
-# the rest stay, windows whose blocks need several chunks of shared memory, block lengths that
-# are no power of two or no multiple of four, and a gradient buffer that is not 16-byte aligned.
+# Sparsely touched arrays, and blocks of more than 128 elements on any, take the position-tile kernel; the slots
+# of an id that a batch repeats often go on in the long-walk kernel after 64 terms, 64 a step.  Chains that end
+# inside the first step, with a step and one past it, and of dozens of steps (its buffers and its ring of keys
+# go round several times); chains of different lengths side by side.
+@pytest.mark.parametrize("d,Z,M,batch,vocab", [
+    (32, 8, 3_000_017, 100, (1, 3, 10**6)), (32, 8, 3_000_017, 448, (1, 3, 10**6)), (32, 8, 3_000_017, 449, (1, 3, 10**6)),
+    (32, 8, 5_000_011, 9000, (1, 3, 10**6)), (64, 64, 9_000_011, 6000, (2, 1, 40)), (33, 1, 2_000_003, 3000, (1, 2, 10**6)),
+    (160, 160, 50_021, 3000, (1, 3, 1000)), (256, 512, 70_001, 2500, (2, 5, 10**6)),
+])
+def test_deterministic_long_walks(d, Z, M, batch, vocab):
+    w = small(d=d, Z=Z, M=M, batch=batch, vocab_arg=vocab)
+    with Case(w) as c:
+        zb = min(Z, d)
+        nb = c.indices.numel() * -(-d // zb)
+        assert d % zb == 0 and (zb > 128 or 2 * nb * zb < M), "the case must not be one for the strips"
+        g_h, g_d = _grad(c, 51)
+        can, touched = c.oracle.backward_canonical(g_h, c.indices_h, c.offsets_h, c.B)
+        assert_bits_equal(c.backward(g_d, "det").cpu().numpy(), can, "dense gradient")
+        arr = c.array_h.copy()
+        c.backward(g_d, "det", sgd=True, lr=0.125)
+        orc.sgd_apply(arr, can, touched, 0.125)
+        assert_bits_equal(c.array.cpu().numpy(), arr, "SGD")
+        ws = torch.empty(robe.robe_backward_workspace_bytes(c.h, c.B, c.indices.numel()), dtype=torch.uint8, device=c.dev)
+        m1, m2, ssq = (np.zeros(M, np.float32) for _ in range(3))
+        m1_d, m2_d, ssq_d = (torch.zeros(M, device=c.dev) for _ in range(3))
+        robe.robe_backward_adam(c.h, g_d, c.indices, c.offsets, c.B, m1_d, m2_d, 0.05, 0.9, 0.999, 1e-8, 1, ws)
+        orc.adam_apply(arr, m1, m2, can, touched, 0.05, 0.9, 0.999, 1e-8, 1)
+        assert_bits_equal(c.array.cpu().numpy(), arr, "Adam")
+        assert_bits_equal(m1_d.cpu().numpy(), m1, "Adam, first moment")
+        assert_bits_equal(m2_d.cpu().numpy(), m2, "Adam, second moment")
+        robe.robe_backward_adagrad(c.h, g_d, c.indices, c.offsets, c.B, ssq_d, 0.05, 1e-8, ws)
+        orc.adagrad_apply(arr, ssq, can, touched, 0.05, 1e-8)
+        assert_bits_equal(c.array.cpu().numpy(), arr, "Adagrad")
+        assert_bits_equal(ssq_d.cpu().numpy(), ssq, "Adagrad, accumulators")
+
+
+# Densely touched arrays are served slot by slot, strip after strip; the cases span strips of every length, a
+# ragged last one, blocks that wrap, ids repeated so often that their strips go to the kernel for hot ones
+# while the rest stay, block lengths that are no power of two or no multiple of four, a block of 64 of 256 that
+# rows share, and a gradient buffer that is not 16-byte aligned.
 WINDOW_CASES = [
     # d, Z, M, batch, tables/vocab, bags, id_dist
     dict(d=64, Z=16, M=300_007, batch=1500, vocab_arg=(10**6, 10**6, 50_000), bag_rule=(6, 0, 20)),
@@ -750,8 +811,7 @@ def test_cfg3_forward_backward_full_size(Z):
         det = c.backward(g_d, "det").cpu().numpy()
         assert_within_l1(det, delta64, l1, what=f"cfg3 Z={Z} det vs fp64")
         assert_bits_equal(c.backward(g_d, "det").cpu().numpy(), det, "cfg3 det repeat")
-        # the same step with the forward's block starts: same bits (window, position-tile and
-        # long-walk kernels all take part at this size)
+        # the same step with the forward's block starts: same bits
         _, detk = c.step_sharing_keys(g_d, "det")
         assert_bits_equal(detk.cpu().numpy(), det, "cfg3 det on kept starts")
         del detk
