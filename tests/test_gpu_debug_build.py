@@ -1,8 +1,8 @@
 """The index-check build of the library (librobe_debug.so: the same sources with -DROBE_DEBUG, every
 computed index compared with its bound before use; it stands in for a memory checker, which cannot
-be run on the machines this is tested on).  The small shape lists of the parity tests - every kernel
-family, wrap-heavy arrays, ragged blocks, windows, long walks, kept block starts - are run against
-it in a child process; each test there must match the oracle as usual AND leave the debug word at
+be run on the machines this is tested on).  The shape lists of the parity tests - every kernel family, at the
+sizes that its dispatch asks for, wrap-heavy arrays, ragged blocks, strips, long walks, kept block starts - are
+run against it in a child process; each test there must match the oracle as usual AND leave the debug word at
 zero (tests/conftest.py checks it after every test)."""
 import os
 import subprocess
@@ -46,7 +46,8 @@ def test_shape_lists_run_clean_on_the_index_check_build():
     if os.environ.get("ROBE_LIBRARY"):
         pytest.skip("already inside the child run")
     pick = ("forward_shapes or backward_shapes or window_apply or step_sharing or vector_kernel or "
-            "lane_hashed or adam or adagrad or merged_rows or table_major or int32 or cfg1 or hot_id or bit_reproducible")
+            "lane_hashed or adam or adagrad or merged_rows or table_major or int32 or cfg1 or hot_id or bit_reproducible "
+            "or large_one_hot or short_bags or repeated_blocks or strips or strip_rooms or long_walks or back_to_back")
     r = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_parity.py", "tests/test_zz_no_alloc.py",
                         "-m", "gpu", "-x", "-q", "-k", pick + " or two_calls or fused_sgd"],
                        env=_debug_env(), cwd=ROOT, capture_output=True, text=True, timeout=3000)
