@@ -376,10 +376,6 @@ def run_ours(args, w):
     if table_major:
         robe.robe_set_option(h, robe.ROBE_OPT_BAG_LAYOUT, robe.ROBE_BAGS_TABLE_MAJOR)
     robe.robe_set_option(h, robe.ROBE_OPT_FWD_KERNEL, args.fwd_kernel)
-    if (args.bwd_kernel == 0 and not bags and w.id_dist.startswith("zipf") and min(w.Z, w.d) >= 64 and d <= 128):
-        # skewed ids, long blocks: the repeats of an id are merged in the warp (the caller knows its
-        # ids; the library cannot tell from the shapes)
-        args.bwd_kernel = 5
     robe.robe_set_option(h, robe.ROBE_OPT_BWD_KERNEL, args.bwd_kernel)
     l2_keep = args.l2_keep
     robe.robe_set_option(h, robe.ROBE_OPT_ARRAY_L2_KEEP, l2_keep)
@@ -397,6 +393,10 @@ def run_ours(args, w):
         ws = torch.empty(robe.robe_backward_workspace_bytes(h, B, max(len(b[0]) for b in batches)),
                          dtype=torch.uint8, device=dev)
         bwd_launches = (1 if bags else 0) + 5  # (bag numbers,) keys, count, scan, scatter, apply
+        # from 8 M blocks on a sample of the sorted list says whether starts repeat
+        nblocks = float(np.mean([len(b[0]) for b in batches])) * -(-w.d // min(w.Z, w.d))
+        if min(w.Z, w.d) <= 128 and nblocks >= 8 << 20:
+            bwd_launches += 1
     # a bf16 array is read-only for the library: its gradient goes to a dense fp32 array instead
     # of the fused SGD step (the array stays as it is)
     dense = torch.zeros(w.M, dtype=torch.float32, device=dev) if w.array_dtype != "f32" else None
