@@ -64,11 +64,17 @@ typedef enum {
                                returns ROBE_OK.  Read it with robe_last_device_status
                                and zero it yourself before going on.                      */
 #define ROBE_OPT_FWD_KERNEL 4 /* forward kernel; every variant gives the same bits.
-                                 0 automatic (default).  One-hot: the rows kernel (repeats of an id
-                                   gathered once) for large batches with more than 16 chunks per row,
-                                   else the flat kernel (rows of any length as one run of elements);
-                                   pooled: the lane-hashed kernel for Z <= 2 on arrays of up to 192 MB,
-                                   the staged kernel for rows of up to 128 elements, else the direct one
+                                 0 automatic (default).  One-hot, sign off, block starts not kept: the
+                                   rows kernel (repeats of an id gathered once) from 32768 rows on with
+                                   more than 16 chunks per row (d <= 128, Z <= d); else, in large calls,
+                                   the staged kernel for rows of 64 or 128 elements in blocks of 8 or 16
+                                   and more (of 32 elements on arrays over 192 MB; of bf16 arrays with
+                                   any block) and for most rows with a short last block; else the flat
+                                   kernel (rows of any length as one run of elements).
+                                   Pooled: the lane-hashed kernel for Z <= 2 on arrays of up to 192 MB,
+                                   sign off; the pool kernel (a run of bags per warp) for many short
+                                   bags, d <= 128.
+                                   What is left: the staged kernel for d <= 128, else the direct one
                                  1 direct: any (Z, d); every lane hashes its element's chunk per id
                                  2 staged: d <= 128; block starts of a batch of ids through shared
                                    memory, 4-byte loads, lanes on consecutive slots of a block
@@ -80,9 +86,12 @@ typedef enum {
                                  A variant asked for a call it cannot take returns
                                  ROBE_ERR_UNSUPPORTED and launches nothing.                          */
 #define ROBE_OPT_BWD_KERNEL 5 /* kernel of the ATOMIC backward (all within the atomic bound):
-                                 0 automatic (default).  One-hot: the rows kernel (repeats of an id
-                                   summed first) for large batches, else the flat kernel; pooled:
-                                   staged for d <= 128, else direct
+                                 0 automatic (default).  One-hot, sign off: the rows kernel (repeats of
+                                   an id summed first) from 131072 rows on, from 32768 with more than 16
+                                   chunks per row (d <= 128, Z <= d); else the flat kernel.
+                                   Pooled: the pool kernel (a run of bags per warp) for many short bags,
+                                   d <= 128.
+                                   What is left: staged for d <= 128, else direct
                                  1 direct   2 staged (scalar red.global.add.f32, lanes on consecutive slots)
                                  3 vector: red.global.add.v4.f32 on the aligned middle of a block,
                                    scalar head and tail; d, Z, M multiples of 4, d <= 128, sign off
@@ -90,9 +99,10 @@ typedef enum {
                                  4 vector, repeats of an id inside a staged batch merged first
                                  5 merged rows: one-hot input, sign off, d <= 128; a warp takes up to 64
                                    rows of ONE table, sums the gradient rows of repeated ids in
-                                   registers and issues one reduction per element for all of them -
-                                   pays for skewed (Zipf) ids with long blocks (Z = 128: 1.34 x), costs
-                                   10-40 % on uniform ids, so it is the caller's choice
+                                   registers and issues one reduction per element for all of them
+                                   (skewed ids, Z = 128: 1.34 x over 2, 10-40 % slower on uniform ids;
+                                   the rows kernel of the automatic choice, which looks for repeats
+                                   among up to 512 rows, is faster on both)
                                  6 lane-hashed: d <= 128, Z <= d, sign off (the reductions, not the
                                    hashing, bound this pass: measured no faster than 2)              */
 
