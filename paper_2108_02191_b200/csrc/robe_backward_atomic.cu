@@ -549,9 +549,10 @@ cudaError_t launch_backward_atomic(const Problem& pb, const float* grad_out, flo
         // A large batch repeats ids - Zipf ids and small tables most of all - and the repeats, served
         // together, are one reduction instead of many on the same address (B200, 26 x 32768 rows of
         // 128 on 100 MB, Zipf ids, us: Z = 1 688 -> 435, Z = 8 225 -> 155, Z = 32 187 -> 129, Z = 128
-        // 241 -> 123; ids that never repeat 938 -> 1012, 281 -> 289, 176 -> 176, 158 -> 160).  Fewer rows
-        // hold fewer repeats: the flat kernel then (53248 rows of 128, Z = 32: 15 .. 18 us against 20;
-        // with short blocks, where a reduction costs most, 27 against 20).
+        // 241 -> 123; ids that never repeat, 26 x 131072 rows: 3604 -> 4003, 1038 -> 1053, 610 -> 611, 551 -> 563:
+        // where that is known, the caller may ask for kernel 2).  Fewer rows hold fewer repeats: the flat
+        // kernel then (53248 rows of 128, Z = 32: 15 .. 18 us against 20; with short blocks, where a reduction
+        // costs most, 27 against 20).
         if ((pb.nbags >= 131072 || (pb.mp.C > 16 && pb.nbags >= 32768)) && rows_ok(pb))
             return launch_backward_rows(pb, grad_out, target, scale, st);
         if (flat_ok(pb)) return launch_backward_flat(pb, grad_out, target, scale, st);

@@ -39,6 +39,7 @@ struct RowsArgs {
     uint32_t nbags, batch;
     uint64_t batch_magic;   // floor((2^64 - 1) / batch) + 1
     uint32_t rows_per_cta;
+    uint32_t shares;        // CTAs per table where tables are taken side by side, else 0 (see rows_first)
     uint32_t shift;         // bin = (base mod m) >> shift
     uint32_t padj;          // lane_padj
     int l2_keep;
@@ -62,6 +63,13 @@ __device__ __forceinline__ uint32_t rows_position(const RowsArgs& a, uint32_t v,
     e = a.batch == 1 ? v : (uint32_t)__umul64hi(a.batch_magic, (uint64_t)v);
     if (a.mp.B != 0) return v;
     return (v - e * a.batch) * a.mp.T + e;
+}
+
+// First row of this CTA in the table-by-table order.  Side by side: CTAs that run at the same time take the
+// same samples of different tables, whose rows lie next to each other in a sample-major call.
+__device__ __forceinline__ uint32_t rows_first(const RowsArgs& a) {
+    const uint32_t b = blockIdx.x;
+    return (a.shares == 0 ? b : (b % a.mp.T) * a.shares + b / a.mp.T) * a.rows_per_cta;
 }
 
 // Hashes rows [row0, row0 + rows) of the table-by-table order and sorts them; returns whether it did
@@ -213,7 +221,7 @@ fwd_rows_kernel(RowsArgs a) {
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     follow();
     if (a.status != nullptr && *a.status != 0) return;
-    const uint32_t first = blockIdx.x * a.rows_per_cta;
+    const uint32_t first = rows_first(a);
     if (first >= a.nbags) return;
     const uint32_t rows = a.nbags - first < a.rows_per_cta ? a.nbags - first : a.rows_per_cta;
     const bool sorted = rows_sort<false>(a, sm, first, rows);
@@ -267,7 +275,7 @@ bwd_rows_kernel(RowsArgs a) {
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     follow();
     if (a.status != nullptr && *a.status != 0) return;
-    const uint32_t first = blockIdx.x * a.rows_per_cta;
+    const uint32_t first = rows_first(a);
     if (first >= a.nbags) return;
     const uint32_t rows = a.nbags - first < a.rows_per_cta ? a.nbags - first : a.rows_per_cta;
     uint32_t* list = lists[LISTED ? w : 0];
@@ -346,9 +354,15 @@ bool rows_ok(const Problem& pb) {
            pb.nbags % pb.mp.T == 0;
 }
 
+// side_by_side: see rows_first.  In calls of millions of rows the order in which the gradient rows are read tells
+// (B200, sample-major, rows of 128, 100 MB, us, table after table -> side by side; 26 x 131072 rows, ids that never
+// repeat: Z = 8 1100 -> 1053, Z = 32 653 -> 611, Z = 128 588 -> 563, the staged kernel 1038, 610, 551; Zipf ids 521
+// -> 518, 430 -> 431, 435 -> 425).  In smaller ones a table's hot blocks, met again by the CTAs of the same time,
+// are worth as much or more (26 x 65536 rows, never repeating 321 -> 313, Zipf 231 -> 236; 8 x 32768 43 -> 46), and
+// with many chunks per row always (Zipf, Z = 1, 420 -> 469, though 4003 -> 3817 / 3604 where nothing repeats).
 // whole_waves: the rows are spread evenly over full waves of resident CTAs (the forward, whose CTAs take
 // about equally long); otherwise the CTAs take kRowsCap rows each (the backward, whose repeats matter more)
-static RowsArgs rows_args(const Problem& pb, bool whole_waves, unsigned& grid) {
+static RowsArgs rows_args(const Problem& pb, bool whole_waves, bool side_by_side, unsigned& grid) {
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     (void)cudaGetLastError();
@@ -366,6 +380,10 @@ static RowsArgs rows_args(const Problem& pb, bool whole_waves, unsigned& grid) {
     if (!whole_waves && waves > 1) a.rows_per_cta = kRowsCap;
     if (a.rows_per_cta < kRowsMin) a.rows_per_cta = kRowsMin;
     grid = (a.nbags + a.rows_per_cta - 1) / a.rows_per_cta;
+    if (side_by_side && pb.mp.B == 0) {
+        a.shares = (grid + pb.mp.T - 1) / pb.mp.T;
+        grid = a.shares * pb.mp.T;  // (CTAs past the last row return)
+    }
     while (((pb.mp.m - 1) >> a.shift) >= kRowsBins) ++a.shift;
     a.padj = lane_padj(pb.mp);
     a.l2_keep = pb.l2_keep;
@@ -386,7 +404,7 @@ static void launch_fwd_rows(const RowsArgs& a, int dtype, unsigned grid, cudaStr
 
 cudaError_t launch_forward_rows(const Problem& pb, float* out, cudaStream_t st) {
     unsigned grid;
-    RowsArgs a = rows_args(pb, true, grid);
+    RowsArgs a = rows_args(pb, true, false, grid);
     a.io = out;
     if (a.mp.d <= 32) launch_fwd_rows<1>(a, pb.dtype, grid, st);
     else if (a.mp.d <= 64) launch_fwd_rows<2>(a, pb.dtype, grid, st);
@@ -405,7 +423,7 @@ static void launch_bwd_rows(const RowsArgs& a, unsigned grid, cudaStream_t st) {
 cudaError_t launch_backward_rows(const Problem& pb, const float* grad_out, float* target, float scale,
                                  cudaStream_t st) {
     unsigned grid;
-    RowsArgs a = rows_args(pb, false, grid);
+    RowsArgs a = rows_args(pb, false, pb.mp.C <= kRowsMaxC && pb.nbags >= (1 << 21), grid);
     a.grad_out = grad_out;
     a.io = target;
     a.scale = scale;

@@ -353,6 +353,23 @@ def test_large_one_hot_batches(d, Z, M, table_major):
                           delta64.astype(np.float32), "backward, integer gradient")
 
 
+# Millions of rows of many tables: the backward then takes tables side by side, the rows of a CTA are part of one
+# table or of two, and CTAs past the last row have nothing to do.
+@pytest.mark.parametrize("table_major", [False, True])
+@pytest.mark.parametrize("d,Z", [(8, 8), (33, 8)])
+def test_millions_of_one_hot_rows(d, Z, table_major):
+    T, batch = 700, 3001
+    w = small(d=d, Z=Z, M=50_021, batch=batch, num_tables=T, vocab_arg=tuple([3, 10**6] * (T // 2)))
+    with Case(w, table_major=table_major) as c:
+        assert c.nbags >= 1 << 21
+        shape = (c.T, c.B, d) if table_major else (c.B, c.T, d)
+        g_h = np.random.default_rng(5).integers(-2, 3, size=shape).astype(np.float32)
+        delta64, _ = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+        assert np.abs(delta64).max() < 2**24  # small integers: exact in any order
+        assert_bits_equal(c.backward(torch.from_numpy(g_h).to(c.dev), "atomic").cpu().numpy(),
+                          delta64.astype(np.float32), "backward, integer gradient")
+
+
 # A run of short bags per warp: runs that end inside the last warp, empty bags at either end of a run and in
 # rows, bags that go on over several batches of staged ids, one element and 128 per row, arrays that wrap,
 # rows clubbed into one block, and offsets that are no stretch (a warp then takes its bags one by one).
