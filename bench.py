@@ -44,16 +44,16 @@ UNIT = "ids/s"
 NCU_TRAFFIC_RECORDS = {
     # (workload, backward variant, block starts shared, id type, bag layout)
     ("cfg4_multihot", "binned", True, "int64", "sample-major"): {
-        "forward": 4_411_400_000, "backward": 4_822_100_000,
+        "forward": 4_411_600_000, "backward": 4_819_600_000,
         "source": "profiles/launches_cfg4_multihot.md: full-size one-pass ncu capture of `python bench.py --steps 3 "
                   "--warmup 3 --no-cpu-baseline`; forward = fwd_staged_kernel, backward = sort_count + sort_scan + "
-                  "sort_scatter + binned_apply_blocks"},
+                  "sort_scatter + binned_sample + binned_apply_blocks"},
     ("cfg4_multihot", "atomic", False, "int64", "sample-major"): {
-        "forward": 4_130_800_000, "backward": 7_378_600_000,
+        "forward": 4_130_800_000, "backward": 7_378_900_000,
         "source": "profiles/launches_cfg4_multihot.md: full-size one-pass ncu capture of `python bench.py --steps 3 "
                   "--warmup 3 --no-cpu-baseline --backward atomic`"},
     ("cfg4_multihot", "det", True, "int64", "sample-major"): {
-        "forward": 4_411_900_000, "backward": 7_445_500_000,
+        "forward": 4_411_400_000, "backward": 7_446_600_000,
         "source": "profiles/launches_cfg4_multihot.md: full-size one-pass ncu capture of `python bench.py --steps 3 "
                   "--warmup 3 --no-cpu-baseline --backward det`; backward = 4 sort passes, strip bounds, "
                   "apply kernels"},
@@ -568,7 +568,7 @@ def run_ours(args, w):
     fwd_bytes, bwd_bytes = algorithmic_bytes(w, nbags, nnz_per_step, bags, id_bytes)
     fwd_kernel = "fwd_staged_kernel" if bags and d <= 128 else "forward kernel (automatic choice)"
     bwd_label = {"atomic": "bwd_atomic_staged_kernel" if bags and d <= 128 else "atomic backward kernel (automatic choice)",
-                 "binned": "composite: keys, sort_count, sort_scan, sort_scatter, binned_apply_blocks kernels",
+                 "binned": "composite: keys, sort_count, sort_scan, sort_scatter, binned_sample, binned_apply_blocks kernels",
                  "det": "composite: keys, sort passes, strip bounds, apply kernels"}[args.backward]
     if share_keys:
         bwd_label = bwd_label.replace("keys, ", "")
