@@ -1193,8 +1193,8 @@ struct SideStream {
     cudaEvent_t fork_event, join_event;
 };
 
-// Strips where they pay, and the low slots beside them: the hot strips (a few long-running CTAs) and the
-// low slots in the second stream (of higher priority), all other strips in the caller's.
+// Strips where they pay: the hot strips (a few long-running CTAs) and the low slots in the second stream (of
+// higher priority), all other strips in the caller's.
 template <int MODE>
 void launch_apply_strips(const ApplyArgs& aa, const uint32_t* K, const uint32_t* V, int mode, void* workspace,
                          const SideStream& side, cudaStream_t st) {
@@ -1208,11 +1208,6 @@ void launch_apply_strips(const ApplyArgs& aa, const uint32_t* K, const uint32_t*
     }
     const cudaStream_t ts = forked ? side.st : st;
     launch_strips(sp, mode, st, ts);
-    if (mp.Z > 1) {
-        const unsigned low_blocks = (mp.Z - 1 + kLowWarps - 1) / kLowWarps;
-        if (mp.d % mp.Z != 0) det_apply_low_kernel<false, MODE, true><<<low_blocks, 32 * kLowWarps, 0, ts>>>(aa, K, V, nullptr);
-        else det_apply_low_kernel<false, MODE, false><<<low_blocks, 32 * kLowWarps, 0, ts>>>(aa, K, V, nullptr);
-    }
     if (forked) {
         cudaEventRecord(side.join_event, side.st);
         cudaStreamWaitEvent(st, side.join_event, 0);

@@ -22,7 +22,7 @@
 // A strip reached by very many blocks (an id that the batch repeats hundreds of times) would keep one group
 // busy for long; such strips go to strip_hot_kernel, one CTA each: eight warps copy gradient elements
 // ahead (cp.async), a warp per 32 slots adds.
-// Slots [0, Z-1) also receive the wrapped tails of the array's last blocks: another kernel's.
+// Slots [0, Z-1) also receive the wrapped tails of the array's last blocks: strip_low_slot serves them.
 #include "robe_internal.h"
 #include "robe_update.cuh"
 
@@ -35,6 +35,7 @@ constexpr int kStripWarps = 8;
 constexpr uint32_t kStripMaxZ = 128;
 constexpr int kHotCopiers = 8;            // warps of the hot kernel that copy
 constexpr int kHotAdders = 8;             // and that add: 32 slots each
+constexpr int kHotWarps = kHotCopiers + kHotAdders;
 constexpr uint32_t kHotAhead = 3;         // steps that the copies, and again as many that the keys, are asked for ahead
 constexpr uint32_t kHotBufs = kHotAhead + 1;
 constexpr uint32_t kHotMin = 256;         // a strip is hot from this many blocks on, at least
@@ -52,11 +53,13 @@ struct StripArgs {
     const uint32_t* hi_of;     // [strips + 1]: first sorted position whose key is in the strip or beyond
     uint32_t strips, log2w;    // strips of 2^log2w slots
     uint32_t n_hot;
+    uint32_t low_ctas;         // the first CTAs of strip_hot_kernel, which serve slots [0, Z-1)
     uint32_t* hot_count;       // [0] strips at the front of the list, [1] at its back, [2] taken
     uint32_t* hot_list;
     uint32_t hot_cap;
     int vec_commit;            // target and moments are 16-byte aligned
-    uint64_t grad_elems, nb;   // of grad_out; sorted blocks (read by the debug build's index checks only)
+    uint64_t grad_elems;       // of grad_out (read by the debug build's index checks only)
+    uint64_t nb;               // sorted blocks
 };
 
 constexpr uint32_t kBoundsGap = 256;  // longer gaps are filled by the whole warp
@@ -350,6 +353,48 @@ __device__ __forceinline__ float hot_add_step(float acc, uint32_t at, uint32_t p
     return acc;
 }
 
+// First sorted position whose key is at least `least`: 32 probes at a time by a warp.
+__device__ __forceinline__ uint64_t strip_first(const StripArgs& a, uint64_t least, uint32_t lane) {
+    uint64_t from = 0, to = a.nb;  // keys before `from` are below, those from `to` on are not
+    while (from < to) {
+        const uint64_t step = (to - from + 31) / 32, at = from + step * lane;
+        const uint32_t not_below = __ballot_sync(0xFFFFFFFFu, at >= to || (uint64_t)__ldca(a.K + at) >= least);
+        const uint32_t f = not_below != 0 ? (uint32_t)__ffs((int)not_below) - 1 : 32u;
+        if (f == 0) return from;
+        const uint64_t next = from + step * f;
+        from += step * (f - 1) + 1;
+        if (next < to) to = next;
+    }
+    return from;
+}
+
+// Slot j in [0, Z-1), by a warp: the blocks that begin at or before it, then the wrapped tails of those that
+// begin in the last Z-1-j slots; the terms of 32 sorted positions at a time, all lanes adding them in order.
+template <int MODE, bool SHORT>
+__device__ __forceinline__ void strip_low_slot(const StripArgs& a, uint32_t j, uint32_t lane) {
+    float acc = 0.0f;
+    bool touched = false;
+    auto walk = [&](uint64_t from, uint64_t to, uint64_t j_plus) {
+        for (uint64_t i0 = from; i0 < to; i0 += 32) {
+            const uint64_t i = i0 + lane;
+            float term = 0.0f;
+            bool ok = false;
+            if (i < to && ROBE_CHK(i < a.nb, ROBE_DBG_SORT_POS)) {
+                const uint32_t v = __ldca(a.V + i), o = (uint32_t)(j_plus - __ldca(a.K + i));
+                ok = o < strip_len<SHORT>(a.mp, v) && ROBE_CHK((uint64_t)v + o < a.grad_elems, ROBE_DBG_GRAD_POS);
+                if (ok) term = __ldca(a.grad_out + (uint64_t)v + o);
+            }
+            const uint32_t oks = __ballot_sync(0xFFFFFFFFu, ok);
+            touched = touched || oks != 0;
+            for (uint32_t rest = oks; rest != 0; rest &= rest - 1)
+                acc = __fadd_rn(acc, __shfl_sync(0xFFFFFFFFu, term, __ffs((int)rest) - 1));
+        }
+    };
+    walk(0, strip_first(a, (uint64_t)j + 1, lane), j);
+    walk(strip_first(a, (uint64_t)a.mp.m - (a.mp.Z - 1) + j, lane), a.nb, (uint64_t)j + a.mp.m);  // (m >= Z)
+    if (touched && lane == 0) commit_slot<MODE>(a, j, acc, a.target[j]);
+}
+
 // Hot strips.  The chain of dependent adds of a slot is the definition's, and one warp's issue is what it
 // costs beyond that: the copies are laid out slot by slot, so that a lane reads four blocks' terms at once,
 // and a whole step of repeats of one start is one loop.  One barrier per step of eight copiers' blocks,
@@ -357,7 +402,7 @@ __device__ __forceinline__ float hot_add_step(float acc, uint32_t at, uint32_t p
 // Measured (B200, ns per repeat of one start): 9.3 with a row per block, 4.1 with divisions and a pass over all
 // blocks in the copiers, 3.7 here (of a step, 1308 clocks are adds, 330 what stands before them); the chain itself: 2.1.
 template <int MODE, int LP, int EPL, bool SHORT>
-__global__ void __launch_bounds__(32 * (kHotCopiers + kHotAdders), 2)
+__global__ void __launch_bounds__(32 * kHotWarps, 2)
 strip_hot_kernel(StripArgs a) {
     extern __shared__ float4 strip_smem[];
     __shared__ int2 ent_s[kHotBufs][kHotCopiers][32];  // (start relative to the strip, length) of each block
@@ -367,6 +412,11 @@ strip_hot_kernel(StripArgs a) {
     follow();
     if (a.status != nullptr && *a.status != 0) return;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (blockIdx.x < a.low_ctas) {  // (in a kernel of their own after this one: Adam on 852 K blocks 125 us against 116)
+        const uint32_t j = blockIdx.x * kHotWarps + w;
+        if (j + 1 < a.mp.Z) strip_low_slot<MODE, SHORT>(a, j, lane);
+        return;
+    }
     const bool copier = w >= (uint32_t)kHotAdders;
     const uint32_t cw = w - kHotAdders;
     const uint32_t Z = a.mp.Z, W = 1u << a.log2w;
@@ -558,7 +608,7 @@ void launch_strip_kernels(const StripArgs& a, cudaStream_t st, cudaStream_t hot_
     const uint32_t per_sm = (uint32_t)(220 * 1024 / (hot_smem + 26 * 1024));  // (26 KB: the static part and a margin)
     uint32_t hot_grid = 148 * (per_sm > 2 ? 2 : (per_sm < 1 ? 1 : per_sm));
     if (hot_grid > a.hot_cap) hot_grid = a.hot_cap;
-    launch_next(strip_hot_kernel<MODE, LP, EPL, SHORT>, hot_grid, 32 * (kHotCopiers + kHotAdders), hot_smem, hot_st, a);
+    launch_next(strip_hot_kernel<MODE, LP, EPL, SHORT>, a.low_ctas + hot_grid, 32 * kHotWarps, hot_smem, hot_st, a);
     const uint32_t per_cta = kStripWarps * (32 / LP);
     const size_t smem = ((size_t)per_cta << a.log2w) * sizeof(float);
     launch_next(strip_apply_kernel<MODE, LP, EPL, SHORT>, (a.strips + per_cta - 1) / per_cta, 32 * kStripWarps, smem, st, a);
@@ -602,6 +652,7 @@ StripArgs strip_args(const StripProblem& sp) {
     a.hot_cap = L.hot_cap;
     a.vec_commit = aligned(sp.target) && aligned(sp.adam.m1) && aligned(sp.adam.m2);
     a.grad_elems = sp.grad_elems;
+    a.low_ctas = (mp.Z - 1 + kHotWarps - 1) / kHotWarps;
     a.nb = sp.nb;
     // hot: twice the average number of blocks, and enough of them to be worth a CTA (26 x 16384 Zipf rows on
     // 540 K slots, twice / four times: 34 / 53 us beside the hot kernel's 50; a floor of 128 blocks instead
