@@ -398,6 +398,19 @@ def test_short_bags(d, Z, M, batch, bags):
                 assert_bits_equal(c.forward().cpu().numpy(), one, "offsets out of order")
 
 
+# More tables than a CTA works out the hash terms of once (64 in robe_pool.cu): both sides of that line in one call.
+@pytest.mark.parametrize("d,Z,M", [(16, 8, 4099), (100, 32, 50_021)])
+def test_short_bags_of_many_tables(d, Z, M):
+    w = small(d=d, Z=Z, M=M, bag_rule=(2, 0, 9), batch=301, num_tables=67, vocab_arg=tuple([1000] * 67))
+    for sign in (False, True):
+        with Case(w, sign=sign) as c:
+            assert_bits_equal(c.forward().cpu().numpy(), c.oracle_forward(), "forward")
+            g_h, g_d = _grad(c, 23, integer=True)
+            delta64, _ = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+            assert np.abs(delta64).max() < 2**24  # small integers: exact in any order
+            assert_bits_equal(c.backward(g_d, "atomic").cpu().numpy(), delta64.astype(np.float32), "backward")
+
+
 # The same in calls of so many bags that a warp takes up to 16 (mean 2) or 10 (mean 3) of them, unsigned rows of
 # every length in the backward too; full batches of staged ids inside a run, long bags among the short ones
 # that go on over several batches, and in the middle of a run.
