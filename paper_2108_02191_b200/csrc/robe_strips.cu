@@ -600,13 +600,20 @@ StripLayout strip_layout(uint64_t nb, uint32_t m) {
     return L;
 }
 
+size_t hot_smem_bytes(uint32_t Z, int epl) { return (size_t)kHotBufs * kHotCopiers * (hot_blocks(epl) + 4) * Z * sizeof(float); }
+
+// CTAs of the hot kernel that run at a time
+uint32_t hot_ctas(size_t hot_smem) {
+    const uint32_t per_sm = (uint32_t)(220 * 1024 / (hot_smem + 26 * 1024));  // (26 KB: the static part and a margin)
+    return 148 * (per_sm > 2 ? 2 : (per_sm < 1 ? 1 : per_sm));
+}
+
 template <int MODE, int LP, int EPL, bool SHORT>
 void launch_strip_kernels(const StripArgs& a, cudaStream_t st, cudaStream_t hot_st) {
-    const size_t hot_smem = (size_t)kHotBufs * kHotCopiers * (hot_blocks(EPL) + 4) * a.mp.Z * sizeof(float);
+    const size_t hot_smem = hot_smem_bytes(a.mp.Z, EPL);
     if (hot_smem > 23 * 1024)  // (with the static part above the default limit)
         cudaFuncSetAttribute(strip_hot_kernel<MODE, LP, EPL, SHORT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hot_smem);
-    const uint32_t per_sm = (uint32_t)(220 * 1024 / (hot_smem + 26 * 1024));  // (26 KB: the static part and a margin)
-    uint32_t hot_grid = 148 * (per_sm > 2 ? 2 : (per_sm < 1 ? 1 : per_sm));
+    uint32_t hot_grid = hot_ctas(hot_smem);
     if (hot_grid > a.hot_cap) hot_grid = a.hot_cap;
     launch_next(strip_hot_kernel<MODE, LP, EPL, SHORT>, a.low_ctas + hot_grid, 32 * kHotWarps, hot_smem, hot_st, a);
     const uint32_t per_cta = kStripWarps * (32 / LP);
@@ -658,7 +665,13 @@ StripArgs strip_args(const StripProblem& sp) {
     // 540 K slots, twice / four times: 34 / 53 us beside the hot kernel's 50; a floor of 128 blocks instead
     // of 256 made a 250 M-slot array 3 % slower, 512 none faster)
     const uint64_t mean = (uint64_t)((double)((1u << L.log2w) + mp.Z) * (double)sp.nb / mp.m) + 1;
-    const uint64_t hot = mean * 2 > kHotMin ? mean * 2 : kHotMin;
+    // A short array has so few strips, each reached by so many blocks, that a group of lanes to a strip leaves most
+    // of the chip idle: then every strip above the floor goes to the hot kernel.  The two costs in clocks: strips
+    // come to about 7700 + 8 blocks each in the hot kernel, over its CTAs, and 137 a block (and element of a lane)
+    // in strip_apply_kernel, all at a time.
+    const int epl = mp.Z <= 32 ? 1 : (mp.Z <= 64 ? 2 : 4);
+    const bool few = (double)L.strips * (7700.0 + 8.0 * mean) < 137.0 * epl * mean * hot_ctas(hot_smem_bytes(mp.Z, epl));
+    const uint64_t hot = !few && mean * 2 > kHotMin ? mean * 2 : kHotMin;
     a.n_hot = (uint32_t)(hot < 0x20000000ull ? hot : 0x20000000ull);
     return a;
 }

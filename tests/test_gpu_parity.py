@@ -671,6 +671,9 @@ STRIP_CASES = [
     dict(d=128, Z=128, M=129, batch=300, vocab_arg=(2, 30, 10**6)),
     dict(d=6, Z=3, M=7, batch=700, vocab_arg=(2, 30, 10**6)),
     dict(d=33, Z=1, M=65, batch=90, vocab_arg=(4, 30, 10**6)),
+    # few strips of very many blocks, all of them the hot kernel's (one and two elements to a lane)
+    dict(d=16, Z=8, M=50_003, batch=70_000, vocab_arg=(10**6, 10**6, 10**6)),
+    dict(d=64, Z=64, M=50_007, batch=40_000, vocab_arg=(10**6, 10**6, 10**6)),
 ]
 
 
