@@ -28,26 +28,42 @@ namespace {
 
 constexpr int kSortThreads = 512;                       // of the count and scatter kernels
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 8;                           // keys per thread per tile
-constexpr int kSortTile = kSortThreads * kSortItems;    // 4096
+// Keys per thread and tile: 8, or 4 in a call whose tiles of 2048 pairs are resident all at a time: the SMs with two
+// CTAs of 4096 would be waited for by those with one.  Measured (B200, us per step, 4096 -> 2048): Adam on 852 K
+// blocks 114 -> 111, ids that do not repeat 108 -> 100, on 52 K blocks 72 -> 66; 1.04 M blocks, 508 tiles for 444
+// CTAs, 238 -> 243.
+constexpr int kSortItems = 8, kSortItemsSmall = 4;
+__host__ __device__ constexpr int sort_tile(int items) { return kSortThreads * items; }  // 4096 pairs, 2048
 constexpr int kRadix = 256;
 constexpr int kSortCtas = 2;                            // per SM (3, with 40 registers: spills, 6 % slower)
 constexpr int kSortMaxGrid = 148 * kSortCtas;
-constexpr int kScanThreads = 256;
+constexpr int kSortMaxGridSmall = 148 * (kSortCtas + 1);  // tiles of kSortItemsSmall: 40 registers, 3 CTAs
+static_assert(128 * kSortMaxGridSmall <= kRadix * kSortMaxGrid, "counts of passes of up to 7 bits");
+constexpr int kScanThreads = 512;
 
 inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct SortPlan {
     uint64_t nb;        // number of (key,val) pairs
     uint32_t grid;      // CTAs of the count / scatter kernels
+    int items;          // keys per thread and tile
     uint64_t tiles;     // total tiles
 };
 
-SortPlan make_plan(uint64_t nb) {
+// for passes of up to `width` bits
+SortPlan make_plan(uint64_t nb, uint32_t width) {
     SortPlan sp;
     sp.nb = nb;
-    sp.tiles = (nb + kSortTile - 1) / kSortTile;
-    sp.grid = (uint32_t)(sp.tiles < (uint64_t)kSortMaxGrid ? sp.tiles : (uint64_t)kSortMaxGrid);
+    const uint64_t small = (nb + sort_tile(kSortItemsSmall) - 1) / sort_tile(kSortItemsSmall);
+    if (small <= (uint64_t)(width <= 7 ? kSortMaxGridSmall : kSortMaxGrid)) {
+        sp.items = kSortItemsSmall;
+        sp.tiles = small;
+        sp.grid = (uint32_t)small;
+    } else {
+        sp.items = kSortItems;
+        sp.tiles = (nb + sort_tile(kSortItems) - 1) / sort_tile(kSortItems);
+        sp.grid = (uint32_t)(sp.tiles < (uint64_t)kSortMaxGrid ? sp.tiles : (uint64_t)kSortMaxGrid);
+    }
     if (sp.grid == 0) sp.grid = 1;
     return sp;
 }
@@ -129,7 +145,7 @@ det_keys_by_block_kernel(KeyArgs a, const uint32_t* bag_of, uint32_t* keys, uint
 
 // ---- radix sort pass, kernel 1: digit histogram of each CTA's contiguous key range
 __global__ void __launch_bounds__(kSortThreads)
-sort_count_kernel(const uint32_t* keys, uint32_t* counts, uint64_t nb, uint64_t tiles,
+sort_count_kernel(const uint32_t* keys, uint32_t* counts, uint64_t nb, uint64_t tiles, uint32_t tile,
                   uint32_t shift, uint32_t mask) {
     __shared__ uint32_t hist[kSortWarps][kRadix];
     follow<true>();
@@ -137,14 +153,14 @@ sort_count_kernel(const uint32_t* keys, uint32_t* counts, uint64_t nb, uint64_t 
     __syncthreads();
     uint64_t first, count;
     cta_tiles(tiles, gridDim.x, blockIdx.x, first, count);
-    const uint64_t begin = first * kSortTile;
-    uint64_t end = (first + count) * kSortTile;
+    const uint64_t begin = first * tile;
+    uint64_t end = (first + count) * tile;
     if (end > nb) end = nb;
     uint32_t* mine = hist[threadIdx.x >> 5];
     for (uint64_t i = begin + threadIdx.x; i < end; i += kSortThreads)
         atomicAdd(&mine[(keys[i] >> shift) & mask], 1u);
     __syncthreads();
-    if (threadIdx.x >= kRadix) return;
+    if (threadIdx.x > mask) return;
     uint32_t total = 0;
     for (int k = 0; k < kSortWarps; ++k) total += hist[k][threadIdx.x];
     counts[(uint64_t)threadIdx.x * gridDim.x + blockIdx.x] = total;
@@ -204,9 +220,9 @@ sort_scan_kernel(uint32_t* counts, uint32_t* totals, uint32_t grid) {
 // next tile's pairs asked for before this one is written out.  Measured (B200, same pairs, us per pass,
 // before -> here): 247 -> 192; unstable with 6-bit digits 142 -> 130.  Finding the lanes of a digit by an
 // atomicOr into a shared word instead of ballots takes as long.
-template <bool STABLE, int BITS>
+template <bool STABLE, int BITS, int ITEMS>
 struct ScatterSmem {
-    uint2 pair[kSortTile];
+    uint2 pair[sort_tile(ITEMS)];
     // STABLE: per warp, pairs of each digit, then where they start in the tile
     uint16_t warp_digit[STABLE ? kSortWarps : 1][1 << BITS];
     uint32_t counter[1 << BITS];  // not STABLE: the same for the whole tile
@@ -216,36 +232,37 @@ struct ScatterSmem {
 
 // The pairs of the tile that starts at tbegin, warp-striped.  (nb may be close to 2^32: positions are
 // compared relative to the tile, so that nothing overflows.)
+template <int ITEMS>
 __device__ __forceinline__ void scatter_load(const uint32_t* kin, const uint32_t* vin,
-                                             uint32_t tbegin, uint32_t nb, uint32_t (&key)[kSortItems],
-                                             uint32_t (&val)[kSortItems]) {
-    const uint32_t left = nb - tbegin, local = (threadIdx.x >> 5) * (32 * kSortItems) + (threadIdx.x & 31);
+                                             uint32_t tbegin, uint32_t nb, uint32_t (&key)[ITEMS],
+                                             uint32_t (&val)[ITEMS]) {
+    const uint32_t left = nb - tbegin, local = (threadIdx.x >> 5) * (32 * ITEMS) + (threadIdx.x & 31);
     kin += tbegin;
     vin += tbegin;
-    if (left >= (uint32_t)kSortTile) {
+    if (left >= (uint32_t)sort_tile(ITEMS)) {
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) key[r] = __ldcs(kin + (local + r * 32));
+        for (int r = 0; r < ITEMS; ++r) key[r] = __ldcs(kin + (local + r * 32));
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) val[r] = __ldcs(vin + (local + r * 32));
+        for (int r = 0; r < ITEMS; ++r) val[r] = __ldcs(vin + (local + r * 32));
     } else {
 #pragma unroll
-        for (int r = 0; r < kSortItems; ++r) {
+        for (int r = 0; r < ITEMS; ++r) {
             key[r] = local + r * 32 < left ? __ldcs(kin + (local + r * 32)) : 0u;
             val[r] = local + r * 32 < left ? __ldcs(vin + (local + r * 32)) : 0u;
         }
     }
 }
 
-template <bool STABLE, int BITS, bool FULL>
-__device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, const uint32_t* kin,
+template <bool STABLE, int BITS, int ITEMS, bool FULL>
+__device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS, ITEMS>& sm, const uint32_t* kin,
                                              const uint32_t* vin, uint32_t* kout,
                                              uint32_t* vout, uint32_t nb, uint32_t tbegin,
-                                             uint32_t shift, uint32_t (&key)[kSortItems],
-                                             uint32_t (&val)[kSortItems], bool more) {
+                                             uint32_t shift, uint32_t (&key)[ITEMS],
+                                             uint32_t (&val)[ITEMS], bool more) {
     constexpr uint32_t R = 1u << BITS, mask = R - 1u;
     const uint32_t tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
-    const uint32_t left = nb - tbegin, local = w * (32 * kSortItems) + lane;  // (see scatter_load)
+    const uint32_t left = nb - tbegin, local = w * (32 * ITEMS) + lane;  // (see scatter_load)
     if (STABLE) {
         for (uint32_t k = tid; k < kSortWarps * R / 2; k += kSortThreads)
             reinterpret_cast<uint32_t*>(&sm.warp_digit[0][0])[k] = 0;
@@ -253,9 +270,9 @@ __device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, cons
         sm.counter[tid] = 0;
     }
     __syncthreads();
-    uint32_t rank[kSortItems];
+    uint32_t rank[ITEMS];
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         const bool valid = FULL || local + r * 32 < left;
         const uint32_t dg = (key[r] >> shift) & mask;
         rank[r] = 0;
@@ -306,17 +323,17 @@ __device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, cons
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
+    for (int r = 0; r < ITEMS; ++r) {
         if (FULL || local + r * 32 < left) {
             const uint32_t dg = (key[r] >> shift) & mask;
             const uint32_t lp = (STABLE ? sm.warp_digit[w][dg] : sm.counter[dg]) + rank[r];
-            if (!ROBE_CHK(lp < (uint32_t)kSortTile, ROBE_DBG_SHARED)) continue;
+            if (!ROBE_CHK(lp < (uint32_t)sort_tile(ITEMS), ROBE_DBG_SHARED)) continue;
             sm.pair[lp] = make_uint2(key[r], val[r]);
         }
     }
     __syncthreads();
-    if (more) scatter_load(kin, vin, tbegin + kSortTile, nb, key, val);
-    const uint32_t in_tile = FULL ? kSortTile : left;
+    if (more) scatter_load(kin, vin, tbegin + sort_tile(ITEMS), nb, key, val);
+    const uint32_t in_tile = FULL ? sort_tile(ITEMS) : left;
 #pragma unroll 4
     for (uint32_t lp = tid; lp < in_tile; lp += kSortThreads) {
         const uint2 p = sm.pair[lp];
@@ -330,13 +347,13 @@ __device__ __forceinline__ void scatter_tile(ScatterSmem<STABLE, BITS>& sm, cons
     // (the next tile's first barrier orders this update before its readers)
 }
 
-template <bool STABLE, int BITS>
-__global__ void __launch_bounds__(kSortThreads, kSortCtas)
+template <bool STABLE, int BITS, int ITEMS>
+__global__ void __launch_bounds__(kSortThreads, ITEMS == kSortItems ? kSortCtas : kSortCtas + 1)
 sort_scatter_kernel(const uint32_t* kin, const uint32_t* vin,
                     uint32_t* kout, uint32_t* vout,
                     const uint32_t* cta_offsets, const uint32_t* totals,
                     uint32_t nb, uint32_t tiles, uint32_t shift) {
-    __shared__ ScatterSmem<STABLE, BITS> sm;
+    __shared__ ScatterSmem<STABLE, BITS, ITEMS> sm;
     const uint32_t tid = threadIdx.x;
     follow<true>();
     {
@@ -349,15 +366,15 @@ sort_scatter_kernel(const uint32_t* kin, const uint32_t* vin,
     uint64_t first, count;
     cta_tiles(tiles, gridDim.x, blockIdx.x, first, count);
     if (count == 0) return;
-    uint32_t key[kSortItems], val[kSortItems];
-    scatter_load(kin, vin, (uint32_t)first * kSortTile, nb, key, val);
+    uint32_t key[ITEMS], val[ITEMS];
+    scatter_load(kin, vin, (uint32_t)first * sort_tile(ITEMS), nb, key, val);
     for (uint32_t t = (uint32_t)first; t < (uint32_t)(first + count); ++t) {
-        const uint32_t tbegin = t * kSortTile;
+        const uint32_t tbegin = t * sort_tile(ITEMS);
         const bool more = t + 1 < (uint32_t)(first + count);
-        if (nb - tbegin >= (uint32_t)kSortTile)
-            scatter_tile<STABLE, BITS, true>(sm, kin, vin, kout, vout, nb, tbegin, shift, key, val, more);
+        if (nb - tbegin >= (uint32_t)sort_tile(ITEMS))
+            scatter_tile<STABLE, BITS, ITEMS, true>(sm, kin, vin, kout, vout, nb, tbegin, shift, key, val, more);
         else
-            scatter_tile<STABLE, BITS, false>(sm, kin, vin, kout, vout, nb, tbegin, shift, key, val, more);
+            scatter_tile<STABLE, BITS, ITEMS, false>(sm, kin, vin, kout, vout, nb, tbegin, shift, key, val, more);
     }
 }
 
@@ -366,10 +383,14 @@ sort_scatter_kernel(const uint32_t* kin, const uint32_t* vin,
 template <bool STABLE, int BITS>
 void launch_sort_pass_bits(const SortPlan& sp, const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
                            uint32_t* counts, uint32_t* totals, uint32_t shift, cudaStream_t st) {
-    launch_next(sort_count_kernel, sp.grid, kSortThreads, 0, st, kin, counts, sp.nb, sp.tiles, shift, (1u << BITS) - 1u);
+    launch_next(sort_count_kernel, sp.grid, kSortThreads, 0, st, kin, counts, sp.nb, sp.tiles, (uint32_t)sort_tile(sp.items), shift,
+                (1u << BITS) - 1u);
     launch_next(sort_scan_kernel, 1 << BITS, kScanThreads, 0, st, counts, totals, sp.grid);
-    launch_next(sort_scatter_kernel<STABLE, BITS>, sp.grid, kSortThreads, 0, st, kin, vin, kout, vout, counts, totals,
-                                                                       (uint32_t)sp.nb, (uint32_t)sp.tiles, shift);
+    auto scatter = [&](auto kernel) {
+        launch_next(kernel, sp.grid, kSortThreads, 0, st, kin, vin, kout, vout, counts, totals, (uint32_t)sp.nb, (uint32_t)sp.tiles, shift);
+    };
+    if (sp.items == kSortItems) scatter(sort_scatter_kernel<STABLE, BITS, kSortItems>);
+    else scatter(sort_scatter_kernel<STABLE, BITS, kSortItemsSmall>);
 }
 
 template <bool STABLE>
@@ -1312,7 +1333,6 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
         launch_bag_of(pb, L, ws, st);  // the signed terms look the id's bag up again
     }
 
-    const SortPlan sp = make_plan(nb);
     const uint32_t bits = bits_for(mp.m);
     if (mode == 3) {
         // binned: one pass on the top key bits, then atomic adds in bin order.  A bin spans 2^22
@@ -1320,6 +1340,7 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
         // be updated in L2, large enough that the scatter writes long runs; 32 MB: adds 850 us against
         // 805) unless that would need more than 256 bins or the array is smaller than one such span.
         const uint32_t shift = bits > 30 ? bits - 8 : (bits > 22 ? 22 : (bits > 8 ? bits - 8 : 0));
+        const SortPlan sp = make_plan(nb, bits - shift);
         launch_sort_pass<false>(sp, kA, vA, kB, vB, counts, totals, shift, bits - shift, st);
         // (an array that does not fit the L2 passes through it bin by bin: lines that outlive their bin would
         // only be in the way of the gradient rows; 34 M blocks of 16 on 1 GB, us: 951 -> 925)
@@ -1351,6 +1372,7 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
     }
     const uint32_t npass = (bits + 7) / 8;
     const uint32_t bpp = (bits + npass - 1) / npass;
+    const SortPlan sp = make_plan(nb, bpp);
     for (uint32_t pass = 0; pass < npass; ++pass) {
         const uint32_t shift = pass * bpp;
         const uint32_t width = bits - shift < bpp ? bits - shift : bpp;

@@ -697,6 +697,12 @@ def test_deterministic_strip_rooms(case):
     test_deterministic_window_apply(case)
 
 
+# Either side of the size from which the sort takes 4096 pairs to a tile instead of 2048 (444 full tiles of them).
+@pytest.mark.parametrize("batch", [75_776, 75_777])
+def test_deterministic_sort_tiles(batch):
+    test_deterministic_window_apply(dict(d=16, Z=4, M=540_001, batch=batch, vocab_arg=(10**6, 10**6, 3000)))
+
+
 # robe_forward_keep + robe_backward_kept: one hash of every id per training step.  The pair must
 # give what robe_forward and robe_backward give: the forward bit for bit, the deterministic
 # backward bit for bit, the binned and atomic ones within the atomic bound.  Shapes: rows of every
