@@ -11,8 +11,8 @@
 //   * The sums start from -0 and a -0 element is made +0 first: x + -0 is x for every x, and -0 remains
 //     exactly where nothing was added (the canonical sum starts from +0, adds the same terms, and is never
 //     -0).  So an untouched slot is known by its sum.
-// No barriers between warps, nothing waits but a warp for its own loads.  Bound by instruction issue
-// (12 per block and lane group) and the random gradient reads.
+// No barriers between warps, nothing waits but a warp for its own loads.  Bound by the LSU pipe (shuffles, sums
+// in shared memory) and the random gradient reads.
 // Measured (B200, us, a CTA per 2048 slots with position-tile and long-walk kernels for often repeated ids
 // -> here): 34 M blocks of 16 on 250 M slots 1690 -> 895; Adam on 852 K blocks of 8 from Zipf ids, 540 K slots
 // 137 -> 50 (the longest id's chain: 9100 terms); the whole Adam step 257 -> 157.
@@ -202,7 +202,7 @@ __device__ __forceinline__ bool strip_touched(float sum) { return __float_as_uin
 // blocks that a copying warp of the hot kernel takes at a time, by the elements per lane of a block
 __host__ __device__ constexpr uint32_t hot_blocks(int epl) { return epl == 1 ? 32u : (epl == 2 ? 16u : 8u); }
 
-template <int MODE, int LP, int EPL, bool SHORT>
+template <int MODE, int LP, int EPL, bool SHORT, bool BANKED>
 __global__ void __launch_bounds__(32 * kStripWarps, 5)
 strip_apply_kernel(StripArgs a) {
     extern __shared__ float4 strip_smem[];
@@ -214,7 +214,15 @@ strip_apply_kernel(StripArgs a) {
     const uint32_t g = lane / LP, ol = lane % LP;
     const uint32_t b = (blockIdx.x * kStripWarps + w) * G + g;
     const uint32_t Z = a.mp.Z, W = 1u << a.log2w;
-    volatile float* const sum = reinterpret_cast<float*>(strip_smem) + (w * G + g) * W;
+    // BANKED: groups whose strips' sums lie one after the other would meet in the same banks.  Slot s of group g's
+    // strip lies at place(s) of the warp's sums, every group having LP banks to itself; past the sums there is a
+    // place in the same bank for slots that are not the strip's.
+    const uint32_t sums_at = BANKED ? w * (G * W + 32) : (w * G + g) * W;
+    volatile float* const sum = reinterpret_cast<float*>(strip_smem) + sums_at;
+    auto place = [&](uint32_t s) {
+        const uint32_t row = s & ~(LP - 1u);
+        return (row < W ? row : W) * G + (s & (LP - 1u)) + g * LP;
+    };
     uint32_t lo = 0, n = 0;
     if (b < a.strips) {
         lo = a.lo_of[b];
@@ -226,8 +234,8 @@ strip_apply_kernel(StripArgs a) {
     const uint32_t w0 = b << a.log2w;
     if (n != 0 && ol < W / 32 && (uint64_t)w0 + 32 * ol < a.mp.m)  // wanted at the end: the lines of the target
         asm volatile("prefetch.global.L2 [%0];" ::"l"(a.target + w0 + 32 * ol));
-    for (uint32_t i = ol; i < W / 4; i += LP)
-        reinterpret_cast<float4*>(strip_smem)[((w * G + g) * W >> 2) + i] = make_float4(-0.0f, -0.0f, -0.0f, -0.0f);
+    for (uint32_t i = BANKED ? lane : ol; i < (BANKED ? G * W / 4 : W / 4); i += BANKED ? 32 : LP)
+        strip_smem[(sums_at >> 2) + i] = make_float4(-0.0f, -0.0f, -0.0f, -0.0f);
     // lane ol holds block ol of the present LP: start relative to the strip, payload
     uint32_t nk = 0, nv = 0;
     if (ol < n && ROBE_CHK((uint64_t)lo + ol < a.nb, ROBE_DBG_SORT_POS)) {
@@ -260,6 +268,7 @@ strip_apply_kernel(StripArgs a) {
                         ROBE_CHK((uint64_t)p + 32 * q < a.grad_elems, ROBE_DBG_GRAD_POS))
                         x[u][q] = load_settled(a.grad_out + (p + 32 * q)) + 0.0f;  // -0 -> +0
                 }
+                if constexpr (BANKED) slot[u] = place(slot[u]);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -267,7 +276,7 @@ strip_apply_kernel(StripArgs a) {
                 for (int q = 0; q < EPL; ++q) {
                     // (a lane past the block's end adds -0 to a slot that is no other lane's in this step)
                     const uint32_t s = slot[u] + 32 * q;
-                    if (s < W) sum[s] = __fadd_rn(sum[s], x[u][q]);
+                    if (BANKED || s < W) sum[s] = __fadd_rn(sum[s], x[u][q]);
                 }
                 __syncwarp();
             }
@@ -275,9 +284,9 @@ strip_apply_kernel(StripArgs a) {
     }
     if (n == 0) return;
     const bool inner = a.vec_commit && w0 + 1 >= Z && (uint64_t)w0 + W <= a.mp.m;
-    const float4* const sum4 = strip_smem + ((w * G + g) * W >> 2);
+    const float4* const sum4 = strip_smem + (sums_at >> 2);
     for (uint32_t i = ol; i < W / 4; i += LP) {
-        const float4 s = sum4[i];
+        const float4 s = sum4[BANKED ? place(4 * i) >> 2 : i];
         const bool t0 = strip_touched(s.x), t1 = strip_touched(s.y), t2 = strip_touched(s.z), t3 = strip_touched(s.w);
         const uint32_t j = w0 + 4 * i;
         if (!(t0 || t1 || t2 || t3)) continue;
@@ -617,8 +626,20 @@ void launch_strip_kernels(const StripArgs& a, cudaStream_t st, cudaStream_t hot_
     if (hot_grid > a.hot_cap) hot_grid = a.hot_cap;
     launch_next(strip_hot_kernel<MODE, LP, EPL, SHORT>, a.low_ctas + hot_grid, 32 * kHotWarps, hot_smem, hot_st, a);
     const uint32_t per_cta = kStripWarps * (32 / LP);
+    const unsigned grid = (a.strips + per_cta - 1) / per_cta;
     const size_t smem = ((size_t)per_cta << a.log2w) * sizeof(float);
-    launch_next(strip_apply_kernel<MODE, LP, EPL, SHORT>, (a.strips + per_cta - 1) / per_cta, 32 * kStripWarps, smem, st, a);
+    // Banks of their own for the lane groups of a warp: 39 .. 48 registers instead of 32 .. 40, against shared-memory
+    // reads and writes that no longer meet (LSU pipe 92 % busy before).  Four groups always gain, two where the rows
+    // come from L2 rather than memory.  Measured (B200, us per step): 68 M blocks of 8 on 250 M slots 5454 -> 4912,
+    // on 10 M 4017 -> 3267; 34 M blocks of 16 on 10 M 1922 -> 1854, on 250 M 2762 -> 2838; 33 M blocks of 8 and
+    // a short one on 10 M 2555 -> 2543, on 250 M 4043 -> 4118.
+    if constexpr (LP < 32) {
+        if ((LP == 8 && !SHORT) || (uint64_t)a.mp.m * 4 <= (192ull << 20)) {
+            launch_next(strip_apply_kernel<MODE, LP, EPL, SHORT, true>, grid, 32 * kStripWarps, smem + kStripWarps * 32 * sizeof(float), st, a);
+            return;
+        }
+    }
+    if constexpr (LP > 8 || SHORT) launch_next(strip_apply_kernel<MODE, LP, EPL, SHORT, false>, grid, 32 * kStripWarps, smem, st, a);
 }
 
 template <int MODE, bool SHORT>

@@ -682,6 +682,29 @@ def test_deterministic_strips(case):
     test_deterministic_window_apply(case)
 
 
+# Lane groups with banks of their own beside those without: four groups to a warp on an array beyond the L2, two
+# on either side of the size at which they change, short last blocks.
+BANK_CASES = [
+    dict(d=16, Z=8, M=52_000_003, batch=1_100_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=32, Z=16, M=50_331_648, batch=550_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=32, Z=16, M=50_331_649, batch=550_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=20, Z=8, M=50_331_000, batch=700_000, vocab_arg=(10**6, 10**6, 3000)),
+]
+
+
+@pytest.mark.parametrize("case", BANK_CASES, ids=lambda k: f"d{k['d']}_Z{k['Z']}_M{k['M']}")
+def test_deterministic_strip_banks(case):
+    w = small(**case)
+    with Case(w, host_array=False) as c:
+        nb = c.indices.numel() * -(-w.d // w.Z)
+        assert nb * w.Z * 2 >= w.M, "the case must touch the array densely"
+        g_h, g_d = _grad(c, 12)
+        det = c.backward(g_d, "det")
+        for j0 in (0, w.M // 2, w.M - 300_000):
+            can, _ = c.oracle.backward_canonical(g_h, c.indices_h, c.offsets_h, c.B, j0=j0, jn=300_000)
+            assert_bits_equal(det[j0:j0 + 300_000].cpu().numpy(), can, f"slots from {j0}")
+
+
 # Where the strips' bounds and lists go: room of their own on a short array; on a longer one where the last sort
 # pass read from, or, at just under a block per strip, nowhere (the position-tile kernel then serves a densely
 # touched array).
