@@ -1220,7 +1220,10 @@ template <int MODE>
 void launch_apply_strips(const ApplyArgs& aa, const uint32_t* K, const uint32_t* V, int mode, void* workspace,
                          const SideStream& side, cudaStream_t st) {
     const MapParams& mp = aa.mp;
-    const StripProblem sp{mp, aa.grad_out, aa.grad_elems, aa.target, aa.lr, aa.adam, K, V, aa.nb, aa.status, workspace};
+    // (the list of long walks, free where strips serve the call, has room for that of the hot strips: 3 bytes a block and
+    // 25 KB at least, 400 MB at most, against 4 bytes for every 32 blocks, or every 85 in a large call)
+    const StripProblem sp{mp, aa.grad_out, aa.grad_elems, aa.target, aa.lr, aa.adam, K, V, aa.nb, aa.status, workspace,
+                          (uint32_t*)aa.long_walks};
     launch_strips_prepare(sp, st);
     const bool forked = side.st != nullptr;
     if (forked) {

@@ -97,7 +97,8 @@ struct StripProblem {
     const uint32_t* V;
     uint64_t nb;
     const int32_t* status;
-    void* workspace;  // strips_workspace_bytes, 256-byte aligned
+    void* workspace;     // strips_workspace_bytes, 256-byte aligned
+    uint32_t* hot_list;  // room for the hot strips' list: nb / 8 bytes and a few more
 };
 bool strips_ok(const MapParams& mp, uint64_t nb, bool sign);
 size_t strips_workspace_bytes(const MapParams& mp, uint64_t nb);

@@ -38,7 +38,7 @@ constexpr int kHotAdders = 8;             // and that add: 32 slots each
 constexpr int kHotWarps = kHotCopiers + kHotAdders;
 constexpr uint32_t kHotAhead = 3;         // steps that the copies, and again as many that the keys, are asked for ahead
 constexpr uint32_t kHotBufs = kHotAhead + 1;
-constexpr uint32_t kHotMin = 256;         // a strip is hot from this many blocks on, at least
+constexpr uint32_t kHotLeast = 96;        // blocks that make a strip hot, at least (see strip_args)
 
 struct StripArgs {
     MapParams mp;
@@ -590,8 +590,8 @@ strip_hot_kernel(StripArgs a) {
 inline size_t align_256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct StripLayout {
-    size_t lo_of, hi_of, list, total;
-    uint32_t strips, hot_cap, log2w;
+    size_t lo_of, hi_of, total;
+    uint32_t strips, log2w;
 };
 
 StripLayout strip_layout(uint64_t nb, uint32_t m) {
@@ -600,12 +600,12 @@ StripLayout strip_layout(uint64_t nb, uint32_t m) {
     L.log2w = kStripMaxLog2;
     while (L.log2w > kStripMinLog2 && (m >> L.log2w) < 148u * 64u) --L.log2w;
     L.strips = ((m - 1) >> L.log2w) + 1;
-    const uint64_t cap = 3 * nb / kHotMin + 1;  // (a block of up to 128 elements reaches at most three strips)
-    L.hot_cap = (uint32_t)(cap < L.strips ? cap : L.strips);
     L.lo_of = 256;  // the counters come first
     L.hi_of = L.lo_of + align_256(((size_t)L.strips + 1) * sizeof(uint32_t));
-    L.list = L.hi_of + align_256(((size_t)L.strips + 1) * sizeof(uint32_t));
-    L.total = L.list + align_256((size_t)L.hot_cap * sizeof(uint32_t));
+    L.total = L.hi_of + align_256(((size_t)L.strips + 1) * sizeof(uint32_t));
+    // (what a list of one strip in 256 blocks would take: the figure that callers have sized workspaces by)
+    const uint64_t list = 3 * nb / 256 + 1;
+    L.total += align_256((size_t)(list < L.strips ? list : L.strips) * sizeof(uint32_t));
     return L;
 }
 
@@ -676,15 +676,13 @@ StripArgs strip_args(const StripProblem& sp) {
     a.strips = L.strips;
     a.log2w = L.log2w;
     a.hot_count = (uint32_t*)ws;
-    a.hot_list = (uint32_t*)(ws + L.list);
-    a.hot_cap = L.hot_cap;
+    a.hot_list = sp.hot_list;
     a.vec_commit = aligned(sp.target) && aligned(sp.adam.m1) && aligned(sp.adam.m2);
     a.grad_elems = sp.grad_elems;
     a.low_ctas = (mp.Z - 1 + kHotWarps - 1) / kHotWarps;
     a.nb = sp.nb;
     // hot: twice the average number of blocks, and enough of them to be worth a CTA (26 x 16384 Zipf rows on
-    // 540 K slots, twice / four times: 34 / 53 us beside the hot kernel's 50; a floor of 128 blocks instead
-    // of 256 made a 250 M-slot array 3 % slower, 512 none faster)
+    // 540 K slots, twice / four times: 34 / 53 us beside the hot kernel's 50)
     const uint64_t mean = (uint64_t)((double)((1u << L.log2w) + mp.Z) * (double)sp.nb / mp.m) + 1;
     // A short array has so few strips, each reached by so many blocks, that a group of lanes to a strip leaves most
     // of the chip idle: then every strip above the floor goes to the hot kernel.  The two costs in clocks: strips
@@ -692,7 +690,14 @@ StripArgs strip_args(const StripProblem& sp) {
     // in strip_apply_kernel, all at a time.
     const int epl = mp.Z <= 32 ? 1 : (mp.Z <= 64 ? 2 : 4);
     const bool few = (double)L.strips * (7700.0 + 8.0 * mean) < 137.0 * epl * mean * hot_ctas(hot_smem_bytes(mp.Z, epl));
-    const uint64_t hot = !few && mean * 2 > kHotMin ? mean * 2 : kHotMin;
+    // A strip is hot from this many blocks on, at least: 256 in large calls, fewer in small ones, whose last strips'
+    // chains are what the call waits for (us, floor 256 / 192 / 128 / 96: Adam on 52 K blocks of 8, 540 K slots 63.4 /
+    // 60.5 / 56.0 / 54.0; on 52 K of 128, 1 M slots 135 / 122 / 109 / 101; 416 K of 16, 1 M 107 / 103 / 99 / 99; but 852 K
+    // of 8, 3.9 M 122 / 125 / 129 / 131, and 34 M of 16 from Zipf ids, 250 M 2941 / 2978 / 3080 / 3199).
+    const uint64_t least = sp.nb / 3072 < kHotLeast ? kHotLeast : (sp.nb / 3072 > 256 ? 256 : sp.nb / 3072);
+    const uint64_t hot = !few && mean * 2 > least ? mean * 2 : least;
+    const uint64_t cap = 3 * sp.nb / least + 1;  // (a block of up to 128 elements reaches at most three strips)
+    a.hot_cap = (uint32_t)(cap < L.strips ? cap : L.strips);
     a.n_hot = (uint32_t)(hot < 0x20000000ull ? hot : 0x20000000ull);
     return a;
 }
