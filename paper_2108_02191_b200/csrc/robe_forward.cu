@@ -380,14 +380,16 @@ static void launch_vec(const FwdArgs& a, bool bags, cudaStream_t st) {
 // for (MINB, see kStagedCtas*).  Measured on B200: the time of the HBM-resident gather does not move
 // between 4 and 16 ids in flight - the random 64-byte requests themselves are the limit.
 
-// One-hot rows of 128 from a bf16 array are the exception (131072 x 26 rows on 50 MB, us): 6 CTAs and 2 ids
-// 498, 5 and 4 484, 4 and 8 477, 3 and 8 505, 8 and 2 566.
+// One-hot rows of up to 128 elements take more ids at fewer CTAs (us): fp32, 65536 x 26 Zipf rows of 128, Z = 32, 100 MB,
+// 6 CTAs and 2 ids 219.8, 5 and 4 215.9, 4 and 4 221.7, 8 and 1 256; 8000 x 26 of them 30.0, 29.1, 30.3, 38.4. bf16,
+// 131072 x 26 rows on 50 MB, 6 and 2 498, 5 and 4 484, 4 and 8 477, 3 and 8 505, 8 and 2 566.
 
 template <int EPL, int DT, bool SIGN, bool FULLD, int MINB>
 static void launch_staged_minb(const FwdArgs& a, bool bags, cudaStream_t st) {
     constexpr int UB = (EPL == 4) ? 2 : 4;
-    constexpr int UO = (EPL == 4) ? (DT == 1 && !SIGN ? 8 : 2) : 4;
-    constexpr int MINO = (EPL == 4 && DT == 1 && !SIGN) ? 4 : MINB;
+    constexpr bool WIDE = EPL == 4 && !SIGN;
+    constexpr int UO = WIDE && DT == 1 ? 8 : (EPL == 4 && SIGN ? 2 : 4);
+    constexpr int MINO = WIDE ? (DT == 1 ? 4 : 5) : MINB;
     const uint32_t ipb = staged_ids_per_batch(a.mp, bags, SIGN);
     const uint32_t cmagic = chunk_magic(a.mp);
     const int64_t warps = bags ? a.nbags : (a.nbags + ipb - 1) / ipb;
