@@ -20,7 +20,13 @@ constexpr int kFlatWarps = 8;
 constexpr int kFlatCtas = 6;            // per SM; loads in flight (8) x CTAs of 8 / 5, 8 / 4, 16 / 4, 4 / 8: 0-5 % slower
 constexpr uint32_t kFlatEntries = 256;  // block starts per warp
 constexpr uint32_t kFlatRows = 64;      // rows per warp
-constexpr uint32_t kFlatElems = 4096;   // elements per warp, about
+// Elements per warp, about.  In large calls the CTAs of fewer rows follow one another more evenly (B200, us per step,
+// 4096 -> 2048 (1536, 1024): 13 x 16384 rows of 256, Z = 64, 100 MB 147.0 -> 141.7 (141.6, 141.9), of 200 139.8 ->
+// 127.8 (128.6, 130.3), of 150, Z = 32 123.9 -> 105.4 (103.9, 107.8), 13 x 8000 of 256 80.8 -> 77.0; 26 x 32768 of 64, Z = 64,
+// 122.3 -> 119.3 (119.9, 123.7); 65536 x 26 of 128, Z = 128 177 -> 176 (181, 196)); calls of a wave or less lose
+// (13 x 4000 rows of 256, 13.3 M elements, 37.7 -> 38.2).
+constexpr uint32_t kFlatElems = 2048, kFlatElemsSmall = 4096;
+constexpr int64_t kFlatLarge = 1 << 24;  // elements of a large call
 
 struct FlatArgs {
     MapParams mp;
@@ -45,7 +51,7 @@ struct FlatSmem {
     uint32_t start[kFlatWarps][kFlatEntries];  // block starts, row after row
 };
 
-// f / divisor, exact while f * divisor < 2^32 (f < 16384 + kFlatElems here, the divisors at most 16384)
+// f / divisor, exact while f * divisor < 2^32 (f < 16384 + kFlatElemsSmall here, the divisors at most 16384)
 __device__ __forceinline__ uint32_t flat_div(uint32_t f, uint32_t magic) { return magic != 0 ? __umulhi(f, magic) : f; }
 
 // Hash phase: the block starts of rows [row0, row0 + cnt).  Returns whether some block wraps.
@@ -204,7 +210,8 @@ static cudaError_t launch_flat(const Problem& pb, const float* grad_out, float* 
     // rows per warp: as many as the staging holds, but few enough for small calls to reach every SM
     uint32_t rows = kFlatEntries / mp.C;
     if (rows > kFlatRows) rows = kFlatRows;
-    if (rows > kFlatElems / mp.d) rows = kFlatElems / mp.d;
+    const uint32_t elems = pb.nbags * (int64_t)mp.d >= kFlatLarge ? kFlatElems : kFlatElemsSmall;
+    if (rows > elems / mp.d) rows = elems / mp.d;
     const int64_t spread = pb.nbags / (148 * 32) + 1;
     if ((int64_t)rows > spread) rows = (uint32_t)spread;
     if (rows < 1) rows = 1;
