@@ -29,6 +29,7 @@ struct PoolArgs {
     uint32_t* keep_keys;   // see KeepBlocks
     uint32_t* keep_vals;
     uint32_t bags;         // per warp
+    uint64_t share;        // forward: the same in units of 2^-32, warp i takes bags [i share, (i + 1) share)
     uint32_t ids;          // per batch
     uint32_t cmagic;
     int l2_keep;
@@ -111,11 +112,21 @@ struct PoolRun {
     bool stretch;
 };
 
+template <bool EVEN>
 __device__ __forceinline__ PoolRun pool_run(const PoolArgs& a, uint32_t w, uint32_t lane) {
     PoolRun r;
-    r.k0 = ((int64_t)blockIdx.x * 8 + w) * a.bags;
-    const int64_t left = a.nbags - r.k0;
-    r.bags = left <= 0 ? 0u : (left < (int64_t)a.bags ? (uint32_t)left : a.bags);
+    const uint64_t warp = (uint64_t)blockIdx.x * 8 + w;
+    if (EVEN) {
+        auto first = [&](uint64_t i) { return (int64_t)(__umul64hi(i, a.share) << 32 | (i * a.share) >> 32); };
+        r.k0 = first(warp);
+        int64_t end = first(warp + 1);
+        if (end > a.nbags) end = a.nbags;
+        r.bags = end > r.k0 ? (uint32_t)(end - r.k0) : 0u;
+    } else {
+        r.k0 = (int64_t)warp * a.bags;
+        const int64_t left = a.nbags - r.k0;
+        r.bags = left <= 0 ? 0u : (left < (int64_t)a.bags ? (uint32_t)left : a.bags);
+    }
     r.off = 0;
     if (r.bags != 0) r.off = clamp64(__ldca(a.offsets + r.k0 + (lane < r.bags ? lane : r.bags)), 0, a.nnz);
     const int64_t next = __shfl_down_sync(0xFFFFFFFFu, r.off, 1);
@@ -209,7 +220,7 @@ pool_kernel(PoolArgs a) {
     stage_init(sm.stage, mp);
     follow();
     if (a.status != nullptr && *a.status != 0) return;
-    const PoolRun run = pool_run(a, w, lane);
+    const PoolRun run = pool_run<MODE != 2>(a, w, lane);
     if (run.bags == 0) return;
 
     PoolLane<EPL> l;
@@ -271,6 +282,8 @@ void launch_pool_epl(const PoolArgs& a, unsigned blocks, cudaStream_t st) {
 
 uint32_t pool_ids(const Problem& pb) { return staged_ids_per_batch(pb.mp, true, pb.sign != 0); }
 
+int64_t pool_wave(const Problem& pb) { return 148 * 8 * (pb.sign != 0 ? kPoolCtasSign : kPoolCtas); }  // warps at a time
+
 // Bags per warp, 1 where a warp per bag is the better kernel.  A run of about 16 ids is what a warp gains
 // by (32 in calls of hundreds of thousands of bags, which have warps enough); how long the bags may be
 // for that follows a sweep over 7 x 3001, 26 x 512 and 26 x 16384 bags of 2 .. 12 ids on 4 and 400 MB (B200, us,
@@ -296,7 +309,7 @@ uint32_t pool_bags(const Problem& pb, bool backward) {
     const int64_t spread = pb.nbags / (148 * 40) + 1;
     if (bags > spread) bags = spread;
     // a last wave that is nearly empty costs a whole one: rather a bag more per warp
-    const int64_t wave = 148 * 8 * (pb.sign != 0 ? kPoolCtasSign : kPoolCtas);
+    const int64_t wave = pool_wave(pb);
     if (bags > 1) {
         const int64_t waves = ((pb.nbags + bags - 1) / bags + wave / 2) / wave;
         if (waves >= 1 && waves <= 3) bags = (pb.nbags + waves * wave - 1) / (waves * wave);
@@ -320,10 +333,17 @@ static cudaError_t launch_pool(const Problem& pb, PoolArgs& a, int mode, cudaStr
     a.nnz = pb.nnz;
     a.status = pb.status;
     a.ids = pool_ids(pb);
-    a.bags = pool_bags(pb, mode == 2);
     a.cmagic = chunk_magic(pb.mp);
     a.l2_keep = pb.l2_keep;
-    const int64_t warps = (pb.nbags + a.bags - 1) / a.bags;
+    // Forward: up to three waves are filled to the last warp, the bags spread evenly over them, unless the runs get much
+    // shorter (B200, us, runs of one length -> even: 7 x 3001 signed bags of 4, d = 100, 17.7 -> 16.7, d = 60 12.4 ->
+    // 11.2; unsigned bags of 2 11.3 -> 10.3; 26 x 1024 bags of 4, d = 64 13.4 -> 12.7; 7 x 1500 of 4, 3 -> 2.2 bags to a
+    // run, 10.3 -> 11.2).  The backward gains where rows are short and loses where bags are (19.0 -> 17.8, 18.7 -> 19.6).
+    const int64_t bags = pool_bags(pb, mode == 2), wave = pool_wave(pb), waves = (pb.nbags + bags * wave - 1) / (bags * wave);
+    const bool fill = mode != 2 && waves <= 3 && 20 * pb.nbags >= 17 * waves * wave * bags;
+    const int64_t warps = fill ? waves * wave : (pb.nbags + bags - 1) / bags;
+    a.bags = (uint32_t)bags;
+    a.share = fill ? (((uint64_t)pb.nbags << 32) + (uint64_t)warps - 1) / (uint64_t)warps : (uint64_t)bags << 32;
     const unsigned blocks = (unsigned)((warps + 7) / 8);
     if (mode == 0) { if (pb.sign) launch_pool_epl<0, true>(a, blocks, st); else launch_pool_epl<0, false>(a, blocks, st); }
     else if (mode == 1) { if (pb.sign) launch_pool_epl<1, true>(a, blocks, st); else launch_pool_epl<1, false>(a, blocks, st); }

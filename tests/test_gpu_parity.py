@@ -411,6 +411,17 @@ def test_short_bags_of_many_tables(d, Z, M):
             assert_bits_equal(c.backward(g_d, "atomic").cpu().numpy(), delta64.astype(np.float32), "backward")
 
 
+# Forward runs spread evenly over a full wave of warps (5920 of them, unsigned): runs of 4 and 5 bags, the last warps,
+# and one bag more than five to a warp.
+@pytest.mark.parametrize("batch", [9472, 9866, 9867])
+@pytest.mark.parametrize("d,Z,M", [(16, 8, 4099), (64, 16, 100_003)])
+def test_short_bags_spread_evenly(d, Z, M, batch):
+    w = small(d=d, Z=Z, M=M, bag_rule=(2, 0, 9), batch=batch)
+    for sign in (False, True):
+        with Case(w, sign=sign) as c:
+            assert_bits_equal(c.forward().cpu().numpy(), c.oracle_forward(), "forward")
+
+
 # The same in calls of so many bags that a warp takes up to 16 (mean 2) or 10 (mean 3) of them, unsigned rows of
 # every length in the backward too; full batches of staged ids inside a run, long bags among the short ones
 # that go on over several batches, and in the middle of a run.
