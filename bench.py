@@ -417,11 +417,11 @@ def run_ours(args, w):
         zb = min(w.Z, w.d)
         bwd_launches = ((1 if bags else 0) + 1 + 3 * npass + 1 + (1 if w.d % zb == 0 else 0)
                         + (1 if zb > 1 else 0))
-        # a densely touched array is served by strips: their bounds, the list of hot ones, the two apply
-        # kernels (and the low slots) instead
+        # a densely touched array is served by strips: their bounds, the list of hot ones and the two apply
+        # kernels instead (the low slots in one of them)
         nblocks = float(np.mean([len(b[0]) for b in batches])) * -(-w.d // zb)
         if zb <= 128 and 2 * nblocks * zb >= w.M:
-            bwd_launches = (1 if bags else 0) + 1 + 3 * npass + 4 + (1 if zb > 1 else 0)
+            bwd_launches = (1 if bags else 0) + 1 + 3 * npass + 4
     # One training step hashes every id once: the forward leaves the block starts in the workspace
     # and the sort-based backward takes them from there (rows of up to 128 elements; longer rows
     # use a forward kernel that keeps nothing, and the key kernels then run inside the forward call).

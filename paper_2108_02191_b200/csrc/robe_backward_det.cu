@@ -209,7 +209,7 @@ sort_scan_kernel(uint32_t* counts, uint32_t* totals, uint32_t grid) {
 }
 
 // ---- kernel 3: ranked scatter (STABLE: keeps the input order inside a digit - the LSD sort needs
-// that; the binned backward does not and takes ranks from shared-memory counters).  Per tile of 4096
+// that; the binned backward does not and takes ranks from shared-memory counters).  Per tile of 4096 or 2048
 // pairs: every warp ranks its 256 pairs by digit (8 rounds of ballots, earlier rounds and lower lanes
 // first), the ranks are extended over the warps, the pairs are laid out in shared memory in (digit,
 // original order), and then written out so that each digit's pairs go to consecutive addresses.

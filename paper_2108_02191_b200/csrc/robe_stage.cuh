@@ -26,7 +26,8 @@ __device__ __forceinline__ void bag_range(const int64_t* offsets, int64_t nnz, i
 // thread) for arrays of L2 size, where the gather is bound by L2 latency and the extra warps pay
 // (2-8 % measured on B200), and 6 CTAs (40 registers, no spill) for arrays in HBM, where occupancy buys
 // nothing and the spill traffic costs DRAM bandwidth (cfg 4 forward 0.895 -> 0.864 ms).  Rows of up to
-// 128 elements: 6 CTAs (42 registers).  With the sign hash on: 4 CTAs (it needs the registers).
+// 128 elements: 6 CTAs (40 registers; one-hot forwards have their own, see launch_staged_minb).  With the sign
+// hash on: 4 CTAs (it needs the registers).
 constexpr int kStagedCtasL2 = 8, kStagedCtasHbm = 6, kStagedCtasWide = 6, kStagedCtasSign = 4;
 constexpr uint64_t kL2SizedBytes = 192ull << 20;  // arrays up to this size count as "of L2 size"
 
