@@ -1177,7 +1177,7 @@ struct Layout {
 };
 
 // Arrays whose strips can never ask for more than this (up to 5.5 M slots) have room for them in the workspace.
-constexpr size_t kStripRoom = 256 << 10;
+constexpr size_t kStripRoom = 171 << 10;
 
 Layout make_layout(uint64_t nb, int64_t nnz, bool bags, const MapParams& mp) {
     Layout L;
@@ -1200,8 +1200,11 @@ Layout make_layout(uint64_t nb, int64_t nnz, bool bags, const MapParams& mp) {
     // (The sign option may be switched after the workspace was sized: room for the strips either way.)  The total
     // must not fall as nb grows: a caller sizes for its largest call.  On a longer array the strips go to the
     // free pair; where they do not fit that, there is less than a block per strip, and the call goes without.
-    const size_t strips = strips_ok(mp, nb, false) ? strips_workspace_bytes(mp, nb) : 0;
-    L.strips_own = strips != 0 && strips_workspace_bytes(mp, 1ull << 40) <= kStripRoom;
+    // The list of hot strips takes the place of that of long walks, which strips do without (400 bytes for every 128
+    // blocks against 4 for every 32 at most; for a list beyond that there would be no strips).
+    const bool listed = strips_ok(mp, nb, false) && strips_list_bytes(mp, nb) <= (size_t)cap * sizeof(LongWalk);
+    const size_t strips = listed ? strips_workspace_bytes(mp) : 0;
+    L.strips_own = strips != 0 && strips <= kStripRoom;
     L.strips_spare = strips != 0 && !L.strips_own && strips <= 2 * kb;
     L.strips = off; off += L.strips_own ? strips : 0;
     L.total = off;
@@ -1220,8 +1223,6 @@ template <int MODE>
 void launch_apply_strips(const ApplyArgs& aa, const uint32_t* K, const uint32_t* V, int mode, void* workspace,
                          const SideStream& side, cudaStream_t st) {
     const MapParams& mp = aa.mp;
-    // (the list of long walks, free where strips serve the call, has room for that of the hot strips: 3 bytes a block and
-    // 25 KB at least, 400 MB at most, against 4 bytes for every 32 blocks, or every 85 in a large call)
     const StripProblem sp{mp, aa.grad_out, aa.grad_elems, aa.target, aa.lr, aa.adam, K, V, aa.nb, aa.status, workspace,
                           (uint32_t*)aa.long_walks};
     launch_strips_prepare(sp, st);

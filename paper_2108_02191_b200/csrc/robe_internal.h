@@ -98,10 +98,11 @@ struct StripProblem {
     uint64_t nb;
     const int32_t* status;
     void* workspace;     // strips_workspace_bytes, 256-byte aligned
-    uint32_t* hot_list;  // room for the hot strips' list: nb / 8 bytes and a few more
+    uint32_t* hot_list;  // strips_list_bytes
 };
 bool strips_ok(const MapParams& mp, uint64_t nb, bool sign);
-size_t strips_workspace_bytes(const MapParams& mp, uint64_t nb);
+size_t strips_workspace_bytes(const MapParams& mp);
+size_t strips_list_bytes(const MapParams& mp, uint64_t nb);
 // first sorted position of every strip; in st
 void launch_strips_prepare(const StripProblem& sp, cudaStream_t st);
 // all slots but [0, Z-1), mode as launch_backward_det's 0, 1, 2, 4.  Strips of often repeated ids are served

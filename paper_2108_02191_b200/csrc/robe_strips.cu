@@ -38,7 +38,7 @@ constexpr int kHotAdders = 8;             // and that add: 32 slots each
 constexpr int kHotWarps = kHotCopiers + kHotAdders;
 constexpr uint32_t kHotAhead = 3;         // steps that the copies, and again as many that the keys, are asked for ahead
 constexpr uint32_t kHotBufs = kHotAhead + 1;
-constexpr uint32_t kHotLeast = 96;        // blocks that make a strip hot, at least (see strip_args)
+constexpr uint32_t kHotLeast = 96;        // blocks that make a strip hot, at least (see hot_least)
 
 struct StripArgs {
     MapParams mp;
@@ -594,7 +594,7 @@ struct StripLayout {
     uint32_t strips, log2w;
 };
 
-StripLayout strip_layout(uint64_t nb, uint32_t m) {
+StripLayout strip_layout(uint32_t m) {
     StripLayout L;
     // Long strips (fewer blocks that reach two of them), unless that leaves warps without work
     L.log2w = kStripMaxLog2;
@@ -603,10 +603,19 @@ StripLayout strip_layout(uint64_t nb, uint32_t m) {
     L.lo_of = 256;  // the counters come first
     L.hi_of = L.lo_of + align_256(((size_t)L.strips + 1) * sizeof(uint32_t));
     L.total = L.hi_of + align_256(((size_t)L.strips + 1) * sizeof(uint32_t));
-    // (what a list of one strip in 256 blocks would take: the figure that callers have sized workspaces by)
-    const uint64_t list = 3 * nb / 256 + 1;
-    L.total += align_256((size_t)(list < L.strips ? list : L.strips) * sizeof(uint32_t));
     return L;
+}
+
+// A strip is hot from this many blocks on, at least: 256 in large calls, fewer in small ones, whose last strips'
+// chains are what the call waits for (us, floor 256 / 192 / 128 / 96: Adam on 52 K blocks of 8, 540 K slots 63.4 /
+// 60.5 / 56.0 / 54.0; on 52 K of 128, 1 M slots 135 / 122 / 109 / 101; 416 K of 16, 1 M 107 / 103 / 99 / 99; but 852 K
+// of 8, 3.9 M 122 / 125 / 129 / 131, and 34 M of 16 from Zipf ids, 250 M 2941 / 2978 / 3080 / 3199).
+uint64_t hot_least(uint64_t nb) { return nb / 3072 < kHotLeast ? kHotLeast : (nb / 3072 > 256 ? 256 : nb / 3072); }
+
+// Entries of the hot strips' list.  (A block of up to 128 elements reaches at most three strips.)
+uint32_t hot_list_cap(uint64_t nb, uint32_t strips) {
+    const uint64_t cap = 3 * nb / hot_least(nb) + 1;
+    return (uint32_t)(cap < strips ? cap : strips);
 }
 
 size_t hot_smem_bytes(uint32_t Z, int epl) { return (size_t)kHotBufs * kHotCopiers * (hot_blocks(epl) + 4) * Z * sizeof(float); }
@@ -659,7 +668,7 @@ void launch_strip_mode(const StripArgs& a, cudaStream_t st, cudaStream_t hot_st)
 
 StripArgs strip_args(const StripProblem& sp) {
     const MapParams& mp = sp.mp;
-    const StripLayout L = strip_layout(sp.nb, mp.m);
+    const StripLayout L = strip_layout(mp.m);
     char* ws = (char*)sp.workspace;
     auto aligned = [](const void* p) { return ((uintptr_t)p & 15u) == 0; };
     StripArgs a{};
@@ -690,14 +699,8 @@ StripArgs strip_args(const StripProblem& sp) {
     // in strip_apply_kernel, all at a time.
     const int epl = mp.Z <= 32 ? 1 : (mp.Z <= 64 ? 2 : 4);
     const bool few = (double)L.strips * (7700.0 + 8.0 * mean) < 137.0 * epl * mean * hot_ctas(hot_smem_bytes(mp.Z, epl));
-    // A strip is hot from this many blocks on, at least: 256 in large calls, fewer in small ones, whose last strips'
-    // chains are what the call waits for (us, floor 256 / 192 / 128 / 96: Adam on 52 K blocks of 8, 540 K slots 63.4 /
-    // 60.5 / 56.0 / 54.0; on 52 K of 128, 1 M slots 135 / 122 / 109 / 101; 416 K of 16, 1 M 107 / 103 / 99 / 99; but 852 K
-    // of 8, 3.9 M 122 / 125 / 129 / 131, and 34 M of 16 from Zipf ids, 250 M 2941 / 2978 / 3080 / 3199).
-    const uint64_t least = sp.nb / 3072 < kHotLeast ? kHotLeast : (sp.nb / 3072 > 256 ? 256 : sp.nb / 3072);
-    const uint64_t hot = !few && mean * 2 > least ? mean * 2 : least;
-    const uint64_t cap = 3 * sp.nb / least + 1;  // (a block of up to 128 elements reaches at most three strips)
-    a.hot_cap = (uint32_t)(cap < L.strips ? cap : L.strips);
+    const uint64_t least = hot_least(sp.nb), hot = !few && mean * 2 > least ? mean * 2 : least;
+    a.hot_cap = hot_list_cap(sp.nb, L.strips);
     a.n_hot = (uint32_t)(hot < 0x20000000ull ? hot : 0x20000000ull);
     return a;
 }
@@ -710,10 +713,14 @@ bool strips_ok(const MapParams& mp, uint64_t nb, bool sign) {
     return !sign && mp.Z <= kStripMaxZ && nb != 0 && nb < 0xFFFFF000ull && nb * mp.Z * 2 >= mp.m;
 }
 
-size_t strips_workspace_bytes(const MapParams& mp, uint64_t nb) { return strip_layout(nb, mp.m).total; }
+size_t strips_workspace_bytes(const MapParams& mp) { return strip_layout(mp.m).total; }
+
+size_t strips_list_bytes(const MapParams& mp, uint64_t nb) {
+    return (size_t)hot_list_cap(nb, strip_layout(mp.m).strips) * sizeof(uint32_t);
+}
 
 void launch_strips_prepare(const StripProblem& sp, cudaStream_t st) {
-    const StripLayout L = strip_layout(sp.nb, sp.mp.m);
+    const StripLayout L = strip_layout(sp.mp.m);
     char* ws = (char*)sp.workspace;
     uint32_t *lo_of = (uint32_t*)(ws + L.lo_of), *hi_of = (uint32_t*)(ws + L.hi_of);
     if (L.strips > 148u * 256u)

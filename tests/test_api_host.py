@@ -130,6 +130,21 @@ def test_workspace_asks_for_no_more_than_it_used_to():
     assert asked[300_000_000, 1_300_000] <= robe.ROBE_STATIC_SCRATCH_BYTES
 
 
+def test_workspace_holds_the_strips_bounds_and_nothing_more():
+    # the bounds of strips go by the array's length alone, whatever the number of blocks; a longer array's go to
+    # buffers that are there anyway
+    for M, strips in [(540_000, 8438), (1_200_000, 18_750), (5_400_000, 21_094), (5_800_000, 0), (25_000_000, 0)]:
+        room = 256 + 2 * -(-4 * (strips + 1) // 256) * 256 if strips else 0
+        for nnz in [M // 32 + 1, M // 4, 2 * M]:  # touched densely: blocks of 16 on half of the slots or more
+            figures = []
+            for m in (M, 1 << 31):
+                h = robe.robe_create(m, 16, 16, 1, 1)
+                robe.robe_set_option(h, robe.ROBE_OPT_BWD_MODE, robe.ROBE_BWD_DETERMINISTIC)
+                figures.append(robe.robe_backward_workspace_bytes(h, nnz, nnz))
+                robe.robe_destroy(h)
+            assert figures[0] - figures[1] == room, (M, nnz, figures)
+
+
 def test_sort_based_variants_refuse_sizes_beyond_their_32_bit_numbering():
     # block numbers, bag numbers and gradient positions are 32-bit in the binned / deterministic /
     # Adam paths: larger calls are refused before anything is launched (dummy pointers are never read)

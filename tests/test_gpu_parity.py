@@ -723,6 +723,7 @@ ROOM_CASES = [
     dict(d=128, Z=128, M=5_400_007, batch=7300, vocab_arg=(10**6, 10**6, 30)),
     dict(d=128, Z=128, M=25_000_000, batch=33_000, vocab_arg=(10**6, 10**6, 30)),
     dict(d=128, Z=128, M=25_000_000, batch=32_567, vocab_arg=(10**6, 10**6, 30)),
+    dict(d=128, Z=128, M=25_000_000, batch=32_553, vocab_arg=(10**6, 10**6, 30)),
 ]
 
 
