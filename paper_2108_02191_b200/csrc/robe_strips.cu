@@ -694,12 +694,18 @@ StripArgs strip_args(const StripProblem& sp) {
     // 540 K slots, twice / four times: 34 / 53 us beside the hot kernel's 50)
     const uint64_t mean = (uint64_t)((double)((1u << L.log2w) + mp.Z) * (double)sp.nb / mp.m) + 1;
     // A short array has so few strips, each reached by so many blocks, that a group of lanes to a strip leaves most
-    // of the chip idle: then every strip above the floor goes to the hot kernel.  The two costs in clocks: strips
-    // come to about 7700 + 8 blocks each in the hot kernel, over its CTAs, and 137 a block (and element of a lane)
-    // in strip_apply_kernel, all at a time.
+    // of the chip idle.  `gain` sets the two costs in clocks against each other: 137 a block (and element of a lane) in
+    // strip_apply_kernel, all strips at a time, and 7700 + 8 a block in the hot kernel, strips over its CTAs.  Spread ids
+    // reach every strip alike, repeated ones leave the apply kernel with strips just below `hot`.  So from a gain of 2.25 (1.75
+    // with many blocks to a strip, or long ones) on every strip above the floor is hot, and from 1 on those a tenth
+    // above the average: spread ids have few of them.  Measured (B200, us per Adam step on 60 K slots, 300 K blocks of 16, a
+    // gain of 1.6; hot from twice the average / 1.1 times it / the floor): spread ids 75.1 / 74.3 / 92.8, Zipf ids 98.4 /
+    // 74.1 / 82.7.  Over 360 shapes of Z = 2 .. 128, relative to twice the average: between the two lines spread 1 / 0.99 / 1.22,
+    // Zipf 1 / 0.74 / 0.75; beyond, up to a gain of 5, spread 1 / 1.00 / 0.88, Zipf 1 / 0.65 / 0.49.
     const int epl = mp.Z <= 32 ? 1 : (mp.Z <= 64 ? 2 : 4);
-    const bool few = (double)L.strips * (7700.0 + 8.0 * mean) < 137.0 * epl * mean * hot_ctas(hot_smem_bytes(mp.Z, epl));
-    const uint64_t least = hot_least(sp.nb), hot = !few && mean * 2 > least ? mean * 2 : least;
+    const double gain = 137.0 * epl * mean * hot_ctas(hot_smem_bytes(mp.Z, epl)) / (L.strips * (7700.0 + 8.0 * mean));
+    const uint64_t least = hot_least(sp.nb), above = gain >= (epl > 1 || mean >= 1000 ? 1.75 : 2.25) ? 0 : (gain >= 1 ? mean + mean / 10 : 2 * mean);
+    const uint64_t hot = above > least ? above : least;
     a.hot_cap = hot_list_cap(sp.nb, L.strips);
     a.n_hot = (uint32_t)(hot < 0x20000000ull ? hot : 0x20000000ull);
     return a;

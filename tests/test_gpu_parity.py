@@ -685,6 +685,9 @@ STRIP_CASES = [
     # few strips of very many blocks, all of them the hot kernel's (one and two elements to a lane)
     dict(d=16, Z=8, M=50_003, batch=70_000, vocab_arg=(10**6, 10**6, 10**6)),
     dict(d=64, Z=64, M=50_007, batch=40_000, vocab_arg=(10**6, 10**6, 10**6)),
+    # fewer blocks: those a little above the average only
+    dict(d=64, Z=16, M=60_003, batch=25_000, vocab_arg=(10**6, 10**6, 10**6)),
+    dict(d=64, Z=16, M=60_004, batch=25_000, vocab_arg=(10**6, 40, 10**6), id_dist="zipf1.05"),
 ]
 
 
