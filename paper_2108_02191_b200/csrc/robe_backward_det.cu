@@ -28,10 +28,12 @@ namespace {
 
 constexpr int kSortThreads = 512;                       // of the count and scatter kernels
 constexpr int kSortWarps = kSortThreads / 32;
-// Keys per thread and tile: 8, or 4 in a call whose tiles of 2048 pairs are resident all at a time: the SMs with two
-// CTAs of 4096 would be waited for by those with one.  Measured (B200, us per step, 4096 -> 2048): Adam on 852 K
-// blocks 114 -> 111, ids that do not repeat 108 -> 100, on 52 K blocks 72 -> 66; 1.04 M blocks, 508 tiles for 444
-// CTAs, 238 -> 243.
+// Keys per thread and tile: 8, or 4 where that leaves the busiest SM fewer pairs (up to 148 tiles of 2048, and from 297
+// to 444: three CTAs of them to an SM against two of 4096).  Measured (B200, us per step, 4096 -> 2048): 304 K .. 606 K
+// pairs, two tiles of 2048 to an SM or one of 4096: deterministic SGD on 400 K blocks of 16, 24-bit keys, 79 -> 86, on
+// 600 K 96 -> 103, binned adds on 400 K 28.3 -> 29.7, Adam on 350 K and 550 K, 7-bit digits, 0.99 .. 1.01; outside: Adam on
+// 200 K 0.97, 100 K 0.95 .. 0.99, 30 K 0.96, binned adds on 30 K and 150 K 0.95; Adam on 852 K 114 -> 111, ids that do not
+// repeat 108 -> 100; 1.04 M, 508 tiles for 444 CTAs, 238 -> 243.
 constexpr int kSortItems = 8, kSortItemsSmall = 4;
 __host__ __device__ constexpr int sort_tile(int items) { return kSortThreads * items; }  // 4096 pairs, 2048
 constexpr int kRadix = 256;
@@ -55,14 +57,17 @@ SortPlan make_plan(uint64_t nb, uint32_t width) {
     SortPlan sp;
     sp.nb = nb;
     const uint64_t small = (nb + sort_tile(kSortItemsSmall) - 1) / sort_tile(kSortItemsSmall);
-    if (small <= (uint64_t)(width <= 7 ? kSortMaxGridSmall : kSortMaxGrid)) {
+    const uint64_t large = (nb + sort_tile(kSortItems) - 1) / sort_tile(kSortItems);
+    auto of_busiest_sm = [](uint64_t tiles, int items) { return (tiles + 147) / 148 * items; };
+    if (small <= (uint64_t)(width <= 7 ? kSortMaxGridSmall : kSortMaxGrid) &&
+        of_busiest_sm(small, kSortItemsSmall) < of_busiest_sm(large, kSortItems)) {
         sp.items = kSortItemsSmall;
         sp.tiles = small;
         sp.grid = (uint32_t)small;
     } else {
         sp.items = kSortItems;
-        sp.tiles = (nb + sort_tile(kSortItems) - 1) / sort_tile(kSortItems);
-        sp.grid = (uint32_t)(sp.tiles < (uint64_t)kSortMaxGrid ? sp.tiles : (uint64_t)kSortMaxGrid);
+        sp.tiles = large;
+        sp.grid = (uint32_t)(large < (uint64_t)kSortMaxGrid ? large : (uint64_t)kSortMaxGrid);
     }
     if (sp.grid == 0) sp.grid = 1;
     return sp;
@@ -209,8 +214,8 @@ sort_scan_kernel(uint32_t* counts, uint32_t* totals, uint32_t grid) {
 }
 
 // ---- kernel 3: ranked scatter (STABLE: keeps the input order inside a digit - the LSD sort needs
-// that; the binned backward does not and takes ranks from shared-memory counters).  Per tile of 4096 or 2048
-// pairs: every warp ranks its 256 pairs by digit (8 rounds of ballots, earlier rounds and lower lanes
+// that; the binned backward does not and takes ranks from shared-memory counters).  Per tile of 4096 (2048)
+// pairs: every warp ranks its 256 (128) pairs by digit (8 (4) rounds of ballots, earlier rounds and lower lanes
 // first), the ranks are extended over the warps, the pairs are laid out in shared memory in (digit,
 // original order), and then written out so that each digit's pairs go to consecutive addresses.
 //

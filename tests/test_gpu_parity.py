@@ -741,6 +741,14 @@ def test_deterministic_sort_tiles(batch):
     test_deterministic_window_apply(dict(d=16, Z=4, M=540_001, batch=batch, vocab_arg=(10**6, 10**6, 3000)))
 
 
+# The other sizes at which the sort changes between tiles of 2048 and of 4096 pairs (148 and 296 full tiles of 2048), with
+# 7-bit and with 8-bit digits; a workspace holds the counts of no more than 296 tiles of the latter.
+@pytest.mark.parametrize("M", [60_001, 540_001])
+@pytest.mark.parametrize("batch", [37_888, 37_889, 75_776, 75_777])
+def test_deterministic_sort_tiles_by_digits(batch, M):
+    test_deterministic_window_apply(dict(d=16, Z=4, M=M, batch=batch, num_tables=2, vocab_arg=(10**6, 3000)))
+
+
 # robe_forward_keep + robe_backward_kept: one hash of every id per training step.  The pair must
 # give what robe_forward and robe_backward give: the forward bit for bit, the deterministic
 # backward bit for bit, the binned and atomic ones within the atomic bound.  Shapes: rows of every
