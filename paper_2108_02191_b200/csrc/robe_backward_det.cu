@@ -1355,7 +1355,7 @@ cudaError_t launch_backward_det(const Problem& pb, const float* grad_out, float*
         launch_sort_pass<false>(sp, kA, vA, kB, vB, counts, totals, shift, bits - shift, st);
         // (an array that does not fit the L2 passes through it bin by bin: lines that outlive their bin would
         // only be in the way of the gradient rows; 34 M blocks of 16 on 1 GB, us: 951 -> 925)
-        const int keep = (uint64_t)mp.m * 4 <= (192ull << 20) ? pb.l2_keep : 0;
+        const int keep = (uint64_t)mp.m * 4 <= kL2SizedBytes ? pb.l2_keep : 0;
         ApplyArgs ab{mp, grad_out, pb.indices, target, lr, nb, pb.status, AdamState{}, nullptr, nullptr, 0,
                      (uint64_t)pb.nbags * mp.d, keep};
         if (!pb.sign && mp.Z <= 128) {

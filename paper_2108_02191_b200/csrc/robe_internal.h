@@ -28,6 +28,8 @@ inline void launch_next(void (*kernel)(P...), unsigned grid, unsigned block, siz
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // (an error stays for cudaGetLastError)
 }
 
+constexpr uint64_t kL2SizedBytes = 192ull << 20;  // arrays up to this size count as "of L2 size"
+
 struct Problem {
     MapParams mp;
     const void* array;       // device, M elements

@@ -29,7 +29,6 @@ __device__ __forceinline__ void bag_range(const int64_t* offsets, int64_t nnz, i
 // 128 elements: 6 CTAs (40 registers; one-hot forwards have their own, see launch_staged_minb).  With the sign
 // hash on: 4 CTAs (it needs the registers).
 constexpr int kStagedCtasL2 = 8, kStagedCtasHbm = 6, kStagedCtasWide = 6, kStagedCtasSign = 4;
-constexpr uint64_t kL2SizedBytes = 192ull << 20;  // arrays up to this size count as "of L2 size"
 
 constexpr int kStageEntries = 256;  // block starts per warp
 constexpr int kStageIds = 64;       // ids per warp batch

@@ -637,13 +637,22 @@ void launch_strip_kernels(const StripArgs& a, cudaStream_t st, cudaStream_t hot_
     const uint32_t per_cta = kStripWarps * (32 / LP);
     const unsigned grid = (a.strips + per_cta - 1) / per_cta;
     const size_t smem = ((size_t)per_cta << a.log2w) * sizeof(float);
-    // Banks of their own for the lane groups of a warp: 39 .. 48 registers instead of 32 .. 40, against shared-memory
-    // reads and writes that no longer meet (LSU pipe 92 % busy before).  Four groups always gain, two where the rows
-    // come from L2 rather than memory.  Measured (B200, us per step): 68 M blocks of 8 on 250 M slots 5454 -> 4912,
-    // on 10 M 4017 -> 3267; 34 M blocks of 16 on 10 M 1922 -> 1854, on 250 M 2762 -> 2838; 33 M blocks of 8 and
-    // a short one on 10 M 2555 -> 2543, on 250 M 4043 -> 4118.
-    if constexpr (LP < 32) {
-        if ((LP == 8 && !SHORT) || (uint64_t)a.mp.m * 4 <= (192ull << 20)) {
+    // Banks of their own for the lane groups of a warp, for up to seven registers more and no more shared-memory conflicts
+    // (LSU pipe 92 % busy with them).  Measured (B200, us per step):
+    //   four groups of full blocks gain on any array: 68 M blocks of 8 on 250 M slots 5454 -> 4912, on 10 M 4017 -> 3267;
+    //   four with short last blocks only in the optimizers' steps, on arrays of L2 size (Adam on 300 K slots 0.92 .. 0.98);
+    //     SGD on 4 M blocks of 8, 8 and 4, 300 K slots 494 -> 565, on 4 M 281 -> 297, on 30 M 368 -> 397;
+    //   two with short last blocks there too: 15 M of 16 and a short one on 4 M 853 -> 817, 4 M on 300 K 421 -> 404;
+    //   two of full blocks pay with six CTAs to an SM instead of eight (39 registers, 32 before): only in the SGD step, where
+    //     rows come from L2 and fewer CTAs at a time are not a wave more of a wave or two.  34 M blocks of 16 on 4 M (977 CTAs)
+    //     1805 -> 1893, from Zipf ids 2044 -> 2564, on 10 M 1723 -> 1643, 2140 -> 2118, on 20 M 1740 -> 1700, on 48 M 1728 -> 1747;
+    //     1.2 M on 540 K slots (528 CTAs) 141 -> 129, on 2 M (977) 130 -> 141; 8 M on 7 M (1709) 499 -> 475; Adam 1.00 .. 1.05.
+    if constexpr (LP < 32 && (LP == 8 ? !SHORT || MODE >= 2 : SHORT || MODE < 2)) {
+        const uint64_t bytes = (uint64_t)a.mp.m * sizeof(float);
+        auto waves = [&](unsigned per_sm) { return (grid + 148 * per_sm - 1) / (148 * per_sm); };
+        const bool banked = SHORT ? bytes <= kL2SizedBytes
+                                  : LP == 8 || (bytes <= (128ull << 20) && (waves(6) <= waves(8) || grid > 2 * 8 * 148));
+        if (banked) {
             launch_next(strip_apply_kernel<MODE, LP, EPL, SHORT, true>, grid, 32 * kStripWarps, smem + kStripWarps * 32 * sizeof(float), st, a);
             return;
         }

@@ -703,6 +703,13 @@ BANK_CASES = [
     dict(d=32, Z=16, M=50_331_648, batch=550_000, vocab_arg=(10**6, 10**6, 3000)),
     dict(d=32, Z=16, M=50_331_649, batch=550_000, vocab_arg=(10**6, 10**6, 3000)),
     dict(d=20, Z=8, M=50_331_000, batch=700_000, vocab_arg=(10**6, 10**6, 3000)),
+    # either side of the lines for two groups of full blocks: 888 and 1184 CTAs of 16 strips, and 128 MB
+    dict(d=32, Z=16, M=909_312, batch=30_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=32, Z=16, M=909_313, batch=30_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=32, Z=16, M=4_849_664, batch=60_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=32, Z=16, M=4_849_665, batch=60_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=32, Z=16, M=33_554_432, batch=400_000, vocab_arg=(10**6, 10**6, 3000)),
+    dict(d=32, Z=16, M=33_554_433, batch=400_000, vocab_arg=(10**6, 10**6, 3000)),
 ]
 
 
