@@ -384,20 +384,40 @@ static void launch_vec(const FwdArgs& a, bool bags, cudaStream_t st) {
 // 6 CTAs and 2 ids 219.8, 5 and 4 215.9, 4 and 4 221.7, 8 and 1 256; 8000 x 26 of them 30.0, 29.1, 30.3, 38.4. bf16,
 // 131072 x 26 rows on 50 MB, 6 and 2 498, 5 and 4 484, 4 and 8 477, 3 and 8 505, 8 and 2 566.
 
+// Ids of a one-hot batch in whole groups of `group` ids in flight (the rest of one waits as long as a whole one), on
+// arrays of L2 size in calls that still are a wave of warps.  Measured (B200, us, as many ids as 64 (id, chunk) pairs take
+// -> whole groups): 60000 x 26 Zipf rows of 100, Z = 8, 100 MB 284 -> 238, 20000 x 26 in bf16 156 -> 75; Z = 16 73 -> 71 and
+// 89 -> 67; but 20000 x 26 rows of 127, Z = 9, 1 GB 1.02, 1500 x 26, Z = 13 1.08 (fewer ids, one group of four: 1.07).
+static uint32_t whole_groups(const FwdArgs& a, uint32_t ids, uint32_t group, int64_t wave) {
+    const uint32_t whole = (ids + group - 1) / group * group;
+    const bool fits = whole * a.mp.C <= (uint32_t)kStageEntries && whole <= (uint32_t)kStageIds;
+    return fits && a.nbags >= wave * whole ? whole : ids;
+}
+
 template <int EPL, int DT, bool SIGN, bool FULLD, int MINB>
 static void launch_staged_minb(const FwdArgs& a, bool bags, cudaStream_t st) {
     constexpr int UB = (EPL == 4) ? 2 : 4;
     constexpr bool WIDE = EPL == 4 && !SIGN;
     constexpr int UO = WIDE && DT == 1 ? 8 : (EPL == 4 && SIGN ? 2 : 4);
     constexpr int MINO = WIDE ? (DT == 1 ? 4 : 5) : MINB;
-    const uint32_t ipb = staged_ids_per_batch(a.mp, bags, SIGN);
+    uint32_t ipb = staged_ids_per_batch(a.mp, bags, SIGN);
+    if (!bags && WIDE && (uint64_t)a.mp.m * (DT == 0 ? 4u : 2u) <= kL2SizedBytes) ipb = whole_groups(a, ipb, UO, 148 * 8 * MINO);
     const uint32_t cmagic = chunk_magic(a.mp);
     const int64_t warps = bags ? a.nbags : (a.nbags + ipb - 1) / ipb;
     const unsigned blocks = (unsigned)((warps + 7) / 8);
-    if (bags)
+    if (bags) {
         launch_next(fwd_staged_kernel<EPL, DT, SIGN, true, FULLD, MINB, UB>, blocks, 256, 0, st, a, ipb, cmagic);
-    else
-        launch_next(fwd_staged_kernel<EPL, DT, SIGN, false, FULLD, MINO, UO>, blocks, 256, 0, st, a, ipb, cmagic);
+        return;
+    }
+    if constexpr (WIDE && DT == 0) {
+        // The rest of a group of four costs more than four in flight gain: 520 K rows of 127, Z = 13, on 1 GB 106.3 -> 101.6,
+        // 78 K of Z = 19 .. 26 15.3 -> 14.4, 13.8 -> 12.8.
+        if (ipb % UO != 0) {
+            launch_next(fwd_staged_kernel<EPL, DT, SIGN, false, FULLD, MINB, 2>, blocks, 256, 0, st, a, ipb, cmagic);
+            return;
+        }
+    }
+    launch_next(fwd_staged_kernel<EPL, DT, SIGN, false, FULLD, MINO, UO>, blocks, 256, 0, st, a, ipb, cmagic);
 }
 
 template <int EPL, int DT, bool SIGN, bool FULLD>

@@ -370,6 +370,26 @@ def test_millions_of_one_hot_rows(d, Z, table_major):
                           delta64.astype(np.float32), "backward, integer gradient")
 
 
+# One-hot rows of 65 to 128 elements by the staged kernel: batches of whole groups of ids (4 fp32, 8 bf16) where they are
+# a wave of warps and fit the staging area, in small calls with a rest.
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d,Z,M", [(100, 8, 4099), (100, 16, 1013), (127, 25, 100_003), (72, 10, 777), (128, 2, 4099), (128, 1, 4099),
+                                   (66, 3, 5003), (128, 512, 5003)])
+def test_staged_rows_in_whole_groups(d, Z, M, dtype):
+    for batch in (1, 97, 20_011 if Z >= 8 else 4_001):
+        w = small(d=d, Z=Z, M=M, batch=batch, array_dtype=dtype, vocab_arg=(3, 1000, 40_000_000))
+        with Case(w) as c:
+            want = c.oracle_forward()
+            assert_bits_equal(c.forward(2).cpu().numpy(), want, "forward")
+            if batch != 97:
+                continue
+            g_h, g_d = _grad(c, 31)
+            can, _ = c.oracle.backward_canonical(g_h, c.indices_h, c.offsets_h, c.B)
+            out, det = c.step_sharing_keys(g_d, "det", fwd_kernel=2)
+            assert_bits_equal(out.cpu().numpy(), want, "forward that keeps its block starts")
+            assert_bits_equal(det.cpu().numpy(), can, "deterministic on the kept starts")
+
+
 # A run of short bags per warp: runs that end inside the last warp, empty bags at either end of a run and in
 # rows, bags that go on over several batches of staged ids, one element and 128 per row, arrays that wrap,
 # rows clubbed into one block, and offsets that are no stretch (a warp then takes its bags one by one).
