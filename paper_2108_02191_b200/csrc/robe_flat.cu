@@ -20,13 +20,19 @@ constexpr int kFlatWarps = 8;
 constexpr int kFlatCtas = 6;            // per SM; loads in flight (8) x CTAs of 8 / 5, 8 / 4, 16 / 4, 4 / 8: 0-5 % slower
 constexpr uint32_t kFlatEntries = 256;  // block starts per warp
 constexpr uint32_t kFlatRows = 64;      // rows per warp
-// Elements per warp, about.  In large calls the CTAs of fewer rows follow one another more evenly (B200, us per step,
-// 4096 -> 2048 (1536, 1024): 13 x 16384 rows of 256, Z = 64, 100 MB 147.0 -> 141.7 (141.6, 141.9), of 200 139.8 ->
-// 127.8 (128.6, 130.3), of 150, Z = 32 123.9 -> 105.4 (103.9, 107.8), 13 x 8000 of 256 80.8 -> 77.0; 26 x 32768 of 64, Z = 64,
-// 122.3 -> 119.3 (119.9, 123.7); 65536 x 26 of 128, Z = 128 177 -> 176 (181, 196)); calls of a wave or less lose
-// (13 x 4000 rows of 256, 13.3 M elements, 37.7 -> 38.2).
-constexpr uint32_t kFlatElems = 2048, kFlatElemsSmall = 4096;
-constexpr int64_t kFlatLarge = 1 << 24;  // elements of a large call
+// Elements per warp, about: 4096, or 2048 in large calls, whose CTAs then follow one another more evenly:
+//   in calls of 0.86 to 2.3 waves of CTAs of 4096 elements a warp, whose last wave then is a smaller part - but not in the forward
+//     on arrays of up to 16 MB, which issue bounds: a rest of a group of 256 elements, whose loads are in flight together, takes
+//     a warp as long as a whole one, and half the elements are half as many to share it;
+//   in the forward from 16 M elements on where the run of rows is whole groups.
+// Measured (B200, us, 4096 -> 2048): 13 x 16384 rows of 256, Z = 64, 100 MB (54 M elements), both passes 147.0 -> 141.7
+// (1536: 141.6, 1024: 141.9).  Over 500 shapes, forward: whole groups 16 M .. 30 M elements 0.93 .. 0.98, more 0.96 .. 1.00,
+// with a rest 1.02 .. 1.09 on arrays of up to 16 MB (13 x 12000 rows of 257, Z = 32 43 -> 48), on larger ones 25 M .. 60 M
+// elements 0.92 .. 0.99, fewer or more 1.02; backward 26 M .. 60 M elements 0.89 .. 0.98, 17 M .. 22 M 1.00 .. 1.10 (13 x 3605 rows
+// of 384, Z = 128 30.7 -> 36.2), 70 M 1.00 .. 1.04.
+constexpr uint32_t kFlatElems = 4096, kFlatElemsHalf = 2048;
+constexpr int64_t kFlatWholeHalf = 1 << 24, kFlatHalf = 24 << 20, kFlatHalfEnd = 64 << 20;  // elements of such calls
+constexpr uint64_t kFlatFewBytes = 16 << 20;
 
 struct FlatArgs {
     MapParams mp;
@@ -51,7 +57,7 @@ struct FlatSmem {
     uint32_t start[kFlatWarps][kFlatEntries];  // block starts, row after row
 };
 
-// f / divisor, exact while f * divisor < 2^32 (f < 16384 + kFlatElemsSmall here, the divisors at most 16384)
+// f / divisor, exact while f * divisor < 2^32 (f < 16384 + kFlatElems here, the divisors at most 16384)
 __device__ __forceinline__ uint32_t flat_div(uint32_t f, uint32_t magic) { return magic != 0 ? __umulhi(f, magic) : f; }
 
 // Hash phase: the block starts of rows [row0, row0 + cnt).  Returns whether some block wraps.
@@ -210,8 +216,11 @@ static cudaError_t launch_flat(const Problem& pb, const float* grad_out, float* 
     // rows per warp: as many as the staging holds, but few enough for small calls to reach every SM
     uint32_t rows = kFlatEntries / mp.C;
     if (rows > kFlatRows) rows = kFlatRows;
-    const uint32_t elems = pb.nbags * (int64_t)mp.d >= kFlatLarge ? kFlatElems : kFlatElemsSmall;
-    if (rows > elems / mp.d) rows = elems / mp.d;
+    const int64_t all = pb.nbags * (int64_t)mp.d;
+    const uint32_t half = rows < kFlatElemsHalf / mp.d ? rows : kFlatElemsHalf / mp.d;
+    const bool few = mode != 2 && (uint64_t)mp.m * (pb.dtype == 0 ? 4u : 2u) <= kFlatFewBytes;
+    if ((all >= kFlatHalf && all < kFlatHalfEnd && !few) || (mode != 2 && all >= kFlatWholeHalf && half * mp.d % 256 == 0)) rows = half;
+    if (rows > kFlatElems / mp.d) rows = kFlatElems / mp.d;
     const int64_t spread = pb.nbags / (148 * 32) + 1;
     if ((int64_t)rows > spread) rows = (uint32_t)spread;
     if (rows < 1) rows = 1;

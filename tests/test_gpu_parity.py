@@ -370,6 +370,25 @@ def test_millions_of_one_hot_rows(d, Z, table_major):
                           delta64.astype(np.float32), "backward, integer gradient")
 
 
+# Rows of more than 128 elements in calls on both sides of the sizes at which the flat kernels change the rows per warp:
+# 2^24 elements (forward, runs of whole groups of 256), 24 and 64 times 2^20 (the forward on more than 16 MB); short last
+# blocks, bf16 arrays.
+@pytest.mark.parametrize("d,Z,M,batch,dtype", [
+    (256, 32, 5_000_011, 21_845, "f32"), (256, 32, 5_000_011, 21_846, "f32"), (200, 64, 5_000_011, 41_943, "f32"),
+    (200, 64, 5_000_011, 41_944, "f32"), (256, 100, 70_001, 87_381, "f32"), (256, 100, 70_001, 87_382, "f32"),
+    (512, 512, 8_388_609, 10_923, "bf16"), (200, 50, 8_388_608, 41_944, "bf16"), (200, 50, 8_388_609, 41_944, "bf16"),
+])
+def test_flat_rows_of_large_calls(d, Z, M, batch, dtype):
+    w = small(d=d, Z=Z, M=M, batch=batch, array_dtype=dtype, vocab_arg=(3, 1000, 40_000_000))
+    with Case(w) as c:
+        assert_bits_equal(c.forward().cpu().numpy(), c.oracle_forward(), "forward")
+        if dtype == "f32":
+            g_h, g_d = _grad(c, 33, integer=True)
+            delta64, _ = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+            assert np.abs(delta64).max() < 2**24  # small integers: exact in any order
+            assert_bits_equal(c.backward(g_d, "atomic").cpu().numpy(), delta64.astype(np.float32), "backward")
+
+
 # One-hot rows of 65 to 128 elements by the staged kernel: batches of whole groups of ids (4 fp32, 8 bf16) where they are
 # a wave of warps and fit the staging area, in small calls with a rest.
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
