@@ -144,16 +144,16 @@ struct PoolLane {
     float acc[EPL];  // forward: the sum; backward: the gradient row
 };
 
-// Ids g0 .. g0+n-1 of the batch, n <= U (PLAIN: n == U and no block wraps): all their loads first, then, id by
-// id, the adds.
-template <int MODE, int EPL, bool SIGN, int U, bool PLAIN>
+// Ids g0 .. g0+n-1 of the batch, n <= U (FULL: n == U): all their loads first, then, id by id, the adds.  WRAP 0: no block
+// wraps; 1, 2: some may, 2 in one instruction (which in the kernel for longer arrays costs the forward 9 %, by the registers).
+template <int MODE, int EPL, bool SIGN, int U, bool FULL, int WRAP>
 __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* bag_s, const uint64_t* gbase_s, PoolLane<EPL>& l,
                                            int64_t k0, uint32_t g0, uint32_t n, bool begins, uint32_t lane, uint64_t pol) {
     const MapParams& mp = a.mp;
     float v[U][EPL];
     uint32_t bag[U];
 #pragma unroll
-    for (int g = 0; g < U; ++g) bag[g] = PLAIN || (uint32_t)g < n ? bag_s[g0 + g] : 0u;
+    for (int g = 0; g < U; ++g) bag[g] = FULL || (uint32_t)g < n ? bag_s[g0 + g] : 0u;
     if (MODE == 2) {  // the gradient row of every id (ids of one bag read the same one)
 #pragma unroll
         for (int g = 0; g < U; ++g) {
@@ -161,7 +161,7 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
             const bool fresh = g == 0 ? begins : (bag[g - 1] & kPoolLast) != 0;  // (warp-uniform)
 #pragma unroll
             for (int u = 0; u < EPL; ++u)
-                v[g][u] = fresh && l.live[u] && (PLAIN || (uint32_t)g < n) && ROBE_CHK_GRAD(row + 32 * u, a) ? __ldcs(row + 32 * u) : 0.0f;
+                v[g][u] = fresh && l.live[u] && (FULL || (uint32_t)g < n) && ROBE_CHK_GRAD(row + 32 * u, a) ? __ldcs(row + 32 * u) : 0.0f;
         }
 #pragma unroll
         for (int g = 0; g < U; ++g) {
@@ -170,8 +170,9 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
             for (int u = 0; u < EPL; ++u) {
                 if (fresh) l.acc[u] = v[g][u] * a.scale;
                 uint32_t j = l.col[u][g0 + g] + l.off[u];
-                if (!PLAIN && j >= mp.m) j -= mp.m;
-                if ((PLAIN || (uint32_t)g < n) && l.live[u] && ROBE_CHK(j < mp.m, ROBE_DBG_ARRAY_SLOT))
+                if (WRAP == 1 && j >= mp.m) j -= mp.m;
+                if (WRAP == 2) j = __viaddmin_u32(j, 0u - mp.m, j);  // j - m unless that is below 0
+                if ((FULL || (uint32_t)g < n) && l.live[u] && ROBE_CHK(j < mp.m, ROBE_DBG_ARRAY_SLOT))
                     red_add(a.io + j, SIGN ? with_sign(gbase_s[g0 + g], l.gelem[u], (uint32_t)l.gelem[u] << 31, l.acc[u]) : l.acc[u], pol);
             }
         }
@@ -181,15 +182,16 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
 #pragma unroll
             for (int u = 0; u < EPL; ++u) {
                 v[g][u] = 0.0f;
-                if (l.live[u] && (PLAIN || (uint32_t)g < n)) {
+                if (l.live[u] && (FULL || (uint32_t)g < n)) {
                     uint32_t j = l.col[u][g0 + g] + l.off[u];  // < m + d <= 2^32
-                    if (!PLAIN && j >= mp.m) j -= mp.m;
+                    if (WRAP == 1 && j >= mp.m) j -= mp.m;
+                    if (WRAP == 2) j = __viaddmin_u32(j, 0u - mp.m, j);  // j - m unless that is below 0
                     if (ROBE_CHK(j < mp.m, ROBE_DBG_ARRAY_SLOT)) v[g][u] = gather_elem<MODE == 1 ? 1 : 0>(a.array, j);
                 }
             }
 #pragma unroll
         for (int g = 0; g < U; ++g) {
-            if (!PLAIN && (uint32_t)g >= n) break;
+            if (!FULL && (uint32_t)g >= n) break;
 #pragma unroll
             for (int u = 0; u < EPL; ++u)
                 l.acc[u] = l.acc[u] + (SIGN ? with_sign(gbase_s[g0 + g], l.gelem[u], (uint32_t)l.gelem[u] << 31, v[g][u]) : v[g][u]);
@@ -206,7 +208,9 @@ __device__ __forceinline__ void pool_group(const PoolArgs& a, const uint32_t* ba
 }
 
 // MODE 0: forward, fp32 array; 1: forward, bf16 array; 2: backward
-template <int MODE, int EPL, bool SIGN>
+// WRAPS: most batches of ids hold a block that wraps.  Then every full group takes the (one-instruction) wrap along; else
+// those of a batch that wraps do so together with the rest of a batch, which is slower for them.
+template <int MODE, int EPL, bool SIGN, bool WRAPS>
 __global__ void __launch_bounds__(256, SIGN ? kPoolCtasSign : kPoolCtas)
 pool_kernel(PoolArgs a) {
     __shared__ PoolSmem sm;
@@ -262,22 +266,31 @@ pool_kernel(PoolArgs a) {
             const bool wraps = pool_stage<SIGN>(sm, a, k0, at, bags, p0, cnt, w, lane);
             uint32_t g0 = 0;
             // (a batch that goes on with a bag reads its gradient row again)
-            for (; !wraps && g0 + U <= cnt; g0 += U)
-                pool_group<MODE, EPL, SIGN, U, true>(a, sm.bag[w], gbase_s, l, k0, g0, U,
-                                                     g0 == 0 || (sm.bag[w][g0 - 1] & kPoolLast) != 0, lane, pol);
+            for (; (WRAPS || !wraps) && g0 + U <= cnt; g0 += U)
+                pool_group<MODE, EPL, SIGN, U, true, WRAPS ? 2 : 0>(a, sm.bag[w], gbase_s, l, k0, g0, U,
+                                                                    g0 == 0 || (sm.bag[w][g0 - 1] & kPoolLast) != 0, lane, pol);
             for (; g0 < cnt; g0 += U)
-                pool_group<MODE, EPL, SIGN, U, false>(a, sm.bag[w], gbase_s, l, k0, g0, cnt - g0 < U ? cnt - g0 : U,
-                                                      g0 == 0 || (sm.bag[w][g0 - 1] & kPoolLast) != 0, lane, pol);
+                pool_group<MODE, EPL, SIGN, U, false, WRAPS ? 2 : 1>(a, sm.bag[w], gbase_s, l, k0, g0, cnt - g0 < U ? cnt - g0 : U,
+                                                                     g0 == 0 || (sm.bag[w][g0 - 1] & kPoolLast) != 0, lane, pol);
             __syncwarp();  // the staging area is rewritten by the next batch
         }
     }
 }
 
+template <int MODE, bool SIGN, bool WRAPS>
+void launch_pool_build(const PoolArgs& a, unsigned blocks, cudaStream_t st) {
+    if (a.mp.d <= 32) launch_next(pool_kernel<MODE, 1, SIGN, WRAPS>, blocks, 256, 0, st, a);
+    else if (a.mp.d <= 64) launch_next(pool_kernel<MODE, 2, SIGN, WRAPS>, blocks, 256, 0, st, a);
+    else launch_next(pool_kernel<MODE, 4, SIGN, WRAPS>, blocks, 256, 0, st, a);
+}
+
+// Arrays of up to 512 rows have a block that wraps in every other batch of a few dozen ids or more.  Measured (B200, us, one
+// build for all -> here): forward of 26 x 9000 bags of 2, d = 128 on 5000 slots 67.0 -> 48.7, d = 100 69.6 -> 51.9, signed bags of 6,
+// d = 100 on 20 K slots, both passes, 459 -> 437; 0.89 .. 0.97 on 150 .. 20 K slots, 1.00 on 100 K, on 1 M 1.01 .. 1.05.
 template <int MODE, bool SIGN>
 void launch_pool_epl(const PoolArgs& a, unsigned blocks, cudaStream_t st) {
-    if (a.mp.d <= 32) launch_next(pool_kernel<MODE, 1, SIGN>, blocks, 256, 0, st, a);
-    else if (a.mp.d <= 64) launch_next(pool_kernel<MODE, 2, SIGN>, blocks, 256, 0, st, a);
-    else launch_next(pool_kernel<MODE, 4, SIGN>, blocks, 256, 0, st, a);
+    if (a.mp.m <= 512ull * a.mp.d) launch_pool_build<MODE, SIGN, true>(a, blocks, st);
+    else launch_pool_build<MODE, SIGN, false>(a, blocks, st);
 }
 
 uint32_t pool_ids(const Problem& pb) { return staged_ids_per_batch(pb.mp, true, pb.sign != 0); }

@@ -450,6 +450,24 @@ def test_short_bags_of_many_tables(d, Z, M):
             assert_bits_equal(c.backward(g_d, "atomic").cpu().numpy(), delta64.astype(np.float32), "backward")
 
 
+# Arrays on both sides of the length (512 rows) from which full groups of ids test for blocks that wrap only in batches that
+# have one: runs with and without such blocks, full batches and rests of groups, one, two and four elements to a lane.
+@pytest.mark.parametrize("d,Z", [(16, 8), (60, 20), (100, 32), (128, 128)])
+@pytest.mark.parametrize("past", [0, 1])
+def test_short_bags_on_short_arrays(d, Z, past):
+    for dtype in ("f32", "bf16"):
+        w = small(d=d, Z=Z, M=512 * d + past, bag_rule=(2, 0, 9), batch=4001, array_dtype=dtype)
+        for sign in (False, True):
+            with Case(w, sign=sign) as c:
+                assert_bits_equal(c.forward().cpu().numpy(), c.oracle_forward(), "forward")
+                if dtype == "bf16":
+                    continue
+                g_h, g_d = _grad(c, 24, integer=True)
+                delta64, _ = c.oracle.backward_f64(g_h, c.indices_h, c.offsets_h, c.B)
+                assert np.abs(delta64).max() < 2**24  # small integers: exact in any order
+                assert_bits_equal(c.backward(g_d, "atomic").cpu().numpy(), delta64.astype(np.float32), "backward")
+
+
 # Forward runs spread evenly over a full wave of warps (5920 of them, unsigned): runs of 4 and 5 bags, the last warps,
 # and one bag more than five to a warp.
 @pytest.mark.parametrize("batch", [9472, 9866, 9867])
