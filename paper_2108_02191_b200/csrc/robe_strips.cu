@@ -276,7 +276,7 @@ strip_apply_kernel(StripArgs a) {
                 for (int q = 0; q < EPL; ++q) {
                     // (a lane past the block's end adds -0 to a slot that is no other lane's in this step)
                     const uint32_t s = slot[u] + 32 * q;
-                    if (BANKED || s < W) sum[s] = __fadd_rn(sum[s], x[u][q]);
+                    if (BANKED ? ROBE_CHK(s < G * W + 32, ROBE_DBG_SHARED) : s < W) sum[s] = __fadd_rn(sum[s], x[u][q]);
                 }
                 __syncwarp();
             }

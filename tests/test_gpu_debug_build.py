@@ -47,7 +47,8 @@ def test_shape_lists_run_clean_on_the_index_check_build():
         pytest.skip("already inside the child run")
     pick = ("forward_shapes or backward_shapes or window_apply or step_sharing or vector_kernel or "
             "lane_hashed or adam or adagrad or merged_rows or table_major or int32 or cfg1 or hot_id or bit_reproducible "
-            "or large_one_hot or millions_of or short_bags or repeated_blocks or strips or strip_rooms or long_walks or back_to_back")
+            "or large_one_hot or millions_of or short_bags or repeated_blocks or strips or strip_rooms or strip_banks or sort_tiles "
+            "or staged_rows or flat_rows or long_walks or back_to_back")
     r = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_parity.py", "tests/test_zz_no_alloc.py",
                         "-m", "gpu", "-x", "-q", "-k", pick + " or two_calls or fused_sgd"],
                        env=_debug_env(), cwd=ROOT, capture_output=True, text=True, timeout=3000)

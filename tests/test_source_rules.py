@@ -67,3 +67,15 @@ def test_every_gradient_read_is_checked_in_the_index_check_build(path):
     for n, line in enumerate(lines):
         if re.search(r"(__ldcs|__ldca|load_settled)\((rows? \+|grad \+|ge\)|a\.grad_out)", line):
             assert re.search("ROBE_CHK_GRAD|ROBE_DBG_GRAD_POS", " ".join(lines[max(0, n - 4):n + 1])), (n + 1, line)
+
+
+def test_index_check_run_picks_every_test_of_a_kernel_path():
+    # a test of the parity file runs on the index-check build too, unless it is one of those named here: workloads at full
+    # size (run against it by hand), and what launches no kernel of its own
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    pick = re.search(r"pick = \((.*?)\)\n", open(os.path.join(root, "tests", "test_gpu_debug_build.py")).read(), re.S).group(1)
+    words = re.sub(r'["\s]+', " ", pick).replace(" or ", "|").strip().split("|") + ["two_calls", "fused_sgd"]
+    tests = re.findall(r"^def (test_\w+)\(", open(os.path.join(root, "tests", "test_gpu_parity.py")).read(), re.M)
+    left = {t for t in tests if not any(w.strip() in t for w in words)}
+    assert {t for t in left if not re.search(r"full_size|full_batch|whole_array|reduced_batch|cfg5|cfg2|errors|refuse|validate|empty|share_one_array|"
+                                             r"bf16|huge_ids|max_array|many_tables_and_large", t)} == set()
