@@ -13,7 +13,8 @@
 //                      slot j is the one at the first sorted block of that key window, so it only
 //                      ever walks forward through the sorted list.  Slots [0, Z-1), which also
 //                      receive the wrapped tails of blocks near the end of the array, are handled
-//                      by a small second kernel (those terms come last: their keys are the largest).
+//                      by a small second kernel (those terms come last: their keys are the largest), with the
+//                      strips below by the first CTAs of the hot strips' kernel.
 //                      Walks over hundreds of blocks (an id repeated many times in the batch)
 //                      are finished by a third kernel that keeps a whole step of terms in flight.
 //                      Arrays that the call touches densely are served slot by slot instead

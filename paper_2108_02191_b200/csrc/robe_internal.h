@@ -107,8 +107,8 @@ size_t strips_workspace_bytes(const MapParams& mp);
 size_t strips_list_bytes(const MapParams& mp, uint64_t nb);
 // first sorted position of every strip; in st
 void launch_strips_prepare(const StripProblem& sp, cudaStream_t st);
-// all slots but [0, Z-1), mode as launch_backward_det's 0, 1, 2, 4.  Strips of often repeated ids are served
-// in hot_st (st itself, or a stream that has been made to wait for launch_strips_prepare).
+// all slots, mode as launch_backward_det's 0, 1, 2, 4.  Slots [0, Z-1) and strips of often repeated ids are served in
+// hot_st (st itself, or a stream that has been made to wait for launch_strips_prepare), the others in st.
 void launch_strips(const StripProblem& sp, int mode, cudaStream_t st, cudaStream_t hot_st);
 
 // mode 0: target[j] += delta; 1: target = attached array, target[j] = fma(-lr, delta, target[j]);
